@@ -31,7 +31,7 @@ __global__ void k_restrict_u(BatchDev, int);
 __global__ void k_zero_u(BatchDev);
 __global__ void k_init_state(BatchDev, int);
 __global__ void k_plan(BatchDev);
-__global__ void k_prolong(BatchDev);
+__global__ void k_final(BatchDev);
 void launch_grad(int bf16, int grid, cudaStream_t st, const BatchDev &b);
 void launch_trial(int bf16, int J, int grid, cudaStream_t st, const BatchDev &b);
 void launch_smooth(int grid, cudaStream_t st, const BatchDev &b);
@@ -149,7 +149,7 @@ struct reg_series {
     reg_params p{};
     int bf16 = 0;
     int nsm = 0;
-    int grid_P = 0, grid_G = 0, grid_T = 0;  // resident-block grids of the step kernels
+    int grid_G = 0, grid_T = 0;  // resident-block grids of the step kernels
     // strip rows of the gradient and trial tiles per level l (2^l + 1 nodes)
     int tile_hg[REG_TILE_LEVELS] = {0}, tile_ht[REG_TILE_LEVELS] = {0};
     std::vector<SeriesInfo> S;
@@ -160,7 +160,8 @@ struct reg_series {
     size_t cap_ws = 0;
     OpDesc *d_ops = nullptr;
     OpState *d_st = nullptr;
-    int *d_lists = nullptr;  // listP, listG, listT, prefP, prefG, prefT
+    int *d_lists = nullptr;  // listG, listT, prefG, prefT
+    int4 *d_plan = nullptr;  // per op: its work of the next step
     int *d_ctr = nullptr;
     double *d_partG = nullptr, *d_partT = nullptr;
     unsigned long long *d_work = nullptr;
@@ -275,12 +276,11 @@ BatchDev make_batch(reg_series *s)
     b.ops = s->d_ops;
     b.st = s->d_st;
     int c = s->cap_ops;
-    b.listP = s->d_lists;
-    b.listG = s->d_lists + c;
-    b.listT = s->d_lists + 2 * c;
-    b.prefP = s->d_lists + 3 * c;
-    b.prefG = s->d_lists + 4 * c + 1;
-    b.prefT = s->d_lists + 5 * c + 2;
+    b.listG = s->d_lists;
+    b.listT = s->d_lists + c;
+    b.prefG = s->d_lists + 2 * c;
+    b.prefT = s->d_lists + 3 * c + 1;
+    b.plan = s->d_plan;
     b.ctr = s->d_ctr;
     b.partG = s->d_partG;
     b.partT = s->d_partT;
@@ -289,6 +289,7 @@ BatchDev make_batch(reg_series *s)
     b.trace_len = s->d_trace_len;
     b.trace_cap = s->trace_cap;
     b.lambda = s->p.lambda;
+    b.lam6 = (float)(s->p.lambda / 6.0);
     b.sigma = s->p.armijo_sigma;
     b.tau_init = s->p.tau_init;
     b.tau_max = s->p.tau_max;
@@ -308,15 +309,14 @@ BatchDev make_batch(reg_series *s)
     return b;
 }
 
-// Work items per operator at a level of n nodes per side: the largest of the
-// prolongation block tiles and the gradient and trial strip tiles.
+// Work items per operator at a level of n nodes per side: the larger of the
+// gradient and trial strip tiles.
 int max_tiles(const reg_series *s, int n)
 {
     const int l = level_of(n);
-    int p = cdiv(n, REG_TX) * cdiv(n, REG_TY);
     int g = cdiv(n, REG_GW) * cdiv(n, s->tile_hg[l]);
     int t = cdiv(n - 1, REG_CW) * cdiv(n - 1, s->tile_ht[l]);
-    return std::max(p, std::max(g, t));
+    return std::max(g, t);
 }
 
 // The largest max_tiles over the levels of a series (from level index k0).
@@ -349,10 +349,12 @@ reg_status ensure_capacity(reg_series *s, int n_ops, size_t ws_total, int64_t it
         untrack(s, s->d_ops);
         untrack(s, s->d_st);
         untrack(s, s->d_lists);
+        untrack(s, s->d_plan);
         if (s->h_ops) cudaFreeHost(s->h_ops);
         RET(track(s, (void **)&s->d_ops, sizeof(OpDesc) * c));
         RET(track(s, (void **)&s->d_st, sizeof(OpState) * c));
-        RET(track(s, (void **)&s->d_lists, sizeof(int) * (6 * c + 3)));
+        RET(track(s, (void **)&s->d_lists, sizeof(int) * (4 * c + 2)));
+        RET(track(s, (void **)&s->d_plan, sizeof(int4) * c));
         if (s->p.smooth > 0.0) {
             untrack(s, s->d_partS);
             RET(track(s, (void **)&s->d_partS, sizeof(double) * 2 * (size_t)s->sm_cch * c));
@@ -381,7 +383,7 @@ reg_status ensure_capacity(reg_series *s, int n_ops, size_t ws_total, int64_t it
     return REG_OK;
 }
 
-// Capture GRAPH_STEPS steps [P G T C plan] into one executable graph.
+// Capture GRAPH_STEPS steps [G T C] into one executable graph.
 reg_status build_graph(reg_series *s)
 {
     if (s->gexec && s->graph_gen == s->buf_gen) return REG_OK;
@@ -397,12 +399,10 @@ reg_status build_graph(reg_series *s)
     cudaStream_t cs = s->cap_stream;
     CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < GRAPH_STEPS; k++) {
-        k_prolong<<<s->grid_P, REG_THREADS, 0, cs>>>(b);
         launch_grad(s->bf16, s->grid_G, cs, b);
         if (b.smooth) launch_smooth(s->grid_S, cs, b);
         launch_trial(s->bf16, s->p.trials_per_pass, s->grid_T, cs, b);
-        k_control<<<std::min(s->cap_ops, 2048), 256, 0, cs>>>(b);
-        k_plan<<<1, 1024, 0, cs>>>(b);
+        k_control<<<std::min(s->cap_ops, 2048), REG_CTL_THREADS, 0, cs>>>(b);
     }
     cudaError_t e = cudaStreamEndCapture(cs, &g);
     if (e != cudaSuccess) return fail(REG_ECUDA, "graph capture: %s", cudaGetErrorString(e));
@@ -417,11 +417,11 @@ void collect_profile(reg_series *s)
 {
     if (!((s->p.flags & REG_FLAG_PROFILE) && s->ev_ok)) return;
     for (int k = 0; k < GRAPH_STEPS; k++) {
-        cudaEvent_t seq[NFAM] = {s->ev[k][F_P], s->ev[k][F_G], s->ev[k][F_T], s->ev[k][F_C], s->ev[k][F_PLAN], s->ev_end[k]};
-        for (int f = 0; f < 5; f++) {
+        cudaEvent_t seq[4] = {s->ev[k][F_G], s->ev[k][F_T], s->ev[k][F_C], s->ev_end[k]};
+        for (int f = 0; f < 3; f++) {
             float ms = 0.f;
             cudaError_t e = cudaEventElapsedTime(&ms, seq[f], seq[f + 1]);
-            if (e == cudaSuccess) s->fam[f].ms += ms;
+            if (e == cudaSuccess) s->fam[F_G + f].ms += ms;
             else {
                 cudaGetLastError();
                 s->ev_ok = false;
@@ -540,9 +540,10 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
     CK(cudaGetLastError());
     RET(pre_iter());
     k_init_state<<<cdiv(n, 256), 256, 0, s->stream>>>(b, n);
-    k_plan<<<1, 1024, 0, s->stream>>>(b);
+    k_plan<<<1, REG_CTL_THREADS, 0, s->stream>>>(b);
     CK(cudaGetLastError());
-    s->fam[F_SETUP].launches += 4 + nl;
+    s->fam[F_SETUP].launches += 3 + nl;
+    s->fam[F_PLAN].launches++;
     const bool prof = (s->p.flags & REG_FLAG_PROFILE) && s->ev_ok;
     if (!prof) RET(build_graph(s));  // profiling launches the same kernels directly
     int max_steps = s->p.max_steps > 0 ? s->p.max_steps
@@ -552,17 +553,13 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
         if (prof) {
             // profiling: the same step kernels launched one by one between events
             for (int k = 0; k < GRAPH_STEPS; k++) {
-                cudaEventRecord(s->ev[k][F_P], s->stream);
-                k_prolong<<<s->grid_P, REG_THREADS, 0, s->stream>>>(b);
                 cudaEventRecord(s->ev[k][F_G], s->stream);
                 launch_grad(s->bf16, s->grid_G, s->stream, b);
                 if (b.smooth) launch_smooth(s->grid_S, s->stream, b);  // timed with the gradient family
                 cudaEventRecord(s->ev[k][F_T], s->stream);
                 launch_trial(s->bf16, s->p.trials_per_pass, s->grid_T, s->stream, b);
                 cudaEventRecord(s->ev[k][F_C], s->stream);
-                k_control<<<std::min(s->cap_ops, 2048), 256, 0, s->stream>>>(b);
-                cudaEventRecord(s->ev[k][F_PLAN], s->stream);
-                k_plan<<<1, 1024, 0, s->stream>>>(b);
+                k_control<<<std::min(s->cap_ops, 2048), REG_CTL_THREADS, 0, s->stream>>>(b);
                 cudaEventRecord(s->ev_end[k], s->stream);
             }
             CK(cudaGetLastError());
@@ -573,7 +570,7 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
         CK(cudaStreamSynchronize(s->stream));
         steps += GRAPH_STEPS;
         collect_profile(s);
-        for (int f = 0; f < 5; f++) s->fam[f].launches += GRAPH_STEPS;
+        for (int f : {F_G, F_T, F_C}) s->fam[f].launches += GRAPH_STEPS;
         if (s->h_ctr[8]) return fail(REG_EKERNEL, "operator state machine reported an internal error");
         if (s->h_ctr[7] == 0) break;
         if (steps > max_steps) return fail(REG_ETIMEOUT, "batch did not finish within %d steps", max_steps);
@@ -585,8 +582,19 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
         CK(cudaMallocHost((void **)&s->h_st, sizeof(OpState) * n));
         s->h_st_cap = n;
     }
+    // results into the destination slots
+    if (prof) cudaEventRecord(s->ev[0][F_P], s->stream);
+    k_final<<<dim3(cdiv(nLmax, 32), cdiv(nLmax, 8), n), blk, 0, s->stream>>>(b);
+    if (prof) cudaEventRecord(s->ev_end[0], s->stream);
+    CK(cudaGetLastError());
+    s->fam[F_P].launches++;
     CK(cudaMemcpyAsync(s->h_st, s->d_st, sizeof(OpState) * n, cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
+    if (prof) {
+        float ms = 0.f;
+        if (cudaEventElapsedTime(&ms, s->ev[0][F_P], s->ev_end[0]) == cudaSuccess) s->fam[F_P].ms += ms;
+        else cudaGetLastError();
+    }
     for (int i = 0; i < n; i++) {
         const OpState &st = s->h_st[i];
         s->tot_iters += st.iters_total;
@@ -921,7 +929,6 @@ void set_grids(reg_series *s)
         int occ = step_blocks_per_sm(which, s->p.trials_per_pass);
         return s->nsm * std::max(1, std::min(occ, 32));
     };
-    s->grid_P = grid_of(0);
     s->grid_G = grid_of(1);
     s->grid_T = grid_of(2);
 }
@@ -1422,12 +1429,12 @@ reg_status reg_prefix_scan(reg_series_t s, reg_scan_kind kind, int32_t chunks, r
                  "\"preprocessing_iters\": %lld, \"learned\": {\"ops\": %d, \"mean_correction_px\": %.5f, "
                  "\"max_correction_px\": %.5f, \"fallbacks\": %d}, \"scan_ops\": %d, \"scan_batches\": %d, "
                  "\"ops\": %lld, \"iters\": %lld, \"trials\": %lld, \"evals\": %lld, \"steps\": %lld, \"ms\": %.3f, "
-                 "\"grids\": [%d, %d, %d], "
+                 "\"grids\": [0, %d, %d], "
                  "\"status\": {\"converged\": %d, \"maxiter\": %d, \"stalled\": %d, \"nonfinite\": %d, \"zero_gradient\": %d}}",
                  (int)kind, pre.size(), pre_ms, (long long)pre_iters, n_judged,
                  n_judged ? corr_sum / n_judged : 0.0, corr_max, n_fallback, scan_ops, batches, (long long)(s->tot_ops - ops0),
                  (long long)(s->tot_iters - it0), (long long)(s->tot_trials - tr0), (long long)(s->tot_evals - ev0),
-                 (long long)(s->tot_steps - st0), ms, s->grid_P, s->grid_G, s->grid_T, counts[0], counts[1], counts[2],
+                 (long long)(s->tot_steps - st0), ms, s->grid_G, s->grid_T, counts[0], counts[1], counts[2],
                  counts[3], counts[4]);
     }
     return REG_OK;
@@ -1713,9 +1720,9 @@ static reg_status diag_setup(reg_series *s, int series, int fi, int fk, int leve
     st.tau = s->p.tau_init;
     CK(cudaMemcpyAsync(s->d_st, &st, sizeof(OpState), cudaMemcpyHostToDevice, s->stream));
     // START: plan, T, C
-    k_plan<<<1, 1024, 0, s->stream>>>(b);
+    k_plan<<<1, REG_CTL_THREADS, 0, s->stream>>>(b);
     launch_trial(s->bf16, s->p.trials_per_pass, s->grid_T, s->stream, b);
-    k_control<<<1, 256, 0, s->stream>>>(b);
+    k_control<<<1, REG_CTL_THREADS, 0, s->stream>>>(b);  // also plans the next step
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(s->stream));
     return REG_OK;
@@ -1755,7 +1762,6 @@ reg_status reg_eval_direction(reg_series_t s, int32_t series, int32_t frame_i, i
     RET(diag_setup(s, series, frame_i, frame_k, level, u_grid, k));
     BatchDev b = make_batch(s);
     // state is now PH_GRAD with src = 0, cur = 1 (no pending step)
-    k_plan<<<1, 1024, 0, s->stream>>>(b);
     launch_grad(s->bf16, s->grid_G, s->stream, b);
     CK(cudaGetLastError());
     OpState st;
@@ -1795,7 +1801,6 @@ reg_status reg_eval_trials(reg_series_t s, int32_t series, int32_t frame_i, int3
     BatchDev b = make_batch(s);
     // gradient pass at u (state PH_GRAD, no pending step), then one trial pass
     // over the given step sizes (still PH_GRAD, so that it also forms d^T K d)
-    k_plan<<<1, 1024, 0, s->stream>>>(b);
     launch_grad(s->bf16, s->grid_G, s->stream, b);
     CK(cudaGetLastError());
     OpState st;
@@ -1803,7 +1808,10 @@ reg_status reg_eval_trials(reg_series_t s, int32_t series, int32_t frame_i, int3
     CK(cudaStreamSynchronize(s->stream));
     if (st.phase != PH_GRAD) return fail(REG_ESTATE, "energy at the given displacement is not finite");
     st.ntr = n_tau;
-    for (int j = 0; j < REG_MAX_TRIALS; j++) st.trial_tau[j] = j < n_tau ? taus[j] : 0.0;
+    for (int j = 0; j < REG_MAX_TRIALS; j++) {
+        st.trial_tau[j] = j < n_tau ? taus[j] : 0.0;
+        st.f_tau[j] = (float)st.trial_tau[j];
+    }
     CK(cudaMemcpyAsync(s->d_st, &st, sizeof(OpState), cudaMemcpyHostToDevice, s->stream));
     launch_trial(s->bf16, s->p.trials_per_pass, s->grid_T, s->stream, b);
     CK(cudaGetLastError());
@@ -1890,11 +1898,13 @@ reg_status reg_get_kernel_stats(reg_series_t s, reg_kernel_stats *buf, int32_t b
             k.bytes = w[KW_G] * (16.0 + 8.0 + 4.0 + img + 16.0 + 8.0 + 4.0);
         } else if (f == F_T) {
             k.items = (int64_t)(w[KW_T] + w[KW_TSTART]);
-            // trial: reads u, d, M~That, M~R~, the template; start: u, M~R~, the template
-            k.bytes = w[KW_T] * (16.0 + 8.0 + 4.0 + 4.0 + img) + w[KW_TSTART] * (16.0 + 4.0 + img);
+            // trial: reads u, d, M~That, M~R~, the template; start: u (read, or written
+            // from a quarter of the coarser level's 24 B), M~R~, the template
+            k.bytes = w[KW_T] * (16.0 + 8.0 + 4.0 + 4.0 + img) + w[KW_TSTART] * (16.0 + 4.0 + img) +
+                      w[KW_PPROL] * 6.0;
         } else if (f == F_P) {
-            k.items = (int64_t)(w[KW_PPROL] + w[KW_PFIN]);
-            k.bytes = w[KW_PPROL] * (16.0 + 6.0) + w[KW_PFIN] * (16.0 + 8.0 + 8.0);
+            k.items = (int64_t)w[KW_PFIN];
+            k.bytes = w[KW_PFIN] * (16.0 + 8.0 + 8.0);  // the result into the slots
         }
     }
     return REG_OK;

@@ -387,8 +387,7 @@ __global__ void k_init_state(BatchDev b, int n_ops)
 // Work planning: compacted per-family op lists and tile prefix sums
 // ---------------------------------------------------------------------------
 
-// work items per operator: prolongation block tiles, gradient and trial strip tiles
-__device__ __forceinline__ int node_tiles(int n) { return ((n + REG_TX - 1) / REG_TX) * ((n + REG_TY - 1) / REG_TY); }
+// work items per operator: gradient and trial strip tiles
 __device__ __forceinline__ int grad_tiles(const LevelDesc &L)
 {
     return ((L.n + REG_GW - 1) / REG_GW) * ((L.n + L.hg - 1) / L.hg);
@@ -398,196 +397,161 @@ __device__ __forceinline__ int trial_tiles(const LevelDesc &L)
     return ((L.n - 1 + REG_CW - 1) / REG_CW) * ((L.n - 1 + L.ht - 1) / L.ht);
 }
 
-// Block-wide exclusive scan of one int per thread (blockDim.x == 1024).
-__device__ int block_excl_scan(int v, int *tmp, int *total)
+// An operator's work of the next step: {gradient tiles, trial tiles, active}.
+__device__ __forceinline__ int4 op_plan(const OpState &s, const OpDesc &op)
 {
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) tmp[w] = x;
-    __syncthreads();
-    if (w == 0) {
-        int t = tmp[lane];
-        int s = t;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        tmp[lane] = s - t;
-        if (lane == 31) tmp[32] = s;
-    }
-    __syncthreads();
-    int res = x - v + tmp[w];
-    *total = tmp[32];
-    __syncthreads();
-    return res;
+    if (s.phase == PH_DONE) return make_int4(0, 0, 0, 0);
+    const LevelDesc &L = op.lv[s.lvl];
+    return make_int4(s.phase == PH_GRAD ? grad_tiles(L) : 0, trial_tiles(L), 1, 0);
 }
 
-__global__ void __launch_bounds__(1024) k_plan(BatchDev b)
+// The lists and tile prefixes of the next step from the operators' plan entries,
+// by one block of REG_CTL_THREADS threads: one scan of {entries, gradient tiles,
+// trial tiles} per REG_CTL_THREADS operators.  (An operator with gradient tiles
+// always has trial tiles.)
+__device__ void plan_lists(const BatchDev &b)
 {
-    __shared__ int tmp[33];
-    int n_ops = b.ctr[0];
-    int offE[3] = {0, 0, 0}, offI[3] = {0, 0, 0};
-    int active = 0;
-    for (int base = 0; base < n_ops; base += 1024) {
-        int o = base + threadIdx.x;
-        int inP = 0, inG = 0, inT = 0, tP = 0, tG = 0, tT = 0;
-        if (o < n_ops) {
-            const OpState &s = b.st[o];
-            const OpDesc &op = b.ops[o];
-            const LevelDesc &L = op.lv[s.lvl];
-            if (s.phase != PH_DONE) active++;
-            if (s.phase == PH_PROLONG || s.phase == PH_FINAL) { inP = 1; tP = node_tiles(L.n); }
-            if (s.phase == PH_GRAD) { inG = 1; tG = grad_tiles(L); }
-            if (s.phase == PH_START || s.phase == PH_GRAD || s.phase == PH_TRIAL || s.phase == PH_PROLONG) {
-                inT = 1; tT = trial_tiles(L);
-            }
+    __shared__ int4 wsum[REG_CTL_THREADS / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int n_ops = b.ctr[0];
+    int offG = 0, offT = 0, itG = 0, itT = 0;  // entries and tiles of the operators before this chunk
+    for (int base = 0; base < n_ops; base += REG_CTL_THREADS) {
+        const int o = base + threadIdx.x;
+        // other blocks wrote the entries in this launch: past L1
+        const int4 p = o < n_ops ? __ldcg(b.plan + o) : make_int4(0, 0, 0, 0);
+        // entries of both lists in one word (at most REG_CTL_THREADS each)
+        const int inc = (p.x > 0 ? 1 : 0) | (p.y > 0 ? 1 << 16 : 0);
+        int e = inc, g = p.x, t = p.y;
+#pragma unroll
+        for (int k = 1; k < 32; k <<= 1) {
+            const int ye = __shfl_up_sync(0xffffffffu, e, k), yg = __shfl_up_sync(0xffffffffu, g, k),
+                      yt = __shfl_up_sync(0xffffffffu, t, k);
+            if (lane >= k) { e += ye; g += yg; t += yt; }
         }
-        int tot;
-        int eP = block_excl_scan(inP, tmp, &tot); int nP = tot;
-        int eG = block_excl_scan(inG, tmp, &tot); int nG = tot;
-        int eT = block_excl_scan(inT, tmp, &tot); int nT = tot;
-        int iP = block_excl_scan(tP, tmp, &tot); int sP = tot;
-        int iG = block_excl_scan(tG, tmp, &tot); int sG = tot;
-        int iT = block_excl_scan(tT, tmp, &tot); int sT = tot;
+        if (lane == 31) wsum[wid] = make_int4(e, g, t, 0);
+        __syncthreads();
+        int4 before = make_int4(0, 0, 0, 0), all = before;
+#pragma unroll
+        for (int w = 0; w < REG_CTL_THREADS / 32; w++) {
+            const int4 x = wsum[w];
+            if (w < wid) { before.x += x.x; before.y += x.y; before.z += x.z; }
+            all.x += x.x; all.y += x.y; all.z += x.z;
+        }
         if (o < n_ops) {
+            const int ex = e - inc + before.x;
+            const int eG = offG + (ex & 0xffff), eT = offT + (ex >> 16);
+            const int iG = itG + g - p.x + before.y, iT = itT + t - p.y + before.z;
             OpState &s = b.st[o];
-            if (inP) { b.listP[offE[0] + eP] = o; b.prefP[offE[0] + eP] = offI[0] + iP; }
-            if (inG) { b.listG[offE[1] + eG] = o; b.prefG[offE[1] + eG] = offI[1] + iG; s.g_entry = offE[1] + eG; }
-            if (inT) { b.listT[offE[2] + eT] = o; b.prefT[offE[2] + eT] = offI[2] + iT; }
-            s.g_begin = offI[1] + iG; s.g_end = s.g_begin + tG;
-            s.t_begin = offI[2] + iT; s.t_end = s.t_begin + tT;
+            if (p.x > 0) {
+                b.listG[eG] = o;
+                b.prefG[eG] = iG;
+                s.g_entry = eG;
+            }
+            if (p.y > 0) {
+                b.listT[eT] = o;
+                b.prefT[eT] = iT;
+            }
+            s.g_begin = iG;
+            s.g_end = iG + p.x;
+            s.t_begin = iT;
+            s.t_end = iT + p.y;
         }
-        offE[0] += nP; offE[1] += nG; offE[2] += nT;
-        offI[0] += sP; offI[1] += sG; offI[2] += sT;
+        offG += all.x & 0xffff;
+        offT += all.x >> 16;
+        itG += all.y;
+        itT += all.z;
+        __syncthreads();
     }
-    // active ops
-    int tot;
-    block_excl_scan(active, tmp, &tot);
     if (threadIdx.x == 0) {
-        b.prefP[offE[0]] = offI[0];
-        b.prefG[offE[1]] = offI[1];
-        b.prefT[offE[2]] = offI[2];
-        b.ctr[1] = offE[0]; b.ctr[2] = offE[1]; b.ctr[3] = offE[2];
-        b.ctr[4] = offI[0]; b.ctr[5] = offI[1]; b.ctr[6] = offI[2];
-        b.ctr[7] = tot;
+        b.prefG[offG] = itG;
+        b.prefT[offT] = itT;
+        b.ctr[2] = offG;
+        b.ctr[3] = offT;
+        b.ctr[5] = itG;
+        b.ctr[6] = itT;
+        b.ctr[7] = offT;  // every operator that is not done has trial tiles
     }
+}
+
+// Plan of a batch's first step (the control kernel plans the others): the
+// entries from the operators' states, then the lists.
+__global__ void __launch_bounds__(REG_CTL_THREADS) k_plan(BatchDev b)
+{
+    const int n_ops = b.ctr[0];
+    for (int o = threadIdx.x; o < n_ops; o += REG_CTL_THREADS) b.plan[o] = op_plan(b.st[o], b.ops[o]);
+    __threadfence_block();
+    __syncthreads();
+    plan_lists(b);
 }
 
 // ---------------------------------------------------------------------------
-// Work distribution of the step kernels: a fixed grid, each block takes one
-// contiguous range of the step's work items (tiles of 32 x 32 nodes or
-// cells), so that it locates its first op once and then walks forward.
+// Prolongation to the next level of the multilevel flow, and the result.
 // ---------------------------------------------------------------------------
 namespace {
 
-struct ItemWalker {
-    const int *pref;
-    int e, e_end;
-    __device__ ItemWalker(const int *p, int nent, int first) : pref(p)
-    {
-        e = find_entry(p, nent, first);
-        e_end = __ldg(p + e + 1);
-    }
-    // entry (index into the compacted op list) of a work item >= the previous one
-    __device__ int entry(int item)
-    {
-        while (item >= e_end) {
-            e++;
-            e_end = __ldg(pref + e + 1);
-        }
-        return e;
-    }
-};
-
-__device__ __forceinline__ void block_range(int items, int &b0, int &b1)
+// u + tau d of the coarser level at node (r, c) of the next one: 2 x bilinear
+// prolongation (coarse grid unit = 2 fine units); the weights 2, 1, 1/2 are
+// exact, the sum is compensated.
+__device__ __forceinline__ float4 prolong_node(const NodeRec *V, int cpitch, float tau, int r, int c)
 {
-    int per = (items + gridDim.x - 1) / gridDim.x;
-    b0 = blockIdx.x * per;
-    b1 = min(items, b0 + per);
+    const int I = r >> 1, J = c >> 1, oi = r & 1, oj = c & 1;
+    const float w2 = (oi ? 0.5f : 1.f) * (oj ? 0.5f : 1.f) * 2.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int a = 0; a <= 1; a++)
+#pragma unroll
+        for (int bb = 0; bb <= 1; bb++) {
+            if ((a && !oi) || (bb && !oj)) continue;
+            const int64_t idx = (int64_t)(I + a) * cpitch + (J + bb);
+            float4 u = V[idx].u;
+            if (tau != 0.f) {
+                float2 d = V[idx].d;
+                u = df_add2(u, tau * d.x, tau * d.y);
+            }
+            df_add(acc.x, acc.z, w2 * u.x);
+            df_add(acc.x, acc.z, w2 * u.z);
+            df_add(acc.y, acc.w, w2 * u.y);
+            df_add(acc.y, acc.w, w2 * u.w);
+        }
+    return acc;
 }
 
 }  // namespace
 
-// ---------------------------------------------------------------------------
-// P: apply the pending step and prolongate to the next level (or write the
-// finest-level result into the destination slot).  Tile: 32 x 32 fine nodes.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(REG_THREADS, 4) k_prolong(BatchDev b)
+// The finest level's u with its pending step into the destination slots, once
+// all operators of the batch are done (their workspaces are their own, so the
+// records wait there).  grid (x tiles, y tiles, ops), block (32, 8).
+__global__ void __launch_bounds__(256) k_final(BatchDev b)
 {
-    int nent = b.ctr[1], items = b.ctr[4];
-    int b0, b1;
-    block_range(items, b0, b1);
-    if (b0 >= b1) return;
-    ItemWalker wk(b.prefP, nent, b0);
-    const int lx = threadIdx.x % REG_TX, ly = threadIdx.x / REG_TX;
-    for (int item = b0; item < b1; item++) {
-        int e = wk.entry(item);
-        int o = b.listP[e];
-        int t = item - b.prefP[e];
-        const OpState &s = b.st[o];
-        const OpDesc &op = b.ops[o];
-        const LevelDesc &Lv = op.lv[s.lvl];
-        const int n = Lv.n, tx = (n + REG_TX - 1) / REG_TX;
-        const int r0 = (t / tx) * REG_TY, c = (t % tx) * REG_TX + lx;
-        const float tau = (float)s.tau_acc;
-        const bool fin = (s.phase == PH_FINAL);
-        float corr = 0.f;  // judged ops: |final - learned start| over this thread's nodes
-#pragma unroll
-        for (int k = 0; k < REG_RPT; k++) {
-            const int r = r0 + ly + k * REG_ROWSTEP;
-            if (r >= n || c >= n) continue;
-            if (fin) {
-                const NodeRec &v = Lv.V[s.src][(int64_t)r * Lv.pitch + c];
-                float4 u = v.u;
-                if (tau != 0.f) {
-                    float2 d = v.d;
-                    u = df_add2(u, tau * d.x, tau * d.y);
-                }
-                const float2 res = make_float2(u.x + u.z, u.y + u.w);
-                float2 &dst = op.out[(int64_t)r * op.slot_pitch + c];
-                if (op.judge) {
-                    const float2 g0 = dst;
-                    corr += fabsf(res.x - g0.x) + fabsf(res.y - g0.y);
-                }
-                dst = res;
-            } else {
-                const LevelDesc &Cv = op.lv[s.lvl - 1];
-                const NodeRec *V = Cv.V[s.src];
-                int I = r >> 1, J = c >> 1, oi = r & 1, oj = c & 1;
-                // 2 x bilinear prolongation (coarse grid unit = 2 fine units); the
-                // weights 2, 1, 1/2 are exact, the sum is compensated
-                float w2 = (oi ? 0.5f : 1.f) * (oj ? 0.5f : 1.f) * 2.f;
-                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int a = 0; a <= 1; a++)
-#pragma unroll
-                    for (int bb = 0; bb <= 1; bb++) {
-                        if ((a && !oi) || (bb && !oj)) continue;
-                        int64_t idx = (int64_t)(I + a) * Cv.pitch + (J + bb);
-                        float4 u = V[idx].u;
-                        if (tau != 0.f) {
-                            float2 d = V[idx].d;
-                            u = df_add2(u, tau * d.x, tau * d.y);
-                        }
-                        df_add(acc.x, acc.z, w2 * u.x);
-                        df_add(acc.x, acc.z, w2 * u.z);
-                        df_add(acc.y, acc.w, w2 * u.y);
-                        df_add(acc.y, acc.w, w2 * u.w);
-                    }
-                Lv.V[0][(int64_t)r * Lv.pitch + c].u = acc;
-            }
+    const OpDesc &op = b.ops[blockIdx.z];
+    const LevelDesc &Lv = op.lv[op.nl - 1];
+    const int n = Lv.n;
+    if ((int)(blockIdx.x * 32) >= n || (int)(blockIdx.y * 8) >= n) return;  // block-uniform
+    const int c = blockIdx.x * 32 + threadIdx.x, r = blockIdx.y * 8 + threadIdx.y;
+    const OpState &s = b.st[blockIdx.z];
+    float corr = 0.f;  // judged ops: |final - learned start|
+    if (r < n && c < n) {
+        const float tau = s.f_tau_acc;
+        const NodeRec &v = Lv.V[s.src][(int64_t)r * Lv.pitch + c];
+        float4 u = v.u;
+        if (tau != 0.f) {
+            float2 d = v.d;
+            u = df_add2(u, tau * d.x, tau * d.y);
         }
-        if (fin && op.judge) {  // block-uniform: the whole block works on this item
-            const float w = warp_sum(corr);
-            if ((threadIdx.x & 31) == 0) atomicAdd(&b.st[o].corr, (double)w);
+        const float2 res = make_float2(u.x + u.z, u.y + u.w);
+        float2 &dst = op.out[(int64_t)r * op.slot_pitch + c];
+        if (op.judge) {
+            const float2 g0 = dst;
+            corr = fabsf(res.x - g0.x) + fabsf(res.y - g0.y);
         }
+        dst = res;
     }
+    if (op.judge) {  // block-uniform
+        const float w = warp_sum(corr);
+        if (threadIdx.x == 0) atomicAdd(&b.st[blockIdx.z].corr, (double)w);
+    }
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0)
+        atomicAdd(&b.work[KW_PFIN], (unsigned long long)n * n);
 }
 
 // ---------------------------------------------------------------------------
@@ -628,15 +592,13 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, 8) k_grad(BatchDev b)
         const bool cEdge = (c == 0 || c == n - 1);
         const float cx6 = cEdge ? 2.f : 4.f;  // 6 M1 on the diagonal
         const float wx = cEdge ? 0.5f : 1.f, iwx = cEdge ? 2.f : 1.f;
-        const float tau = (float)s.tau_acc;
+        const float tau = s.f_tau_acc;
         const NodeRec *Vs = Lv.V[s.src];
         NodeRec *Vc = Lv.V[s.cur];
         // the stencils run on the integer weights 6 M1 and 6 K1 (36 M~, 6 K); their
-        // scale goes into these per-tile coefficients, each rounded once
-        const float isig = (float)(1.0 / s.sigT);
-        const float c36 = (float)(s.ncc / (s.sigT * s.sigT) / 36.0);  // NCC / sigma^2 / 36
-        const float cT = (float)(s.ncc / (s.sigT * s.sigT) * s.Tbar);  // NCC / sigma^2 T_bar
-        const float lam6 = (float)(b.lambda / 6.0);
+        // scale is in these per-operator coefficients, each rounded once by the
+        // control kernel: 1 / sigma, NCC / sigma^2 / 36, NCC / sigma^2 T_bar
+        const float isig = s.f_isig, c36 = s.f_c36, cT = s.f_cT, lam6 = b.lam6;
         const float ih2 = 1.f / Lv.h2;  // exact: h^2 is a power of two
         // rows r-2 (suffix A) and r-1 (suffix M) of this column; row r is read
         // in the iteration and row r-1 is completed by it
@@ -1111,12 +1073,20 @@ __device__ __forceinline__ bool patch_delta(const Patch &P, int n, float ex, flo
 
 // Level-start sums of one strip tile at u, accumulated in double: they seed
 // every search of the level (the trial passes only add changes to them), and
-// the pass runs once per level.
+// the pass runs once per level.  After a level change (PH_PROLONG) the tile forms
+// u itself from the coarser level's records and stores the nodes it owns: the
+// prolongation is needed here only, once per level and operator, and as a kernel
+// of its own it cost every step an (almost always empty) launch of 3 us.
 template <bool BF16>
-__device__ __forceinline__ void start_tile(const OpState &s, const LevelDesc &Lv, const StripGeom &g, double *v)
+__device__ __forceinline__ void start_tile(const OpState &s, const OpDesc &op, const LevelDesc &Lv, const StripGeom &g,
+                                           double *v)
 {
     const unsigned FULL = 0xffffffffu;
-    const NodeRec *V = Lv.V[s.cur];
+    const bool prol = s.phase == PH_PROLONG;
+    NodeRec *V = Lv.V[s.cur];
+    const LevelDesc &Cv = op.lv[prol ? s.lvl - 1 : s.lvl];
+    const NodeRec *VC = Cv.V[s.src];
+    const float ptau = s.f_tau_acc;
     double s1 = 0.0, s3 = 0.0, q2 = 0.0, quu = 0.0;
     float tP = 0.f, tPR = 0.f, pux = 0.f, puy = 0.f;
     float4 uP = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1125,7 +1095,12 @@ __device__ __forceinline__ void start_tile(const OpState &s, const LevelDesc &Lv
         float t0 = 0.f, mr = 0.f;
         if (g.colIn) {
             const int64_t idx = (int64_t)r * g.pitch + g.c;
-            u = V[idx].u;
+            if (prol) {
+                u = prolong_node(VC, Cv.pitch, ptau, r, g.c);
+                if (g.nodeCol && (r < g.r0 + g.h || r == g.n - 1)) V[idx].u = u;
+            } else {
+                u = V[idx].u;
+            }
             mr = Lv.MR[idx];
             t0 = sample_df<BF16, false>(Lv.T, g.n, g.pitch, g.c, r, u, nullptr, nullptr);
         }
@@ -1313,7 +1288,7 @@ __device__ __forceinline__ void steps_tile(const OpState &s, const LevelDesc &Lv
     float tmax = 0.f;
 #pragma unroll
     for (int j = 0; j < JM; j++) {
-        tau[j] = (j < J) ? (float)s.trial_tau[j] : 0.f;
+        tau[j] = (j < J) ? s.f_tau[j] : 0.f;
         tmax = fmaxf(tmax, tau[j]);
 #pragma unroll
         for (int k = 0; k < 3; k++) sh.sn[k][j][lane] = 0.f;
@@ -1498,13 +1473,14 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, 4) k_trial(BatchDev b)
         const int e = find_entry(b.prefT, nent, item);
         const int o = b.listT[e];
         const OpState &s = b.st[o];
-        const LevelDesc &Lv = b.ops[o].lv[s.lvl];
+        const OpDesc &op = b.ops[o];
+        const LevelDesc &Lv = op.lv[s.lvl];
         const StripGeom g = strip_geom(Lv, item - b.prefT[e], lane);
         const bool start = (s.phase == PH_START || s.phase == PH_PROLONG);
         if (start) {
             // sums in double, reduced in double: [0..2] and the Dirichlet form of u
             double v[4];
-            start_tile<BF16>(s, Lv, g, v);
+            start_tile<BF16>(s, op, Lv, g, v);
             double mine = 0.0;
 #pragma unroll
             for (int k = 0; k < 4; k++) {
@@ -1525,16 +1501,31 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, 4) k_trial(BatchDev b)
 }
 
 // ---------------------------------------------------------------------------
-// C: per-operator FP64 reduction and the Armijo state machine
+// C: per-operator FP64 reduction, the Armijo state machine, and the plan of the
+// next step
 // ---------------------------------------------------------------------------
 namespace {
 
-// NCC from the FE sums S1 = int That, S2 = int That^2, S3 = int That R~ (R~
-// normalised: mean 0, FE sigma 1): NCC = S3 / sqrt(S2 - S1^2).
-__device__ __forceinline__ double ncc_of(double S1, double S2, double S3)
+// An energy's scalars from the FE sums S1 = int That, S2 = int That^2, S3 = int
+// That R~ (R~ normalised: mean 0, FE sigma 1): sigma = sqrt(S2 - S1^2), NCC =
+// S3 / sigma, and the gradient pass's coefficients there.
+struct EvalAt {
+    double S1, S2, S3, ncc, sig, dE;
+    float isig, c36, cT;
+};
+
+__device__ __forceinline__ void eval_at(EvalAt &v, double S1, double S2, double S3)
 {
-    double var = S2 - S1 * S1;
-    return S3 / (var > 0.0 ? sqrt(var) : 0.0);
+    const double var = S2 - S1 * S1;
+    v.S1 = S1;
+    v.S2 = S2;
+    v.S3 = S3;
+    v.sig = var > 0.0 ? sqrt(var) : 0.0;
+    v.ncc = S3 / v.sig;
+    v.isig = (float)(1.0 / v.sig);
+    const double q = v.ncc / (v.sig * v.sig);
+    v.c36 = (float)(q / 36.0);
+    v.cT = (float)(q * S1);
 }
 
 __device__ void level_end(OpState &s, const OpDesc &op, int status, double pending)
@@ -1542,13 +1533,14 @@ __device__ void level_end(OpState &s, const OpDesc &op, int status, double pendi
     if (status == OPST_NONFINITE) s.nonfinite_seen = 1;
     s.status = status;
     s.tau_acc = pending;
+    s.f_tau_acc = (float)pending;
     s.src = s.cur;
     if (s.lvl < op.nl - 1) {
         s.phase = PH_PROLONG;
         s.lvl += 1;
         s.cur = 0;
     } else {
-        s.phase = PH_FINAL;
+        s.phase = PH_DONE;
     }
 }
 
@@ -1563,11 +1555,17 @@ __device__ __forceinline__ int lock_count(const OpState &s, const OpDesc &op)
     return op.lock_off[s.lvl + 1] - op.lock_off[s.lvl];
 }
 
+__device__ __forceinline__ void set_trial(OpState &s, int k, double t)
+{
+    s.trial_tau[k] = t;
+    s.f_tau[k] = (float)t;
+}
+
 __device__ void set_init_trials(OpState &s, const BatchDev &b, const OpDesc &op)
 {
     if (op.lock_tau) {
         // replay: the one step size the reference sequence accepted here
-        s.trial_tau[0] = lock_step(s, op);
+        set_trial(s, 0, lock_step(s, op));
         s.ntr = 1;
         s.search = SEARCH_INIT;
         return;
@@ -1576,11 +1574,11 @@ __device__ void set_init_trials(OpState &s, const BatchDev &b, const OpDesc &op)
     // pass covers the most likely continuations of both branches.
     int J = b.J;
     int k = 0;
-    s.trial_tau[k++] = s.tau;
     double up = s.tau, dn = s.tau;
+    set_trial(s, k++, up);
     while (k < J) {
-        if (2.0 * up <= b.tau_max) { up *= 2.0; s.trial_tau[k++] = up; }
-        if (k < J && 0.5 * dn >= b.tau_min) { dn *= 0.5; s.trial_tau[k++] = dn; }
+        if (2.0 * up <= b.tau_max) { up *= 2.0; set_trial(s, k++, up); }
+        if (k < J && 0.5 * dn >= b.tau_min) { dn *= 0.5; set_trial(s, k++, dn); }
         if (2.0 * up > b.tau_max && 0.5 * dn < b.tau_min) break;
     }
     s.ntr = k;
@@ -1591,125 +1589,43 @@ __device__ void schedule_grad(OpState &s, const BatchDev &b, const OpDesc &op, d
 {
     s.phase = PH_GRAD;
     s.tau_acc = pending;
+    s.f_tau_acc = (float)pending;
     s.src = s.cur;
     s.cur = 1 - s.cur;
     set_init_trials(s, b, op);
 }
 
-}  // namespace
-
-__device__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int o, int ph, const double *S,
-                           double slope, double qud);
-
-__global__ void __launch_bounds__(256) k_control(BatchDev b)
+// The scalars at the new u: of a level start, or of the accepted trial.
+__device__ __forceinline__ void take_eval(OpState &s, const EvalAt &v)
 {
-    __shared__ double red[8][2];
-    __shared__ double redT[9][PT_STRIDE];
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int n_ops = b.ctr[0];
-    // grid-stride over ops: one block per op, the block reduces the op's tile
-    // partials, thread 0 runs the op's Armijo state machine
-    for (int o = blockIdx.x; o < n_ops; o += gridDim.x) {
-    OpState &s = b.st[o];
-    const OpDesc &op = b.ops[o];
-    int ph = s.phase;
-    if (ph == PH_DONE) continue;
-    if (threadIdx.x == 0) {
-        // algorithmic work of this step (nodes of the level each kernel swept)
-        unsigned long long nn = (unsigned long long)op.lv[s.lvl].n * op.lv[s.lvl].n;
-        if (ph == PH_FINAL) atomicAdd(&b.work[KW_PFIN], nn);
-        if (ph == PH_PROLONG) { atomicAdd(&b.work[KW_PPROL], nn); atomicAdd(&b.work[KW_TSTART], nn); }
-        if (ph == PH_START) atomicAdd(&b.work[KW_TSTART], nn);
-        if (ph == PH_GRAD) atomicAdd(&b.work[KW_G], nn);
-        if (ph == PH_GRAD || ph == PH_TRIAL) {
-            atomicAdd(&b.work[KW_T], nn);
-            atomicAdd(&b.work[KW_TSAMPLES], nn * (unsigned long long)s.ntr);
-        }
-    }
-    if (ph == PH_FINAL) {
-        __syncthreads();
-        if (threadIdx.x == 0) s.phase = PH_DONE;
-        __syncthreads();
-        continue;
-    }
-    // reduce the T partials (and G slope partials) of this op over the block:
-    // thread t < 9 PT_STRIDE sums entry t % PT_STRIDE of every ninth record
-    // from t / PT_STRIDE on, so that a warp's loads are consecutive doubles;
-    // thread 0 then adds the nine partial sums of each entry in order
-    // (deterministic)
-    const int tb = s.t_begin, te = s.t_end;
-    if (threadIdx.x < 9 * PT_STRIDE) {
-        const int kk = threadIdx.x % PT_STRIDE, g = threadIdx.x / PT_STRIDE;
-        double acc = 0.0;
-        for (int it = tb + g; it < te; it += 9) acc += b.partT[(int64_t)it * PT_STRIDE + kk];
-        redT[g][kk] = acc;
-    }
-    double slope = 0.0, qud = 0.0;
-    if (ph == PH_GRAD) {
-        for (int it = s.g_begin + threadIdx.x; it < s.g_end; it += blockDim.x) {
-            slope += b.partG[(int64_t)it * PG_STRIDE];
-            qud += b.partG[(int64_t)it * PG_STRIDE + 1];
-        }
-    }
-    slope = warp_sum_d(slope);
-    qud = warp_sum_d(qud);
-    if (lane == 0) {
-        red[wid][0] = slope;
-        red[wid][1] = qud;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double S[PT_STRIDE];
-        for (int k = 0; k < PT_STRIDE; k++) {
-            double v = 0.0;
-            for (int g = 0; g < 9; g++) v += redT[g][k];
-            S[k] = v;
-        }
-        slope = 0.0;
-        qud = 0.0;
-        for (int w = 0; w < 8; w++) {
-            slope += red[w][0];
-            qud += red[w][1];
-        }
-        control_op(b, s, op, o, ph, S, slope, qud);
-    }
-    __syncthreads();
+    s.S1 = v.S1; s.S2 = v.S2; s.S3 = v.S3;
+    s.Tbar = v.S1;
+    s.sigT = v.sig;
+    s.ncc = v.ncc;
+    s.f_isig = v.isig; s.f_c36 = v.c36; s.f_cT = v.cT;
+}
+
+__device__ __forceinline__ void trace_trial(const BatchDev &b, const OpState &s, int o, int n, double want, double dE,
+                                            bool acc)
+{
+    if (!b.trace) return;
+    unsigned long long k = atomicAdd(b.trace_len, 1ull);
+    if ((long long)k < b.trace_cap) {
+        double *rec = b.trace + 7 * k;
+        rec[0] = o; rec[1] = n; rec[2] = s.iter - 1; rec[3] = want;
+        rec[4] = dE; rec[5] = b.sigma * want * s.slope; rec[6] = acc;
     }
 }
 
-// The Armijo state machine of one operator after a step (thread 0 of its block).
-__device__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int o, int ph, const double *S,
-                           double slope, double qud)
+// The Armijo state machine of one operator after a step (one thread; s in shared
+// memory).  ev: the evaluated trials' scalars, or ev[0] those of a level start.
+__device__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int o, int n, double h2, const EvalAt *ev,
+                           double quu, double slope)
 {
-    const LevelDesc &Lv = op.lv[s.lvl];
-    const double h2 = Lv.h2d;
-    if (ph == PH_GRAD && b.smooth) {
-        // the smoothed direction's slope and u^T K d (smoother partials, fixed order)
-        double sl = 0.0, qd = 0.0;
-        const int nch = (Lv.n + REG_GW - 1) / REG_GW;
-        for (int ch = 0; ch < nch; ch++) {
-            sl += b.partS[((int64_t)s.g_entry * b.cch + ch) * 2];
-            qd += b.partS[((int64_t)s.g_entry * b.cch + ch) * 2 + 1];
-        }
-        slope = -h2 * h2 * sl;
-        qud = qd;
-    }
-    if (ph == PH_GRAD) {
-        // the Dirichlet forms of the new search: u^T K d from the gradient pass
-        // (or the smoother), d^T K d from its first trial pass
-        s.Qud = qud;
-        s.Qdd = S[3 * REG_MAX_TRIALS + 2];
-    }
-    const double Qud = s.Qud, Qdd = s.Qdd;
+    const int ph = s.phase;
     if (ph == PH_START || ph == PH_PROLONG) {
-        s.S1 = h2 * S[0];
-        s.S2 = h2 * S[1];
-        s.S3 = h2 * S[2];
-        s.Tbar = s.S1;
-        double var = s.S2 - s.S1 * s.S1;
-        s.sigT = var > 0.0 ? sqrt(var) : 0.0;
-        s.ncc = ncc_of(s.S1, s.S2, s.S3);
-        s.E = -s.ncc + 0.5 * b.lambda * h2 * S[3 * REG_MAX_TRIALS];
+        take_eval(s, ev[0]);
+        s.E = -s.ncc + 0.5 * b.lambda * h2 * quu;
         s.iter = 0;
         s.tau = b.tau_init;
         s.evals += 1;
@@ -1728,30 +1644,16 @@ __device__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int 
         }
     }
     s.evals += s.ntr;
+    const unsigned long long nn = (unsigned long long)n * n;
     if (op.lock_tau) {
         // lockstep replay: take the given step whatever the test says (the
         // trace records the test), end the level after the last given step
         const double want = s.trial_tau[0];
-        double S1 = s.S1 + h2 * S[0], S2 = s.S2 + h2 * S[1], S3 = s.S3 + h2 * S[2];
-        double nc = ncc_of(S1, S2, S3);
-        double dE = -(nc - s.ncc) + 0.5 * b.lambda * h2 * (2.0 * want * Qud + want * want * Qdd);
         s.trials_seq += 1;
-        atomicAdd(&b.work[KW_TSEQ], (unsigned long long)Lv.n * Lv.n);
-        bool acc = (dE <= b.sigma * want * s.slope);
-        if (b.trace) {
-            unsigned long long k = atomicAdd(b.trace_len, 1ull);
-            if ((long long)k < b.trace_cap) {
-                double *rec = b.trace + 7 * k;
-                rec[0] = o; rec[1] = Lv.n; rec[2] = s.iter - 1; rec[3] = want;
-                rec[4] = dE; rec[5] = b.sigma * want * s.slope; rec[6] = acc;
-            }
-        }
-        s.E += dE;
-        s.S1 = S1; s.S2 = S2; s.S3 = S3;
-        s.Tbar = S1;
-        double var = S2 - S1 * S1;
-        s.sigT = var > 0.0 ? sqrt(var) : 0.0;
-        s.ncc = nc;
+        atomicAdd(&b.work[KW_TSEQ], nn);
+        trace_trial(b, s, o, n, want, ev[0].dE, ev[0].dE <= b.sigma * want * s.slope);
+        s.E += ev[0].dE;
+        take_eval(s, ev[0]);
         s.tau = want;
         if (s.iter >= lock_count(s, op)) level_end(s, op, OPST_MAXITER, want);
         else schedule_grad(s, b, op, want);
@@ -1775,30 +1677,25 @@ __device__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int 
                 int k = 0;
                 double t = want;
                 if (s.search == SEARCH_WIDEN) {
-                    while (k < b.J && t <= b.tau_max) { s.trial_tau[k++] = t; t *= 2.0; }
+                    while (k < b.J && t <= b.tau_max) { set_trial(s, k++, t); t *= 2.0; }
                 } else {
-                    while (k < b.J && t >= b.tau_min) { s.trial_tau[k++] = t; t *= 0.5; }
+                    while (k < b.J && t >= b.tau_min) { set_trial(s, k++, t); t *= 0.5; }
                 }
                 s.ntr = k;
                 s.phase = PH_TRIAL;
                 return;
             }
             // energy change E(u + tau d) - E(u) from the accumulated sums at u
-            double S1 = s.S1 + h2 * S[3 * j], S2 = s.S2 + h2 * S[3 * j + 1], S3 = s.S3 + h2 * S[3 * j + 2];
-            double nc = ncc_of(S1, S2, S3);
-            double dE = -(nc - s.ncc) + 0.5 * b.lambda * h2 * (2.0 * want * Qud + want * want * Qdd);
+            const EvalAt &v = ev[j];
             s.trials_seq += 1;
-            atomicAdd(&b.work[KW_TSEQ], (unsigned long long)Lv.n * Lv.n);
-            bool acc = (dE <= b.sigma * want * s.slope);
-            if (b.trace) {
-                unsigned long long k = atomicAdd(b.trace_len, 1ull);
-                if ((long long)k < b.trace_cap) {
-                    double *rec = b.trace + 7 * k;
-                    rec[0] = o; rec[1] = Lv.n; rec[2] = s.iter - 1; rec[3] = want;
-                    rec[4] = dE; rec[5] = b.sigma * want * s.slope; rec[6] = acc;
-                }
+            atomicAdd(&b.work[KW_TSEQ], nn);
+            const bool acc = (v.dE <= b.sigma * want * s.slope);
+            trace_trial(b, s, o, n, want, v.dE, acc);
+            if (acc) {
+                s.bS1 = v.S1; s.bS2 = v.S2; s.bS3 = v.S3; s.bncc = v.ncc; s.bdE = v.dE;
+                s.bsig = v.sig;
+                s.b_isig = v.isig; s.b_c36 = v.c36; s.b_cT = v.cT;
             }
-            if (acc) { s.bS1 = S1; s.bS2 = S2; s.bS3 = S3; s.bncc = nc; s.bdE = dE; }
             if (s.search == SEARCH_INIT) {
                 if (acc) { s.search = SEARCH_WIDEN; s.btau = want; }
                 else { s.search = SEARCH_SHRINK; s.sh_tau = want; }
@@ -1822,9 +1719,9 @@ __device__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int 
             s.E += s.bdE;
             s.S1 = s.bS1; s.S2 = s.bS2; s.S3 = s.bS3;
             s.Tbar = s.S1;
-            double var = s.S2 - s.S1 * s.S1;
-            s.sigT = var > 0.0 ? sqrt(var) : 0.0;
+            s.sigT = s.bsig;
             s.ncc = s.bncc;
+            s.f_isig = s.b_isig; s.f_c36 = s.b_c36; s.f_cT = s.b_cT;
             s.tau = s.btau;
             if (dec < b.eps * scale) level_end(s, op, OPST_CONVERGED, s.btau);
             else if (s.iter >= b.iter_max) level_end(s, op, OPST_MAXITER, s.btau);
@@ -1834,6 +1731,151 @@ __device__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int 
     }
     atomicExch(&b.ctr[8], 1);  // the search did not terminate: internal error
     s.phase = PH_DONE;
+}
+
+}  // namespace
+
+// One block per operator (grid stride): the block sums the operator's tile
+// partials in FP64, the lanes of a warp form the scalars of all evaluated trials
+// side by side (FP64 square roots and divisions are slow here: one after the
+// other in one thread they were most of the kernel), thread 0 runs the state
+// machine on a copy of the state in shared memory, and the last block to finish
+// plans the next step.  Latency bound at every size: 22 us as one thread working
+// in global memory after a 9-way split of the records, plus 6 us for a plan
+// kernel of its own (33 x 1024^2 scan).
+//
+// The sums: thread (g, kk) adds entry kk of every ng-th record (kk fastest, so a
+// warp reads neighbouring doubles), only the entries that the pass wrote: 3 per
+// step size and one Dirichlet form, at most 16 for up to four step sizes (32
+// groups), 32 otherwise (16 groups); then one warp per entry adds the groups.
+__global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
+{
+    constexpr int NW = REG_CTL_THREADS / 32;
+    __shared__ OpState s;
+    __shared__ double red[REG_CTL_THREADS + 32];
+    __shared__ double redG[NW][2];
+    __shared__ double S[32];
+    __shared__ double SG[2];
+    __shared__ EvalAt ev[REG_MAX_TRIALS];
+    __shared__ int last;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int n_ops = b.ctr[0];
+    if ((int)blockIdx.x >= n_ops) return;
+    for (int o = blockIdx.x; o < n_ops; o += gridDim.x) {
+        const OpDesc &op = b.ops[o];
+        static_assert(sizeof(OpState) % 8 == 0 && sizeof(OpState) / 8 <= REG_CTL_THREADS, "state copied by one pass");
+        if (threadIdx.x < sizeof(OpState) / 8)
+            reinterpret_cast<double *>(&s)[threadIdx.x] = reinterpret_cast<const double *>(b.st + o)[threadIdx.x];
+        __syncthreads();
+        const int ph = s.phase;
+        if (ph != PH_DONE) {
+            const LevelDesc &Lv = op.lv[s.lvl];
+            const int n = Lv.n, ntr = s.ntr;
+            const double h2 = Lv.h2d;
+            const bool start = ph == PH_START || ph == PH_PROLONG;
+            if (threadIdx.x == REG_CTL_THREADS - 1) {
+                // algorithmic work of this step (nodes of the level each kernel swept)
+                const unsigned long long nn = (unsigned long long)n * n;
+                if (ph == PH_PROLONG) atomicAdd(&b.work[KW_PPROL], nn);
+                if (start) atomicAdd(&b.work[KW_TSTART], nn);
+                if (ph == PH_GRAD) atomicAdd(&b.work[KW_G], nn);
+                if (!start) {
+                    atomicAdd(&b.work[KW_T], nn);
+                    atomicAdd(&b.work[KW_TSAMPLES], nn * (unsigned long long)ntr);
+                }
+            }
+            const int lg = b.J <= 4 ? 4 : 5, ng = REG_CTL_THREADS >> lg;
+            const int kk = threadIdx.x & ((1 << lg) - 1), g = threadIdx.x >> lg;
+            // entries 0 .. ne-2 of a record, then the Dirichlet form: of u
+            // (level start) or of d (first pass of a search)
+            const int ne = (start ? 3 : 3 * ntr) + 1;
+            if (kk < ne) {
+                const double *rec = b.partT + (kk < ne - 1 ? kk : 3 * REG_MAX_TRIALS + (start ? 0 : 2));
+                const int te = s.t_end;
+                double acc = 0.0;
+#pragma unroll 8
+                for (int it = s.t_begin + g; it < te; it += ng) acc += rec[(int64_t)it * PT_STRIDE];
+                red[kk * (ng + 1) + g] = acc;
+            }
+            double slope = 0.0, qud = 0.0;
+            if (ph == PH_GRAD) {
+                if (b.smooth) {
+                    // the smoothed direction's slope and u^T K d (smoother partials)
+                    const double *pS = b.partS + (int64_t)s.g_entry * b.cch * 2;
+                    const int nch = (n + REG_GW - 1) / REG_GW;
+                    for (int ch = threadIdx.x; ch < nch; ch += REG_CTL_THREADS) {
+                        slope += pS[2 * ch];
+                        qud += pS[2 * ch + 1];
+                    }
+                } else {
+                    const int ge = s.g_end;
+#pragma unroll 4
+                    for (int it = s.g_begin + threadIdx.x; it < ge; it += REG_CTL_THREADS) {
+                        const double2 p = reinterpret_cast<const double2 *>(b.partG)[it];
+                        slope += p.x;
+                        qud += p.y;
+                    }
+                }
+                slope = warp_sum_d(slope);
+                qud = warp_sum_d(qud);
+                if (lane == 0) {
+                    redG[wid][0] = slope;
+                    redG[wid][1] = qud;
+                }
+            }
+            __syncthreads();
+            for (int k = wid; k < ne; k += NW) {
+                const double v = warp_sum_d(lane < ng ? red[k * (ng + 1) + lane] : 0.0);
+                if (lane == 0) S[k] = v;
+            }
+            if (ph == PH_GRAD && wid == NW - 1) {
+                const double v = warp_sum_d(lane < NW ? redG[lane][0] : 0.0);
+                const double w = warp_sum_d(lane < NW ? redG[lane][1] : 0.0);
+                if (lane == 0) {
+                    SG[0] = b.smooth ? -h2 * h2 * v : v;
+                    SG[1] = w;
+                }
+            }
+            __syncthreads();
+            if (wid == 0) {
+                if (ph == PH_GRAD && lane == 0) {
+                    // the Dirichlet forms of the new search: u^T K d from the gradient
+                    // pass (or the smoother), d^T K d from its first trial pass
+                    s.Qud = SG[1];
+                    s.Qdd = S[ne - 1];
+                }
+                __syncwarp();
+                if (start) {
+                    if (lane == 0) eval_at(ev[0], h2 * S[0], h2 * S[1], h2 * S[2]);
+                } else if (lane < ntr) {
+                    EvalAt v;
+                    const double want = s.trial_tau[lane];
+                    eval_at(v, s.S1 + h2 * S[3 * lane], s.S2 + h2 * S[3 * lane + 1], s.S3 + h2 * S[3 * lane + 2]);
+                    v.dE = -(v.ncc - s.ncc) + 0.5 * b.lambda * h2 * (2.0 * want * s.Qud + want * want * s.Qdd);
+                    ev[lane] = v;
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    control_op(b, s, op, o, n, h2, ev, S[ne - 1], SG[0]);
+                    b.plan[o] = op_plan(s, op);
+                }
+            }
+            __syncthreads();
+            if (threadIdx.x < sizeof(OpState) / 8)
+                reinterpret_cast<double *>(b.st + o)[threadIdx.x] = reinterpret_cast<const double *>(&s)[threadIdx.x];
+        }
+        __syncthreads();
+    }
+    // the last block plans: its reads of the other blocks' entries follow their fences
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&b.ctr[9], 1) == min((int)gridDim.x, n_ops) - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    plan_lists(b);
+    if (threadIdx.x == 0) b.ctr[9] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -2115,9 +2157,7 @@ static int occupancy(K kernel, int threads, int carveout)
 int step_blocks_per_sm(int which, int J)
 {
     int occ = 0;
-    if (which == 0) {
-        occ = occupancy(k_prolong, REG_THREADS, 0);
-    } else if (which == 1) {
+    if (which == 1) {
         occupancy(k_grad<true>, REG_STRIP_THREADS, 0);
         occ = occupancy(k_grad<false>, REG_STRIP_THREADS, 0);
     } else {

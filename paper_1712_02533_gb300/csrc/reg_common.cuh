@@ -6,11 +6,7 @@
 
 #define REG_MAX_LEVELS 8
 #define REG_MAX_TRIALS 8
-#define REG_TX 32        // prolongation block tile width (nodes along x_0)
-#define REG_TY 32        // prolongation block tile height
-#define REG_THREADS 256  // threads per step-kernel block (8 warps)
-#define REG_ROWSTEP (REG_THREADS / REG_TX)  // thread (lx, ly) handles rows ly + k REG_ROWSTEP
-#define REG_RPT (REG_TY / REG_ROWSTEP)      // rows per thread
+#define REG_CTL_THREADS 512  // threads per block of the control kernel
 // Warp strips of the gradient and trial kernels: the 32 lanes of a warp hold 32
 // adjacent node columns and walk down the rows of a tile together, so that
 // vertical neighbours stay in registers and horizontal ones are a shuffle away.
@@ -33,9 +29,8 @@ enum {
     PH_START = 0,    // evaluate the energy at the level's initial u (tau = 0)
     PH_GRAD = 1,     // apply the pending step, then gradient + first trial pass
     PH_TRIAL = 2,    // more step sizes of the same Armijo search
-    PH_PROLONG = 3,  // apply pending step, prolongate to the next level, then START there
-    PH_FINAL = 4,    // apply pending step on the finest level into the output slot
-    PH_DONE = 5
+    PH_PROLONG = 3,  // prolongate u + pending step from the level below, START at the result
+    PH_DONE = 4      // the batch's final pass applies the pending step and writes the output slot
 };
 enum { SEARCH_INIT = 0, SEARCH_WIDEN = 1, SEARCH_SHRINK = 2 };
 enum { OPST_CONVERGED = 0, OPST_MAXITER = 1, OPST_STALLED = 2, OPST_NONFINITE = 3, OPST_ZERO_GRAD = 4 };
@@ -104,11 +99,17 @@ struct OpState {
     double sh_tau;    // shrinking: last rejected step
     double E, Tbar, sigT, ncc;      // at the current u
     double S1, S2, S3;              // FE sums int That, int That^2, int That R~ at the current u
-    double bS1, bS2, bS3, bncc, bdE;  // last accepted trial of the search
+    double bS1, bS2, bS3, bncc, bsig, bdE;  // last accepted trial of the search
     double btau;
     double slope;
     double Qud, Qdd;  // Dirichlet forms u^T K d and d^T K d of the current search
     double trial_tau[REG_MAX_TRIALS];
+    // What the gradient and trial passes read, rounded once per step by the
+    // control kernel instead of once per tile: the pending step, the step sizes
+    // of the pass, and 1 / sigma, NCC / sigma^2 / 36, NCC / sigma^2 T_bar at u
+    // (b*: of the last accepted trial of the search).
+    float f_tau_acc, f_isig, f_c36, f_cT, b_isig, b_c36, b_cT, f_pad;
+    float f_tau[REG_MAX_TRIALS];
     double corr;  // judged ops: sum over finest nodes of |u_final - u_start| (x + y, px)
 };
 
@@ -118,10 +119,11 @@ struct OpState {
 struct BatchDev {
     OpDesc *ops;
     OpState *st;
-    int *listP, *listG, *listT;  // compacted op indices per family
-    int *prefP, *prefG, *prefT;  // exclusive prefix of tile counts (n+1 entries)
-    int *ctr;                    // [0] n_ops [1] nP [2] nG [3] nT [4] itemsP [5] itemsG [6] itemsT
-                                 // [7] n_active [8] error flag
+    int *listG, *listT;          // compacted op indices per family
+    int *prefG, *prefT;          // exclusive prefix of tile counts (n+1 entries)
+    int4 *plan;                  // per op: {gradient tiles, trial tiles, active, -} of the next step
+    int *ctr;                    // [0] n_ops [2] nG [3] nT [5] itemsG [6] itemsT [7] n_active
+                                 // [8] error flag [9] blocks of the control kernel that are done
     double *partG;               // per G item: slope and u^T K d partials (PG_STRIDE)
     double *partT;               // per T item: 3 sums per step size, then 3 Dirichlet forms (PT_STRIDE)
     unsigned long long *work;    // per kernel family: nodes processed
@@ -129,7 +131,8 @@ struct BatchDev {
     unsigned long long *trace_len;
     long long trace_cap;
     double lambda, sigma, tau_init, tau_max, tau_min, eps;
-    int iter_max, J, bf16, pad;
+    float lam6;                  // lambda / 6
+    int iter_max, J, bf16;
     // H1-type smoother (smooth != 0): per gradient-pass op and column chunk of
     // REG_GW columns, the partial sums {sum omega d_L2 . d, sum d . 6 K u}
     double *partS;

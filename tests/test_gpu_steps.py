@@ -1,0 +1,53 @@
+"""The device step loop (gradient, trial and control kernels) at the sizes
+where its work planning changes: batches wider than one planning pass, and
+every number of step sizes per trial pass."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def reg():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1712_02533_gb300 import _build
+    _build.build()
+    import paper_1712_02533_gb300 as r
+    return r
+
+
+@pytest.mark.parametrize("n_ops", [1, 2, 511, 512, 513, 1100])
+def test_operators_of_a_wide_batch_are_those_run_alone(reg, syn, n_ops):
+    """Operators of one batch are independent: whatever the batch's width, each
+    result, status and iteration count is bit for bit that of the operator run
+    alone (the tile records and their FP64 sums do not depend on the batch)."""
+    n_fr = min(n_ops + 1, 12)
+    fr = syn.series(11, n_fr, 32, spacing=8.0, sigma=1.5, peak=20.0)
+    # n_ops pairs (i, i + 1), repeated, into as many slots: several series share the frames
+    per = n_fr - 1
+    m = -(-n_ops // per)
+    p = reg.default_params(n_levels=2, iter_max=8, lam=10.0)
+    ops = [(k // per, -1, -1, k % per, k % per, k % per + 1) for k in range(n_ops)]
+    with reg.Series([fr] * m, p) as s:
+        st, it = s.apply_operator_batch(ops)
+        got = {k: s.get_slot(ops[k][3], series=ops[k][0])[0] for k in {0, n_ops // 2, n_ops - 1}}
+    with reg.Series(fr, p) as s:
+        for k, u in got.items():
+            a, b = s.apply_operator_batch([(0, -1, -1, ops[k][3], ops[k][4], ops[k][5])])
+            assert (a[0], b[0]) == (st[k], it[k])
+            assert np.array_equal(s.get_slot(ops[k][3])[0], u)
+
+
+@pytest.mark.parametrize("J", [1, 2, 3, 4, 5, 8])
+def test_step_sizes_per_pass_do_not_change_the_accepted_steps(reg, orc, syn, J):
+    """A stable pair (no shot noise, 64^2, 2 levels): for every number of step
+    sizes per pass the field is within 1e-3 px of the oracle's, the bound of
+    the other stable-series tests."""
+    fr = syn.series(7, 2, 64, noise=False, drift_sd=1.0, dist_amp=0.0, spacing=10.0, sigma=2.5)
+    want, _, _ = orc.register(orc.embed(fr[0]), orc.embed(fr[1]), orc.params(n_levels=2, iter_max=20, lam=10.0))
+    with reg.Series(fr, reg.default_params(n_levels=2, iter_max=20, lam=10.0, trials_per_pass=J)) as s:
+        s.apply_operator_batch([(0, -1, -1, 0, 0, 1)])
+        got = s.get_slot(0)[0]
+    assert np.abs(got - want * 64).max() <= 1e-3
