@@ -161,7 +161,7 @@ struct reg_series {
     OpDesc *d_ops = nullptr;
     OpState *d_st = nullptr;
     int *d_lists = nullptr;  // listG, listT, prefG, prefT
-    int4 *d_plan = nullptr;  // per op: its work of the next step
+    int2 *d_plan = nullptr;  // per op: its work of the next step
     int *d_ctr = nullptr;
     double *d_partG = nullptr, *d_partT = nullptr;
     unsigned long long *d_work = nullptr;
@@ -333,6 +333,8 @@ void fill_level(const reg_series *s, LevelDesc &L, int n, int pitch)
     L.pitch = pitch;
     L.hg = s->tile_hg[level_of(n)];
     L.ht = s->tile_ht[level_of(n)];
+    L.tg = cdiv(n, REG_GW) * cdiv(n, L.hg);
+    L.tt = cdiv(n - 1, REG_CW) * cdiv(n - 1, L.ht);
     const double h = 1.0 / (n - 1);
     L.h2d = h * h;
     L.h2 = (float)L.h2d;
@@ -354,7 +356,7 @@ reg_status ensure_capacity(reg_series *s, int n_ops, size_t ws_total, int64_t it
         RET(track(s, (void **)&s->d_ops, sizeof(OpDesc) * c));
         RET(track(s, (void **)&s->d_st, sizeof(OpState) * c));
         RET(track(s, (void **)&s->d_lists, sizeof(int) * (4 * c + 2)));
-        RET(track(s, (void **)&s->d_plan, sizeof(int4) * c));
+        RET(track(s, (void **)&s->d_plan, sizeof(int2) * std::max(c, 32)));
         if (s->p.smooth > 0.0) {
             untrack(s, s->d_partS);
             RET(track(s, (void **)&s->d_partS, sizeof(double) * 2 * (size_t)s->sm_cch * c));
@@ -454,6 +456,7 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
     // batch without every op taking the largest one's room); the step's work
     // items are at most the sum of the ops' largest tile counts
     std::vector<size_t> ws_off(n);
+    std::vector<int> part0(n);  // first tile record of each op
     size_t ws = 0;
     int64_t items = 0;
     int nl = 0, nLmax = 0;
@@ -462,10 +465,12 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
         const SeriesInfo &si = s->S[o.series];
         ws_off[i] = ws;
         ws += (si.ws_bytes + 255) / 256 * 256;
+        part0[i] = (int)items;
         items += max_tiles_series(s, si, o.skip);
         nl = std::max(nl, si.nl);
         nLmax = std::max(nLmax, si.n[si.nl - 1]);
     }
+    if (items > INT32_MAX) return fail(REG_EINVAL, "batch of %d ops has too many tiles", n);
     RET(ensure_capacity(s, n, ws, items));
     for (int i = 0; i < n; i++) {
         const OpReq &o = ops[i];
@@ -479,6 +484,7 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
         d.out = si.slots + (size_t)o.dst * si.slot_elems;
         d.slot_pitch = si.pitch[si.nl - 1];
         d.judge = o.judge;
+        d.part0 = part0[i];
         char *w = s->d_ws + ws_off[i];
         for (int j = 0; j < d.nl; j++) {
             const int k = o.skip + j;  // level index within the series' pyramid
@@ -1769,7 +1775,7 @@ reg_status reg_eval_direction(reg_series_t s, int32_t series, int32_t frame_i, i
     CK(cudaStreamSynchronize(s->stream));
     if (st.phase != PH_GRAD) return fail(REG_ESTATE, "energy at the given displacement is not finite");
     if (!s->d_scratch) RET(track(s, (void **)&s->d_scratch, sizeof(double) * 16));
-    k_sum_range<<<1, 32, 0, s->stream>>>(s->d_partG, PG_STRIDE, st.g_begin, st.g_end, s->d_scratch);
+    k_sum_range<<<1, 32, 0, s->stream>>>(s->d_partG, PG_STRIDE, 0, st.tG, s->d_scratch);
     double sl = 0.0;
     CK(cudaMemcpyAsync(&sl, s->d_scratch, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
     const SeriesInfo &si = s->S[series];
@@ -1807,18 +1813,18 @@ reg_status reg_eval_trials(reg_series_t s, int32_t series, int32_t frame_i, int3
     CK(cudaMemcpyAsync(&st, s->d_st, sizeof(OpState), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
     if (st.phase != PH_GRAD) return fail(REG_ESTATE, "energy at the given displacement is not finite");
-    st.ntr = n_tau;
+    st.ntr = st.step.ntr = n_tau;
     for (int j = 0; j < REG_MAX_TRIALS; j++) {
         st.trial_tau[j] = j < n_tau ? taus[j] : 0.0;
-        st.f_tau[j] = (float)st.trial_tau[j];
+        st.step.tau[j] = (float)st.trial_tau[j];
     }
     CK(cudaMemcpyAsync(s->d_st, &st, sizeof(OpState), cudaMemcpyHostToDevice, s->stream));
     launch_trial(s->bf16, s->p.trials_per_pass, s->grid_T, s->stream, b);
     CK(cudaGetLastError());
-    std::vector<double> pt((size_t)(st.t_end - st.t_begin) * PT_STRIDE), pg((size_t)(st.g_end - st.g_begin) * PG_STRIDE);
-    CK(cudaMemcpyAsync(pt.data(), s->d_partT + (size_t)st.t_begin * PT_STRIDE, pt.size() * sizeof(double),
+    std::vector<double> pt((size_t)st.tT * PT_STRIDE), pg((size_t)st.tG * PG_STRIDE);
+    CK(cudaMemcpyAsync(pt.data(), s->d_partT, pt.size() * sizeof(double),
                        cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(pg.data(), s->d_partG + (size_t)st.g_begin * PG_STRIDE, pg.size() * sizeof(double),
+    CK(cudaMemcpyAsync(pg.data(), s->d_partG, pg.size() * sizeof(double),
                        cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
     double S[PT_STRIDE] = {0.0}, qud = 0.0;

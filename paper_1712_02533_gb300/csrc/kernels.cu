@@ -387,22 +387,76 @@ __global__ void k_init_state(BatchDev b, int n_ops)
 // Work planning: compacted per-family op lists and tile prefix sums
 // ---------------------------------------------------------------------------
 
-// work items per operator: gradient and trial strip tiles
-__device__ __forceinline__ int grad_tiles(const LevelDesc &L)
+constexpr int PLAN_WARP = 32;  // batches up to this wide are planned by every warp itself
+
+// The next step of an operator, from its state: the tile counts and the
+// description that the gradient and trial passes read.
+__device__ __forceinline__ void set_step(OpState &s, const OpDesc &op)
 {
-    return ((L.n + REG_GW - 1) / REG_GW) * ((L.n + L.hg - 1) / L.hg);
-}
-__device__ __forceinline__ int trial_tiles(const LevelDesc &L)
-{
-    return ((L.n - 1 + REG_CW - 1) / REG_CW) * ((L.n - 1 + L.ht - 1) / L.ht);
+    const LevelDesc &L = op.lv[s.lvl];
+    s.tG = s.phase == PH_GRAD ? L.tg : 0;
+    s.tT = s.phase == PH_DONE ? 0 : L.tt;
+    StepDesc &d = s.step;
+    d.T = L.T;
+    d.MR = L.MR;
+    d.Vs = s.phase == PH_PROLONG ? L.V[s.cur] : L.V[s.src];
+    d.Vc = L.V[s.cur];
+    const LevelDesc &C = op.lv[s.phase == PH_PROLONG ? s.lvl - 1 : s.lvl];
+    d.VC = C.V[s.src];
+    d.cpitch = C.pitch;
+    d.phase = s.phase;
+    d.n = L.n;
+    d.pitch = L.pitch;
+    d.hg = L.hg;
+    d.ht = L.ht;
+    d.ntr = s.ntr;
+    d.part0 = op.part0;
+    d.ih2 = 1.f / L.h2;
 }
 
-// An operator's work of the next step: {gradient tiles, trial tiles, active}.
-__device__ __forceinline__ int4 op_plan(const OpState &s, const OpDesc &op)
+// A warp's view of the step's work items (tiles of one family).  Batches of up to
+// PLAN_WARP operators: lane l holds operator l's tile range, from one load and a
+// warp scan.  Wider ones: the compacted lists (cnt = -1, incl = their length).
+struct WorkPlan {
+    int items, incl, cnt;
+};
+
+template <bool GRAD>
+__device__ __forceinline__ WorkPlan work_plan(const BatchDev &b, int lane)
 {
-    if (s.phase == PH_DONE) return make_int4(0, 0, 0, 0);
-    const LevelDesc &L = op.lv[s.lvl];
-    return make_int4(s.phase == PH_GRAD ? grad_tiles(L) : 0, trial_tiles(L), 1, 0);
+    WorkPlan w;
+    const int2 p = b.plan[lane];  // (at least PLAN_WARP entries exist)
+    const int n_ops = b.ctr[0];
+    if (n_ops <= PLAN_WARP) {
+        w.cnt = lane < n_ops ? (GRAD ? p.x : p.y) : 0;
+        w.incl = w.cnt;
+#pragma unroll
+        for (int k = 1; k < 32; k <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, w.incl, k);
+            if (lane >= k) w.incl += y;
+        }
+        w.items = __shfl_sync(0xffffffffu, w.incl, 31);
+    } else {
+        w.cnt = -1;
+        w.incl = b.ctr[GRAD ? 2 : 3];
+        w.items = b.ctr[GRAD ? 5 : 6];
+    }
+    return w;
+}
+
+// Operator of a work item and the item's tile index in it (warp-uniform).
+template <bool GRAD>
+__device__ __forceinline__ int find_item(const BatchDev &b, const WorkPlan &w, int item, int &tile)
+{
+    if (w.cnt >= 0) {
+        const int o = __ffs(__ballot_sync(0xffffffffu, w.incl > item)) - 1;
+        tile = item - __shfl_sync(0xffffffffu, w.incl - w.cnt, o);
+        return o;
+    }
+    const int *pref = GRAD ? b.prefG : b.prefT;
+    const int e = find_entry(pref, w.incl, item);
+    tile = item - pref[e];
+    return (GRAD ? b.listG : b.listT)[e];
 }
 
 // The lists and tile prefixes of the next step from the operators' plan entries,
@@ -418,7 +472,7 @@ __device__ void plan_lists(const BatchDev &b)
     for (int base = 0; base < n_ops; base += REG_CTL_THREADS) {
         const int o = base + threadIdx.x;
         // other blocks wrote the entries in this launch: past L1
-        const int4 p = o < n_ops ? __ldcg(b.plan + o) : make_int4(0, 0, 0, 0);
+        const int2 p = o < n_ops ? __ldcg(b.plan + o) : make_int2(0, 0);
         // entries of both lists in one word (at most REG_CTL_THREADS each)
         const int inc = (p.x > 0 ? 1 : 0) | (p.y > 0 ? 1 << 16 : 0);
         int e = inc, g = p.x, t = p.y;
@@ -437,24 +491,14 @@ __device__ void plan_lists(const BatchDev &b)
             if (w < wid) { before.x += x.x; before.y += x.y; before.z += x.z; }
             all.x += x.x; all.y += x.y; all.z += x.z;
         }
-        if (o < n_ops) {
-            const int ex = e - inc + before.x;
-            const int eG = offG + (ex & 0xffff), eT = offT + (ex >> 16);
-            const int iG = itG + g - p.x + before.y, iT = itT + t - p.y + before.z;
-            OpState &s = b.st[o];
-            if (p.x > 0) {
-                b.listG[eG] = o;
-                b.prefG[eG] = iG;
-                s.g_entry = eG;
-            }
-            if (p.y > 0) {
-                b.listT[eT] = o;
-                b.prefT[eT] = iT;
-            }
-            s.g_begin = iG;
-            s.g_end = iG + p.x;
-            s.t_begin = iT;
-            s.t_end = iT + p.y;
+        const int ex = e - inc + before.x;
+        if (p.x > 0) {
+            b.listG[offG + (ex & 0xffff)] = o;
+            b.prefG[offG + (ex & 0xffff)] = itG + g - p.x + before.y;
+        }
+        if (p.y > 0) {
+            b.listT[offT + (ex >> 16)] = o;
+            b.prefT[offT + (ex >> 16)] = itT + t - p.y + before.z;
         }
         offG += all.x & 0xffff;
         offT += all.x >> 16;
@@ -469,19 +513,22 @@ __device__ void plan_lists(const BatchDev &b)
         b.ctr[3] = offT;
         b.ctr[5] = itG;
         b.ctr[6] = itT;
-        b.ctr[7] = offT;  // every operator that is not done has trial tiles
     }
 }
 
-// Plan of a batch's first step (the control kernel plans the others): the
-// entries from the operators' states, then the lists.
+// Plan of a batch's first step from the operators' states (the control kernel
+// plans the others).
 __global__ void __launch_bounds__(REG_CTL_THREADS) k_plan(BatchDev b)
 {
     const int n_ops = b.ctr[0];
-    for (int o = threadIdx.x; o < n_ops; o += REG_CTL_THREADS) b.plan[o] = op_plan(b.st[o], b.ops[o]);
-    __threadfence_block();
+    for (int o = threadIdx.x; o < n_ops; o += REG_CTL_THREADS) {
+        set_step(b.st[o], b.ops[o]);
+        b.plan[o] = make_int2(b.st[o].tG, b.st[o].tT);
+    }
+    __threadfence();
     __syncthreads();
-    plan_lists(b);
+    if (n_ops > PLAN_WARP) plan_lists(b);
+    if (threadIdx.x == 0) b.ctr[7] = n_ops;
 }
 
 // ---------------------------------------------------------------------------
@@ -531,7 +578,7 @@ __global__ void __launch_bounds__(256) k_final(BatchDev b)
     const OpState &s = b.st[blockIdx.z];
     float corr = 0.f;  // judged ops: |final - learned start|
     if (r < n && c < n) {
-        const float tau = s.f_tau_acc;
+        const float tau = (float)s.tau_acc;
         const NodeRec &v = Lv.V[s.src][(int64_t)r * Lv.pitch + c];
         float4 u = v.u;
         if (tau != 0.f) {
@@ -577,14 +624,14 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, 8) k_grad(BatchDev b)
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int nwarps = gridDim.x * (REG_STRIP_THREADS / 32);
-    const int nent = b.ctr[2], items = b.ctr[5];
-    for (int item = blockIdx.x * (REG_STRIP_THREADS / 32) + (threadIdx.x >> 5); item < items; item += nwarps) {
-        const int e = find_entry(b.prefG, nent, item);
-        const int o = b.listG[e];
-        const int t = item - b.prefG[e];
-        const OpState &s = b.st[o];
-        const LevelDesc &Lv = b.ops[o].lv[s.lvl];
-        const int n = Lv.n, pitch = Lv.pitch, ntx = (n + REG_GW - 1) / REG_GW, h = Lv.hg;
+    for (int item = blockIdx.x * (REG_STRIP_THREADS / 32) + (threadIdx.x >> 5);; item += nwarps) {
+        // read again for every tile: held in registers over the row walk it spills
+        const WorkPlan wp = work_plan<true>(b, lane);
+        if (item >= wp.items) break;
+        int t;
+        const StepDesc &s = b.st[find_item<true>(b, wp, item, t)].step;
+        const int n = s.n, pitch = s.pitch, ntx = (n + REG_GW - 1) / REG_GW, h = s.hg;
+        const int part = s.part0 + t;
         const int r0 = (t / ntx) * h, c = (t % ntx) * REG_GW - 1 + lane;
         const int rLast = min(r0 + h - 1, n - 1);
         const bool colIn = c >= 0 && c < n;
@@ -592,14 +639,14 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, 8) k_grad(BatchDev b)
         const bool cEdge = (c == 0 || c == n - 1);
         const float cx6 = cEdge ? 2.f : 4.f;  // 6 M1 on the diagonal
         const float wx = cEdge ? 0.5f : 1.f, iwx = cEdge ? 2.f : 1.f;
-        const float tau = s.f_tau_acc;
-        const NodeRec *Vs = Lv.V[s.src];
-        NodeRec *Vc = Lv.V[s.cur];
+        const float tau = s.tau_acc;
+        const NodeRec *Vs = s.Vs;
+        NodeRec *Vc = s.Vc;
         // the stencils run on the integer weights 6 M1 and 6 K1 (36 M~, 6 K); their
         // scale is in these per-operator coefficients, each rounded once by the
         // control kernel: 1 / sigma, NCC / sigma^2 / 36, NCC / sigma^2 T_bar
-        const float isig = s.f_isig, c36 = s.f_c36, cT = s.f_cT, lam6 = b.lam6;
-        const float ih2 = 1.f / Lv.h2;  // exact: h^2 is a power of two
+        const float isig = s.isig, c36 = s.c36, cT = s.cT, lam6 = b.lam6;
+        const float ih2 = s.ih2;
         // rows r-2 (suffix A) and r-1 (suffix M) of this column; row r is read
         // in the iteration and row r-1 is completed by it
         float tA = 0.f, tM = 0.f, kxAx = 0.f, kxAy = 0.f, kxMx = 0.f, kxMy = 0.f;
@@ -614,7 +661,7 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, 8) k_grad(BatchDev b)
             const float4 *rec = reinterpret_cast<const float4 *>(Vs + idx);
             nu = rec[0];
             nd = rec[1];
-            nmr = Lv.MR[idx];
+            nmr = s.MR[idx];
         }
         for (int r = r0 - 1; r <= rLast + 1; r++) {
             const bool in = colIn && r >= 0 && r < n;
@@ -626,12 +673,12 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, 8) k_grad(BatchDev b)
                 const float4 *rec = reinterpret_cast<const float4 *>(Vs + idx);
                 nu = rec[0];
                 nd = rec[1];
-                nmr = Lv.MR[idx];
+                nmr = s.MR[idx];
             }
             float tv = 0.f, gx = 0.f, gy = 0.f;
             if (in) {
                 if (tau != 0.f) u = df_add2(u, tau * dp.x, tau * dp.y);
-                tv = sample_df<BF16, true>(Lv.T, n, pitch, c, r, u, &gx, &gy);
+                tv = sample_df<BF16, true>(s.T, n, pitch, c, r, u, &gx, &gy);
             } else {
                 u = make_float4(0.f, 0.f, 0.f, 0.f);
             }
@@ -687,7 +734,7 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, 8) k_grad(BatchDev b)
         }
         slope = warp_sum(slope);
         qud = warp_sum(qud / 6.f);
-        if (lane < PG_STRIDE) b.partG[(int64_t)item * PG_STRIDE + lane] = lane == 0 ? slope : qud;
+        if (lane < PG_STRIDE) b.partG[(int64_t)part * PG_STRIDE + lane] = lane == 0 ? slope : qud;
     }
 }
 
@@ -713,12 +760,12 @@ __device__ __forceinline__ float2 *sm_scratch(NodeRec *V, int64_t idx, int k)
 __global__ void __launch_bounds__(128) k_smooth_rows(BatchDev b)
 {
     const int lane = threadIdx.x & 31;
-    const int nwarps = gridDim.x * 4, nG = b.ctr[2];
+    const int nwarps = gridDim.x * 4, n_ops = b.ctr[0];
     const float a = b.sm_a;
-    for (int it = blockIdx.x * 4 + (threadIdx.x >> 5); it < nG * b.rch; it += nwarps) {
-        const int e = it / b.rch, ch = it % b.rch;
-        const int o = b.listG[e];
+    for (int it = blockIdx.x * 4 + (threadIdx.x >> 5); it < n_ops * b.rch; it += nwarps) {
+        const int o = it / b.rch, ch = it % b.rch;
         const OpState &s = b.st[o];
+        if (s.phase != PH_GRAD) continue;
         const LevelDesc &Lv = b.ops[o].lv[s.lvl];
         const int n = Lv.n, pitch = Lv.pitch, r = ch * 32 + lane;
         if (r >= n) continue;
@@ -757,12 +804,12 @@ __global__ void __launch_bounds__(128) k_smooth_cols(BatchDev b)
 {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const int nwarps = gridDim.x * 4, nG = b.ctr[2];
+    const int nwarps = gridDim.x * 4, n_ops = b.ctr[0];
     const float a = b.sm_a;
-    for (int it = blockIdx.x * 4 + (threadIdx.x >> 5); it < nG * b.cch; it += nwarps) {
-        const int e = it / b.cch, ch = it % b.cch;
-        const int o = b.listG[e];
+    for (int it = blockIdx.x * 4 + (threadIdx.x >> 5); it < n_ops * b.cch; it += nwarps) {
+        const int o = it / b.cch, ch = it % b.cch;
         const OpState &s = b.st[o];
+        if (s.phase != PH_GRAD) continue;
         const LevelDesc &Lv = b.ops[o].lv[s.lvl];
         const int n = Lv.n, pitch = Lv.pitch;
         if (ch * REG_GW >= n) continue;  // warp-uniform
@@ -837,8 +884,8 @@ __global__ void __launch_bounds__(128) k_smooth_cols(BatchDev b)
         sl = warp_sum(sl);
         qd = warp_sum(qd / 6.f);
         if (lane == 0) {
-            b.partS[((int64_t)e * b.cch + ch) * 2] = sl;
-            b.partS[((int64_t)e * b.cch + ch) * 2 + 1] = qd;
+            b.partS[((int64_t)o * b.cch + ch) * 2] = sl;
+            b.partS[((int64_t)o * b.cch + ch) * 2 + 1] = qd;
         }
     }
 }
@@ -930,7 +977,7 @@ struct StripGeom {
     float wx;
 };
 
-__device__ __forceinline__ StripGeom strip_geom(const LevelDesc &Lv, int t, int lane)
+__device__ __forceinline__ StripGeom strip_geom(const StepDesc &Lv, int t, int lane)
 {
     StripGeom g;
     g.n = Lv.n;
@@ -1078,15 +1125,13 @@ __device__ __forceinline__ bool patch_delta(const Patch &P, int n, float ex, flo
 // prolongation is needed here only, once per level and operator, and as a kernel
 // of its own it cost every step an (almost always empty) launch of 3 us.
 template <bool BF16>
-__device__ __forceinline__ void start_tile(const OpState &s, const OpDesc &op, const LevelDesc &Lv, const StripGeom &g,
-                                           double *v)
+__device__ __forceinline__ void start_tile(const StepDesc &s, const StripGeom &g, double *v)
 {
     const unsigned FULL = 0xffffffffu;
     const bool prol = s.phase == PH_PROLONG;
-    NodeRec *V = Lv.V[s.cur];
-    const LevelDesc &Cv = op.lv[prol ? s.lvl - 1 : s.lvl];
-    const NodeRec *VC = Cv.V[s.src];
-    const float ptau = s.f_tau_acc;
+    NodeRec *V = s.Vc;
+    const NodeRec *VC = s.VC;
+    const float ptau = s.tau_acc;
     double s1 = 0.0, s3 = 0.0, q2 = 0.0, quu = 0.0;
     float tP = 0.f, tPR = 0.f, pux = 0.f, puy = 0.f;
     float4 uP = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1096,13 +1141,13 @@ __device__ __forceinline__ void start_tile(const OpState &s, const OpDesc &op, c
         if (g.colIn) {
             const int64_t idx = (int64_t)r * g.pitch + g.c;
             if (prol) {
-                u = prolong_node(VC, Cv.pitch, ptau, r, g.c);
+                u = prolong_node(VC, s.cpitch, ptau, r, g.c);
                 if (g.nodeCol && (r < g.r0 + g.h || r == g.n - 1)) V[idx].u = u;
             } else {
                 u = V[idx].u;
             }
-            mr = Lv.MR[idx];
-            t0 = sample_df<BF16, false>(Lv.T, g.n, g.pitch, g.c, r, u, nullptr, nullptr);
+            mr = s.MR[idx];
+            t0 = sample_df<BF16, false>(s.T, g.n, g.pitch, g.c, r, u, nullptr, nullptr);
         }
         if (g.nodeCol && (r < g.r0 + g.h || r == g.n - 1)) {
             const float w = g.wx * ((r == 0 || r == g.n - 1) ? 0.5f : 1.f);
@@ -1163,13 +1208,12 @@ struct TrialScratch {
 // changes go to queue entry q and, for an owned node, into the node sums of
 // the lane that computes them.
 template <bool BF16, int JM>
-__device__ __forceinline__ void node_deltas_exact(const LevelDesc &Lv, const float *tau, int J, int c, int r,
+__device__ __forceinline__ void node_deltas_exact(const void *T, int n, int pitch, const float *tau, int J, int c, int r,
                                                   float4 u, float4 dm, float w, bool own, TrialScratch<JM> &sh,
                                                   int q, int lane)
 {
-    const int n = Lv.n, pitch = Lv.pitch;
     Patch P;
-    make_patch<BF16>(P, Lv.T, n, pitch, c, r, u, dm.x, dm.y);
+    make_patch<BF16>(P, T, n, pitch, c, r, u, dm.x, dm.y);
     const bool cl = P.clx || P.cly;
     // dThat/dx at a_y, dThat/dy at a_x and the mixed derivative of the base cell
     const float sy = P.v0[0] + P.ax * (P.v0[1] - P.v0[0]);
@@ -1186,7 +1230,7 @@ __device__ __forceinline__ void node_deltas_exact(const LevelDesc &Lv, const flo
             } else if (!patch_delta(P, n, ex, ey, del)) {
                 Texel4 t;
                 locate(n, c, r, (u.x + u.z) + ex, (u.y + u.w) + ey, t.jx, t.jy, t.ax, t.ay, t.clx, t.cly);
-                fetch<BF16>(t, Lv.T, pitch);
+                fetch<BF16>(t, T, pitch);
                 del = bil(t) - P.t0;
             }
             sh.dl[j][q] = del;
@@ -1205,7 +1249,7 @@ __device__ __forceinline__ void node_deltas_exact(const LevelDesc &Lv, const flo
 // A and B.  The last row moves to slot 0 with the changes of its queued nodes,
 // for the cells between it and the next window.
 template <bool BF16, int JM>
-__device__ __forceinline__ void trial_flush(const LevelDesc &Lv, const StripGeom &g, const float4 *V,
+__device__ __forceinline__ void trial_flush(const void *T, const StripGeom &g, const float4 *V,
                                             const float *tau, int J, TrialScratch<JM> &sh, int lane, int rlast,
                                             int nrow, int &q0, int &qn, int &qc)
 {
@@ -1218,7 +1262,7 @@ __device__ __forceinline__ void trial_flush(const LevelDesc &Lv, const StripGeom
         const float4 u = V[2 * idx], dm = V[2 * idx + 1];
         const bool own = (ln < REG_CW || c == g.n - 1) && (r < g.r0 + g.h || r == g.n - 1);
         const float w = ((c == 0 || c == g.n - 1) ? 0.5f : 1.f) * ((r == 0 || r == g.n - 1) ? 0.5f : 1.f);
-        node_deltas_exact<BF16, JM>(Lv, tau, J, c, r, u, dm, w, own, sh, q, lane);
+        node_deltas_exact<BF16, JM>(T, g.n, g.pitch, tau, J, c, r, u, dm, w, own, sh, q, lane);
     }
     __syncwarp();
     for (int q = lane; q < qc; q += 32) {
@@ -1276,19 +1320,20 @@ __device__ __forceinline__ void trial_flush(const LevelDesc &Lv, const StripGeom
 // step size, in windows of rows finished by the whole warp (trial_flush).  The
 // node record of the next row is loaded while the current row is worked on.
 template <bool BF16, int JM>
-__device__ __forceinline__ void steps_tile(const OpState &s, const LevelDesc &Lv, const StripGeom &g, float *v,
+__device__ __forceinline__ void steps_tile(const StepDesc &s, const StripGeom &g, float *v,
                                            TrialScratch<JM> &sh, int lane, unsigned &nexact)
 {
     const unsigned FULL = 0xffffffffu;
     const unsigned lt = (1u << lane) - 1u;
     const int J = min(s.ntr, JM);
     const bool withQ = (s.phase == PH_GRAD);
-    const float4 *V = reinterpret_cast<const float4 *>(Lv.V[s.cur]);
+    const float4 *V = reinterpret_cast<const float4 *>(s.Vc);
+    const void *T = s.T;
     float tau[JM];
     float tmax = 0.f;
 #pragma unroll
     for (int j = 0; j < JM; j++) {
-        tau[j] = (j < J) ? s.f_tau[j] : 0.f;
+        tau[j] = (j < J) ? s.tau[j] : 0.f;
         tmax = fmaxf(tmax, tau[j]);
 #pragma unroll
         for (int k = 0; k < 3; k++) sh.sn[k][j][lane] = 0.f;
@@ -1332,7 +1377,7 @@ __device__ __forceinline__ void steps_tile(const OpState &s, const LevelDesc &Lv
             slow = q.jx < 0 || q.jx > g.n - 2 || q.jy < 0 || q.jy > g.n - 2 || !(ax1 >= 0.f && ax1 < 1.f) ||
                    !(ay1 >= 0.f && ay1 < 1.f);
             if (!slow) {
-                fetch<BF16>(q, Lv.T, g.pitch);
+                fetch<BF16>(q, T, g.pitch);
                 const float dtx = q.t01 - q.t00, dtx1 = q.t11 - q.t10;
                 const float sx = dtx + q.ay * (dtx1 - dtx);                            // dThat/dx
                 const float sy = (q.t10 - q.t00) + q.ax * ((q.t11 - q.t01) - (q.t10 - q.t00));  // dThat/dy
@@ -1387,7 +1432,7 @@ __device__ __forceinline__ void steps_tile(const OpState &s, const LevelDesc &Lv
         }
         nrow++;
         if (nrow == TW || qn > TQ - 32 || qc > TC - 32 || r == g.rEnd) {
-            if (qn > q0 || qc > 0) trial_flush<BF16, JM>(Lv, g, V, tau, J, sh, lane, r, nrow, q0, qn, qc);
+            if (qn > q0 || qc > 0) trial_flush<BF16, JM>(T, g, V, tau, J, sh, lane, r, nrow, q0, qn, qc);
             else {
                 // nothing new queued (so the last row has no exact nodes): only
                 // its A, B move to slot 0
@@ -1468,33 +1513,31 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, 4) k_trial(BatchDev b)
     __shared__ TrialScratch<JM> scratch[REG_STRIP_THREADS / 32];
     const int lane = threadIdx.x & 31;
     const int nwarps = gridDim.x * (REG_STRIP_THREADS / 32);
-    const int nent = b.ctr[3], items = b.ctr[6];
-    for (int item = blockIdx.x * (REG_STRIP_THREADS / 32) + (threadIdx.x >> 5); item < items; item += nwarps) {
-        const int e = find_entry(b.prefT, nent, item);
-        const int o = b.listT[e];
-        const OpState &s = b.st[o];
-        const OpDesc &op = b.ops[o];
-        const LevelDesc &Lv = op.lv[s.lvl];
-        const StripGeom g = strip_geom(Lv, item - b.prefT[e], lane);
+    const WorkPlan wp = work_plan<false>(b, lane);
+    for (int item = blockIdx.x * (REG_STRIP_THREADS / 32) + (threadIdx.x >> 5); item < wp.items; item += nwarps) {
+        int tile;
+        const StepDesc &s = b.st[find_item<false>(b, wp, item, tile)].step;
+        const StripGeom g = strip_geom(s, tile, lane);
+        const int part = s.part0 + tile;
         const bool start = (s.phase == PH_START || s.phase == PH_PROLONG);
         if (start) {
             // sums in double, reduced in double: [0..2] and the Dirichlet form of u
             double v[4];
-            start_tile<BF16>(s, op, Lv, g, v);
+            start_tile<BF16>(s, g, v);
             double mine = 0.0;
 #pragma unroll
             for (int k = 0; k < 4; k++) {
                 const double tot = warp_sum_d(v[k]);
                 if (lane == (k < 3 ? k : 3 * REG_MAX_TRIALS)) mine = tot;
             }
-            if (lane < PT_STRIDE) b.partT[(int64_t)item * PT_STRIDE + lane] = mine;
+            if (lane < PT_STRIDE) b.partT[(int64_t)part * PT_STRIDE + lane] = mine;
         } else {
             float v[PT_STRIDE];
 #pragma unroll
             for (int k = 0; k < PT_STRIDE; k++) v[k] = 0.f;
             unsigned nexact = 0;
-            steps_tile<BF16, JM>(s, Lv, g, v, scratch[threadIdx.x >> 5], lane, nexact);
-            write_partials<JM>(b, item, v, 3 * min(s.ntr, JM), lane);
+            steps_tile<BF16, JM>(s, g, v, scratch[threadIdx.x >> 5], lane, nexact);
+            write_partials<JM>(b, part, v, 3 * min(s.ntr, JM), lane);
             if (lane == 0 && nexact) atomicAdd(&b.work[KW_TEXACT], (unsigned long long)nexact);
         }
     }
@@ -1506,34 +1549,60 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, 4) k_trial(BatchDev b)
 // ---------------------------------------------------------------------------
 namespace {
 
-// An energy's scalars from the FE sums S1 = int That, S2 = int That^2, S3 = int
-// That R~ (R~ normalised: mean 0, FE sigma 1): sigma = sqrt(S2 - S1^2), NCC =
-// S3 / sigma, and the gradient pass's coefficients there.
+// An evaluated energy: the FE sums S1 = int That, S2 = int That^2, S3 = int That
+// R~ (R~ normalised: mean 0, FE sigma 1), sigma = sqrt(S2 - S1^2), NCC = S3 /
+// sigma, the gradient pass's coefficients there, and of a trial the energy
+// change, the Armijo test and the stopping test.
 struct EvalAt {
     double S1, S2, S3, ncc, sig, dE;
     float isig, c36, cT;
+    int acc, conv;
 };
 
+// One reciprocal square root serves sigma, NCC and the coefficients: a double
+// division or square root takes 600-670 cycles on this chip (a multiplication
+// 62), and a chain of five of them was a third of the control kernel.
 __device__ __forceinline__ void eval_at(EvalAt &v, double S1, double S2, double S3)
 {
     const double var = S2 - S1 * S1;
     v.S1 = S1;
     v.S2 = S2;
     v.S3 = S3;
-    v.sig = var > 0.0 ? sqrt(var) : 0.0;
-    v.ncc = S3 / v.sig;
-    v.isig = (float)(1.0 / v.sig);
-    const double q = v.ncc / (v.sig * v.sig);
-    v.c36 = (float)(q / 36.0);
-    v.cT = (float)(q * S1);
+    if (var > 0.0 && var < 1e300) {
+        const double r = rsqrt(var);
+        v.sig = var * r;
+        v.ncc = S3 * r;
+        v.isig = (float)r;
+        const double q = v.ncc * (r * r);
+        v.c36 = (float)(q * (1.0 / 36.0));
+        v.cT = (float)(q * S1);
+    } else {  // no variance, or not finite: no energy
+        v.sig = var > 0.0 ? sqrt(var) : 0.0;
+        v.ncc = S3 / v.sig;
+        v.isig = v.c36 = v.cT = 0.f;
+    }
 }
 
-__device__ void level_end(OpState &s, const OpDesc &op, int status, double pending)
+// Positive doubles compare like their bits, and doubling one adds to its
+// exponent field: the step sizes of the search stay off the slow FP64 pipe.
+// (Numbers near the ends of the exponent range take the multiplication.)
+__device__ __forceinline__ double pow2_scale(double x, int e, double f)
+{
+    const long long w = __double_as_longlong(x);
+    const int ex = (int)(w >> 52);
+    return ex >= 2 && ex <= 0x7fc ? __longlong_as_double(w + ((long long)e << 52)) : x * f;
+}
+__device__ __forceinline__ double twice(double x) { return pow2_scale(x, 1, 2.0); }
+__device__ __forceinline__ double half_of(double x) { return pow2_scale(x, -1, 0.5); }
+__device__ __forceinline__ bool pos_le(double a, double b) { return __double_as_longlong(a) <= __double_as_longlong(b); }
+__device__ __forceinline__ bool pos_eq(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
+
+__device__ __forceinline__ void level_end(OpState &s, const OpDesc &op, int status, double pending)
 {
     if (status == OPST_NONFINITE) s.nonfinite_seen = 1;
     s.status = status;
     s.tau_acc = pending;
-    s.f_tau_acc = (float)pending;
+    s.step.tau_acc = (float)pending;
     s.src = s.cur;
     if (s.lvl < op.nl - 1) {
         s.phase = PH_PROLONG;
@@ -1558,74 +1627,68 @@ __device__ __forceinline__ int lock_count(const OpState &s, const OpDesc &op)
 __device__ __forceinline__ void set_trial(OpState &s, int k, double t)
 {
     s.trial_tau[k] = t;
-    s.f_tau[k] = (float)t;
+    s.step.tau[k] = (float)t;
 }
 
-__device__ void set_init_trials(OpState &s, const BatchDev &b, const OpDesc &op)
+__device__ __forceinline__ void schedule_grad(OpState &s, const BatchDev &b, const OpDesc &op, double pending)
 {
+    s.phase = PH_GRAD;
+    s.tau_acc = pending;
+    s.step.tau_acc = (float)pending;
+    s.src = s.cur;
+    s.cur = 1 - s.cur;
+    s.search = SEARCH_INIT;
     if (op.lock_tau) {
         // replay: the one step size the reference sequence accepted here
         set_trial(s, 0, lock_step(s, op));
         s.ntr = 1;
-        s.search = SEARCH_INIT;
         return;
     }
     // sequential Armijo order: tau, then 2 tau (if accepted), else tau/2; the
     // pass covers the most likely continuations of both branches.
-    int J = b.J;
+    const int J = b.J;
     int k = 0;
     double up = s.tau, dn = s.tau;
     set_trial(s, k++, up);
     while (k < J) {
-        if (2.0 * up <= b.tau_max) { up *= 2.0; set_trial(s, k++, up); }
-        if (k < J && 0.5 * dn >= b.tau_min) { dn *= 0.5; set_trial(s, k++, dn); }
-        if (2.0 * up > b.tau_max && 0.5 * dn < b.tau_min) break;
+        const double u2 = twice(up), d2 = half_of(dn);
+        const bool canUp = pos_le(u2, b.tau_max), canDn = pos_le(b.tau_min, d2);
+        if (!canUp && !canDn) break;
+        if (canUp) { up = u2; set_trial(s, k++, up); }
+        if (k < J && canDn) { dn = d2; set_trial(s, k++, dn); }
     }
     s.ntr = k;
-    s.search = SEARCH_INIT;
 }
 
-__device__ void schedule_grad(OpState &s, const BatchDev &b, const OpDesc &op, double pending)
-{
-    s.phase = PH_GRAD;
-    s.tau_acc = pending;
-    s.f_tau_acc = (float)pending;
-    s.src = s.cur;
-    s.cur = 1 - s.cur;
-    set_init_trials(s, b, op);
-}
-
-// The scalars at the new u: of a level start, or of the accepted trial.
-__device__ __forceinline__ void take_eval(OpState &s, const EvalAt &v)
-{
-    s.S1 = v.S1; s.S2 = v.S2; s.S3 = v.S3;
-    s.Tbar = v.S1;
-    s.sigT = v.sig;
-    s.ncc = v.ncc;
-    s.f_isig = v.isig; s.f_c36 = v.c36; s.f_cT = v.cT;
-}
-
-__device__ __forceinline__ void trace_trial(const BatchDev &b, const OpState &s, int o, int n, double want, double dE,
-                                            bool acc)
+__device__ __forceinline__ void trace_trial(const BatchDev &b, const OpState &s, int o, int n, double want,
+                                            const EvalAt &v)
 {
     if (!b.trace) return;
     unsigned long long k = atomicAdd(b.trace_len, 1ull);
     if ((long long)k < b.trace_cap) {
         double *rec = b.trace + 7 * k;
         rec[0] = o; rec[1] = n; rec[2] = s.iter - 1; rec[3] = want;
-        rec[4] = dE; rec[5] = b.sigma * want * s.slope; rec[6] = acc;
+        rec[4] = v.dE; rec[5] = b.sigma * want * s.slope; rec[6] = v.acc;
     }
 }
 
-// The Armijo state machine of one operator after a step (one thread; s in shared
-// memory).  ev: the evaluated trials' scalars, or ev[0] those of a level start.
-__device__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int o, int n, double h2, const EvalAt *ev,
-                           double quu, double slope)
+// The Armijo state machine of one operator after a step (one thread; s and op in
+// shared memory).  ev: the evaluated trials, or ev[0] the level's start (dE: its
+// energy).  sgn: 1 the slope of a new search is negative, 0 it is zero, -1 else.
+__device__ __forceinline__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int o, int n,
+                                           const EvalAt *ev, double slope, int sgn)
 {
     const int ph = s.phase;
+    auto take = [&](const EvalAt &v) {
+        s.S1 = v.S1; s.S2 = v.S2; s.S3 = v.S3;
+        s.Tbar = v.S1;
+        s.sigT = v.sig;
+        s.ncc = v.ncc;
+        s.step.isig = v.isig; s.step.c36 = v.c36; s.step.cT = v.cT;
+    };
     if (ph == PH_START || ph == PH_PROLONG) {
-        take_eval(s, ev[0]);
-        s.E = -s.ncc + 0.5 * b.lambda * h2 * quu;
+        take(ev[0]);
+        s.E = ev[0].dE;
         s.iter = 0;
         s.tau = b.tau_init;
         s.evals += 1;
@@ -1638,8 +1701,8 @@ __device__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int 
         s.iter += 1;
         s.iters_total += 1;
         s.slope = slope;
-        if (!(slope < 0.0)) {
-            level_end(s, op, slope == 0.0 ? OPST_ZERO_GRAD : OPST_NONFINITE, 0.0);
+        if (sgn != 1) {
+            level_end(s, op, sgn == 0 ? OPST_ZERO_GRAD : OPST_NONFINITE, 0.0);
             return;
         }
     }
@@ -1651,98 +1714,97 @@ __device__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int 
         const double want = s.trial_tau[0];
         s.trials_seq += 1;
         atomicAdd(&b.work[KW_TSEQ], nn);
-        trace_trial(b, s, o, n, want, ev[0].dE, ev[0].dE <= b.sigma * want * s.slope);
+        trace_trial(b, s, o, n, want, ev[0]);
         s.E += ev[0].dE;
-        take_eval(s, ev[0]);
+        take(ev[0]);
         s.tau = want;
         if (s.iter >= lock_count(s, op)) level_end(s, op, OPST_MAXITER, want);
         else schedule_grad(s, b, op, want);
         return;
     }
     // Walk the sequential Armijo search over the step sizes evaluated this pass.
-    for (int guard = 0; guard < 4 * REG_MAX_TRIALS + 8; guard++) {
-        double want;
-        if (s.search == SEARCH_INIT) want = s.tau;
-        else if (s.search == SEARCH_WIDEN) want = 2.0 * s.btau;
-        else want = 0.5 * s.sh_tau;
-        bool finish = false, stall = false;
-        if (s.search == SEARCH_WIDEN && want > b.tau_max) finish = true;
-        if (s.search == SEARCH_SHRINK && want < b.tau_min) stall = true;
-        if (!finish && !stall) {
-            int j = -1;
-            for (int k = 0; k < s.ntr; k++)
-                if (s.trial_tau[k] == want) { j = k; break; }
-            if (j < 0) {
-                // continue the search in another pass
-                int k = 0;
-                double t = want;
-                if (s.search == SEARCH_WIDEN) {
-                    while (k < b.J && t <= b.tau_max) { set_trial(s, k++, t); t *= 2.0; }
-                } else {
-                    while (k < b.J && t >= b.tau_min) { set_trial(s, k++, t); t *= 0.5; }
-                }
-                s.ntr = k;
-                s.phase = PH_TRIAL;
-                return;
-            }
-            // energy change E(u + tau d) - E(u) from the accumulated sums at u
-            const EvalAt &v = ev[j];
-            s.trials_seq += 1;
-            atomicAdd(&b.work[KW_TSEQ], nn);
-            const bool acc = (v.dE <= b.sigma * want * s.slope);
-            trace_trial(b, s, o, n, want, v.dE, acc);
-            if (acc) {
-                s.bS1 = v.S1; s.bS2 = v.S2; s.bS3 = v.S3; s.bncc = v.ncc; s.bdE = v.dE;
-                s.bsig = v.sig;
-                s.b_isig = v.isig; s.b_c36 = v.c36; s.b_cT = v.cT;
-            }
-            if (s.search == SEARCH_INIT) {
-                if (acc) { s.search = SEARCH_WIDEN; s.btau = want; }
-                else { s.search = SEARCH_SHRINK; s.sh_tau = want; }
-                continue;
-            }
-            if (s.search == SEARCH_WIDEN) {
-                if (acc) { s.btau = want; continue; }
-                finish = true;
+    const int ntr = s.ntr;
+    int search = s.search, seq = 0, best = -1;  // best: the last trial accepted in this pass
+    double btau = s.btau, sh_tau = s.sh_tau;
+    bool finish = false, stall = false;
+    int guard = 0;
+    for (; guard < 4 * REG_MAX_TRIALS + 8 && !finish && !stall; guard++) {
+        const double want = search == SEARCH_INIT ? s.tau : (search == SEARCH_WIDEN ? twice(btau) : half_of(sh_tau));
+        if (search == SEARCH_WIDEN && !pos_le(want, b.tau_max)) { finish = true; break; }
+        if (search == SEARCH_SHRINK && !pos_le(b.tau_min, want)) { stall = true; break; }
+        int j = -1;
+        for (int k = 0; k < ntr; k++)
+            if (pos_eq(s.trial_tau[k], want)) { j = k; break; }
+        if (j < 0) {
+            // continue the search in another pass
+            int k = 0;
+            double t = want;
+            if (search == SEARCH_WIDEN) {
+                while (k < b.J && pos_le(t, b.tau_max)) { set_trial(s, k++, t); t = twice(t); }
             } else {
-                if (acc) { s.btau = want; finish = true; }
-                else { s.sh_tau = want; continue; }
+                while (k < b.J && pos_le(b.tau_min, t)) { set_trial(s, k++, t); t = half_of(t); }
             }
+            s.ntr = k;
+            s.phase = PH_TRIAL;
+            break;
         }
-        if (stall) {
-            level_end(s, op, OPST_STALLED, 0.0);
-            return;
-        }
-        if (finish) {
-            double dec = -s.bdE;
-            double scale = fabs(s.E) > 1.0 ? fabs(s.E) : 1.0;
-            s.E += s.bdE;
-            s.S1 = s.bS1; s.S2 = s.bS2; s.S3 = s.bS3;
-            s.Tbar = s.S1;
-            s.sigT = s.bsig;
-            s.ncc = s.bncc;
-            s.f_isig = s.b_isig; s.f_c36 = s.b_c36; s.f_cT = s.b_cT;
-            s.tau = s.btau;
-            if (dec < b.eps * scale) level_end(s, op, OPST_CONVERGED, s.btau);
-            else if (s.iter >= b.iter_max) level_end(s, op, OPST_MAXITER, s.btau);
-            else schedule_grad(s, b, op, s.btau);
-            return;
+        seq++;
+        trace_trial(b, s, o, n, want, ev[j]);
+        const bool acc = ev[j].acc != 0;
+        if (acc) best = j;
+        if (search == SEARCH_SHRINK) {
+            if (acc) { btau = want; finish = true; }
+            else sh_tau = want;
+        } else if (acc) {
+            search = SEARCH_WIDEN;
+            btau = want;
+        } else if (search == SEARCH_INIT) {
+            search = SEARCH_SHRINK;
+            sh_tau = want;
+        } else {
+            finish = true;
         }
     }
-    atomicExch(&b.ctr[8], 1);  // the search did not terminate: internal error
-    s.phase = PH_DONE;
+    s.trials_seq += seq;
+    if (seq) atomicAdd(&b.work[KW_TSEQ], nn * seq);
+    if (best >= 0) {
+        const EvalAt &v = ev[best];
+        s.bS1 = v.S1; s.bS2 = v.S2; s.bS3 = v.S3; s.bncc = v.ncc; s.bdE = v.dE;
+        s.bsig = v.sig;
+        s.b_isig = v.isig; s.b_c36 = v.c36; s.b_cT = v.cT;
+        s.b_conv = v.conv;
+    }
+    s.search = search;
+    s.btau = btau;
+    s.sh_tau = sh_tau;
+    if (stall) {
+        level_end(s, op, OPST_STALLED, 0.0);
+    } else if (finish) {
+        s.E += s.bdE;
+        s.S1 = s.bS1; s.S2 = s.bS2; s.S3 = s.bS3;
+        s.Tbar = s.bS1;
+        s.sigT = s.bsig;
+        s.ncc = s.bncc;
+        s.step.isig = s.b_isig; s.step.c36 = s.b_c36; s.step.cT = s.b_cT;
+        s.tau = btau;
+        if (s.b_conv) level_end(s, op, OPST_CONVERGED, btau);
+        else if (s.iter >= b.iter_max) level_end(s, op, OPST_MAXITER, btau);
+        else schedule_grad(s, b, op, btau);
+    } else if (s.phase != PH_TRIAL || guard >= 4 * REG_MAX_TRIALS + 8) {
+        atomicExch(&b.ctr[8], 1);  // the search did not terminate: internal error
+        s.phase = PH_DONE;
+    }
 }
 
 }  // namespace
 
 // One block per operator (grid stride): the block sums the operator's tile
-// partials in FP64, the lanes of a warp form the scalars of all evaluated trials
-// side by side (FP64 square roots and divisions are slow here: one after the
-// other in one thread they were most of the kernel), thread 0 runs the state
-// machine on a copy of the state in shared memory, and the last block to finish
-// plans the next step.  Latency bound at every size: 22 us as one thread working
-// in global memory after a 9-way split of the records, plus 6 us for a plan
-// kernel of its own (33 x 1024^2 scan).
+// partials in FP64, the lanes of a warp evaluate all trials side by side, and
+// thread 0 runs the state machine on copies of the state and the descriptor in
+// shared memory.  Batches of more than PLAN_WARP operators: the last block to
+// finish makes the lists of the next step (narrower ones need none).  Latency
+// bound at every size; what was spent was chains of FP64 operations (62 cycles
+// each, 600 and more for a square root or a division) and of dependent loads.
 //
 // The sums: thread (g, kk) adds entry kk of every ng-th record (kk fastest, so a
 // warp reads neighbouring doubles), only the entries that the pass wrote: 3 per
@@ -1751,29 +1813,31 @@ __device__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int 
 __global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
 {
     constexpr int NW = REG_CTL_THREADS / 32;
-    __shared__ OpState s;
+    constexpr int NS = sizeof(OpState) / 8, ND = sizeof(OpDesc) / 8;
+    static_assert(sizeof(OpState) % 8 == 0 && sizeof(OpDesc) % 8 == 0 && NS + ND <= REG_CTL_THREADS,
+                  "state and descriptor copied in one pass");
+    __shared__ __align__(16) double sbuf[NS], dbuf[ND];
     __shared__ double red[REG_CTL_THREADS + 32];
     __shared__ double redG[NW][2];
     __shared__ double S[32];
     __shared__ double SG[2];
     __shared__ EvalAt ev[REG_MAX_TRIALS];
     __shared__ int last;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    OpState &s = *reinterpret_cast<OpState *>(sbuf);
+    const OpDesc &op = *reinterpret_cast<const OpDesc *>(dbuf);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int n_ops = b.ctr[0];
     if ((int)blockIdx.x >= n_ops) return;
     for (int o = blockIdx.x; o < n_ops; o += gridDim.x) {
-        const OpDesc &op = b.ops[o];
-        static_assert(sizeof(OpState) % 8 == 0 && sizeof(OpState) / 8 <= REG_CTL_THREADS, "state copied by one pass");
-        if (threadIdx.x < sizeof(OpState) / 8)
-            reinterpret_cast<double *>(&s)[threadIdx.x] = reinterpret_cast<const double *>(b.st + o)[threadIdx.x];
+        if (tid < NS) sbuf[tid] = reinterpret_cast<const double *>(b.st + o)[tid];
+        else if (tid < NS + ND) dbuf[tid - NS] = reinterpret_cast<const double *>(b.ops + o)[tid - NS];
         __syncthreads();
         const int ph = s.phase;
         if (ph != PH_DONE) {
-            const LevelDesc &Lv = op.lv[s.lvl];
-            const int n = Lv.n, ntr = s.ntr;
-            const double h2 = Lv.h2d;
+            const int n = s.step.n, ntr = s.ntr;
+            const double h2 = op.lv[s.lvl].h2d;
             const bool start = ph == PH_START || ph == PH_PROLONG;
-            if (threadIdx.x == REG_CTL_THREADS - 1) {
+            if (tid == REG_CTL_THREADS - 1) {
                 // algorithmic work of this step (nodes of the level each kernel swept)
                 const unsigned long long nn = (unsigned long long)n * n;
                 if (ph == PH_PROLONG) atomicAdd(&b.work[KW_PPROL], nn);
@@ -1785,36 +1849,39 @@ __global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
                 }
             }
             const int lg = b.J <= 4 ? 4 : 5, ng = REG_CTL_THREADS >> lg;
-            const int kk = threadIdx.x & ((1 << lg) - 1), g = threadIdx.x >> lg;
+            const int kk = tid & ((1 << lg) - 1), g = tid >> lg;
             // entries 0 .. ne-2 of a record, then the Dirichlet form: of u
             // (level start) or of d (first pass of a search)
             const int ne = (start ? 3 : 3 * ntr) + 1;
             if (kk < ne) {
-                const double *rec = b.partT + (kk < ne - 1 ? kk : 3 * REG_MAX_TRIALS + (start ? 0 : 2));
-                const int te = s.t_end;
-                double acc = 0.0;
-#pragma unroll 8
-                for (int it = s.t_begin + g; it < te; it += ng) acc += rec[(int64_t)it * PT_STRIDE];
-                red[kk * (ng + 1) + g] = acc;
+                const double *rec = b.partT + (int64_t)op.part0 * PT_STRIDE +
+                                    (kk < ne - 1 ? kk : 3 * REG_MAX_TRIALS + (start ? 0 : 2));
+                const int nt = s.tT;
+                double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0, acc3 = 0.0;
+                int it = g;
+#pragma unroll 2
+                for (; it + 3 * ng < nt; it += 4 * ng) {
+                    acc0 += rec[(int64_t)it * PT_STRIDE];
+                    acc1 += rec[(int64_t)(it + ng) * PT_STRIDE];
+                    acc2 += rec[(int64_t)(it + 2 * ng) * PT_STRIDE];
+                    acc3 += rec[(int64_t)(it + 3 * ng) * PT_STRIDE];
+                }
+                if (it < nt) acc0 += rec[(int64_t)it * PT_STRIDE];
+                if (it + ng < nt) acc1 += rec[(int64_t)(it + ng) * PT_STRIDE];
+                if (it + 2 * ng < nt) acc2 += rec[(int64_t)(it + 2 * ng) * PT_STRIDE];
+                red[kk * (ng + 1) + g] = (acc0 + acc1) + (acc2 + acc3);
             }
-            double slope = 0.0, qud = 0.0;
             if (ph == PH_GRAD) {
-                if (b.smooth) {
-                    // the smoothed direction's slope and u^T K d (smoother partials)
-                    const double *pS = b.partS + (int64_t)s.g_entry * b.cch * 2;
-                    const int nch = (n + REG_GW - 1) / REG_GW;
-                    for (int ch = threadIdx.x; ch < nch; ch += REG_CTL_THREADS) {
-                        slope += pS[2 * ch];
-                        qud += pS[2 * ch + 1];
-                    }
-                } else {
-                    const int ge = s.g_end;
+                double slope = 0.0, qud = 0.0;
+                // the gradient pass's tiles, or the smoother's column chunks
+                const double2 *p = b.smooth ? reinterpret_cast<const double2 *>(b.partS) + (int64_t)o * b.cch
+                                            : reinterpret_cast<const double2 *>(b.partG) + op.part0;
+                const int np = b.smooth ? (n + REG_GW - 1) / REG_GW : s.tG;
 #pragma unroll 4
-                    for (int it = s.g_begin + threadIdx.x; it < ge; it += REG_CTL_THREADS) {
-                        const double2 p = reinterpret_cast<const double2 *>(b.partG)[it];
-                        slope += p.x;
-                        qud += p.y;
-                    }
+                for (int it = tid; it < np; it += REG_CTL_THREADS) {
+                    const double2 v = p[it];
+                    slope += v.x;
+                    qud += v.y;
                 }
                 slope = warp_sum_d(slope);
                 qud = warp_sum_d(qud);
@@ -1828,46 +1895,56 @@ __global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
                 const double v = warp_sum_d(lane < ng ? red[k * (ng + 1) + lane] : 0.0);
                 if (lane == 0) S[k] = v;
             }
-            if (ph == PH_GRAD && wid == NW - 1) {
-                const double v = warp_sum_d(lane < NW ? redG[lane][0] : 0.0);
-                const double w = warp_sum_d(lane < NW ? redG[lane][1] : 0.0);
-                if (lane == 0) {
-                    SG[0] = b.smooth ? -h2 * h2 * v : v;
-                    SG[1] = w;
-                }
+            if (ph == PH_GRAD && wid >= NW - 2) {
+                // (the two last warps have no entry of a pass with four step sizes)
+                const int w = wid - (NW - 2);
+                const double v = warp_sum_d(lane < NW ? redG[lane][w] : 0.0);
+                if (lane == 0) SG[w] = w == 0 && b.smooth ? -h2 * h2 * v : v;
             }
             __syncthreads();
             if (wid == 0) {
-                if (ph == PH_GRAD && lane == 0) {
-                    // the Dirichlet forms of the new search: u^T K d from the gradient
-                    // pass (or the smoother), d^T K d from its first trial pass
-                    s.Qud = SG[1];
-                    s.Qdd = S[ne - 1];
-                }
-                __syncwarp();
+                // the Dirichlet forms of the search: u^T K d from the gradient pass
+                // (or the smoother), d^T K d from its first trial pass
+                const double Qud = ph == PH_GRAD ? SG[1] : s.Qud, Qdd = ph == PH_GRAD ? S[ne - 1] : s.Qdd;
+                const double slope = ph == PH_GRAD ? SG[0] : s.slope;
                 if (start) {
-                    if (lane == 0) eval_at(ev[0], h2 * S[0], h2 * S[1], h2 * S[2]);
+                    if (lane == 0) {
+                        eval_at(ev[0], h2 * S[0], h2 * S[1], h2 * S[2]);
+                        ev[0].dE = -ev[0].ncc + 0.5 * b.lambda * h2 * S[3];
+                    }
                 } else if (lane < ntr) {
                     EvalAt v;
-                    const double want = s.trial_tau[lane];
+                    const double want = s.trial_tau[lane], E = s.E;
+                    const double reg = 0.5 * b.lambda * h2 * (2.0 * want * Qud + want * want * Qdd);
+                    const double bound = b.sigma * want * slope, stop = b.eps * (fabs(E) > 1.0 ? fabs(E) : 1.0);
                     eval_at(v, s.S1 + h2 * S[3 * lane], s.S2 + h2 * S[3 * lane + 1], s.S3 + h2 * S[3 * lane + 2]);
-                    v.dE = -(v.ncc - s.ncc) + 0.5 * b.lambda * h2 * (2.0 * want * s.Qud + want * want * s.Qdd);
+                    // energy change E(u + tau d) - E(u) from the accumulated sums at u
+                    v.dE = -(v.ncc - s.ncc) + reg;
+                    v.acc = v.dE <= bound;
+                    v.conv = -v.dE < stop;
                     ev[lane] = v;
                 }
                 __syncwarp();
                 if (lane == 0) {
-                    control_op(b, s, op, o, n, h2, ev, S[ne - 1], SG[0]);
-                    b.plan[o] = op_plan(s, op);
+                    if (ph == PH_GRAD) {
+                        s.Qud = Qud;
+                        s.Qdd = Qdd;
+                    }
+                    control_op(b, s, op, o, n, ev, slope, slope < 0.0 ? 1 : (slope == 0.0 ? 0 : -1));
+                    set_step(s, op);
+                    b.plan[o] = make_int2(s.tG, s.tT);
+                    if (s.phase == PH_DONE) atomicAdd(&b.ctr[7], -1);
                 }
             }
             __syncthreads();
-            if (threadIdx.x < sizeof(OpState) / 8)
-                reinterpret_cast<double *>(b.st + o)[threadIdx.x] = reinterpret_cast<const double *>(&s)[threadIdx.x];
+            if (tid < NS) reinterpret_cast<double *>(b.st + o)[tid] = sbuf[tid];
         }
         __syncthreads();
     }
-    // the last block plans: its reads of the other blocks' entries follow their fences
-    if (threadIdx.x == 0) {
+    if (n_ops <= PLAN_WARP) return;
+    // the last block makes the lists: its reads of the other blocks' entries follow
+    // their fences
+    if (tid == 0) {
         __threadfence();
         last = atomicAdd(&b.ctr[9], 1) == min((int)gridDim.x, n_ops) - 1;
     }
@@ -1875,7 +1952,7 @@ __global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
     if (!last) return;
     __threadfence();
     plan_lists(b);
-    if (threadIdx.x == 0) b.ctr[9] = 0;
+    if (tid == 0) b.ctr[9] = 0;
 }
 
 // ---------------------------------------------------------------------------

@@ -62,6 +62,7 @@ struct LevelDesc {
     int n;            // nodes per side (2^l + 1)
     int pitch;        // row pitch in elements (float2 for U/D, scalar for images)
     int hg, ht;       // strip rows of the gradient and trial tiles at this level
+    int tg, tt;       // tiles of a gradient and a trial pass at this level
     float h2;         // h^2 = 4^-l (as float for scaling, exact)
     double h2d;       // h^2 in double
     const void *R;    // normalised reference frame (mean 0, FE sigma 1) at this level
@@ -79,6 +80,7 @@ struct OpDesc {
     float2 *out;            // destination slot (finest level)
     int slot_pitch;
     int judge;              // the output slot holds a learned start: measure the correction
+    int part0;              // first of the operator's tile records in partG and partT
     // Lockstep replay (diagnostic; null: free-running search).  Level k
     // (0 = coarsest) takes exactly the accepted step sizes
     // lock_tau[lock_off[k] .. lock_off[k+1]), one per gradient iteration, and
@@ -88,12 +90,30 @@ struct OpDesc {
     LevelDesc lv[REG_MAX_LEVELS];  // index 0 = coarsest level m0
 };
 
+// What the gradient and trial passes of a step read of an operator, gathered by
+// the control kernel in two cache lines: the passes reach their first node
+// records three dependent loads after their start (plan, this, record), and the
+// scalars are rounded to float once per step instead of once per tile.
+struct __align__(16) StepDesc {
+    const void *T;       // template at the level
+    const float *MR;
+    const NodeRec *Vs;   // records before the gradient pass (or the only ones of a level start)
+    NodeRec *Vc;         // records the gradient pass writes and the trial pass reads
+    const NodeRec *VC;   // PH_PROLONG: the coarser level's records
+    int cpitch;          // and their pitch
+    int phase, n, pitch, hg, ht, ntr, part0;
+    float ih2;           // 1 / h^2 (exact: a power of two)
+    float tau_acc;       // pending step
+    float isig, c36, cT; // 1 / sigma, NCC / sigma^2 / 36, NCC / sigma^2 T_bar at u
+    float tau[REG_MAX_TRIALS];  // step sizes of the trial pass
+};
+
 struct OpState {
+    StepDesc step;
     int phase, lvl, cur, src;
     int iter, iters_total, trials_seq, evals;
     int status, nonfinite_seen, search, ntr;
-    int t_begin, t_end, g_begin, g_end;
-    int g_entry;      // index in the gradient pass's op list of this step (smoother partials)
+    int tG, tT;       // gradient and trial tiles of this step
     double tau;       // base step of the current search
     double tau_acc;   // step to apply at the start of the next G/P pass
     double sh_tau;    // shrinking: last rejected step
@@ -104,12 +124,10 @@ struct OpState {
     double slope;
     double Qud, Qdd;  // Dirichlet forms u^T K d and d^T K d of the current search
     double trial_tau[REG_MAX_TRIALS];
-    // What the gradient and trial passes read, rounded once per step by the
-    // control kernel instead of once per tile: the pending step, the step sizes
-    // of the pass, and 1 / sigma, NCC / sigma^2 / 36, NCC / sigma^2 T_bar at u
-    // (b*: of the last accepted trial of the search).
-    float f_tau_acc, f_isig, f_c36, f_cT, b_isig, b_c36, b_cT, f_pad;
-    float f_tau[REG_MAX_TRIALS];
+    // of the last accepted trial of the search: the gradient pass's coefficients
+    // there, and whether its energy decrease meets the stopping rule
+    float b_isig, b_c36, b_cT;
+    int b_conv;
     double corr;  // judged ops: sum over finest nodes of |u_final - u_start| (x + y, px)
 };
 
@@ -119,13 +137,13 @@ struct OpState {
 struct BatchDev {
     OpDesc *ops;
     OpState *st;
-    int *listG, *listT;          // compacted op indices per family
-    int *prefG, *prefT;          // exclusive prefix of tile counts (n+1 entries)
-    int4 *plan;                  // per op: {gradient tiles, trial tiles, active, -} of the next step
+    int2 *plan;                  // per op: {gradient tiles, trial tiles} of the next step
+    int *listG, *listT;          // batches of more than 32 ops: compacted op indices per family
+    int *prefG, *prefT;          // and exclusive prefix of tile counts (n+1 entries)
     int *ctr;                    // [0] n_ops [2] nG [3] nT [5] itemsG [6] itemsT [7] n_active
                                  // [8] error flag [9] blocks of the control kernel that are done
-    double *partG;               // per G item: slope and u^T K d partials (PG_STRIDE)
-    double *partT;               // per T item: 3 sums per step size, then 3 Dirichlet forms (PT_STRIDE)
+    double *partG;               // per gradient tile: slope and u^T K d partials (PG_STRIDE)
+    double *partT;               // per trial tile: 3 sums per step size, then 3 Dirichlet forms (PT_STRIDE)
     unsigned long long *work;    // per kernel family: nodes processed
     double *trace;               // optional Armijo trial records (7 doubles each)
     unsigned long long *trace_len;
@@ -133,7 +151,7 @@ struct BatchDev {
     double lambda, sigma, tau_init, tau_max, tau_min, eps;
     float lam6;                  // lambda / 6
     int iter_max, J, bf16;
-    // H1-type smoother (smooth != 0): per gradient-pass op and column chunk of
+    // H1-type smoother (smooth != 0): per op and column chunk of
     // REG_GW columns, the partial sums {sum omega d_L2 . d, sum d . 6 K u}
     double *partS;
     int smooth, rch, cch;  // row chunks of 32 and column chunks of REG_GW per op (maxima)
