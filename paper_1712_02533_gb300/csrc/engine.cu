@@ -34,7 +34,9 @@ __global__ void k_plan(BatchDev);
 __global__ void k_final(BatchDev);
 void launch_grad(int bf16, int grid, cudaStream_t st, const BatchDev &b);
 void launch_trial(int bf16, int J, int grid, cudaStream_t st, const BatchDev &b);
-void launch_smooth(int grid, cudaStream_t st, const BatchDev &b);
+void launch_smooth(int nsm, int ops, int n, cudaStream_t st, const BatchDev &b);
+int smooth_row_chunks(int n);
+int smooth_prepare();
 int step_blocks_per_sm(int which, int J);
 __global__ void k_control(BatchDev);
 __global__ void k_slot_to_planes(const float2 *, int, int, float *);
@@ -192,7 +194,7 @@ struct reg_series {
     // H1-type smoother: Thomas pivots per level l (2^l + 1 nodes), partial sums
     float2 *d_smtab[REG_TILE_LEVELS] = {nullptr};
     double *d_partS = nullptr;
-    int sm_rch = 0, sm_cch = 0, grid_S = 0;
+    int sm_rch = 0, sm_cch = 0, sm_n = 0;  // row and column chunks per op, largest level
     // rigid variant buffers
     RigidLevel *d_rlv = nullptr, *h_rlv = nullptr;
     RigidReq *d_rreq = nullptr, *h_rreq = nullptr;
@@ -402,7 +404,7 @@ reg_status build_graph(reg_series *s)
     CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < GRAPH_STEPS; k++) {
         launch_grad(s->bf16, s->grid_G, cs, b);
-        if (b.smooth) launch_smooth(s->grid_S, cs, b);
+        if (b.smooth) launch_smooth(s->nsm, s->cap_ops, s->sm_n, cs, b);
         launch_trial(s->bf16, s->p.trials_per_pass, s->grid_T, cs, b);
         k_control<<<std::min(s->cap_ops, 2048), REG_CTL_THREADS, 0, cs>>>(b);
     }
@@ -561,7 +563,7 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
             for (int k = 0; k < GRAPH_STEPS; k++) {
                 cudaEventRecord(s->ev[k][F_G], s->stream);
                 launch_grad(s->bf16, s->grid_G, s->stream, b);
-                if (b.smooth) launch_smooth(s->grid_S, s->stream, b);  // timed with the gradient family
+                if (b.smooth) launch_smooth(s->nsm, s->cap_ops, s->sm_n, s->stream, b);  // timed with the gradient family
                 cudaEventRecord(s->ev[k][F_T], s->stream);
                 launch_trial(s->bf16, s->p.trials_per_pass, s->grid_T, s->stream, b);
                 cudaEventRecord(s->ev[k][F_C], s->stream);
@@ -1153,9 +1155,10 @@ reg_status reg_create_series(const float *frames, int32_t n_series, const int32_
                     return cleanup(fail(REG_ECUDA, "smoother table upload"));
                 if (cudaStreamSynchronize(s->stream) != cudaSuccess) return cleanup(fail(REG_ECUDA, "sync"));
             }
-        s->sm_rch = cdiv(nmax, 32);
+        s->sm_n = nmax;
+        s->sm_rch = smooth_row_chunks(nmax);
         s->sm_cch = cdiv(nmax, REG_GW);
-        s->grid_S = s->nsm * 8;
+        if (smooth_prepare() != 0) return cleanup(fail(REG_ECUDA, "smoother shared memory"));
     }
     // Pyramid construction in chunks of frames: raw level L, restriction chain,
     // per-level FE mean/sigma, normalisation into the stored pyramid.  The

@@ -749,138 +749,287 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, 8) k_grad(BatchDev b)
 // solve along every row, then one along every column (Thomas elimination
 // with the level's precomputed pivots).  The previous iterate's node records
 // (not read again before the next gradient pass overwrites them) hold the
-// intermediate fields.
+// intermediate fields: the row solutions in u.x, u.y, 6 K u in d, the columns'
+// elimination in mt, mr.
+//
+// The sweeps are serial chains of two or three FP32 operations per element.  With
+// their loads in the chain (each element read from global memory when its turn
+// came) a row took 145 us and a column 192 us at 257^2; here the elements come
+// from shared memory, filled ahead by whole-warp copies: 236 -> 42 us for the
+// gradient pass and both smoother passes of a step (5 operators of 257^2 and
+// coarser levels), 263 -> 63 ms for a 6 x 256^2 scan.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float2 *sm_scratch(NodeRec *V, int64_t idx, int k)
-{
-    return reinterpret_cast<float2 *>(&V[idx].u) + k;  // k = 0: u.x, u.y; k = 1: u.z, u.w
-}
+namespace {
 
-// Rows: lane = one row of one operator, sequential over its columns.
-__global__ void __launch_bounds__(128) k_smooth_rows(BatchDev b)
+__device__ __forceinline__ float2 *sm_x(NodeRec *V, int64_t idx) { return reinterpret_cast<float2 *>(&V[idx].u); }
+__device__ __forceinline__ float2 *sm_y(NodeRec *V, int64_t idx) { return reinterpret_cast<float2 *>(&V[idx].mt); }
+
+constexpr int SM_BATCH = 8;     // elements of a sweep held in registers at a time
+constexpr int SM_RING = 32;     // rows of the column sweeps' ring, filled SM_GROUP at a time
+constexpr int SM_GROUP = 8;
+
+// Rows per block of the row pass: what fits 131 KB of shared memory at a side of
+// n nodes, at most 16 (one warp sweeps 16 rows x 2 components).
+__host__ __device__ __forceinline__ int smooth_row_chunk(int n) { return n <= 1025 ? 16 : (n <= 2049 ? 8 : 4); }
+
+__device__ __forceinline__ void copy_async8(void *dst, const void *src)
 {
-    const int lane = threadIdx.x & 31;
-    const int nwarps = gridDim.x * 4, n_ops = b.ctr[0];
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+__device__ __forceinline__ void copy_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N)); }
+
+}  // namespace
+
+// Rows: a block holds smooth_row_chunk(n) rows of one operator in shared memory.
+// Warp 0 sweeps them (lane = row and component: with n = 2^l + 1 the 32 lanes hit
+// 32 banks) while the other warps form 6 K u of the same rows for the column
+// pass (strips of 30 columns and a halo, by the gradient pass's integer
+// stencils, hi and lo parts of u differenced separately).
+__global__ void __launch_bounds__(256) k_smooth_rows(BatchDev b)
+{
+    extern __shared__ __align__(16) float2 smem_rows[];
+    const unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int n_ops = b.ctr[0];
     const float a = b.sm_a;
-    for (int it = blockIdx.x * 4 + (threadIdx.x >> 5); it < n_ops * b.rch; it += nwarps) {
+    for (int it = blockIdx.x; it < n_ops * b.rch; it += gridDim.x) {
         const int o = it / b.rch, ch = it % b.rch;
-        const OpState &s = b.st[o];
+        const StepDesc &s = b.st[o].step;
         if (s.phase != PH_GRAD) continue;
-        const LevelDesc &Lv = b.ops[o].lv[s.lvl];
-        const int n = Lv.n, pitch = Lv.pitch, r = ch * 32 + lane;
-        if (r >= n) continue;
-        const NodeRec *Vc = Lv.V[s.cur];
-        NodeRec *Vs = Lv.V[s.src];
-        const float omr = (r == 0 || r == n - 1) ? 0.5f : 1.f;
-        float2 y = make_float2(0.f, 0.f);
-        for (int c = 0; c < n; c++) {
-            const int64_t idx = (int64_t)r * pitch + c;
-            const float2 d = Vc[idx].d;
-            const float om = omr * ((c == 0 || c == n - 1) ? 0.5f : 1.f);
-            const float m = Lv.sm_tab[c].y;
-            y.x = (om * d.x - a * y.x) * m;
-            y.y = (om * d.y - a * y.y) * m;
-            *sm_scratch(Vs, idx, 0) = y;
+        const int n = s.n, pitch = s.pitch, R = smooth_row_chunk(n), r0 = ch * R;
+        if (r0 >= n) continue;
+        const int nr = min(R, n - r0);
+        const NodeRec *Vc = s.Vc;
+        NodeRec *Vs = const_cast<NodeRec *>(s.Vs);
+        const float2 *gtab = b.ops[o].lv[b.st[o].lvl].sm_tab;
+        float2 *tab = smem_rows, *ys = smem_rows + n;  // ys[row n + c]
+        for (int c = tid; c < n; c += 256) tab[c] = gtab[c];
+        for (int q = wid; q < nr; q += 8) {
+            const int r = r0 + q;
+            const float omr = (r == 0 || r == n - 1) ? 0.5f : 1.f;
+            const NodeRec *row = Vc + (int64_t)r * pitch;
+#pragma unroll 8
+            for (int c = lane; c < n; c += 32) {
+                const float2 d = row[c].d;
+                const float om = omr * ((c == 0 || c == n - 1) ? 0.5f : 1.f);
+                ys[q * n + c] = make_float2(om * d.x, om * d.y);
+            }
         }
-        float2 x = make_float2(0.f, 0.f);
-        for (int c = n - 1; c >= 0; c--) {
-            const int64_t idx = (int64_t)r * pitch + c;
-            const float2 yc = *sm_scratch(Vs, idx, 0);
-            const float cp = c < n - 1 ? Lv.sm_tab[c].x : 0.f;
-            x.x = yc.x - cp * x.x;
-            x.y = yc.y - cp * x.y;
-            *sm_scratch(Vs, idx, 0) = x;
+        __syncthreads();
+        if (wid == 0) {
+            if ((lane >> 1) < nr) {
+                float *p = reinterpret_cast<float *>(ys + (lane >> 1) * n) + (lane & 1);
+                float v[SM_BATCH], m[SM_BATCH], nv[SM_BATCH], nm[SM_BATCH];
+                // elimination, then substitution: the next batch is read while a
+                // batch is worked on
+                float y = 0.f;
+#pragma unroll
+                for (int k = 0; k < SM_BATCH; k++) { nv[k] = p[2 * min(k, n - 1)]; nm[k] = tab[min(k, n - 1)].y; }
+                for (int c = 0; c < n; c += SM_BATCH) {
+#pragma unroll
+                    for (int k = 0; k < SM_BATCH; k++) { v[k] = nv[k]; m[k] = nm[k]; }
+#pragma unroll
+                    for (int k = 0; k < SM_BATCH; k++) {
+                        const int cc = min(c + SM_BATCH + k, n - 1);
+                        nv[k] = p[2 * cc];
+                        nm[k] = tab[cc].y;
+                    }
+#pragma unroll
+                    for (int k = 0; k < SM_BATCH; k++)
+                        if (c + k < n) {
+                            y = __fsub_rn(v[k], __fmul_rn(a, y)) * m[k];  // (a y rounded first)
+                            p[2 * (c + k)] = y;
+                        }
+                }
+                float x = 0.f;
+#pragma unroll
+                for (int k = 0; k < SM_BATCH; k++) { const int cc = max(n - 1 - k, 0); nv[k] = p[2 * cc]; nm[k] = tab[cc].x; }
+                for (int c = n - 1; c >= 0; c -= SM_BATCH) {
+#pragma unroll
+                    for (int k = 0; k < SM_BATCH; k++) { v[k] = nv[k]; m[k] = nm[k]; }
+#pragma unroll
+                    for (int k = 0; k < SM_BATCH; k++) {
+                        const int cc = max(c - SM_BATCH - k, 0);
+                        nv[k] = p[2 * cc];
+                        nm[k] = tab[cc].x;
+                    }
+#pragma unroll
+                    for (int k = 0; k < SM_BATCH; k++)
+                        if (c - k >= 0) {
+                            const float cp = c - k < n - 1 ? m[k] : 0.f;
+                            x = v[k] - cp * x;
+                            p[2 * (c - k)] = x;
+                        }
+                }
+            }
+        } else {
+            const int nst = (n + REG_GW - 1) / REG_GW;
+            for (int st = wid - 1; st < nst; st += 7) {
+                const int c = st * REG_GW - 1 + lane;
+                const bool colIn = c >= 0 && c < n, own = colIn && lane >= 1 && lane <= REG_GW;
+                const float cx6 = (c == 0 || c == n - 1) ? 2.f : 4.f;
+                // rolling rows r+1 (P), r (C), r-1 (N) of u and of K1 along the row
+                auto ldu = [&](int r) {
+                    return (colIn && r >= 0 && r < n) ? reinterpret_cast<const float4 *>(Vc + (int64_t)r * pitch + c)[0]
+                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+                };
+                auto kx_of = [&](const float4 &u, int r) {
+                    // [u(c) - u(c-1)] - [u(c+1) - u(c)] along the row (0 past the grid)
+                    float4 uR;
+                    uR.x = __shfl_down_sync(FULL, u.x, 1);
+                    uR.y = __shfl_down_sync(FULL, u.y, 1);
+                    uR.z = __shfl_down_sync(FULL, u.z, 1);
+                    uR.w = __shfl_down_sync(FULL, u.w, 1);
+                    const bool rowIn = r >= 0 && r < n, hasR = colIn && rowIn && c + 1 < n;
+                    const float dxx = hasR ? (uR.x - u.x) + (uR.z - u.z) : 0.f;
+                    const float dxy = hasR ? (uR.y - u.y) + (uR.w - u.w) : 0.f;
+                    return make_float2(__shfl_up_sync(FULL, dxx, 1) - dxx, __shfl_up_sync(FULL, dxy, 1) - dxy);
+                };
+                const int rT = r0 + nr - 1;
+                float4 uP = ldu(rT + 1), uC = ldu(rT), uNext = ldu(rT - 1);
+                float2 kP = kx_of(uP, rT + 1), kC = kx_of(uC, rT);
+                for (int r = rT; r >= r0; r--) {
+                    const float4 uN = uNext;
+                    if (r > r0) uNext = ldu(r - 2);
+                    const float2 kN = kx_of(uN, r - 1);
+                    // K1 along the column at (r, c): [u(r) - u(r-1)] - [u(r+1) - u(r)]
+                    const bool hasU = colIn && r >= 1, hasD = colIn && r + 1 < n;
+                    const float kyx = (hasU ? (uC.x - uN.x) + (uC.z - uN.z) : 0.f) - (hasD ? (uP.x - uC.x) + (uP.z - uC.z) : 0.f);
+                    const float kyy = (hasU ? (uC.y - uN.y) + (uC.w - uN.w) : 0.f) - (hasD ? (uP.y - uC.y) + (uP.w - uC.w) : 0.f);
+                    const float KYx = (__shfl_up_sync(FULL, kyx, 1) + __shfl_down_sync(FULL, kyx, 1)) + cx6 * kyx;
+                    const float KYy = (__shfl_up_sync(FULL, kyy, 1) + __shfl_down_sync(FULL, kyy, 1)) + cx6 * kyy;
+                    if (own) {
+                        const float cy6 = (r == 0 || r == n - 1) ? 2.f : 4.f;
+                        const float kux = (kP.x + kN.x) + cy6 * kC.x + KYx;  // 6 (K u)
+                        const float kuy = (kP.y + kN.y) + cy6 * kC.y + KYy;
+                        Vs[(int64_t)r * pitch + c].d = make_float2(kux, kuy);
+                    }
+                    uP = uC; uC = uN;
+                    kP = kC; kC = kN;
+                }
+            }
         }
+        __syncthreads();
+        for (int q = wid; q < nr; q += 8) {
+            const int64_t row = (int64_t)(r0 + q) * pitch;
+            for (int c = lane; c < n; c += 32) *sm_x(Vs, row + c) = ys[q * n + c];
+        }
+        __syncthreads();
     }
 }
 
-// Columns: a warp holds REG_GW owned columns and one halo column on each side
-// (lanes 0 and 31), walks down for the elimination and up for the
-// substitution; on the way up it writes d into the current records and sums
-// the new slope g^T d = -h^4 sum omega d_L2 . d and u^T K d (6 K u by the
-// integer stencils of the gradient pass, hi and lo parts of u differenced
-// separately).
-__global__ void __launch_bounds__(128) k_smooth_cols(BatchDev b)
+// Columns: a one-warp block holds REG_GW owned columns (lanes 1 .. REG_GW) and
+// walks down for the elimination and up for the substitution, its rows arriving in
+// a ring in shared memory; on the way up it writes d into the current records
+// and sums the new slope g^T d = -h^4 sum omega d_L2 . d and u^T K d.
+__global__ void __launch_bounds__(32) k_smooth_cols(BatchDev b)
 {
-    const unsigned FULL = 0xffffffffu;
+    // ring rows: 16 B (6 K u, elimination) and 8 B (d_L2) per column; going down
+    // the first 8 B per column of the same rows hold the row solutions
+    __shared__ float4 ringV[SM_RING][32];
+    __shared__ float2 ringD[SM_RING][32];
+    extern __shared__ __align__(16) float2 tab_cols[];
     const int lane = threadIdx.x & 31;
-    const int nwarps = gridDim.x * 4, n_ops = b.ctr[0];
+    const int n_ops = b.ctr[0];
     const float a = b.sm_a;
-    for (int it = blockIdx.x * 4 + (threadIdx.x >> 5); it < n_ops * b.cch; it += nwarps) {
+    for (int it = blockIdx.x; it < n_ops * b.cch; it += gridDim.x) {
         const int o = it / b.cch, ch = it % b.cch;
-        const OpState &s = b.st[o];
+        const StepDesc &s = b.st[o].step;
         if (s.phase != PH_GRAD) continue;
-        const LevelDesc &Lv = b.ops[o].lv[s.lvl];
-        const int n = Lv.n, pitch = Lv.pitch;
+        const int n = s.n, pitch = s.pitch;
         if (ch * REG_GW >= n) continue;  // warp-uniform
         const int c = ch * REG_GW - 1 + lane;
-        const bool colIn = c >= 0 && c < n, own = colIn && lane >= 1 && lane <= REG_GW;
-        NodeRec *Vc = Lv.V[s.cur];
-        NodeRec *Vs = Lv.V[s.src];
+        const bool own = c < n && lane >= 1 && lane <= REG_GW;
+        NodeRec *Vc = s.Vc + c;
+        NodeRec *Vs = const_cast<NodeRec *>(s.Vs) + c;
+        const float2 *gtab = b.ops[o].lv[b.st[o].lvl].sm_tab;
+        __syncwarp();
+        for (int r = lane; r < n; r += 32) tab_cols[r] = gtab[r];
+        // down: rows r .. r + SM_GROUP - 1 of the row solutions are one copy group
+        float2 *ringX = ringD[0];
+        auto fill_down = [&](int r0) {
+            if (own)
+                for (int k = 0; k < SM_GROUP; k++) {
+                    const int r = r0 + k;
+                    if (r < n) copy_async8(ringX + (r % SM_RING) * 32 + lane, sm_x(Vs, (int64_t)r * pitch));
+                }
+            copy_commit();
+        };
+        for (int k = 0; k < SM_RING - SM_GROUP; k += SM_GROUP) fill_down(k);
         float2 y = make_float2(0.f, 0.f);
-        if (colIn)
-            for (int r = 0; r < n; r++) {
-                const int64_t idx = (int64_t)r * pitch + c;
-                const float2 x = *sm_scratch(Vs, idx, 0);
-                const float m = Lv.sm_tab[r].y;
-                y.x = (x.x - a * y.x) * m;
-                y.y = (x.y - a * y.y) * m;
-                *sm_scratch(Vs, idx, 1) = y;
+        for (int r0 = 0; r0 < n; r0 += SM_GROUP) {
+            fill_down(r0 + SM_RING - SM_GROUP);
+            copy_wait<SM_RING / SM_GROUP - 1>();
+            __syncwarp();
+            if (own) {
+                float2 x[SM_GROUP];
+                float m[SM_GROUP];
+#pragma unroll
+                for (int k = 0; k < SM_GROUP; k++) {
+                    x[k] = ringX[((r0 + k) % SM_RING) * 32 + lane];
+                    m[k] = tab_cols[min(r0 + k, n - 1)].y;
+                }
+#pragma unroll
+                for (int k = 0; k < SM_GROUP; k++)
+                    if (r0 + k < n) {
+                        y.x = (x[k].x - a * y.x) * m[k];
+                        y.y = (x[k].y - a * y.y) * m[k];
+                        *sm_y(Vs, (int64_t)(r0 + k) * pitch) = y;
+                    }
             }
-        const float cx6 = (c == 0 || c == n - 1) ? 2.f : 4.f;
+            __syncwarp();  // the group's slots are free for the next fill
+        }
+        copy_wait<0>();
+        __threadfence();  // the copies below read what the stores above wrote
+        __syncwarp();
+        // up: group g holds rows n-1 - g SM_GROUP .. downwards, slot by distance
+        auto fill_up = [&](int q0) {
+            if (own)
+                for (int k = 0; k < SM_GROUP; k++) {
+                    const int r = n - 1 - (q0 + k);
+                    if (r >= 0) {
+                        copy_async16(&ringV[(q0 + k) % SM_RING][lane], &Vs[(int64_t)r * pitch].d);
+                        copy_async8(&ringD[(q0 + k) % SM_RING][lane], &Vc[(int64_t)r * pitch].d);
+                    }
+                }
+            copy_commit();
+        };
+        for (int k = 0; k < SM_RING - SM_GROUP; k += SM_GROUP) fill_up(k);
         const float omc = (c == 0 || c == n - 1) ? 0.5f : 1.f;
-        // rolling rows r+1 (P), r (C), r-1 (N) of u and of K1 along the row
-        auto ldu = [&](int r) {
-            return (colIn && r >= 0 && r < n) ? reinterpret_cast<const float4 *>(Vc + (int64_t)r * pitch + c)[0]
-                                              : make_float4(0.f, 0.f, 0.f, 0.f);
-        };
-        auto kx_of = [&](const float4 &u, int r) {
-            // [u(c) - u(c-1)] - [u(c+1) - u(c)] along the row (0 past the grid)
-            float4 uR;
-            uR.x = __shfl_down_sync(FULL, u.x, 1);
-            uR.y = __shfl_down_sync(FULL, u.y, 1);
-            uR.z = __shfl_down_sync(FULL, u.z, 1);
-            uR.w = __shfl_down_sync(FULL, u.w, 1);
-            const bool rowIn = r >= 0 && r < n, hasR = colIn && rowIn && c + 1 < n;
-            const float dxx = hasR ? (uR.x - u.x) + (uR.z - u.z) : 0.f;
-            const float dxy = hasR ? (uR.y - u.y) + (uR.w - u.w) : 0.f;
-            return make_float2(__shfl_up_sync(FULL, dxx, 1) - dxx, __shfl_up_sync(FULL, dxy, 1) - dxy);
-        };
-        float4 uP = make_float4(0.f, 0.f, 0.f, 0.f), uC = ldu(n - 1);
-        float2 kP = make_float2(0.f, 0.f), kC = kx_of(uC, n - 1);
         float2 dnext = make_float2(0.f, 0.f);
         float sl = 0.f, qd = 0.f;
-        for (int r = n - 1; r >= 0; r--) {
-            const float4 uN = ldu(r - 1);
-            const float2 kN = kx_of(uN, r - 1);
-            float2 dn = make_float2(0.f, 0.f);
-            const int64_t idx = (int64_t)r * pitch + c;
-            if (colIn) {
-                const float2 yr = *sm_scratch(Vs, idx, 1);
-                const float cp = r < n - 1 ? Lv.sm_tab[r].x : 0.f;
-                dn.x = yr.x - cp * dnext.x;
-                dn.y = yr.y - cp * dnext.y;
-            }
-            dnext = dn;
-            // K1 along the column at (r, c): [u(r) - u(r-1)] - [u(r+1) - u(r)]
-            const bool hasU = colIn && r >= 1, hasD = colIn && r + 1 < n;
-            const float kyx = (hasU ? (uC.x - uN.x) + (uC.z - uN.z) : 0.f) - (hasD ? (uP.x - uC.x) + (uP.z - uC.z) : 0.f);
-            const float kyy = (hasU ? (uC.y - uN.y) + (uC.w - uN.w) : 0.f) - (hasD ? (uP.y - uC.y) + (uP.w - uC.w) : 0.f);
-            const float KYx = (__shfl_up_sync(FULL, kyx, 1) + __shfl_down_sync(FULL, kyx, 1)) + cx6 * kyx;
-            const float KYy = (__shfl_up_sync(FULL, kyy, 1) + __shfl_down_sync(FULL, kyy, 1)) + cx6 * kyy;
+        for (int q0 = 0; q0 < n; q0 += SM_GROUP) {
+            fill_up(q0 + SM_RING - SM_GROUP);
+            copy_wait<SM_RING / SM_GROUP - 1>();
+            __syncwarp();
             if (own) {
-                const float cy6 = (r == 0 || r == n - 1) ? 2.f : 4.f;
-                const float kux = (kP.x + kN.x) + cy6 * kC.x + KYx;  // 6 (K u)
-                const float kuy = (kP.y + kN.y) + cy6 * kC.y + KYy;
-                const float om = omc * ((r == 0 || r == n - 1) ? 0.5f : 1.f);
-                const float2 dl = Vc[idx].d;
-                sl += om * (dl.x * dn.x + dl.y * dn.y);
-                qd += dn.x * kux + dn.y * kuy;
-                Vc[idx].d = dn;
+#pragma unroll
+                for (int k = 0; k < SM_GROUP; k++) {
+                    const int r = n - 1 - (q0 + k);
+                    if (r >= 0) {
+                        const float4 v = ringV[(q0 + k) % SM_RING][lane];  // 6 K u, elimination
+                        const float2 dl = ringD[(q0 + k) % SM_RING][lane];
+                        const float cp = r < n - 1 ? tab_cols[r].x : 0.f;
+                        float2 dn;
+                        dn.x = v.z - cp * dnext.x;
+                        dn.y = v.w - cp * dnext.y;
+                        dnext = dn;
+                        const float om = omc * ((r == 0 || r == n - 1) ? 0.5f : 1.f);
+                        sl += om * (dl.x * dn.x + dl.y * dn.y);
+                        qd += dn.x * v.x + dn.y * v.y;
+                        Vc[(int64_t)r * pitch].d = dn;
+                    }
+                }
             }
-            uP = uC; uC = uN;
-            kP = kC; kC = kN;
+            __syncwarp();
         }
+        copy_wait<0>();
         sl = warp_sum(sl);
         qd = warp_sum(qd / 6.f);
         if (lane == 0) {
@@ -890,10 +1039,29 @@ __global__ void __launch_bounds__(128) k_smooth_cols(BatchDev b)
     }
 }
 
-void launch_smooth(int grid, cudaStream_t st, const BatchDev &b)
+// Row chunks per operator, and the dynamic shared memory of the two passes, for
+// levels of up to n nodes per side.
+int smooth_row_chunks(int n) { return (n + smooth_row_chunk(n) - 1) / smooth_row_chunk(n); }
+static size_t smooth_rows_smem(int n) { return sizeof(float2) * (size_t)n * (smooth_row_chunk(n) + 1); }
+
+// Room for the largest side (per device; cheap enough to repeat per handle).
+int smooth_prepare()
 {
-    k_smooth_rows<<<grid, 128, 0, st>>>(b);
-    k_smooth_cols<<<grid, 128, 0, st>>>(b);
+    return cudaFuncSetAttribute(k_smooth_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smooth_rows_smem(4097)) ==
+                       cudaSuccess &&
+                   cudaFuncSetAttribute(k_smooth_cols, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)(sizeof(float2) * 4097)) == cudaSuccess
+               ? 0
+               : 1;
+}
+
+// n: nodes per side of the handle's finest level; ops: operators of the widest
+// batch.
+void launch_smooth(int nsm, int ops, int n, cudaStream_t st, const BatchDev &b)
+{
+    const int rows = std::min((int64_t)ops * b.rch, (int64_t)2 * nsm), cols = std::min((int64_t)ops * b.cch, (int64_t)8 * nsm);
+    k_smooth_rows<<<rows, 256, smooth_rows_smem(n), st>>>(b);
+    k_smooth_cols<<<cols, 32, sizeof(float2) * (size_t)n, st>>>(b);
 }
 
 // Bilinear sampling helpers of the trial pass.

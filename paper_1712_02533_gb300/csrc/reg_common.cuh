@@ -154,7 +154,7 @@ struct BatchDev {
     // H1-type smoother (smooth != 0): per op and column chunk of
     // REG_GW columns, the partial sums {sum omega d_L2 . d, sum d . 6 K u}
     double *partS;
-    int smooth, rch, cch;  // row chunks of 32 and column chunks of REG_GW per op (maxima)
+    int smooth, rch, cch;  // row chunks and column chunks of REG_GW per op (maxima)
     float sm_a;            // off-diagonal of the dimensionless 1D system (1/6 - s^2/2)
 };
 

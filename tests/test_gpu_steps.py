@@ -51,3 +51,31 @@ def test_step_sizes_per_pass_do_not_change_the_accepted_steps(reg, orc, syn, J):
         s.apply_operator_batch([(0, -1, -1, 0, 0, 1)])
         got = s.get_slot(0)[0]
     assert np.abs(got - want * 64).max() <= 1e-3
+
+
+@pytest.mark.parametrize("side", [32, 64, 512, 1024, 2048, 4096])
+def test_smoothed_direction_is_the_tensor_product_solve(reg, syn, side):
+    """One lockstep step of the smoothed flow from the identity moves by tau d,
+    d = (T (x) T)^-1 (omega d_L2): against an FP64 solve of the library's own
+    lumped direction d_L2, at every row-chunk size of the row pass (16, 8 and 4
+    rows) and sides whose last chunk and column strip are partial.  Tolerance:
+    the sweeps are contractions (|c'| < 1), so their FP32 rounding stays within
+    a few ulp per element: 1e-5 of the largest component."""
+    from scipy.linalg import solve_banded
+    sg, L = 2.0, int(np.log2(side))
+    fr = syn.series(3, 2, side, peak=10.0, spacing=12.0, sigma=2.0)
+    n = side + 1
+    with reg.Series(fr, reg.default_params(n_levels=1, lam=10.0, smooth=sg)) as s:
+        d_l2, _ = s.eval_direction(0, 1, L, np.zeros((2, n, n), np.float32))
+        s.set_lockstep(np.array([[1]]), np.array([1.0]))
+        s.apply_operator_batch([(0, -1, -1, 0, 0, 1)])
+        got = s.get_slot(0)[0]
+    off, diag = 1.0 / 6.0 - 0.5 * sg * sg, np.full(n, 2.0 / 3.0 + sg * sg)
+    diag[[0, -1]] = 1.0 / 3.0 + 0.5 * sg * sg
+    ab = np.stack([np.full(n, off), diag, np.full(n, off)])
+    w = np.ones(n)
+    w[[0, -1]] = 0.5
+    for c in range(2):
+        f = w[:, None] * w[None, :] * d_l2[c].astype(np.float64)
+        want = solve_banded((1, 1), ab, solve_banded((1, 1), ab, f).T).T
+        assert np.abs(got[c] - want).max() <= 1e-5 * np.abs(want).max()
