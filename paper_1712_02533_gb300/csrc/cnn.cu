@@ -392,12 +392,12 @@ __global__ void __launch_bounds__(256) k_wgrad_last(const uint4 *__restrict__ a,
         __syncthreads();
         // all of a thread's loads are issued before its stores
         constexpr int NA = (4 * WL_AR * WL_AC + 255) / 256;
-        float g[2];
+        float g;
         uint4 qa[NA];
-#pragma unroll
-        for (int k = 0; k < 2; k++) {
-            const int i = t + 256 * k, o = i / WL_NP, p = i % WL_NP, y = y0 + p / WL_TW, xx = x0 + p % WL_TW;
-            g[k] = (y < H && xx < H) ? gz[(((int64_t)b * 2 + o) * H + y) * H + xx] : 0.f;
+        {
+            static_assert(2 * WL_NP == 256, "one gradient value per thread");
+            const int o = t / WL_NP, p = t % WL_NP, y = y0 + p / WL_TW, xx = x0 + p % WL_TW;
+            g = (y < H && xx < H) ? gz[(((int64_t)b * 2 + o) * H + y) * H + xx] : 0.f;
         }
 #pragma unroll
         for (int k = 0; k < NA; k++) {
@@ -407,8 +407,7 @@ __global__ void __launch_bounds__(256) k_wgrad_last(const uint4 *__restrict__ a,
             if (i < 4 * WL_AR * WL_AC && iy >= 0 && iy < H && ix >= 0 && ix < H)
                 qa[k] = a[((int64_t)(4 * b + cg) * H + iy) * H + ix];
         }
-#pragma unroll
-        for (int k = 0; k < 2; k++) (&gs[0][0])[t + 256 * k] = g[k];
+        (&gs[0][0])[t] = g;
 #pragma unroll
         for (int k = 0; k < NA; k++) {
             const int i = t + 256 * k, cg = i / (WL_AR * WL_AC), rr = (i / WL_AC) % WL_AR, cc = i % WL_AC;
