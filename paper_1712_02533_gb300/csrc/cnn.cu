@@ -182,74 +182,276 @@ __global__ void __launch_bounds__(128) k_conv_bwd_data(const float *__restrict__
 }
 
 // ---------------------------------------------------------------------------
-// Backward, weights: gW[o, c, dy, dx] = sum_{b, y, x} gz[b, o, y, x]
-// in_pad[b, c, S y + dy, S x + dx] and gb[o] = sum gz[b, o, ., .].  One block per
-// (o, c), a fixed-order reduction (deterministic).
+// The FP32 path's convolutions with 32 output channels, their data and weight
+// gradients.  All are FP32 work of 288 multiply-adds per value moved, so what
+// counts is how many multiply-adds follow a shared-memory load: with one pixel
+// per thread and all 32 channels each 16-byte weight load fed four of them and
+// the loads bounded the kernel (128 us per forward layer of 32 pairs, 64^2
+// outputs; 136 us per data gradient).  Here a thread holds four pixels (one
+// column of four rows: lanes stay on adjacent columns) by 16 channels, so that a
+// weight load feeds 16 (packed in pairs).  Each output's products are added in
+// the order they always were, so the results are bit for bit the same.  Forward
+// layer 128 -> 74 us, data gradient 136 -> 92 us (stride 2: 222 -> 111 us).
 // ---------------------------------------------------------------------------
-//
-// With split > 1 the pixels are cut into `split` contiguous parts, one block
-// each (grid O C split), and each block writes its 10 sums to part; the
-// layers with few (o, c) pairs (2 -> 32, 32 -> 2) keep the GPU busy that way,
-// and k_bwd_weight_sum adds the parts in order.
-template <int C, int O, int S>
-__global__ void __launch_bounds__(256) k_conv_bwd_weight(const float *__restrict__ in, int H,
-                                                         const float *__restrict__ gz, int Ho, int B,
-                                                         float *__restrict__ grad, int split,
-                                                         float *__restrict__ part)
+constexpr int PX = 4, OC = 16;  // pixels and channels per thread
+
+__device__ __forceinline__ void fma_group(float2 (&acc)[PX][OC / 2], const float *w, const float (&v)[PX])
 {
-    const int oc = blockIdx.x / split, sp = blockIdx.x % split;
-    const int o = oc / C, c = oc % C;
-    float acc[10];
 #pragma unroll
-    for (int k = 0; k < 10; k++) acc[k] = 0.f;
-    const int per = Ho * Ho, total = B * per;
-    const int chunk = (total + split - 1) / split, p0 = sp * chunk, p1 = min(total, p0 + chunk);
-    for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-        const int b = p / per, q = p % per, y = q / Ho, x = q % Ho;
-        const float g = gz[((int64_t)b * O + o) * per + q];
-        const float *src = in + ((int64_t)b * C + c) * H * H;
+    for (int q = 0; q < OC / 4; q++) {
+        const float4 wv = reinterpret_cast<const float4 *>(w)[q];
+        const float2 w0 = make_float2(wv.x, wv.y), w1 = make_float2(wv.z, wv.w);
 #pragma unroll
-        for (int dy = 0; dy < 3; dy++)
-#pragma unroll
-            for (int dx = 0; dx < 3; dx++) {
-                const int iy = S * y + dy - 1, ix = S * x + dx - 1;
-                float v = 0.f;
-                if (iy >= 0 && iy < H && ix >= 0 && ix < H) v = src[iy * H + ix];
-                acc[dy * 3 + dx] = fmaf(g, v, acc[dy * 3 + dx]);
-            }
-        acc[9] += g;
-    }
-    __shared__ float red[8][10];
-#pragma unroll
-    for (int k = 0; k < 10; k++) {
-        float v = acc[k];
-        for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 10) {
-        float t = 0.f;
-        for (int w = 0; w < 8; w++) t += red[w][threadIdx.x];
-        if (split > 1) {
-            part[(int64_t)blockIdx.x * 10 + threadIdx.x] = t;
-        } else {
-            if (threadIdx.x < 9) grad[(o * C + c) * 9 + threadIdx.x] = t;
-            else if (c == 0) grad[O * C * 9 + o] = t;
+        for (int p = 0; p < PX; p++) {
+            const float2 vv = make_float2(v[p], v[p]);
+            acc[p][2 * q] = __ffma2_rn(w0, vv, acc[p][2 * q]);
+            acc[p][2 * q + 1] = __ffma2_rn(w1, vv, acc[p][2 * q + 1]);
         }
     }
 }
 
-// The parts of k_conv_bwd_weight in order (one thread per (o, c) and sum).
-template <int C, int O>
-__global__ void k_bwd_weight_sum(const float *__restrict__ part, int split, float *__restrict__ grad)
+// Forward, 32 outputs with ReLU: out[b][o][y][x], rows y = 4 yg .. 4 yg + 3.  grid
+// (column-and-row-group blocks, channel halves).  Sum order (c, tap), as k_conv_fwd.
+template <int C, int S>
+__global__ void __launch_bounds__(128, 4) k_conv_fwd32(const float *__restrict__ in, int H,
+                                                       const float *__restrict__ theta, float *__restrict__ out,
+                                                       int Ho, int nyg, int total)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= O * C * 10) return;
-    const int oc = i / 10, k = i % 10, o = oc / C, c = oc % C;
-    float t = 0.f;
-    for (int sp = 0; sp < split; sp++) t += part[((int64_t)oc * split + sp) * 10 + k];
-    if (k < 9) grad[(o * C + c) * 9 + k] = t;
-    else if (c == 0) grad[O * C * 9 + o] = t;
+    constexpr int NR = S * (PX - 1) + 3;  // input rows of the four output rows
+    __shared__ __align__(16) float w[C * 9 * OC];
+    __shared__ float bias[OC];
+    const int o0 = blockIdx.y * OC;
+    for (int i = threadIdx.x; i < C * 9 * OC; i += blockDim.x) {
+        const int o = i / (C * 9), ck = i - o * (C * 9);
+        w[ck * OC + o] = theta[(o0 + o) * C * 9 + ck];
+    }
+    if (threadIdx.x < OC) bias[threadIdx.x] = theta[32 * C * 9 + o0 + threadIdx.x];
+    __syncthreads();
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= total) return;
+    const int x = p % Ho, yg = (p / Ho) % nyg, b = p / (Ho * nyg), y0 = yg * PX;
+    float2 acc[PX][OC / 2];
+#pragma unroll
+    for (int k = 0; k < PX; k++)
+#pragma unroll
+        for (int o = 0; o < OC / 2; o++) acc[k][o] = make_float2(bias[2 * o], bias[2 * o + 1]);
+    const float *src = in + (int64_t)b * C * H * H;
+    const int ix0 = S * x - 1, iy0 = S * y0 - 1;
+#pragma unroll 1
+    for (int c = 0; c < C; c++, src += (int64_t)H * H) {
+        float v[NR][3];
+#pragma unroll
+        for (int r = 0; r < NR; r++)
+#pragma unroll
+            for (int dx = 0; dx < 3; dx++) {
+                const int iy = iy0 + r, ix = ix0 + dx;
+                v[r][dx] = (iy >= 0 && iy < H && ix >= 0 && ix < H) ? src[iy * H + ix] : 0.f;
+            }
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            float q[PX];
+#pragma unroll
+            for (int j = 0; j < PX; j++) q[j] = v[S * j + k / 3][k % 3];
+            fma_group(acc, w + (c * 9 + k) * OC, q);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < PX; j++)
+        if (y0 + j < Ho) {
+#pragma unroll
+            for (int o = 0; o < OC; o++) {
+                const float a = (o & 1) ? acc[j][o / 2].y : acc[j][o / 2].x;
+                out[(((int64_t)b * 32 + o0 + o) * Ho + y0 + j) * Ho + x] = fmaxf(a, 0.f);
+            }
+        }
+}
+
+// Data gradient of the 32 -> 32 layers with the ReLU mask of the layer below (its
+// FP32 output > 0).  Stride 2: an input pixel takes the taps dy with iy + 1 - dy
+// even, likewise along x, so the pixels of one parity class (blockIdx.z = 2 py +
+// px) share their taps; a thread's rows and the lanes' columns are two apart.  Sum
+// order (dy, dx, o), as k_conv_bwd_data.
+template <int S>
+__global__ void __launch_bounds__(128, 4) k_conv_bwd_data32(const float *__restrict__ gz, int Ho,
+                                                            const float *__restrict__ theta,
+                                                            const float *__restrict__ a_below, float *__restrict__ gx,
+                                                            int H, int nyg, int total)
+{
+    __shared__ __align__(16) float w[32 * 9 * OC];  // [o][tap][c of this half]
+    const int c0 = blockIdx.y * OC, py = S == 2 ? blockIdx.z >> 1 : 0, px = S == 2 ? blockIdx.z & 1 : 0;
+    for (int i = threadIdx.x; i < 32 * 9 * OC; i += blockDim.x) {
+        const int o = i / (9 * OC), r = i - o * (9 * OC), c = r / 9, k = r - c * 9;
+        w[(o * 9 + k) * OC + c] = theta[(o * 32 + c0 + c) * 9 + k];
+    }
+    __syncthreads();
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= total) return;
+    const int nx = H / S;
+    const int xi = p % nx, yg = (p / nx) % nyg, b = p / (nx * nyg), y0 = yg * PX;  // in class rows and columns
+    const int ix = S * xi + px;
+    float2 acc[PX][OC / 2];
+#pragma unroll
+    for (int k = 0; k < PX; k++)
+#pragma unroll
+        for (int o = 0; o < OC / 2; o++) acc[k][o] = make_float2(0.f, 0.f);
+    const int64_t plane = (int64_t)Ho * Ho;
+    const float *gb = gz + (int64_t)b * 32 * plane;
+#pragma unroll 1
+    for (int dy = 0; dy < 3; dy++) {
+        if (S == 2 && ((py + 1 - dy) & 1)) continue;  // block-uniform
+        int off[PX];
+        bool okr[PX];
+#pragma unroll
+        for (int j = 0; j < PX; j++) {
+            const int ty = S * (y0 + j) + py + 1 - dy, oy = S == 2 ? ty >> 1 : ty;
+            okr[j] = ty >= 0 && oy < Ho && y0 + j < nx;
+            off[j] = oy * Ho;
+        }
+#pragma unroll 1
+        for (int dx = 0; dx < 3; dx++) {
+            if (S == 2 && ((px + 1 - dx) & 1)) continue;  // block-uniform
+            const int tx = ix + 1 - dx, ox = S == 2 ? tx >> 1 : tx;
+            const bool okc = tx >= 0 && ox < Ho;
+            const float *g0 = gb + ox;
+            const float *wk = w + (dy * 3 + dx) * OC;
+#pragma unroll 4
+            for (int o = 0; o < 32; o++) {
+                float g[PX];
+#pragma unroll
+                for (int j = 0; j < PX; j++) g[j] = okc && okr[j] ? g0[o * plane + off[j]] : 0.f;
+                fma_group(acc, wk + o * 9 * OC, g);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < PX; j++) {
+        const int iy = S * (y0 + j) + py;
+        if (y0 + j < nx) {
+#pragma unroll
+            for (int c = 0; c < OC; c++) {
+                const int64_t i = (((int64_t)b * 32 + c0 + c) * H + iy) * H + ix;
+                const float a = (c & 1) ? acc[j][c / 2].y : acc[j][c / 2].x;
+                gx[i] = a_below[i] > 0.f ? a : 0.f;
+            }
+        }
+    }
+}
+
+// Weight and bias gradients of the 32 -> 32 layers: gW[o][c][tap] = sum gz[b][o][y][x]
+// in[b][c][S y + dy - 1][S x + dx - 1].  A block stages a tile of output pixels
+// (the gradient as [pixel][o], the input window as [c][row][column]) and its
+// threads (warp = 4 output channels, lane = input channel) sum 4 x 9 products per
+// pixel over a window sliding along the row: one broadcast 16-byte load and 3 S
+// conflict-free loads per 36 multiply-adds.  With a block per (o, c) pair, which
+// read input and gradient 32 times over from L2, a layer took 1155 us (32 pairs);
+// now 66 us and 4 us for the records' sum.
+// Blocks take tiles block, block + grid, ..; each writes one record.
+template <int S>
+struct Wg32 {
+    static constexpr int TR = 4, TC = S == 1 ? 32 : 16, NP = TR * TC;
+    static constexpr int IR = S * (TR - 1) + 3, IC = S * (TC - 1) + 3;
+    static constexpr int CS = (IR * IC) | 1;  // odd channel stride: no bank conflicts across channels
+    static constexpr int GS = 36;             // gradient row: 32 channels, 16-byte aligned
+};
+constexpr int WG32_REC = 32 * 32 * 9 + 32;
+constexpr int WG32_BLOCKS = 2;  // per SM
+
+template <int S>
+__global__ void __launch_bounds__(256, WG32_BLOCKS) k_wgrad32(const float *__restrict__ in, int H,
+                                                              const float *__restrict__ gz, int Ho, int B,
+                                                              float *__restrict__ part)
+{
+    using G = Wg32<S>;
+    __shared__ __align__(16) float gs[G::NP * G::GS];
+    __shared__ float is[32 * G::CS];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    float2 acc[2][9];
+    float gb[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 2; i++)
+#pragma unroll
+        for (int j = 0; j < 9; j++) acc[i][j] = make_float2(0.f, 0.f);
+    const int tx_n = (Ho + G::TC - 1) / G::TC, ty_n = (Ho + G::TR - 1) / G::TR, nt = B * tx_n * ty_n;
+    for (int tile = blockIdx.x; tile < nt; tile += gridDim.x) {
+        const int b = tile / (tx_n * ty_n), rr = tile % (tx_n * ty_n);
+        const int y0 = (rr / tx_n) * G::TR, x0 = (rr % tx_n) * G::TC;
+        __syncthreads();  // the previous tile's reads are done
+        // gradient: warp w its own channels 4 w .. 4 w + 3 (bias sums from the registers)
+        float gv[4][G::NP / 32];
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+#pragma unroll
+            for (int j = 0; j < G::NP / 32; j++) {
+                const int p = 32 * j + lane, y = y0 + p / G::TC, x = x0 + p % G::TC;
+                gv[q][j] = (y < Ho && x < Ho) ? gz[(((int64_t)b * 32 + 4 * wid + q) * Ho + y) * Ho + x] : 0.f;
+            }
+        // input window: warp w channels w, w + 8, ..
+        constexpr int NI = (G::IR * G::IC + 31) / 32;
+#pragma unroll 1
+        for (int k = 0; k < 4; k++) {
+            const int c = wid + 8 * k;
+            const float *src = in + ((int64_t)b * 32 + c) * H * H;
+            float iv[NI];
+#pragma unroll
+            for (int j = 0; j < NI; j++) {
+                const int i = 32 * j + lane, iy = S * y0 - 1 + i / G::IC, ix = S * x0 - 1 + i % G::IC;
+                iv[j] = (i < G::IR * G::IC && iy >= 0 && iy < H && ix >= 0 && ix < H) ? src[iy * H + ix] : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < NI; j++)
+                if (32 * j + lane < G::IR * G::IC) is[c * G::CS + 32 * j + lane] = iv[j];
+        }
+#pragma unroll
+        for (int j = 0; j < G::NP / 32; j++) {
+            *reinterpret_cast<float4 *>(gs + (32 * j + lane) * G::GS + 4 * wid) =
+                make_float4(gv[0][j], gv[1][j], gv[2][j], gv[3][j]);
+#pragma unroll
+            for (int q = 0; q < 4; q++) gb[q] += gv[q][j];
+        }
+        __syncthreads();
+        const float *ic = is + lane * G::CS;
+#pragma unroll 1
+        for (int r = 0; r < G::TR; r++) {
+            float win[3][3];
+#pragma unroll
+            for (int dy = 0; dy < 3; dy++)
+#pragma unroll
+                for (int dx = 0; dx < 3 - S; dx++) win[dy][S + dx] = ic[(S * r + dy) * G::IC + dx];
+#pragma unroll 4
+            for (int x = 0; x < G::TC; x++) {
+#pragma unroll
+                for (int dy = 0; dy < 3; dy++) {
+#pragma unroll
+                    for (int dx = 0; dx < 3 - S; dx++) win[dy][dx] = win[dy][S + dx];
+#pragma unroll
+                    for (int dx = 3 - S; dx < 3; dx++) win[dy][dx] = ic[(S * r + dy) * G::IC + S * x + dx];
+                }
+                const float4 g = *reinterpret_cast<const float4 *>(gs + (r * G::TC + x) * G::GS + 4 * wid);
+                const float2 g0 = make_float2(g.x, g.y), g1 = make_float2(g.z, g.w);
+#pragma unroll
+                for (int j = 0; j < 9; j++) {
+                    const float2 v = make_float2(win[j / 3][j % 3], win[j / 3][j % 3]);
+                    acc[0][j] = __ffma2_rn(g0, v, acc[0][j]);
+                    acc[1][j] = __ffma2_rn(g1, v, acc[1][j]);
+                }
+            }
+        }
+    }
+    float *rec = part + (int64_t)blockIdx.x * WG32_REC;
+#pragma unroll
+    for (int i = 0; i < 2; i++)
+#pragma unroll
+        for (int j = 0; j < 9; j++) {
+            rec[((4 * wid + 2 * i) * 32 + lane) * 9 + j] = acc[i][j].x;
+            rec[((4 * wid + 2 * i + 1) * 32 + lane) * 9 + j] = acc[i][j].y;
+        }
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        float v = gb[q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) rec[32 * 32 * 9 + 4 * wid + q] = v;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -260,7 +462,7 @@ __global__ void k_bwd_weight_sum(const float *__restrict__ part, int split, floa
 // gradient and the input window the tile needs, and its threads form all the
 // layer's weight and bias sums from shared memory.  Each block works through a
 // fixed sequence of tiles (tile = block + k grid) and writes one partial
-// record; k_wgrad_parts_sum adds the records in block order, so the result is
+// record; cnn_sum_records adds the records in a fixed order, so the result is
 // deterministic for a given grid.
 // ---------------------------------------------------------------------------
 constexpr int WF_TR = 2, WF_TW = 64, WF_NP = WF_TR * WF_TW;  // first layer: 2 output rows x 64 columns
@@ -371,12 +573,14 @@ constexpr int WL_CS = WL_AR * WL_AC + 1;                     // channel stride (
 constexpr int WL_REC = 2 * 32 * 9 + 2;
 
 // Last layer: gW[o][c][dy][dx] = sum gz[b][o][y][x] a[b][c][y + dy - 1][x + dx - 1],
-// gb[o] = sum gz[b][o][y][x]; a the planar BF16 input (B x 32 x H x H), gz FP32
-// NCHW (B x 2 x H x H).  Thread (c, seg) = (t % 32, t / 32) walks 16 pixels of
+// gb[o] = sum gz[b][o][y][x]; a the input (B x 32 x H x H), BF16 in the planar
+// layout or FP32 NCHW, gz FP32 NCHW (B x 2 x H x H).  Thread (c, seg) = (t % 32, t / 32) walks 16 pixels of
 // tile row seg / 2 with a sliding 3 x 3 window of channel c.
-__global__ void __launch_bounds__(256) k_wgrad_last(const uint4 *__restrict__ a, int H, const float *__restrict__ gz,
+template <bool PLANAR>
+__global__ void __launch_bounds__(256) k_wgrad_last(const void *__restrict__ act, int H, const float *__restrict__ gz,
                                                     int B, float *__restrict__ part)
 {
+    const uint4 *a = reinterpret_cast<const uint4 *>(act);
     __shared__ float as[32 * WL_CS];
     __shared__ float gs[2][WL_NP];
     __shared__ float red[8][32][18];
@@ -393,23 +597,42 @@ __global__ void __launch_bounds__(256) k_wgrad_last(const uint4 *__restrict__ a,
         // all of a thread's loads are issued before its stores
         constexpr int NA = (4 * WL_AR * WL_AC + 255) / 256;
         float g;
-        uint4 qa[NA];
+        uint4 qa[PLANAR ? NA : 1];
         {
             static_assert(2 * WL_NP == 256, "one gradient value per thread");
             const int o = t / WL_NP, p = t % WL_NP, y = y0 + p / WL_TW, xx = x0 + p % WL_TW;
             g = (y < H && xx < H) ? gz[(((int64_t)b * 2 + o) * H + y) * H + xx] : 0.f;
         }
+        if constexpr (PLANAR) {
 #pragma unroll
-        for (int k = 0; k < NA; k++) {
-            const int i = t + 256 * k, cg = i / (WL_AR * WL_AC), rr = (i / WL_AC) % WL_AR, cc = i % WL_AC;
-            const int iy = y0 - 1 + rr, ix = x0 - 1 + cc;
-            qa[k] = make_uint4(0u, 0u, 0u, 0u);
-            if (i < 4 * WL_AR * WL_AC && iy >= 0 && iy < H && ix >= 0 && ix < H)
-                qa[k] = a[((int64_t)(4 * b + cg) * H + iy) * H + ix];
+            for (int k = 0; k < NA; k++) {
+                const int i = t + 256 * k, cg = i / (WL_AR * WL_AC), rr = (i / WL_AC) % WL_AR, cc = i % WL_AC;
+                const int iy = y0 - 1 + rr, ix = x0 - 1 + cc;
+                qa[k] = make_uint4(0u, 0u, 0u, 0u);
+                if (i < 4 * WL_AR * WL_AC && iy >= 0 && iy < H && ix >= 0 && ix < H)
+                    qa[k] = a[((int64_t)(4 * b + cg) * H + iy) * H + ix];
+            }
+        } else {
+            // warp w channels w, w + 8, ..: lanes on adjacent columns
+            constexpr int NW = (WL_AR * WL_AC + 31) / 32;
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const int ch = (t >> 5) + 8 * k;
+                const float *src = reinterpret_cast<const float *>(act) + ((int64_t)b * 32 + ch) * H * H;
+                float v[NW];
+#pragma unroll
+                for (int j = 0; j < NW; j++) {
+                    const int i = 32 * j + (t & 31), iy = y0 - 1 + i / WL_AC, ix = x0 - 1 + i % WL_AC;
+                    v[j] = (i < WL_AR * WL_AC && iy >= 0 && iy < H && ix >= 0 && ix < H) ? src[iy * H + ix] : 0.f;
+                }
+#pragma unroll
+                for (int j = 0; j < NW; j++)
+                    if (32 * j + (t & 31) < WL_AR * WL_AC) as[ch * WL_CS + 32 * j + (t & 31)] = v[j];
+            }
         }
         (&gs[0][0])[t] = g;
 #pragma unroll
-        for (int k = 0; k < NA; k++) {
+        for (int k = 0; k < (PLANAR ? NA : 0); k++) {
             const int i = t + 256 * k, cg = i / (WL_AR * WL_AC), rr = (i / WL_AC) % WL_AR, cc = i % WL_AC;
             if (i >= 4 * WL_AR * WL_AC) continue;
             const uint32_t wv[4] = {qa[k].x, qa[k].y, qa[k].z, qa[k].w};
@@ -470,27 +693,7 @@ __global__ void __launch_bounds__(256) k_wgrad_last(const uint4 *__restrict__ a,
     }
 }
 
-// grad[e] = sum over blocks of part[block][e], e < rec: one block per entry,
-// a fixed-order tree.
-__global__ void __launch_bounds__(256) k_wgrad_parts_sum(const float *__restrict__ part, int nblk, int rec,
-                                                         float *__restrict__ grad)
-{
-    __shared__ float red[8];
-    const int e = blockIdx.x, t = threadIdx.x;
-    float s = 0.f;
-    for (int k = t; k < nblk; k += 256) s += part[(int64_t)k * rec + e];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((t & 31) == 0) red[t >> 5] = s;
-    __syncthreads();
-    if (t == 0) {
-        float tot = 0.f;
-        for (int w = 0; w < 8; w++) tot += red[w];
-        grad[e] = tot;
-    }
-}
-
-// Grid of the two kernels above: two blocks per SM, at most one per tile.
+// Grid of the weight gradient kernels: two blocks per SM, at most one per tile.
 int wgrad_small_grid(int n_tiles)
 {
     int dev = 0, nsm = 152;
@@ -555,25 +758,54 @@ __global__ void k_adam(float *__restrict__ theta, const float *__restrict__ g, f
     }
 }
 
-template <int C, int O, int S, bool RELU>
-void fwd(const float *in, int H, const float *theta, float *out, int B, cudaStream_t st)
+// FP32 forward of layer k.
+void fwd(int k, const float *in, int H, const float *theta, float *out, int B, cudaStream_t st)
 {
-    const int Ho = (H + 2 - 3) / S + 1, total = B * Ho * Ho;
-    k_conv_fwd<C, O, S, RELU><<<(total + 127) / 128, 128, 0, st>>>(in, H, theta, out, Ho, total);
+    const int Ho = (H + 2 - 3) / LAYERS[k].S + 1;
+    if (k == NL - 1) {
+        const int total = B * Ho * Ho;
+        k_conv_fwd<32, 2, 1, false><<<(total + 127) / 128, 128, 0, st>>>(in, H, theta, out, Ho, total);
+        return;
+    }
+    const int nyg = (Ho + PX - 1) / PX, total = B * nyg * Ho;
+    const dim3 grid((total + 127) / 128, 32 / OC);
+    if (k == 0) k_conv_fwd32<2, 2><<<grid, 128, 0, st>>>(in, H, theta, out, Ho, nyg, total);
+    else if (LAYERS[k].S == 2) k_conv_fwd32<32, 2><<<grid, 128, 0, st>>>(in, H, theta, out, Ho, nyg, total);
+    else k_conv_fwd32<32, 1><<<grid, 128, 0, st>>>(in, H, theta, out, Ho, nyg, total);
 }
 
-template <int C, int O, int S>
-void bwd(const float *in, int H, const float *gz, const float *theta, const float *a_below, float *gx, float *grad,
-         int B, cudaStream_t st, float *part)
+// FP32 weight gradient of layer k into grad and, for k > 0, its data gradient with
+// the ReLU mask of the layer below into gx.
+void bwd(int k, const float *in, int H, const float *gz, const float *theta, float *gx, float *grad, int B,
+         cudaStream_t st, float *part)
 {
-    const int Ho = (H + 2 - 3) / S + 1;
-    // (o, c) pairs times parts of the pixel range: about a thousand blocks
-    const int split = (O * C >= 512) ? 1 : std::min(64, 1024 / (O * C));
-    k_conv_bwd_weight<C, O, S><<<O * C * split, 256, 0, st>>>(in, H, gz, Ho, B, grad, split, part);
-    if (split > 1) k_bwd_weight_sum<C, O><<<(O * C * 10 + 255) / 256, 256, 0, st>>>(part, split, grad);
-    if (gx) {
-        const int total = B * H * H;
-        k_conv_bwd_data<C, O, S><<<(total + 127) / 128, 128, 0, st>>>(gz, Ho, theta, a_below, gx, H, total);
+    const int Ho = (H + 2 - 3) / LAYERS[k].S + 1;
+    auto tiles = [&](int tr, int tc) { return B * ((Ho + tr - 1) / tr) * ((Ho + tc - 1) / tc); };
+    if (k == 0) {
+        const int grid = wgrad_small_grid(tiles(WF_TR, WF_TW));
+        k_wgrad_first<<<grid, 256, 0, st>>>(in, H, gz, Ho, B, part);
+        cnn_sum_records(part, grid, WF_REC, grad, st);
+        return;
+    }
+    if (k == NL - 1) {
+        const int grid = wgrad_small_grid(tiles(WL_TR, WL_TW)), total = B * H * H;
+        k_wgrad_last<false><<<grid, 256, 0, st>>>(in, H, gz, B, part);
+        cnn_sum_records(part, grid, WL_REC, grad, st);
+        k_conv_bwd_data<32, 2, 1><<<(total + 127) / 128, 128, 0, st>>>(gz, Ho, theta, in, gx, H, total);
+        return;
+    }
+    const int S = LAYERS[k].S, nx = H / S, nyg = (nx + PX - 1) / PX, total = B * nyg * nx;
+    const dim3 grid((total + 127) / 128, 32 / OC, S * S);
+    if (S == 2) {
+        const int wg = wgrad_small_grid(tiles(Wg32<2>::TR, Wg32<2>::TC));
+        k_wgrad32<2><<<wg, 256, 0, st>>>(in, H, gz, Ho, B, part);
+        cnn_sum_records(part, wg, WG32_REC, grad, st);
+        k_conv_bwd_data32<2><<<grid, 128, 0, st>>>(gz, Ho, theta, in, gx, H, nyg, total);
+    } else {
+        const int wg = wgrad_small_grid(tiles(Wg32<1>::TR, Wg32<1>::TC));
+        k_wgrad32<1><<<wg, 256, 0, st>>>(in, H, gz, Ho, B, part);
+        cnn_sum_records(part, wg, WG32_REC, grad, st);
+        k_conv_bwd_data32<1><<<grid, 128, 0, st>>>(gz, Ho, theta, in, gx, H, nyg, total);
     }
 }
 
@@ -666,14 +898,7 @@ reg_status cnn_forward(reg_cnn *h, const float *x, int B, float *y, cudaStream_t
             if (rs != REG_OK) return rs;
             h->packed_fwd[k] = h->version;
         } else {
-            switch (k) {
-            case 0: fwd<2, 32, 2, true>(a, H, th, out, B, st); break;
-            case 1: fwd<32, 32, 2, true>(a, H, th, out, B, st); break;
-            case 2:
-            case 3:
-            case 4: fwd<32, 32, 1, true>(a, H, th, out, B, st); break;
-            default: fwd<32, 2, 1, false>(a, H, th, out, B, st); break;
-            }
+            fwd(k, a, H, th, out, B, st);
         }
         if (k == NL - 1 && y && y != h->act[k])
             CKC(cudaMemcpyAsync(h->act[k], y, sizeof(float) * act_elems(k, S) * B, cudaMemcpyDeviceToDevice, st));
@@ -717,7 +942,7 @@ reg_status reg_cnn_create(int32_t side, int32_t max_batch, void *cuda_stream, re
          alloc((void **)&h->wpack_last, sizeof(uint32_t) * cnn_last_umma_words()) &&
          cudaHostAlloc((void **)&h->uerr_host, sizeof(int), cudaHostAllocMapped) == cudaSuccess &&
          cudaHostGetDevicePointer((void **)&h->uerr, h->uerr_host, 0) == cudaSuccess &&
-         alloc((void **)&h->wpart, sizeof(float) * (size_t)std::max(cnn_wgrad32_umma_part_floats(), 2 * 1024 * 608));
+         alloc((void **)&h->wpart, sizeof(float) * (size_t)std::max(cnn_wgrad32_umma_part_floats(), wgrad_small_grid(1 << 30) * WG32_REC));
     if (!ok) {
         reg_cnn_destroy(h);
         return cnn_fail(REG_ENOMEM, "device allocation failed");
@@ -805,7 +1030,6 @@ static reg_status loss_grad(reg_cnn_t h, const float *x, const float *target, in
         const float *th = h->theta + param_offset(k);
         float *gr = h->grad + param_offset(k);
         float *gx = k == 0 ? nullptr : bufs[k & 1];
-        const float *below = k == 0 ? nullptr : h->act[k - 1];
         if (tc && k >= 1 && k <= 4) {
             // the layer's input and the mask below: BF16 planar
             const uint16_t *inb = h->actb[k - 1];
@@ -824,8 +1048,8 @@ static reg_status loss_grad(reg_cnn_t h, const float *x, const float *target, in
             // the last layer's input (and the mask below) is the planar BF16
             // output of layer 4
             const int nt = B * ((H + WL_TW - 1) / WL_TW) * ((H + WL_TR - 1) / WL_TR), grid = wgrad_small_grid(nt);
-            k_wgrad_last<<<grid, 256, 0, st>>>(reinterpret_cast<const uint4 *>(h->actb[k - 1]), H, gz, B, h->wpart);
-            k_wgrad_parts_sum<<<WL_REC, 256, 0, st>>>(h->wpart, grid, WL_REC, gr);
+            k_wgrad_last<true><<<grid, 256, 0, st>>>(h->actb[k - 1], H, gz, B, h->wpart);
+            cnn_sum_records(h->wpart, grid, WL_REC, gr, st);
             const int total = B * H * H;
             k_conv_bwd_data<32, 2, 1, true><<<(total + 127) / 128, 128, 0, st>>>(gz, H, th, h->actb[k - 1], gx, H, total);
             gz = gx;
@@ -835,17 +1059,10 @@ static reg_status loss_grad(reg_cnn_t h, const float *x, const float *target, in
             const int Ho = H / 2, nt = B * ((Ho + WF_TW - 1) / WF_TW) * ((Ho + WF_TR - 1) / WF_TR);
             const int grid = wgrad_small_grid(nt);
             k_wgrad_first<<<grid, 256, 0, st>>>(x, H, gz, Ho, B, h->wpart);
-            k_wgrad_parts_sum<<<WF_REC, 256, 0, st>>>(h->wpart, grid, WF_REC, gr);
+            cnn_sum_records(h->wpart, grid, WF_REC, gr, st);
             continue;
         }
-        switch (k) {
-        case 0: bwd<2, 32, 2>(in, H, gz, th, below, gx, gr, B, st, h->wpart); break;
-        case 1: bwd<32, 32, 2>(in, H, gz, th, below, gx, gr, B, st, h->wpart); break;
-        case 2:
-        case 3:
-        case 4: bwd<32, 32, 1>(in, H, gz, th, below, gx, gr, B, st, h->wpart); break;
-        default: bwd<32, 2, 1>(in, H, gz, th, below, gx, gr, B, st, h->wpart); break;
-        }
+        bwd(k, in, H, gz, th, gx, gr, B, st, h->wpart);
         gz = gx;
     }
     CKC(cudaGetLastError());

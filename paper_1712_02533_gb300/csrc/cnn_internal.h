@@ -24,6 +24,8 @@ int cnn_max_batch(const reg_cnn *h);
 reg_status cnn_wgrad32_umma(const uint16_t *in, int H, const float *gz, int B, int S, float *grad, float *part,
                             cudaStream_t st, int *err);
 int cnn_wgrad32_umma_part_floats();
+// grad[e] = the sum of entry e < rec of nrec records part[record][rec] (fixed order).
+void cnn_sum_records(const float *part, int nrec, int rec, float *grad, cudaStream_t st);
 // 32 -> 32 channel 3x3 convolution (zero padding 1, stride S = 1 or 2) with
 // bias and ReLU on the fifth-generation tensor cores (tcgen05.mma, accumulator
 // in TMEM, BF16 operands, FP32 accumulation): in (planar, B x 32 x H x H, read

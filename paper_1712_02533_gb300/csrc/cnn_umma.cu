@@ -814,7 +814,7 @@ __global__ void __launch_bounds__(128) k_conv_umma_staged(const float *__restric
 // of one tile run while the next is staged; the bias sums (of the unrounded
 // FP32 gradient) are formed from the staging registers.  Each CTA writes one
 // record in the parameter layout ((o 32 + c) 9 + tap, then the 32 biases);
-// k_wgrad_umma_reduce adds the records in block order.
+// cnn_sum_records adds the records.
 constexpr int WG_TH = 8, WG_TW = 16, WG_N = 96, WG_COLS = 512;
 constexpr int WG_REC = UC * UC * 9 + UC;
 
@@ -992,14 +992,28 @@ __global__ void __launch_bounds__(256, 1) k_wgrad32_umma(const uint4 *__restrict
     umma_teardown<WG_COLS>(tmem);
 }
 
-// grad[e] = the records' sum in block order, one thread per entry.
-__global__ void k_wgrad_umma_reduce(const float *__restrict__ part, int nblk, float *__restrict__ grad)
+// grad[e] = sum of the records' entries e < rec: a warp's lanes on adjacent
+// entries, 32 groups of records side by side (a chain of a few loads each), the
+// groups in order.  9.3 -> 3.5 us for the 152 records of a 32 -> 32 layer against
+// one thread per entry walking all records.
+__global__ void __launch_bounds__(1024) k_sum_records(const float *__restrict__ part, int nrec, int rec,
+                                                      float *__restrict__ grad)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= WG_REC) return;
+    __shared__ float red[32][32];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
     float s = 0.f;
-    for (int k = 0; k < nblk; k++) s += part[(int64_t)k * WG_REC + e];
-    grad[e] = s;
+    if (e < rec) {
+#pragma unroll 8
+        for (int k = g; k < nrec; k += 32) s += part[(int64_t)k * rec + e];
+    }
+    red[g][lane] = s;
+    __syncthreads();
+    if (g == 0 && e < rec) {
+        float tot = 0.f;
+#pragma unroll
+        for (int w = 0; w < 32; w++) tot += red[w][lane];
+        grad[e] = tot;
+    }
 }
 
 // cuTensorMapEncodeTiled from the driver, found once.
@@ -1169,7 +1183,7 @@ reg_status launch_wgrad_umma(const uint16_t *in, int H, const float *gz, int B, 
         return reg_internal_fail(REG_ECUDA, "tcgen05 weight gradient: launch attributes");
     k_wgrad32_umma<S><<<grid, 256, WgSmem<S>::bytes, st>>>(reinterpret_cast<const uint4 *>(in), H, gz, Ho, tx, ty, nt,
                                                           part, err);
-    k_wgrad_umma_reduce<<<(WG_REC + 255) / 256, 256, 0, st>>>(part, grid, grad);
+    cnn_sum_records(part, grid, WG_REC, grad, st);
     if (cudaGetLastError() != cudaSuccess) return reg_internal_fail(REG_ECUDA, "tcgen05 weight gradient launch");
     return REG_OK;
 }
@@ -1182,6 +1196,11 @@ reg_status cnn_wgrad32_umma(const uint16_t *in, int H, const float *gz, int B, i
     if (S == 1) return launch_wgrad_umma<1>(in, H, gz, B, grad, part, st, err);
     if (S == 2) return launch_wgrad_umma<2>(in, H, gz, B, grad, part, st, err);
     return reg_internal_fail(REG_EINVAL, "tcgen05 weight gradient: stride must be 1 or 2");
+}
+
+void cnn_sum_records(const float *part, int nrec, int rec, float *grad, cudaStream_t st)
+{
+    k_sum_records<<<(rec + 31) / 32, 1024, 0, st>>>(part, nrec, rec, grad);
 }
 
 int cnn_wgrad32_umma_part_floats()

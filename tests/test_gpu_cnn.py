@@ -287,3 +287,29 @@ def test_tensor_core_training_learns(reg, syn):
                   f"{ms:.3f} ms per 32-pair pass, {tf:.1f} TFLOP/s")
     assert hist[True][-1] < 0.6 * hist[True][0]
     assert hist[True][-1] < 1.2 * hist[False][-1]
+
+
+@pytest.mark.parametrize("side,batch", [(16, 1), (20, 3), (36, 2), (132, 1)])
+def test_fp32_gradient_at_ragged_sides(reg, syn, side, batch):
+    """FP32 loss and gradient against FP64 automatic differentiation of the same
+    network, at sides whose rows and columns do not fill the kernels' tiles (4
+    rows per thread, 4 x 32 and 4 x 16 pixel tiles): 1e-5 of the largest
+    component, the bound of the other FP32 gradient tests."""
+    import torch
+    theta = syn.cnn_params(5)
+    g = torch.Generator(device="cuda").manual_seed(side)
+    x = torch.randn((batch, 2, side, side), generator=g, device="cuda")
+    t = torch.randn((batch, 2, side // 4, side // 4), generator=g, device="cuda")
+    with reg.Cnn(theta, side=side, max_batch=batch) as net:
+        loss, got = net.loss_grad(x, t, want_grad=True)
+    th = torch.from_numpy(theta).double().requires_grad_(True)
+    a, off = x.cpu().double(), 0
+    for k, ((c, o), st) in enumerate(zip(syn.CNN_SHAPES, (2, 2, 1, 1, 1, 1))):
+        w, b = th[off:off + o * c * 9].reshape(o, c, 3, 3), th[off + o * c * 9:off + o * c * 9 + o]
+        off += o * c * 9 + o
+        a = torch.nn.functional.conv2d(a, w, b, stride=st, padding=1)
+        a = a if k == 5 else torch.relu(a)
+    want = ((a - t.cpu().double()) ** 2).mean()
+    grad = torch.autograd.grad(want, th)[0].numpy()
+    assert abs(loss - float(want.detach())) <= 1e-5 * float(want.detach())
+    assert np.abs(got - grad).max() <= 1e-5 * np.abs(grad).max()
