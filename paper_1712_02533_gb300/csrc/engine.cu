@@ -19,13 +19,10 @@
 #include "cnn_internal.h"
 
 // kernels (kernels.cu)
-__global__ void k_embed(const float *, int64_t, int64_t, int, float *, int64_t, int);
-__global__ void k_restrict_img(const float *, int64_t, int, int, float *, int64_t, int);
-void launch_image_stats(const float *img, int64_t stride, int pitch, int n, int n_img, double *part, double *out,
-                        cudaStream_t st);
-int image_stats_part_doubles(int n_img);
-__global__ void k_normalize(const float *, int64_t, int, int, const double *, void *, int64_t, int, int);
-__global__ void k_mass_image(const void *, int64_t, int, int, int, float *, int64_t);
+__global__ void k_restrict_img(const float *, int64_t, int64_t, int, int, float *, int64_t, int);
+void launch_pyramid(const RawLevels &lv, int n_img, int bf16, double *work, double *fstats, void *out, float *mr,
+                    int64_t ostride, cudaStream_t st);
+int image_stats_doubles(int n_img, int nl);
 __global__ void k_compose(BatchDev);
 __global__ void k_restrict_u(BatchDev, int);
 __global__ void k_zero_u(BatchDev);
@@ -959,32 +956,38 @@ reg_status validate_params(const reg_params *p)
     return REG_OK;
 }
 
-// Pyramid levels of nf frames from their raw finest levels (rawf: nf blocks of
-// frame_block floats, level L filled): the restriction chain (1/16 [1 2 1; 2 4
-// 2; 1 2 1], Section "Multilevel"), per level the FE mean and sigma and the
+// Pyramid levels of nf frames from their finest level (node (r, c) of frame z at
+// src[z stride + min(r, lim) pitch + min(c, lim)]): the restriction chain (1/16 [1 2
+// 1; 2 4 2; 1 2 1], Section "Multilevel") into rawf (nf blocks of frame_block
+// floats, the coarser levels' scratch), per level the FE mean and sigma and the
 // normalised image (stored as float or bf16) with its M~ R~ image, into pyramid
 // blocks f0 .. f0+nf-1.  The finest level's mean and sigma are kept in fstats.
-void build_levels(reg_series *s, SeriesInfo &si, float *rawf, int f0, int nf, double *stats)
+void build_levels(reg_series *s, SeriesInfo &si, const float *src, int64_t stride, int64_t pitch, int lim, float *rawf,
+                  int f0, int nf, double *work)
 {
     dim3 blk(32, 8);
-    const int kL = si.nl - 1;
-    for (int k = kL - 1; k >= 0; k--)
-        k_restrict_img<<<dim3(cdiv(si.n[k], 32), cdiv(si.n[k], 8), nf), blk, 0, s->stream>>>(
-            rawf + si.img_off[k + 1], (int64_t)si.frame_block, si.pitch[k + 1], si.n[k + 1],
-            rawf + si.img_off[k], (int64_t)si.frame_block, si.pitch[k]);
-    for (int k = 0; k < si.nl; k++) {
-        launch_image_stats(rawf + si.img_off[k], (int64_t)si.frame_block, si.pitch[k], si.n[k], nf, stats + 2 * nf,
-                           stats, s->stream);
-        size_t esz = s->bf16 ? 2 : 4;
-        char *dst = (char *)si.pyr + ((size_t)f0 * si.frame_block + si.img_off[k]) * esz;
-        k_normalize<<<dim3(cdiv(si.n[k], 32), cdiv(si.n[k], 8), nf), blk, 0, s->stream>>>(
-            rawf + si.img_off[k], (int64_t)si.frame_block, si.pitch[k], si.n[k], (const double *)stats, dst,
-            (int64_t)si.frame_block, si.pitch[k], s->bf16);
-        k_mass_image<<<dim3(cdiv(si.n[k], 32), cdiv(si.n[k], 8), nf), blk, 0, s->stream>>>(
-            dst, (int64_t)si.frame_block, si.pitch[k], si.n[k], s->bf16,
-            si.mr + (size_t)f0 * si.frame_block + si.img_off[k], (int64_t)si.frame_block);
+    RawLevels lv;
+    memset(&lv, 0, sizeof(lv));
+    lv.nl = si.nl;
+    for (int k = si.nl - 1; k >= 0; k--) {
+        RawLevel &L = lv.l[k];
+        const bool fine = k == si.nl - 1;
+        L.img = fine ? src : rawf + si.img_off[k];
+        L.stride = fine ? stride : (int64_t)si.frame_block;
+        L.pitch = fine ? pitch : si.pitch[k];
+        L.lim = fine ? lim : si.n[k] - 1;
+        L.n = si.n[k];
+        L.out = (int64_t)si.img_off[k];
+        L.opitch = si.pitch[k];
+        lv.tiles[k] = cdiv(si.n[k], 32) * cdiv(si.n[k], 32);
+        if (k > 0)
+            k_restrict_img<<<dim3(cdiv(si.n[k - 1], 32), cdiv(si.n[k - 1], 8), nf), blk, 0, s->stream>>>(
+                L.img, L.stride, L.pitch, L.n, L.lim, rawf + si.img_off[k - 1], (int64_t)si.frame_block,
+                si.pitch[k - 1]);
     }
-    cudaMemcpyAsync(si.fstats + 2 * (size_t)f0, stats, sizeof(double) * 2 * nf, cudaMemcpyDeviceToDevice, s->stream);
+    const size_t esz = s->bf16 ? 2 : 4, first = (size_t)f0 * si.frame_block;
+    launch_pyramid(lv, nf, s->bf16, work, si.fstats + 2 * (size_t)f0, (char *)si.pyr + first * esz, si.mr + first,
+                   (int64_t)si.frame_block, s->stream);
 }
 
 // Copy a slot field (device) to another slot.
@@ -1180,7 +1183,7 @@ reg_status reg_create_series(const float *frames, int32_t n_series, const int32_
         void *raw = nullptr, *stage = nullptr, *stats = nullptr;
         size_t raw_bytes = (size_t)chunk * si.frame_block * 4;
         if ((st = dalloc(s, &raw, raw_bytes)) != REG_OK) return cleanup(st);
-        if ((st = dalloc(s, &stats, sizeof(double) * (2 * chunk + image_stats_part_doubles(chunk)))) != REG_OK)
+        if ((st = dalloc(s, &stats, sizeof(double) * image_stats_doubles(chunk, si.nl))) != REG_OK)
             return cleanup(st);
         size_t stage_bytes = (size_t)chunk * frame_bytes;
         if (!frames_on_device && !staged && (st = dalloc(s, &stage, stage_bytes)) != REG_OK) return cleanup(st);
@@ -1207,12 +1210,7 @@ reg_status reg_create_series(const float *frames, int32_t n_series, const int32_
                 fstride = (int64_t)si.side * si.side;
                 pitch = si.side;
             }
-            int kL = si.nl - 1;
-            float *rawf = (float *)raw;
-            dim3 blk(32, 8);
-            k_embed<<<dim3(cdiv(nL, 32), cdiv(nL, 8), nf), blk, 0, s->stream>>>(
-                src, fstride, pitch, si.side, rawf + si.img_off[kL], (int64_t)si.frame_block, si.pitch[kL]);
-            build_levels(s, si, rawf, f0, nf, (double *)stats);
+            build_levels(s, si, src, fstride, pitch, si.side - 1, (float *)raw, f0, nf, (double *)stats);
             if (staged) cudaEventRecord(s->ev_drained[b], s->stream);
             cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return cleanup(fail(REG_ECUDA, "pyramid kernels: %s", cudaGetErrorString(e)));
@@ -1462,7 +1460,7 @@ reg_status reg_average_series(reg_series_t s, int32_t series, int32_t iterations
     const int kL = si.nl - 1, nL = si.n[kL];
     void *raw = nullptr, *stats = nullptr;
     RET(dalloc(s, &raw, si.frame_block * sizeof(float)));
-    reg_status st = dalloc(s, &stats, sizeof(double) * (2 + image_stats_part_doubles(1)));
+    reg_status st = dalloc(s, &stats, sizeof(double) * image_stats_doubles(1, si.nl));
     if (st != REG_OK) {
         dfree(s, raw, 0);
         return st;
@@ -1487,7 +1485,7 @@ reg_status reg_average_series(reg_series_t s, int32_t series, int32_t iterations
             // the average becomes the reference frame (pyramid block n_frames);
             // every frame is registered to it by function A, started from its
             // current deformation (frame 0 from the identity at first)
-            build_levels(s, si, rawf, si.n_frames, 1, (double *)stats);
+            build_levels(s, si, rawf + si.img_off[kL], 0, si.pitch[kL], nL - 1, rawf, si.n_frames, 1, (double *)stats);
             CK(cudaGetLastError());
             std::vector<OpReq> ops;
             for (int k = 0; k < si.n_frames; k++) {

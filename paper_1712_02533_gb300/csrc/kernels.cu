@@ -146,23 +146,11 @@ __device__ __forceinline__ int find_entry(const int *pref, int nent, int item)
 // Pyramid construction
 // ---------------------------------------------------------------------------
 
-// Frame (side x side px, pitch in elements) -> level-L vertex grid; last row
-// and column repeated.  grid: (x tiles, y tiles, frames).
-__global__ void k_embed(const float *__restrict__ frames, int64_t frame_stride, int64_t pitch, int side,
-                        float *__restrict__ out, int64_t out_stride, int out_pitch)
-{
-    int f = blockIdx.z;
-    int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y * blockDim.y + threadIdx.y;
-    int n = side + 1;
-    if (r >= n || c >= n) return;
-    int rr = r < side ? r : side - 1, cc = c < side ? c : side - 1;
-    out[f * out_stride + (int64_t)r * out_pitch + c] = frames[f * frame_stride + (int64_t)rr * pitch + cc];
-}
-
-// Restriction 1/16 [1 2 1; 2 4 2; 1 2 1] with mirrored boundary.
-// grid: (x tiles, y tiles, items); fine/coarse images of item z at
-// fine + z*fstride, coarse + z*cstride.
-__global__ void k_restrict_img(const float *__restrict__ fine, int64_t fstride, int fpitch, int nf,
+// Restriction 1/16 [1 2 1; 2 4 2; 1 2 1] with mirrored boundary.  grid: (x tiles, y
+// tiles, images); node (r, c) of a fine image z is fine[z fstride + min(r, lim)
+// fpitch + min(c, lim)]: lim < nf - 1 embeds a frame of lim + 1 pixels on the
+// vertex grid by repeating its last row and column, without a copy of it.
+__global__ void k_restrict_img(const float *__restrict__ fine, int64_t fstride, int64_t fpitch, int nf, int lim,
                                float *__restrict__ coarse, int64_t cstride, int cpitch)
 {
     int z = blockIdx.z;
@@ -175,21 +163,28 @@ __global__ void k_restrict_img(const float *__restrict__ fine, int64_t fstride, 
 #pragma unroll
     for (int a = -1; a <= 1; a++) {
         int r = 2 * I + a;
-        r = r < 0 ? -r : (r > nf - 1 ? 2 * (nf - 1) - r : r);
+        r = min(r < 0 ? -r : (r > nf - 1 ? 2 * (nf - 1) - r : r), lim);
 #pragma unroll
         for (int b = -1; b <= 1; b++) {
             int c = 2 * J + b;
-            c = c < 0 ? -c : (c > nf - 1 ? 2 * (nf - 1) - c : c);
+            c = min(c < 0 ? -c : (c > nf - 1 ? 2 * (nf - 1) - c : c), lim);
             s += w[a + 1] * w[b + 1] * F[(int64_t)r * fpitch + c];
         }
     }
     coarse[z * cstride + (int64_t)I * cpitch + J] = s;
 }
 
-// Per image: FE mean (w^T F) and FE standard deviation ((F-mean)^T M (F-mean))^1/2,
-// two passes over the cells, summed in double.  Each image's cell rows are cut into
-// STATS_SPLIT parts, one block each (grid: parts, images); the parts' sums
-// go to `part` and are added in order by k_image_stats_fin (deterministic).
+// One raw level of the images under construction, node access as above.
+__device__ __forceinline__ const float *level_row(const RawLevel &L, int z, int r)
+{
+    return L.img + z * L.stride + (int64_t)min(r, L.lim) * L.pitch;
+}
+
+// Per image and level: FE mean (w^T F) and FE standard deviation ((F-mean)^T M
+// (F-mean))^1/2, two passes over the cells, summed in double.  Each image's cell
+// rows are cut into STATS_SPLIT parts, one block each (grid: parts x levels,
+// images); the parts' sums go to `part` and are added in order by
+// k_image_stats_fin (deterministic).
 constexpr int STATS_SPLIT = 32;
 
 __device__ __forceinline__ double block_sum_d(double v, double *red)
@@ -204,106 +199,223 @@ __device__ __forceinline__ double block_sum_d(double v, double *red)
     return t;
 }
 
-// pass 0: sum of the cell means; pass 1: sum of the cell mass forms of F - mean
-__global__ void k_image_stats_part(const float *__restrict__ img, int64_t stride, int pitch, int n, int pass,
-                                   const double *__restrict__ stats, double *__restrict__ part)
+// PASS 0: sum of the cell means; PASS 1: sum of the cell mass forms of F - mean.
+// Each cell's term in FP32, their sum in FP64 (GB300's FP64 rate is a small
+// fraction of its FP32 rate): a thread adds its cells of a row (columns t, t + 256,
+// ..) in FP32, then the row's share in FP64.  PASS 1 centres on the FP64 mean
+// rounded to FP32: the cell form's linear term in that offset sums to zero (M 1 = w
+// and sum w (F - mean) = 0), so only its square, ~1e-14 of the variance, remains.
+// A row is loaded once, two columns per cell (its lower edge is the next row's
+// upper one), STATS_COLS columns per thread at a time with the next row in flight;
+// four loads per cell and one row at a time left the pass at 1.2 TB/s of the images
+// (134 us for 40 x 1025^2).
+constexpr int STATS_COLS = 4;  // 4 x 256 columns: sides up to 1024 in one sweep
+template <int PASS>
+__global__ void __launch_bounds__(256) k_image_stats_part(const RawLevels lv, const double *__restrict__ stats,
+                                                          int n_img, double *__restrict__ part)
 {
-    const float *F = img + blockIdx.y * stride;
     __shared__ double red[32];
-    const int rows = n - 1, per = (rows + STATS_SPLIT - 1) / STATS_SPLIT;
-    const int r0 = blockIdx.x * per, r1 = min(rows, r0 + per);
-    // each cell's term in FP32, their sum in FP64 (GB300's FP64 rate is a
-    // small fraction of its FP32 rate).  Pass 1 centres on the FP64 mean
-    // rounded to FP32: the cell form's linear term in that offset sums to
-    // zero (M 1 = w and sum w (F - mean) = 0), so only its square, ~1e-14 of
-    // the variance, remains.
-    // (a thread adds its few cells of a row in FP32, then the row's share in
-    // FP64)
-    const float mf = pass ? (float)stats[2 * blockIdx.y] : 0.f;
+    const int k = blockIdx.x / STATS_SPLIT, sp = blockIdx.x % STATS_SPLIT, z = blockIdx.y;
+    const RawLevel L = lv.l[k];
+    const int n = L.n, rows = n - 1, per = (rows + STATS_SPLIT - 1) / STATS_SPLIT;
+    const int r0 = sp * per, r1 = min(rows, r0 + per);
+    const float mf = PASS ? (float)stats[2 * ((int64_t)k * n_img + z)] : 0.f;
     double s = 0.0;
-    for (int r = r0; r < r1; r++) {
-        const float *row = F + (int64_t)r * pitch;
-        float rs = 0.f;
-        for (int c = threadIdx.x; c < n - 1; c += blockDim.x) {
-            const float *p = row + c;
-            if (!pass) {
-                rs += 0.25f * ((p[0] + p[1]) + (p[pitch] + p[pitch + 1]));
-            } else {
-                const float a = p[0] - mf, b = p[1] - mf, cc = p[pitch + 1] - mf, d = p[pitch] - mf;  // cyclic
-                rs += 4.f * (a * a + b * b + cc * cc + d * d) + 4.f * (a * b + b * cc + cc * d + d * a) +
-                      2.f * (a * cc + b * d);
+    if (n - 1 <= STATS_COLS * 256) {
+        float p0[STATS_COLS], p1[STATS_COLS], q0[STATS_COLS], q1[STATS_COLS];
+        auto load = [&](int r, float (&x0)[STATS_COLS], float (&x1)[STATS_COLS]) {
+            const float *row = level_row(L, z, r);
+#pragma unroll
+            for (int j = 0; j < STATS_COLS; j++) {
+                const int c = threadIdx.x + 256 * j;
+                x0[j] = c < n - 1 ? row[min(c, L.lim)] : 0.f;
+                x1[j] = c < n - 1 ? row[min(c + 1, L.lim)] : 0.f;
+            }
+        };
+        auto step = [&](const float (&x0)[STATS_COLS], const float (&x1)[STATS_COLS], const float (&y0)[STATS_COLS],
+                        const float (&y1)[STATS_COLS]) {
+            float rs = 0.f;
+#pragma unroll
+            for (int j = 0; j < STATS_COLS; j++)
+                if ((int)threadIdx.x + 256 * j < n - 1) {
+                    if (!PASS) {
+                        rs += 0.25f * ((x0[j] + x1[j]) + (y0[j] + y1[j]));
+                    } else {
+                        const float a = x0[j] - mf, b = x1[j] - mf, cc = y1[j] - mf, d = y0[j] - mf;  // cyclic
+                        rs += 4.f * (a * a + b * b + cc * cc + d * d) + 4.f * (a * b + b * cc + cc * d + d * a) +
+                              2.f * (a * cc + b * d);
+                    }
+                }
+            s += (double)rs;
+        };
+        if (r0 < r1) {
+            load(r0, p0, p1);
+            load(r0 + 1, q0, q1);
+            // the row after the cells' lower edge is loaded while they are summed
+            for (int r = r0; r < r1; r++) {
+                float t0[STATS_COLS], t1[STATS_COLS];
+                load(min(r + 2, n - 1), t0, t1);
+                step(p0, p1, q0, q1);
+#pragma unroll
+                for (int j = 0; j < STATS_COLS; j++) { p0[j] = q0[j]; p1[j] = q1[j]; q0[j] = t0[j]; q1[j] = t1[j]; }
             }
         }
-        s += (double)rs;
-    }
-    const double t = block_sum_d(s, red) * (pass ? 1.0 / 36.0 : 1.0);
-    if (threadIdx.x == 0) part[(int64_t)blockIdx.y * STATS_SPLIT + blockIdx.x] = t;
-}
-
-// One thread per image: the parts in order; pass 0 writes the mean, pass 1 sigma.
-__global__ void k_image_stats_fin(int n_img, int n, int pass, const double *__restrict__ part, double *__restrict__ out)
-{
-    const int z = blockIdx.x * blockDim.x + threadIdx.x;
-    if (z >= n_img) return;
-    double t = 0.0;
-    for (int k = 0; k < STATS_SPLIT; k++) t += part[(int64_t)z * STATS_SPLIT + k];
-    const double h2 = 1.0 / ((double)(n - 1) * (n - 1));
-    if (!pass) out[2 * z] = t * h2;
-    else out[2 * z + 1] = sqrt(t * h2);
-}
-
-void launch_image_stats(const float *img, int64_t stride, int pitch, int n, int n_img, double *part, double *out,
-                        cudaStream_t st)
-{
-    for (int pass = 0; pass < 2; pass++) {
-        k_image_stats_part<<<dim3(STATS_SPLIT, n_img), 256, 0, st>>>(img, stride, pitch, n, pass, out, part);
-        k_image_stats_fin<<<(n_img + 127) / 128, 128, 0, st>>>(n_img, n, pass, part, out);
-    }
-}
-
-int image_stats_part_doubles(int n_img) { return n_img * STATS_SPLIT; }
-
-// F~ = (F - mean) / sigma into float or bf16 storage. grid (x, y, images).
-__global__ void k_normalize(const float *__restrict__ img, int64_t stride, int pitch, int n, const double *stats,
-                            void *out, int64_t ostride, int opitch, int bf16)
-{
-    int z = blockIdx.z;
-    int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y * blockDim.y + threadIdx.y;
-    if (r >= n || c >= n) return;
-    double m = stats[2 * z], s = stats[2 * z + 1];
-    float v = (float)(((double)img[z * stride + (int64_t)r * pitch + c] - m) / s);
-    int64_t o = z * ostride + (int64_t)r * opitch + c;
-    if (bf16) reinterpret_cast<__nv_bfloat16 *>(out)[o] = __float2bfloat16_rn(v);
-    else reinterpret_cast<float *>(out)[o] = v;
-}
-
-// M~ R~ of normalised frames at one level: the FE mass matrix in units of h^2,
-// M1 (x) M1 with the 1D weights 1/6, 4/6, 1/6 (2/6 on the diagonal at the
-// border), applied to the stored (float or bf16) image.  The weights are taken
-// as the integers 36 M~ and the sum is divided by 36 once, so that no rounded
-// weight biases every node the same way.  The gradient and trial passes take
-// the NCC terms int R~ phi_i from it.
-__global__ void k_mass_image(const void *img, int64_t stride, int pitch, int n, int bf16, float *out,
-                             int64_t ostride)
-{
-    int z = blockIdx.z;
-    int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y * blockDim.y + threadIdx.y;
-    if (r >= n || c >= n) return;
-    const void *f = bf16 ? (const void *)(reinterpret_cast<const __nv_bfloat16 *>(img) + z * stride)
-                         : (const void *)(reinterpret_cast<const float *>(img) + z * stride);
-    auto w6 = [n](int i, int a) { return a == 0 ? ((i == 0 || i == n - 1) ? 2.f : 4.f) : 1.f; };
-    float acc = 0.f;
-    for (int a = -1; a <= 1; a++) {
-        if (r + a < 0 || r + a >= n) continue;
-        float row = 0.f;
-        for (int bb = -1; bb <= 1; bb++) {
-            if (c + bb < 0 || c + bb >= n) continue;
-            const int i = (r + a) * pitch + (c + bb);
-            row += w6(c, bb) * (bf16 ? ldimg<true>(f, i) : ldimg<false>(f, i));
+    } else {
+        for (int r = r0; r < r1; r++) {
+            const float *x = level_row(L, z, r), *y = level_row(L, z, r + 1);
+            float rs = 0.f;
+            for (int c = threadIdx.x; c < n - 1; c += 256) {
+                const int c1 = min(c + 1, L.lim);
+                if (!PASS) {
+                    rs += 0.25f * ((x[c] + x[c1]) + (y[c] + y[c1]));
+                } else {
+                    const float a = x[c] - mf, b = x[c1] - mf, cc = y[c1] - mf, d = y[c] - mf;  // cyclic
+                    rs += 4.f * (a * a + b * b + cc * cc + d * d) + 4.f * (a * b + b * cc + cc * d + d * a) +
+                          2.f * (a * cc + b * d);
+                }
+            }
+            s += (double)rs;
         }
-        acc += w6(r, a) * row;
     }
-    out[z * ostride + (int64_t)r * pitch + c] = acc / 36.f;
+    const double t = block_sum_d(s, red) * (PASS ? 1.0 / 36.0 : 1.0);
+    if (threadIdx.x == 0) part[((int64_t)k * n_img + z) * STATS_SPLIT + sp] = t;
+}
+
+// One thread per image and level: the parts in order; pass 0 writes the mean, pass 1
+// sigma, of the finest level into fstats too.
+__global__ void k_image_stats_fin(const RawLevels lv, int n_img, int pass, const double *__restrict__ part,
+                                  double *__restrict__ out, double *__restrict__ fstats)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_img * lv.nl) return;
+    const int k = i / n_img, z = i % n_img, n = lv.l[k].n;
+    double v[STATS_SPLIT];
+#pragma unroll
+    for (int q = 0; q < STATS_SPLIT; q++) v[q] = part[(int64_t)i * STATS_SPLIT + q];
+    double t = 0.0;
+#pragma unroll
+    for (int q = 0; q < STATS_SPLIT; q++) t += v[q];
+    const double h2 = 1.0 / ((double)(n - 1) * (n - 1));
+    const double r = pass ? sqrt(t * h2) : t * h2;
+    out[2 * i + pass] = r;
+    if (k == lv.nl - 1) fstats[2 * z + pass] = r;
+}
+
+// doubles of scratch and results for n_img images of nl levels
+int image_stats_doubles(int n_img, int nl) { return n_img * nl * (STATS_SPLIT + 2); }
+
+// F~ = (F - mean) / sigma rounded to float, as FP64 arithmetic gives it: the
+// quotient as an unevaluated sum of two floats (mean and 1 / sigma each as two), to
+// about 2^-45; where that does not settle the rounding (one value in 10^5), in FP64.
+// FP64 divisions of every pixel made the normalisation 860 us for 40 x 1025^2.
+struct NormScale {
+    float mh, ml, ih, il, eps;
+    double m, s;
+};
+
+__device__ __forceinline__ float normalised(const NormScale &q, float x)
+{
+    float dh, dl;
+    two_sum(x, -q.mh, dh, dl);
+    const float e = dl - q.ml, ph = dh * q.ih;
+    const float lo = fmaf(dh, q.ih, -ph) + fmaf(dh, q.il, e * q.ih);
+    const float tol = fmaf(fabsf(ph), 2.2737368e-13f, q.eps);  // 2^-42
+    const float a = ph + (lo - tol), b = ph + (lo + tol);
+    if (a == b) return a;
+    return (float)(((double)x - q.m) / q.s);
+}
+
+// Normalised images (stored as float or bf16) and their M~ R~ images at all levels:
+// M~ R~ is the FE mass matrix in units of h^2, M1 (x) M1 with the 1D weights 1/6,
+// 4/6, 1/6 (2/6 on the diagonal at the border), applied to the stored image.  The
+// weights are taken as the integers 36 M~ and the sum is divided by 36 once, so that
+// no rounded weight biases every node the same way.  The gradient and trial passes
+// take the NCC terms int R~ phi_i from it.  A block normalises a 32 x 32 node tile
+// and one node around it into shared memory and writes both images from there.
+// grid (tiles of all levels, images).
+template <bool BF16>
+__global__ void __launch_bounds__(256) k_norm_mass(const RawLevels lv, const double *__restrict__ stats, int n_img,
+                                                   char *__restrict__ out, float *__restrict__ mr, int64_t ostride)
+{
+    __shared__ float sh[34][35];
+    __shared__ NormScale scale;
+    const int z = blockIdx.y;
+    int k = 0, tile = blockIdx.x;
+    while (tile >= lv.tiles[k]) tile -= lv.tiles[k++];
+    const RawLevel L = lv.l[k];
+    const int n = L.n, tx = (n + 31) / 32, r0 = (tile / tx) * 32, c0 = (tile % tx) * 32;
+    if (threadIdx.x == 0) {
+        NormScale q;
+        const double *st = stats + 2 * ((int64_t)k * n_img + z);
+        q.m = st[0];
+        q.s = st[1];
+        const double inv = 1.0 / q.s;
+        q.mh = (float)q.m;
+        q.ml = (float)(q.m - (double)q.mh);
+        q.ih = (float)inv;
+        q.il = (float)(inv - (double)q.ih);
+        q.eps = fabsf(q.mh) * q.ih * 2.2737368e-13f;
+        scale = q;
+    }
+    __syncthreads();
+    const int tc = threadIdx.x & 31, tr = threadIdx.x >> 5;
+    auto value = [&](int r, int c) {
+        float v = 0.f;
+        if (r >= 0 && r < n && c >= 0 && c < n) v = normalised(scale, level_row(L, z, r)[min(c, L.lim)]);
+        if (BF16) v = __bfloat162float(__float2bfloat16_rn(v));
+        return v;
+    };
+#pragma unroll
+    for (int q = 0; q < 5; q++) {
+        const int lr = tr + 8 * q;
+        if (lr < 34) sh[lr][tc + 1] = value(r0 - 1 + lr, c0 + tc);
+    }
+    if (threadIdx.x < 68) {
+        const int lr = threadIdx.x >> 1, side = threadIdx.x & 1;
+        sh[lr][side ? 33 : 0] = value(r0 - 1 + lr, side ? c0 + 32 : c0 - 1);
+    }
+    __syncthreads();
+    const int c = c0 + tc;
+    if (c >= n) return;
+    const int64_t base = z * ostride + L.out;
+    const float wc = (c == 0 || c == n - 1) ? 2.f : 4.f;
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const int lr = tr + 8 * q, r = r0 + lr;
+        if (r >= n) continue;
+        const int64_t o = base + (int64_t)r * L.opitch + c;
+        const float v = sh[lr + 1][tc + 1];
+        if (BF16) reinterpret_cast<__nv_bfloat16 *>(out)[o] = __float2bfloat16_rn(v);
+        else reinterpret_cast<float *>(out)[o] = v;
+        // nodes past the grid are zero in the tile
+        const float wr = (r == 0 || r == n - 1) ? 2.f : 4.f;
+        float acc = 0.f;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const float row = (sh[lr + a][tc] + wc * sh[lr + a][tc + 1]) + sh[lr + a][tc + 2];
+            acc += (a == 1 ? wr : 1.f) * row;
+        }
+        mr[o] = acc / 36.f;
+    }
+}
+
+// Statistics, normalised and M~ R~ images of n_img images from their raw levels
+// (finest last): out and mr point at the first image's pyramid block, ostride
+// elements apart; work: image_stats_doubles(n_img, nl).
+void launch_pyramid(const RawLevels &lv, int n_img, int bf16, double *work, double *fstats, void *out, float *mr,
+                    int64_t ostride, cudaStream_t st)
+{
+    double *stats = work, *part = work + 2 * (int64_t)n_img * lv.nl;
+    const dim3 grid(STATS_SPLIT * lv.nl, n_img);
+    const int nf = (n_img * lv.nl + 63) / 64;
+    k_image_stats_part<0><<<grid, 256, 0, st>>>(lv, stats, n_img, part);
+    k_image_stats_fin<<<nf, 64, 0, st>>>(lv, n_img, 0, part, stats, fstats);
+    k_image_stats_part<1><<<grid, 256, 0, st>>>(lv, stats, n_img, part);
+    k_image_stats_fin<<<nf, 64, 0, st>>>(lv, n_img, 1, part, stats, fstats);
+    int tiles = 0;
+    for (int k = 0; k < lv.nl; k++) tiles += lv.tiles[k];
+    if (bf16) k_norm_mass<true><<<dim3(tiles, n_img), 256, 0, st>>>(lv, stats, n_img, (char *)out, mr, ostride);
+    else k_norm_mass<false><<<dim3(tiles, n_img), 256, 0, st>>>(lv, stats, n_img, (char *)out, mr, ostride);
 }
 
 // ---------------------------------------------------------------------------

@@ -158,6 +158,21 @@ struct BatchDev {
     float sm_a;            // off-diagonal of the dimensionless 1D system (1/6 - s^2/2)
 };
 
+// Raw levels of the images whose pyramids are being built (0 = coarsest): node
+// (r, c) of image z is img[z stride + min(r, lim) pitch + min(c, lim)] (lim < n - 1:
+// a frame embedded on the vertex grid by repeating its last row and column); out
+// and opitch: the level inside a pyramid block.
+struct RawLevel {
+    const float *img;
+    int64_t stride, pitch, out;
+    int n, lim, opitch;
+};
+struct RawLevels {
+    RawLevel l[REG_MAX_LEVELS];
+    int tiles[REG_MAX_LEVELS];  // 32 x 32 node tiles per level
+    int nl;
+};
+
 // Rigid variant: one level of one operator, and one requested parameter set
 // (element 0 of an operator's REG_MAX_TRIALS requests carries the count n_e
 // and, with grad, the scalars of the gradient at that parameter set).
