@@ -2243,24 +2243,102 @@ __global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
 // Node (r, c) of the finest level: 1/m sum_k F_k(x + u_k(x)), F_k frame k's
 // stored finest level with its normalisation undone (F = F~ sigma_k + mean_k),
 // sampled bilinearly and clamped to the grid; u_k from fields[k] (float2 grid
-// units of the finest level; null = the identity).  Sums in double.
+// units of the finest level; null = the identity), as sums in double give it.
+// Three FP64 operations per sample (16 cycles of an SM each for a warp) took 345 of
+// the 415 us for 64 frames of 1025^2 (255 us now, bound by issue and the latency of
+// field -> texel chains), so the products and their sum run in float
+// pairs (to 2^-44 of the terms' sum, the means' sum is one FP64 constant); a node
+// whose rounding that does not settle, about one in 10^5, is summed again in FP64.
+constexpr int AVG_FRAMES = 128;  // frames staged in shared memory at a time
+constexpr int AVG_BATCH = 2;     // frames whose fields, then texels, a thread has in flight
 template <bool BF16>
-__global__ void k_average(const void *__restrict__ pyr, int64_t frame_block, int64_t img_off, int n, int pitch,
-                          const double *__restrict__ fstats, const float2 *const *__restrict__ fields, int slot_pitch,
-                          int m, float *__restrict__ out, int opitch)
+__global__ void __launch_bounds__(256) k_average(const void *__restrict__ pyr, int64_t frame_block, int64_t img_off,
+                                                 int n, int pitch, const double *__restrict__ fstats,
+                                                 const float2 *const *__restrict__ fields, int slot_pitch, int m,
+                                                 float *__restrict__ out, int opitch)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y * blockDim.y + threadIdx.y;
-    if (r >= n || c >= n) return;
-    double acc = 0.0;
-    for (int k = 0; k < m; k++) {
-        const float2 *f = fields[k];
-        const float2 u = f ? f[(int64_t)r * slot_pitch + c] : make_float2(0.f, 0.f);
-        const void *img = BF16 ? (const void *)(reinterpret_cast<const __nv_bfloat16 *>(pyr) + k * frame_block + img_off)
-                               : (const void *)(reinterpret_cast<const float *>(pyr) + k * frame_block + img_off);
-        const float v = sample<BF16, false>(img, n, pitch, c, r, u.x, u.y, nullptr, nullptr);
-        acc += (double)v * fstats[2 * k + 1] + fstats[2 * k];
+    __shared__ const float2 *fld[AVG_FRAMES];
+    __shared__ const void *img[AVG_FRAMES];
+    __shared__ float2 sig[AVG_FRAMES];  // sigma_k as two floats
+    __shared__ double mean_sum;
+    const int c = blockIdx.x * 32 + threadIdx.x, r = blockIdx.y * 8 + threadIdx.y;
+    const int tid = threadIdx.y * 32 + threadIdx.x;
+    const bool in = r < n && c < n;
+    const int node = r * slot_pitch + c;
+    auto image = [&](int k) {
+        return BF16 ? (const void *)(reinterpret_cast<const __nv_bfloat16 *>(pyr) + k * frame_block + img_off)
+                    : (const void *)(reinterpret_cast<const float *>(pyr) + k * frame_block + img_off);
+    };
+    if (tid < 32) {
+        double s = 0.0;
+        for (int k = tid; k < m; k += 32) s += fstats[2 * k];
+        s = warp_sum_d(s);
+        if (tid == 0) mean_sum = s;
     }
-    out[(int64_t)r * opitch + c] = (float)(acc / m);
+    float hi = 0.f, lo = 0.f, mag = 0.f;
+    for (int k0 = 0; k0 < m; k0 += AVG_FRAMES) {
+        const int mk = min(AVG_FRAMES, m - k0);
+        __syncthreads();
+        for (int k = tid; k < mk; k += 256) {
+            fld[k] = fields[k0 + k];
+            img[k] = image(k0 + k);
+            const double s = fstats[2 * (k0 + k) + 1];
+            const float sh = (float)s;
+            sig[k] = make_float2(sh, (float)(s - (double)sh));
+        }
+        __syncthreads();
+        if (in) {
+            auto add = [&](int k, float v) {
+                const float2 s = sig[k];
+                const float p = v * s.x, pl = fmaf(v, s.y, fmaf(v, s.x, -p));
+                float e;
+                two_sum(hi, p, hi, e);
+                lo += e + pl;
+                mag += fabsf(p);
+            };
+            for (int k = 0; k < mk; k += AVG_BATCH) {
+                float2 u[AVG_BATCH];
+                float far = 0.f;
+#pragma unroll
+                for (int q = 0; q < AVG_BATCH; q++) {
+                    const float2 *f = fld[min(k + q, mk - 1)];
+                    u[q] = f ? f[node] : make_float2(0.f, 0.f);
+                }
+#pragma unroll
+                for (int q = 0; q < AVG_BATCH; q++) far += fabsf(u[q].x) + fabsf(u[q].y);
+                if (far < 2097152.f) {
+                    Texel4 t[AVG_BATCH];
+#pragma unroll
+                    for (int q = 0; q < AVG_BATCH; q++) {
+                        locate(n, c, r, u[q].x, u[q].y, t[q].jx, t[q].jy, t[q].ax, t[q].ay, t[q].clx, t[q].cly);
+                        fetch<BF16>(t[q], img[min(k + q, mk - 1)], pitch);
+                    }
+#pragma unroll
+                    for (int q = 0; q < AVG_BATCH; q++)
+                        if (k + q < mk) add(k + q, bil(t[q]));
+                } else {  // beyond floor_i's range, or NaN
+                    for (int q = 0; q < AVG_BATCH && k + q < mk; q++)
+                        add(k + q, sample<BF16, false>(img[k + q], n, pitch, c, r, u[q].x, u[q].y, nullptr, nullptr));
+                }
+            }
+        }
+    }
+    if (!in) return;
+    const double t = ((double)hi + (double)lo) + mean_sum;
+    const double tol = ((double)mag + fabs(mean_sum)) * 5.6843418860808015e-14;  // 2^-44
+    const float a = (float)((t - tol) / m), b = (float)((t + tol) / m);
+    float res = a;
+    if (!(a == b)) {
+        double acc = 0.0;
+        for (int k = 0; k < m; k++) {
+            const float2 *f = fields[k];
+            const float2 u = f ? f[(int64_t)r * slot_pitch + c] : make_float2(0.f, 0.f);
+            const float v = sample<BF16, false>(image(k), n, pitch, c, r, u.x, u.y, nullptr, nullptr);
+            acc += (double)v * fstats[2 * k + 1] + fstats[2 * k];
+        }
+        res = (float)(acc / m);
+    }
+    out[(int64_t)r * opitch + c] = res;
 }
 
 void launch_average(int bf16, cudaStream_t st, const void *pyr, int64_t frame_block, int64_t img_off, int n,
