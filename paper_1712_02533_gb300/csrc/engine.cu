@@ -40,7 +40,7 @@ __global__ void k_slot_to_planes(const float2 *, int, int, float *);
 __global__ void k_slots_to_planes(const float2 *slots, int64_t slot_elems, int k0, const float2 *slot0, int pitch,
                                   int side, float *out);
 __global__ void k_planes_to_slot(const float *, int, float2 *, int);
-void launch_rigid(int bf16, int tiles, int n_ops, cudaStream_t st, const RigidLevel *lv, const RigidReq *req,
+void launch_rigid(int bf16, int tiles, int n_ops, int sets, cudaStream_t st, const RigidLevel *lv, const RigidReq *req,
                   double *part, double *sums);
 void launch_rigid_fill(const RigidReq &q, int n, float2 *slot, int pitch, cudaStream_t st);
 void launch_average(int bf16, cudaStream_t st, const void *pyr, int64_t frame_block, int64_t img_off, int n,
@@ -799,8 +799,12 @@ reg_status run_batch_rigid(reg_series *s, const std::vector<OpReq> &ops, F pre_i
             CK(cudaMemcpyAsync(s->d_rreq, s->h_rreq, sizeof(RigidReq) * REG_MAX_TRIALS * n, cudaMemcpyHostToDevice,
                                s->stream));
             int lvl_tiles = 1;
-            for (int i : act) lvl_tiles = std::max(lvl_tiles, cdiv(s->h_rlv[i].n, 32) * cdiv(s->h_rlv[i].n, 32));
-            launch_rigid(s->bf16, lvl_tiles, n, s->stream, s->d_rlv, s->d_rreq, s->d_rpart, s->d_rsums);
+            int sets = 1;
+            for (int i : act) {
+                lvl_tiles = std::max(lvl_tiles, cdiv(s->h_rlv[i].n, 32) * cdiv(s->h_rlv[i].n, 32));
+                sets = std::max(sets, s->h_rreq[(size_t)i * REG_MAX_TRIALS].n_e);
+            }
+            launch_rigid(s->bf16, lvl_tiles, n, sets, s->stream, s->d_rlv, s->d_rreq, s->d_rpart, s->d_rsums);
             CK(cudaGetLastError());
             CK(cudaMemcpyAsync(s->h_rsums, s->d_rsums, sizeof(double) * RIGID_SUMS * n, cudaMemcpyDeviceToHost,
                                s->stream));

@@ -2363,8 +2363,9 @@ __device__ __forceinline__ float2 rigid_u(const RigidReq &q, int c, int r)
     return make_float2(fmaf(q.a, (float)c, fmaf(-q.b, (float)r, q.tx)), fmaf(q.b, (float)c, fmaf(q.a, (float)r, q.ty)));
 }
 
-// One block per 32 x 32 node tile of one operator (grid: tiles, ops).  For
-// every requested parameter set j < q.n_e: the FE sums of the warped template
+// One block per 32 x 32 node tile, operator and requested parameter set (grid:
+// tiles, ops, sets; one block for all sets of a tile left small batches waiting on
+// four serial passes).  For parameter set j < q.n_e: the FE sums of the warped template
 // That = T(x + u) over the tile (nodes and cells it owns): sum omega That,
 // sum of the Q1 element mass forms of That, sum That M~R~ (multiplied by h^2
 // on the host).  With q.grad: the data part of dE/dtheta at parameter set 0,
@@ -2391,8 +2392,9 @@ __global__ void __launch_bounds__(256) k_rigid_eval(const RigidLevel *__restrict
     const RigidReq *qs = req + (int64_t)o * REG_MAX_TRIALS;
     auto omega = [n](int i) { return (i == 0 || i == n - 1) ? 0.5f : 1.f; };
     auto w6 = [n](int i, int a) { return a == 0 ? ((i == 0 || i == n - 1) ? 2.f : 4.f) : 1.f; };
-    const int nsets = qs[0].n_e;
-    for (int j = 0; j < nsets; j++) {
+    const int j = blockIdx.z;
+    if (j >= qs[0].n_e) return;
+    {
         const RigidReq q = qs[j];
         const bool grad = (j == 0) && q.grad;
         // That on the tile plus a one-node halo (nodes outside the grid: 0)
@@ -2456,28 +2458,37 @@ __global__ void __launch_bounds__(256) k_rigid_eval(const RigidLevel *__restrict
             for (int w = 0; w < 8; w++) acc += red[w][threadIdx.x];
             out[(threadIdx.x < 3 ? 3 * j : 3 * REG_MAX_TRIALS - 3) + threadIdx.x] = acc;
         }
-        __syncthreads();
     }
 }
 
-// Per operator: the tiles' partial sums in a fixed order (one block per op).
-__global__ void k_rigid_reduce(const double *__restrict__ part, int tiles_stride, const RigidLevel *__restrict__ lv,
-                               double *__restrict__ sums)
+// Per operator: the tiles' partial sums in a fixed order (one block per op): warp by
+// warp of 32 tiles, then the warps' sums in order, up to 256 tiles; beyond, a lane
+// first adds every 256th.  Each warp takes (sum, group of 32 tiles) pairs of the sums
+// this round asked for; one sum after the other through the whole block took 21 us.
+__global__ void __launch_bounds__(1024) k_rigid_reduce(const double *__restrict__ part, int tiles_stride,
+                                                       const RigidLevel *__restrict__ lv,
+                                                       const RigidReq *__restrict__ req, double *__restrict__ sums)
 {
     const int o = blockIdx.x;
     const int n = lv[o].n, tx = (n + 31) / 32, tiles = tx * tx;
+    const RigidReq &q = req[(int64_t)o * REG_MAX_TRIALS];
     __shared__ double red[RIGID_SUMS][8];
-    for (int m = 0; m < RIGID_SUMS; m++) {
+    const int lane = threadIdx.x & 31, groups = min(8, (tiles + 31) / 32);
+    const int ne = q.n_e > 0 ? 3 * q.n_e + (q.grad ? 3 : 0) : 0;
+    for (int p = threadIdx.x >> 5; p < ne * groups; p += 32) {
+        const int k = p / groups, g = p % groups;
+        const int m = k < 3 * q.n_e ? k : 3 * REG_MAX_TRIALS + (k - 3 * q.n_e);
         double acc = 0.0;
-        for (int t = threadIdx.x; t < tiles; t += blockDim.x) acc += part[((int64_t)o * tiles_stride + t) * RIGID_SUMS + m];
+        for (int t = g * 32 + lane; t < tiles; t += 256) acc += part[((int64_t)o * tiles_stride + t) * RIGID_SUMS + m];
         acc = warp_sum_d(acc);
-        if ((threadIdx.x & 31) == 0) red[m][threadIdx.x >> 5] = acc;
+        if (lane == 0) red[m][g] = acc;
     }
     __syncthreads();
-    if (threadIdx.x < RIGID_SUMS) {
+    for (int k = threadIdx.x; k < ne; k += 1024) {
+        const int m = k < 3 * q.n_e ? k : 3 * REG_MAX_TRIALS + (k - 3 * q.n_e);
         double acc = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) acc += red[threadIdx.x][w];
-        sums[(int64_t)o * RIGID_SUMS + threadIdx.x] = acc;
+        for (int w = 0; w < groups; w++) acc += red[m][w];
+        sums[(int64_t)o * RIGID_SUMS + m] = acc;
     }
 }
 
@@ -2490,13 +2501,13 @@ __global__ void k_rigid_fill(RigidReq q, int n, float2 *__restrict__ slot, int p
     slot[(int64_t)r * pitch + c] = rigid_u(q, c, r);
 }
 
-void launch_rigid(int bf16, int tiles, int n_ops, cudaStream_t st, const RigidLevel *lv, const RigidReq *req,
+void launch_rigid(int bf16, int tiles, int n_ops, int sets, cudaStream_t st, const RigidLevel *lv, const RigidReq *req,
                   double *part, double *sums)
 {
-    dim3 grid(tiles, n_ops);
+    dim3 grid(tiles, n_ops, sets);
     if (bf16) k_rigid_eval<true><<<grid, 256, 0, st>>>(lv, req, part);
     else k_rigid_eval<false><<<grid, 256, 0, st>>>(lv, req, part);
-    k_rigid_reduce<<<n_ops, 256, 0, st>>>(part, tiles, lv, sums);
+    k_rigid_reduce<<<n_ops, 1024, 0, st>>>(part, tiles, lv, req, sums);
 }
 
 void launch_rigid_fill(const RigidReq &q, int n, float2 *slot, int pitch, cudaStream_t st)
