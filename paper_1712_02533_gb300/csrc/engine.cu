@@ -314,7 +314,7 @@ int max_tiles(const reg_series *s, int n)
 {
     const int l = level_of(n);
     int g = cdiv(n, REG_GW) * cdiv(n, s->tile_hg[l]);
-    int t = cdiv(n - 1, REG_CW) * cdiv(n - 1, s->tile_ht[l]);
+    int t = cdiv(n - 1, REG_CW) * cdiv(n - 1, std::min(s->tile_ht[l], REG_TRIAL_ROWS));
     return std::max(g, t);
 }
 
@@ -331,7 +331,7 @@ void fill_level(const reg_series *s, LevelDesc &L, int n, int pitch)
     L.n = n;
     L.pitch = pitch;
     L.hg = s->tile_hg[level_of(n)];
-    L.ht = s->tile_ht[level_of(n)];
+    L.ht = std::min(s->tile_ht[level_of(n)], REG_TRIAL_ROWS);
     L.tg = cdiv(n, REG_GW) * cdiv(n, L.hg);
     L.tt = cdiv(n - 1, REG_CW) * cdiv(n - 1, L.ht);
     const double h = 1.0 / (n - 1);

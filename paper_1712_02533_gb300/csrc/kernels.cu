@@ -1398,41 +1398,87 @@ __device__ __forceinline__ bool patch_delta(const Patch &P, int n, float ex, flo
     return ok;
 }
 
-// Level-start sums of one strip tile at u, accumulated in double: they seed
-// every search of the level (the trial passes only add changes to them), and
-// the pass runs once per level.  After a level change (PH_PROLONG) the tile forms
-// u itself from the coarser level's records and stores the nodes it owns: the
-// prolongation is needed here only, once per level and operator, and as a kernel
-// of its own it cost every step an (almost always empty) launch of 3 us.
+// Shared memory of one block of the trial pass (one tile).
+constexpr int TRIAL_WARPS = REG_STRIP_THREADS / 32;
+constexpr int TRIAL_BLOCKS = 7;   // resident blocks per SM
+constexpr int TRIAL_RB = 1;       // node rows a warp has in flight
+constexpr int TWR = REG_TRIAL_ROWS;  // most cell rows of a tile
+template <int JM>
+struct TrialTile {
+    // per node: A, B, 36 M~That, M~R~ of a node whose moves stay in its cell, else its
+    // changes delta_j (four step sizes per plane)
+    float4 node[(JM + 3) / 4][TWR + 1][32];
+    float qt[TWR + 1][32];                 // Dirichlet form of d over the cells above a row
+    unsigned slow[TWR + 1];                // nodes on the exact path, per row
+    unsigned short qn[(TWR + 1) * 32];     // queued nodes: row << 5 | lane, in row order
+    unsigned short qc[TWR * 32];           // cells with such a corner (between rows row - 1 and row)
+    float mom[9][32];                      // per-lane moments
+    double start[TRIAL_WARPS][4];          // level-start pass: the warps' sums
+};
+
+// The order of the exact sums.  A lane adds the exact changes of every 32nd queued
+// node and cell of a window of rows; a window ends after TW rows, or when more than
+// TQ - 32 nodes (with those of the row above it) or TC - 32 cells are queued.  (The
+// windows are those of a pass that walks the rows with queues of TQ and TC entries;
+// keeping its order of additions keeps every sum, and through the gradient's
+// coefficients every iterate, bit for bit what it was.)
+constexpr int TW = 12, TQ = 96, TC = 192;
+
+// A sum of floats held without rounding beyond 2^-72 of it, as three floats: the
+// FP64 pipe of this chip takes 16 cycles of an SM for a warp's addition and as
+// many for the conversion, which made the level-start pass of 16 x 1025^2 nodes
+// 720 us long; two exact FP32 additions take less than one cycle each.
+struct Sum3 {
+    float a = 0.f, b = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float x)
+    {
+        float e, e2;
+        two_sum(a, x, a, e);
+        two_sum(b, e, b, e2);
+        c += e2;
+    }
+    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
+
+// Level-start sums of node rows ra .. rb-1 of one strip tile at u (and the cells
+// between them; rows ra > r0 of a tile take the row above for their cells), at
+// least in double precision: they seed every search of the level (the trial passes
+// only add changes to them), and the pass runs once per level.  After a level
+// change (PH_PROLONG) the pass forms u itself from the coarser level's records
+// and stores the nodes it owns: the prolongation is needed here only, once per
+// level and operator, and as a kernel of its own it cost every step an (almost
+// always empty) launch of 3 us.
 template <bool BF16>
-__device__ __forceinline__ void start_tile(const StepDesc &s, const StripGeom &g, double *v)
+__device__ __forceinline__ void start_rows(const StepDesc &s, const StripGeom &g, int ra, int rb, double *v)
 {
     const unsigned FULL = 0xffffffffu;
     const bool prol = s.phase == PH_PROLONG;
     NodeRec *V = s.Vc;
     const NodeRec *VC = s.VC;
     const float ptau = s.tau_acc;
-    double s1 = 0.0, s3 = 0.0, q2 = 0.0, quu = 0.0;
+    Sum3 s1, s3, q2, quu;
     float tP = 0.f, tPR = 0.f, pux = 0.f, puy = 0.f;
     float4 uP = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int r = g.r0; r <= g.rEnd; r++) {
+    const int first = ra > g.r0 ? ra - 1 : ra;  // the row above the first one, for the cells between
+    for (int r = first; r < rb; r++) {
         float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
         float t0 = 0.f, mr = 0.f;
+        const bool own = g.nodeCol && r >= ra && (r < g.r0 + g.h || r == g.n - 1);
         if (g.colIn) {
             const int64_t idx = (int64_t)r * g.pitch + g.c;
             if (prol) {
                 u = prolong_node(VC, s.cpitch, ptau, r, g.c);
-                if (g.nodeCol && (r < g.r0 + g.h || r == g.n - 1)) V[idx].u = u;
+                if (own) V[idx].u = u;
             } else {
                 u = V[idx].u;
             }
             mr = s.MR[idx];
             t0 = sample_df<BF16, false>(s.T, g.n, g.pitch, g.c, r, u, nullptr, nullptr);
         }
-        if (g.nodeCol && (r < g.r0 + g.h || r == g.n - 1)) {
+        if (own) {
             const float w = g.wx * ((r == 0 || r == g.n - 1) ? 0.5f : 1.f);
-            s1 += (double)(w * t0);
-            s3 += (double)(mr * t0);
+            s1.add(w * t0);
+            s3.add(mr * t0);
         }
         const float tR = __shfl_down_sync(FULL, t0, 1);
         float4 uR;
@@ -1443,54 +1489,30 @@ __device__ __forceinline__ void start_tile(const StepDesc &s, const StripGeom &g
         const float qx = (uR.x - u.x) + (uR.z - u.z), qy = (uR.y - u.y) + (uR.w - u.w);
         const float rx = (u.x - uP.x) + (u.z - uP.z), ry = (u.y - uP.y) + (u.w - uP.w);
         const float sx = __shfl_down_sync(FULL, rx, 1), sy = __shfl_down_sync(FULL, ry, 1);
-        if (g.cellCol) {
-            const float wrow2 = (float)(2 * ((r > g.r0) + (r < g.rEnd)));
-            q2 += (double)(wrow2 * pform(t0, tR));
-            if (r > g.r0) {
-                q2 += (double)(tP * (2.f * t0 + tR) + tPR * (t0 + 2.f * tR));
-                quu += (double)(pform(pux, qx) + pform(rx, sx) + pform(puy, qy) + pform(ry, sy));
-            }
+        if (g.cellCol && r > first) {
+            // the cell between rows r-1 and r: each row's form twice, the cross terms
+            q2.add(2.f * pform(t0, tR));
+            q2.add(2.f * pform(tP, tPR));
+            q2.add(tP * (2.f * t0 + tR) + tPR * (t0 + 2.f * tR));
+            quu.add(pform(pux, qx) + pform(rx, sx) + pform(puy, qy) + pform(ry, sy));
         }
         tP = t0; tPR = tR;
         pux = qx; puy = qy; uP = u;
     }
-    v[0] = s1;
-    v[1] = q2 * (1.0 / 18.0);
-    v[2] = s3;
-    v[3] = quu * (1.0 / 3.0);
+    v[0] = s1.value();
+    v[1] = q2.value() * (1.0 / 18.0);
+    v[2] = s3.value();
+    v[3] = quu.value() * (1.0 / 3.0);
 }
-
-// Shared memory of one warp in the trial pass.  The row walk sums the nodes
-// and cells that the polynomial moments cover and queues the rest: nodes whose
-// largest move leaves their cell (or whose base point lies outside the grid),
-// and cells with such a corner.  A window of up to TW rows is then finished
-// cooperatively, one queued node or cell per lane, so that the exact path
-// runs on full warps instead of on the few lanes of a row that need it.
-constexpr int TW = 12;   // rows per window
-constexpr int TQ = 96;   // queued nodes (a row adds at most 32)
-constexpr int TC = 192;  // queued cells (a row adds at most 31)
-template <int JM>
-struct TrialScratch {
-    float A[TW + 1][32], B[TW + 1][32];  // A, B of the window's rows; slot 0: the row before the window
-    unsigned char qi[TW + 1][32];        // 1 + queue index of a node on the exact path, else 0
-    unsigned short qn[TQ];               // queued nodes: slot << 5 | lane
-    unsigned short qc[TC];               // queued cells: slot << 5 | lane (between slots slot-1 and slot)
-    float dl[JM][TQ];                    // delta_j of the queued nodes
-    float sn[3][JM][32];                 // per-lane node sums: omega delta, 36 M~That delta, M~R~ delta
-    float sq[JM][32];                    // per-lane cell sums of 18 delta^T M~_e delta
-};
 
 // Exact change of the interpolant at one node for every step size, for a
 // node whose largest move leaves its cell (or whose base point lies outside
 // the grid): the moves that stay in the cell take the polynomial of the base
 // cell, the others the texel patch, or a fresh sample for moves of a cell or
-// more (whose rounding, ~1e-7 of That, is small against such a change).  The
-// changes go to queue entry q and, for an owned node, into the node sums of
-// the lane that computes them.
+// more (whose rounding, ~1e-7 of That, is small against such a change).
 template <bool BF16, int JM>
-__device__ __forceinline__ void node_deltas_exact(const void *T, int n, int pitch, const float *tau, int J, int c, int r,
-                                                  float4 u, float4 dm, float w, bool own, TrialScratch<JM> &sh,
-                                                  int q, int lane)
+__device__ __forceinline__ void node_deltas_exact(const void *T, int n, int pitch, const float *tau, int J, int c,
+                                                  int r, float4 u, float4 dm, float *delta)
 {
     Patch P;
     make_patch<BF16>(P, T, n, pitch, c, r, u, dm.x, dm.y);
@@ -1501,6 +1523,7 @@ __device__ __forceinline__ void node_deltas_exact(const void *T, int n, int pitc
     const float B = dm.x * dm.y * (P.v0[1] - P.v0[0]);
 #pragma unroll
     for (int j = 0; j < JM; j++) {
+        delta[j] = 0.f;
         if (j < J) {
             const float ex = tau[j] * dm.x, ey = tau[j] * dm.y;
             const float ax1 = P.ax + ex, ay1 = P.ay + ey;
@@ -1513,313 +1536,376 @@ __device__ __forceinline__ void node_deltas_exact(const void *T, int n, int pitc
                 fetch<BF16>(t, T, pitch);
                 del = bil(t) - P.t0;
             }
-            sh.dl[j][q] = del;
-            if (own) {
-                sh.sn[0][j][lane] += w * del;
-                sh.sn[1][j][lane] += dm.z * del;
-                sh.sn[2][j][lane] += dm.w * del;
-            }
+            delta[j] = del;
         }
     }
 }
 
-// Finish a window whose rows rlast-nrow+1 .. rlast sit in slots 1..nrow: the
-// queued nodes from entry q0 on (one per lane), then the queued cells, whose
-// corners take either a queued node's exact change or the polynomial of their
-// A and B.  The last row moves to slot 0 with the changes of its queued nodes,
-// for the cells between it and the next window.
-template <bool BF16, int JM>
-__device__ __forceinline__ void trial_flush(const void *T, const StripGeom &g, const float4 *V,
-                                            const float *tau, int J, TrialScratch<JM> &sh, int lane, int rlast,
-                                            int nrow, int &q0, int &qn, int &qc)
+// pform and the rest of a cell's form (below) for two values at a time, rounded as the
+// scalar expressions are.
+__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 pform2(float2 x0, float2 x1)
 {
-    const unsigned FULL = 0xffffffffu;
-    __syncwarp();
-    for (int q = q0 + lane; q < qn; q += 32) {
-        const int e = sh.qn[q], slot = e >> 5, ln = e & 31;
-        const int r = rlast - nrow + slot, c = g.c - lane + ln;
-        const int64_t idx = (int64_t)r * g.pitch + c;
-        const float4 u = V[2 * idx], dm = V[2 * idx + 1];
-        const bool own = (ln < REG_CW || c == g.n - 1) && (r < g.r0 + g.h || r == g.n - 1);
-        const float w = ((c == 0 || c == g.n - 1) ? 0.5f : 1.f) * ((r == 0 || r == g.n - 1) ? 0.5f : 1.f);
-        node_deltas_exact<BF16, JM>(T, g.n, g.pitch, tau, J, c, r, u, dm, w, own, sh, q, lane);
-    }
-    __syncwarp();
-    for (int q = lane; q < qc; q += 32) {
-        const int e = sh.qc[q], slot = e >> 5, ln = e & 31;
-        const int itl = sh.qi[slot - 1][ln], itr = sh.qi[slot - 1][ln + 1];
-        const int ibl = sh.qi[slot][ln], ibr = sh.qi[slot][ln + 1];
-        const float Atl = sh.A[slot - 1][ln], Btl = sh.B[slot - 1][ln];
-        const float Atr = sh.A[slot - 1][ln + 1], Btr = sh.B[slot - 1][ln + 1];
-        const float Abl = sh.A[slot][ln], Bbl = sh.B[slot][ln];
-        const float Abr = sh.A[slot][ln + 1], Bbr = sh.B[slot][ln + 1];
-#pragma unroll
-        for (int j = 0; j < JM; j++) {
-            if (j < J) {
-                const float t = tau[j];
-                const float tl = itl ? sh.dl[j][itl - 1] : t * (Atl + t * Btl);
-                const float tr = itr ? sh.dl[j][itr - 1] : t * (Atr + t * Btr);
-                const float bl = ibl ? sh.dl[j][ibl - 1] : t * (Abl + t * Bbl);
-                const float br = ibr ? sh.dl[j][ibr - 1] : t * (Abr + t * Bbr);
-                sh.sq[j][lane] += 2.f * (pform(tl, tr) + pform(bl, br)) + tl * (2.f * bl + br) + tr * (bl + 2.f * br);
-            }
-        }
-    }
-    __syncwarp();
-    // the last row becomes slot 0
-    const int iq = sh.qi[nrow][lane];
-    const unsigned m = __ballot_sync(FULL, iq != 0);
-    const int np = __popc(m & ((1u << lane) - 1u));
-    float keep[JM];
-#pragma unroll
-    for (int j = 0; j < JM; j++) keep[j] = (iq && j < J) ? sh.dl[j][iq - 1] : 0.f;
-    const float a = sh.A[nrow][lane], b = sh.B[nrow][lane];
-    __syncwarp();
-    sh.A[0][lane] = a;
-    sh.B[0][lane] = b;
-    sh.qi[0][lane] = iq ? (unsigned char)(np + 1) : 0;
-    if (iq) {
-#pragma unroll
-        for (int j = 0; j < JM; j++)
-            if (j < J) sh.dl[j][np] = keep[j];
-    }
-    qn = q0 = __popc(m);
-    qc = 0;
-    __syncwarp();
+    return __ffma2_rn(x1, x1, __fmul2_rn(x0, __fadd2_rn(x0, x1)));
+}
+// 2 (P(top) + P(bottom)) + top . [2 1; 1 2] bottom, the rows' forms given
+__device__ __forceinline__ float2 cell2(float2 pt, float2 pb, float2 tl, float2 tr, float2 bl, float2 br)
+{
+    const float2 two = f2(2.f, 2.f);
+    return __ffma2_rn(tr, __ffma2_rn(two, br, bl),
+                      __ffma2_rn(tl, __ffma2_rn(two, bl, br), __fmul2_rn(two, __fadd2_rn(pt, pb))));
 }
 
-// Trial sums of one strip tile for the step sizes tau_0..tau_{J-1}.  All step
-// sizes move a node along the same ray u + tau d, and while the moved point
-// stays in the base cell the change of the bilinear interpolant is exactly
+// Row counts of the exact path's queues, one row per lane (row 32 apart): the mask
+// of the row's nodes, and inclusive prefixes of the queued nodes and cells.
+struct RowQueues {
+    unsigned s, cells;   // nodes on the exact path; mixed cells between this row and the one above
+    int pn, pc;          // inclusive prefixes over rows 0 .. lane
+    unsigned s32, cells32;
+    int tn, tc;          // totals
+};
+
+template <int JM>
+__device__ __forceinline__ RowQueues row_queues(const TrialTile<JM> &sh, int nr, unsigned cellmask, int lane)
+{
+    RowQueues q;
+    q.s = lane < nr ? sh.slow[lane] : 0u;
+    const unsigned up = __shfl_up_sync(0xffffffffu, q.s, 1);
+    // a cell's corners: columns l and l + 1 of both rows
+    q.cells = lane > 0 && lane < nr ? (up | up >> 1 | q.s | q.s >> 1) & cellmask : 0u;
+    q.pn = __popc(q.s);
+    q.pc = __popc(q.cells);
+#pragma unroll
+    for (int k = 1; k < 32; k <<= 1) {
+        const int a = __shfl_up_sync(0xffffffffu, q.pn, k), b = __shfl_up_sync(0xffffffffu, q.pc, k);
+        if (lane >= k) { q.pn += a; q.pc += b; }
+    }
+    const unsigned s31 = __shfl_sync(0xffffffffu, q.s, 31);
+    q.s32 = nr > 32 ? sh.slow[32] : 0u;
+    q.cells32 = nr > 32 ? (s31 | s31 >> 1 | q.s32 | q.s32 >> 1) & cellmask : 0u;
+    q.tn = __shfl_sync(0xffffffffu, q.pn, 31) + __popc(q.s32);
+    q.tc = __shfl_sync(0xffffffffu, q.pc, 31) + __popc(q.cells32);
+    return q;
+}
+
+// Trial sums of one strip tile for the step sizes tau_0..tau_{J-1}, by one block.
+// All step sizes move a node along the same ray u + tau d, and while the moved
+// point stays in the base cell the change of the bilinear interpolant is exactly
 //   delta(tau) = tau A + tau^2 B,  A = d . grad That (at the base point),
 //   B = d_x d_y (t00 - t01 - t10 + t11),
-// so the sums over such nodes and cells are polynomials in tau of per-node
-// moments (sum omega A, sum omega B, ...; 18 A^T M~ A, 18 A^T M~ B, 18 B^T M~ B
-// per cell) that are gathered once for all step sizes.  A node whose largest
-// move leaves the cell, and every cell touching one, is summed exactly for each
-// step size, in windows of rows finished by the whole warp (trial_flush).  The
-// node record of the next row is loaded while the current row is worked on.
+// so the sums over such nodes are polynomials in tau of per-node moments (sum omega
+// A, sum omega B, ...) and of per-cell ones (18 A^T M~ A, 18 A^T M~ B, 18 B^T M~ B),
+// gathered once for all step sizes.  A node whose largest move leaves the cell, and
+// every cell touching one, is summed exactly for each step size.  Phases, the tile's
+// nodes in shared memory between them:
+//   1. every warp walks some rows, TRIAL_RB at a time without a branch, their texel
+//      loads and the next rows' records in flight together: A, B, and which
+//      nodes take the exact path;
+//   2. lists of those nodes and of the cells that touch one;
+//   3. exact changes, one node per thread; beside them the moments, one kind per
+//      warp, each down the rows;
+//   4. per two step sizes (one warp) the exact nodes and cells.
+// One warp per tile doing all of this row by row held 128 registers (16 warps on an
+// SM) and waited for the record -> template gather of every row: per launch of a 33 x
+// 1024^2 scan 122 -> 104 us, of a 21 x 512^2 one 37 -> 23, of a single 1024^2 operator
+// 24 -> 15, of 7 operators of 64^2 12.6 -> 8.  Seven blocks per SM at one row in flight
+// (72 registers) beat six (80) at one or two rows, 104 against 112 and 109 us.
 template <bool BF16, int JM>
-__device__ __forceinline__ void steps_tile(const StepDesc &s, const StripGeom &g, float *v,
-                                           TrialScratch<JM> &sh, int lane, unsigned &nexact)
+__device__ __forceinline__ void trial_tile(const BatchDev &b, const StepDesc &s, const StripGeom &g, TrialTile<JM> &sh,
+                                           int part, int wid, int lane)
 {
     const unsigned FULL = 0xffffffffu;
     const unsigned lt = (1u << lane) - 1u;
-    const int J = min(s.ntr, JM);
+    const int J = min(s.ntr, JM), n = g.n, pitch = g.pitch;
     const bool withQ = (s.phase == PH_GRAD);
     const float4 *V = reinterpret_cast<const float4 *>(s.Vc);
     const void *T = s.T;
-    float tau[JM];
-    float tmax = 0.f;
+    // node rows r0 .. r0 + nr - 1, this warp's i0 .. i1 - 1
+    const int w0 = g.r0, cells = g.rEnd - w0, nr = cells + 1;
+    const int rw = (cells + TRIAL_WARPS - 1) / TRIAL_WARPS;
+    const int i0 = min(wid * rw, nr), i1 = wid == TRIAL_WARPS - 1 ? nr : min(i0 + rw, nr);
+    {
+        float tmax = 0.f;
 #pragma unroll
-    for (int j = 0; j < JM; j++) {
-        tau[j] = (j < J) ? s.tau[j] : 0.f;
-        tmax = fmaxf(tmax, tau[j]);
-#pragma unroll
-        for (int k = 0; k < 3; k++) sh.sn[k][j][lane] = 0.f;
-        sh.sq[j][lane] = 0.f;
-    }
-    // node moments (owned nodes that stay in their cell) and cell moments
-    float mWA = 0.f, mWB = 0.f, mTA = 0.f, mTB = 0.f, mRA = 0.f, mRB = 0.f;
-    float qaa = 0.f, qab = 0.f, qbb = 0.f;
-    // the previous row: A, B here and at the right neighbour, its row forms
-    float Ap = 0.f, ApR = 0.f, Bp = 0.f, BpR = 0.f, PaaP = 0.f, PabP = 0.f, PbbP = 0.f;
-    bool slowP = false, slowPR = false;
-    float qdd = 0.f, pdx = 0.f, pdy = 0.f, dPx = 0.f, dPy = 0.f;
-    int q0 = 0, qn = 0, qc = 0, nrow = 0;  // queue state (warp-uniform)
-    float4 nu = make_float4(0.f, 0.f, 0.f, 0.f), ndm = nu;  // record of the next row
-    if (g.colIn) {
-        const int64_t idx = (int64_t)g.r0 * g.pitch + g.c;
-        nu = V[2 * idx];
-        ndm = V[2 * idx + 1];
-    }
-    for (int r = g.r0; r <= g.rEnd; r++) {
-        const float4 u = nu, dm = ndm;  // d = (dm.x, dm.y), 36 M~That = dm.z, M~R~ = dm.w
-        if (g.colIn && r < g.rEnd) {
-            const int64_t idx = (int64_t)(r + 1) * g.pitch + g.c;
-            nu = V[2 * idx];
-            ndm = V[2 * idx + 1];
+        for (int j = 0; j < JM; j++) tmax = fmaxf(tmax, j < J ? s.tau[j] : 0.f);
+        // lanes past the grid work on its last column and count nothing
+        const int cc = min(g.c, n - 1);
+        const float4 *Vcol = V + 2 * cc;  // (a level's records: below 2^27 words)
+        float dPx = 0.f, dPy = 0.f, pdx = 0.f, pdy = 0.f;
+        if (withQ && i0 > 0 && i0 < i1) {
+            const float4 dm = Vcol[2 * (w0 + i0 - 1) * pitch + 1];
+            dPx = dm.x;
+            dPy = dm.y;
+            pdx = __shfl_down_sync(FULL, dPx, 1) - dPx;
+            pdy = __shfl_down_sync(FULL, dPy, 1) - dPy;
         }
-        const bool own = g.nodeCol && (r < g.r0 + g.h || r == g.n - 1);
-        const float w = g.wx * ((r == 0 || r == g.n - 1) ? 0.5f : 1.f);
-        float A = 0.f, B = 0.f;
-        bool slow = false;
-        if (g.colIn) {
-            Texel4 q;
-            int ix, iy;
-            df_split(u.x, u.z, ix, q.ax);
-            df_split(u.y, u.w, iy, q.ay);
-            q.jx = g.c + ix;
-            q.jy = r + iy;
-            // a base point outside the grid, or a largest move that leaves the
-            // cell (then every smaller one along the ray stays inside)
-            const float ax1 = q.ax + tmax * dm.x, ay1 = q.ay + tmax * dm.y;
-            slow = q.jx < 0 || q.jx > g.n - 2 || q.jy < 0 || q.jy > g.n - 2 || !(ax1 >= 0.f && ax1 < 1.f) ||
-                   !(ay1 >= 0.f && ay1 < 1.f);
-            if (!slow) {
-                fetch<BF16>(q, T, g.pitch);
+        constexpr int RB = TRIAL_RB;
+        float4 nu[RB], nd[RB];
+#pragma unroll
+        for (int k = 0; k < RB; k++) {
+            const int o = 2 * (w0 + min(i0 + k, cells)) * pitch;
+            nu[k] = Vcol[o];
+            nd[k] = Vcol[o + 1];
+        }
+        for (int i = i0; i < i1; i += RB) {
+            float4 dmr[RB];  // d, 36 M~That, M~R~
+            Texel4 t[RB];
+            bool slw[RB];
+#pragma unroll
+            for (int k = 0; k < RB; k++) {
+                const int r = w0 + min(i + k, cells);
+                dmr[k] = nd[k];
+                int ix, iy;
+                df_split(nu[k].x, nu[k].z, ix, t[k].ax);
+                df_split(nu[k].y, nu[k].w, iy, t[k].ay);
+                const int jx = cc + ix, jy = r + iy;
+                // a base point outside the grid, or a largest move that leaves the
+                // cell (then every smaller one along the ray stays inside)
+                const float ax1 = t[k].ax + tmax * dmr[k].x, ay1 = t[k].ay + tmax * dmr[k].y;
+                slw[k] = (unsigned)jx > (unsigned)(n - 2) || (unsigned)jy > (unsigned)(n - 2) ||
+                         !(ax1 >= 0.f && ax1 < 1.f) || !(ay1 >= 0.f && ay1 < 1.f);
+                t[k].jx = min(max(jx, 0), n - 2);
+                t[k].jy = min(max(jy, 0), n - 2);
+                fetch<BF16>(t[k], T, pitch);
+            }
+#pragma unroll
+            for (int k = 0; k < RB; k++) {
+                const int o = 2 * (w0 + min(i + RB + k, cells)) * pitch;
+                nu[k] = Vcol[o];
+                nd[k] = Vcol[o + 1];
+            }
+#pragma unroll
+            for (int k = 0; k < RB; k++) {
+                if (k > 0 && i + k >= i1) break;  // warp-uniform
+                const Texel4 &q = t[k];
+                const float4 dm = dmr[k];
                 const float dtx = q.t01 - q.t00, dtx1 = q.t11 - q.t10;
                 const float sx = dtx + q.ay * (dtx1 - dtx);                            // dThat/dx
                 const float sy = (q.t10 - q.t00) + q.ax * ((q.t11 - q.t01) - (q.t10 - q.t00));  // dThat/dy
-                A = dm.x * sx + dm.y * sy;
-                B = dm.x * dm.y * (dtx1 - dtx);
-                if (own) {
-                    mWA += w * A; mWB += w * B;
-                    mTA += dm.z * A; mTB += dm.z * B;
-                    mRA += dm.w * A; mRB += dm.w * B;
+                const float A = dm.x * sx + dm.y * sy;
+                const float B = dm.x * dm.y * (dtx1 - dtx);
+                const unsigned ms = __ballot_sync(FULL, slw[k] && g.colIn);
+                if (lane == 0) sh.slow[i + k] = ms;
+                sh.node[0][i + k][lane] = make_float4(A, B, dm.z, dm.w);
+                if (withQ) {
+                    // Dirichlet form of d over the cells between rows r-1 and r
+                    const float dRx = __shfl_down_sync(FULL, dm.x, 1), dRy = __shfl_down_sync(FULL, dm.y, 1);
+                    const float qx = dRx - dm.x, qy = dRy - dm.y;
+                    const float rx = dm.x - dPx, ry = dm.y - dPy;
+                    const float sx = __shfl_down_sync(FULL, rx, 1), sy = __shfl_down_sync(FULL, ry, 1);
+                    sh.qt[i + k][lane] = pform(pdx, qx) + pform(rx, sx) + pform(pdy, qy) + pform(ry, sy);
+                    pdx = qx; pdy = qy; dPx = dm.x; dPy = dm.y;
                 }
             }
         }
-        // this row's slot in the window; queue its nodes on the exact path
-        const int slot = nrow + 1;
-        const unsigned ms = __ballot_sync(FULL, slow);
-        nexact += __popc(ms);
-        const int pos = qn + __popc(ms & lt);
-        sh.A[slot][lane] = A;
-        sh.B[slot][lane] = B;
-        sh.qi[slot][lane] = slow ? (unsigned char)(pos + 1) : 0;
-        if (slow) sh.qn[pos] = (unsigned short)((slot << 5) | lane);
-        qn += __popc(ms);
-        // cells between rows r-1 and r, columns c and c+1
-        const float AR = __shfl_down_sync(FULL, A, 1), BR = __shfl_down_sync(FULL, B, 1);
-        const bool slowR = __shfl_down_sync(FULL, slow, 1);
-        const float Paa = pform(A, AR), Pbb = pform(B, BR);
-        const float Pab = A * B + AR * BR + 0.5f * (A * BR + AR * B);
-        bool mixed = false;
-        if (g.cellCol && r > g.r0) {
-            if (!(slowP || slowPR || slow || slowR)) {
+    }
+    __syncthreads();
+    // lists, each warp its rows'
+    const unsigned cellmask = __ballot_sync(FULL, g.cellCol);
+    const RowQueues rq = row_queues(sh, nr, cellmask, lane);
+    if (rq.tn > 0)
+        for (int i = i0; i < i1; i++) {
+            const int src = i & 31;
+            const unsigned ms = i < 32 ? __shfl_sync(FULL, rq.s, src) : rq.s32;
+            const unsigned mc = i < 32 ? __shfl_sync(FULL, rq.cells, src) : rq.cells32;
+            const int en = i < 32 ? __shfl_sync(FULL, rq.pn, src) : rq.tn, ec = i < 32 ? __shfl_sync(FULL, rq.pc, src) : rq.tc;
+            if (ms >> lane & 1) sh.qn[en - __popc(ms) + __popc(ms & lt)] = (unsigned short)((i << 5) | lane);
+            if (mc >> lane & 1) sh.qc[ec - __popc(mc) + __popc(mc & lt)] = (unsigned short)((i << 5) | lane);
+        }
+    __syncthreads();
+    // exact changes in place of the queued nodes' entries (the moments below skip them)
+    if (rq.tn > 0) {
+        float tau[JM];
+#pragma unroll
+        for (int j = 0; j < JM; j++) tau[j] = j < J ? s.tau[j] : 0.f;
+        for (int k = wid * 32 + lane; k < rq.tn; k += REG_STRIP_THREADS) {
+            const int e = sh.qn[k], i = e >> 5, ln = e & 31;
+            const int r = w0 + i, c = g.c - lane + ln;
+            const int idx = 2 * (r * pitch + c);
+            const float4 u = V[idx], dm = V[idx + 1];
+            float del[(JM + 3) / 4 * 4];
+#pragma unroll
+            for (int j = JM; j < (JM + 3) / 4 * 4; j++) del[j] = 0.f;
+            node_deltas_exact<BF16, JM>(T, n, pitch, tau, J, c, r, u, dm, del);
+#pragma unroll
+            for (int m = 0; m < (JM + 3) / 4; m++)
+                sh.node[m][i][ln] = make_float4(del[4 * m], del[4 * m + 1], del[4 * m + 2], del[4 * m + 3]);
+        }
+    }
+    if (wid == 0) {
+        // node moments (owned nodes that stay in their cell)
+        float mWA = 0.f, mWB = 0.f, mTA = 0.f, mTB = 0.f, mRA = 0.f, mRB = 0.f;
+#pragma unroll 4
+        for (int i = 0; i < nr; i++) {
+            const int r = w0 + i;
+            const float4 q = sh.node[0][i][lane];
+            const bool own = g.nodeCol && (r < g.r0 + g.h || r == n - 1);
+            const float w = g.wx * ((r == 0 || r == n - 1) ? 0.5f : 1.f);
+            if (own && !(sh.slow[i] >> lane & 1)) {
+                mWA += w * q.x; mWB += w * q.y;
+                mTA += q.z * q.x; mTB += q.z * q.y;
+                mRA += q.w * q.x; mRB += q.w * q.y;
+            }
+        }
+        sh.mom[0][lane] = mWA; sh.mom[1][lane] = mWB;
+        sh.mom[2][lane] = mTA; sh.mom[3][lane] = mTB;
+        sh.mom[4][lane] = mRA; sh.mom[5][lane] = mRB;
+    } else if (wid == 1) {
+        // cell moments of A and of B (cells whose four corners stay in their cells)
+        float2 q = f2(0.f, 0.f), Pv = q, ab0 = q, abR0 = q;
+        unsigned mP = 0u;
+        const int rn = min(lane + 1, 31);
+#pragma unroll 4
+        for (int i = 0; i < nr; i++) {
+            const float2 ab = *reinterpret_cast<const float2 *>(&sh.node[0][i][lane]);
+            const float2 abR = *reinterpret_cast<const float2 *>(&sh.node[0][i][rn]);
+            const unsigned m = sh.slow[i];
+            const float2 P = pform2(ab, abR);
+            if (g.cellCol && i > 0 && !((mP | m) >> lane & 3u)) q = __fadd2_rn(q, cell2(Pv, P, ab0, abR0, ab, abR));
+            Pv = P;
+            ab0 = ab;
+            abR0 = abR;
+            mP = m;
+        }
+        sh.mom[6][lane] = q.x;
+        sh.mom[8][lane] = q.y;
+    } else if (wid == 2) {
+        // their mixed moments
+        float qab = 0.f, Ap = 0.f, ApR = 0.f, Bp = 0.f, BpR = 0.f, PabP = 0.f;
+        unsigned mP = 0u;
+        const int rn = min(lane + 1, 31);
+#pragma unroll 4
+        for (int i = 0; i < nr; i++) {
+            const float2 q = *reinterpret_cast<const float2 *>(&sh.node[0][i][lane]);
+            const float2 qr = *reinterpret_cast<const float2 *>(&sh.node[0][i][rn]);
+            const float A = q.x, B = q.y, AR = qr.x, BR = qr.y;
+            const unsigned m = sh.slow[i];
+            const float Pab = A * B + AR * BR + 0.5f * (A * BR + AR * B);
+            if (g.cellCol && i > 0 && !((mP | m) >> lane & 3u)) {
                 const float ha = 2.f * A + AR, haR = A + 2.f * AR, hb = 2.f * B + BR, hbR = B + 2.f * BR;
-                qaa += 2.f * (PaaP + Paa) + Ap * ha + ApR * haR;
-                qbb += 2.f * (PbbP + Pbb) + Bp * hb + BpR * hbR;
                 qab += 2.f * (PabP + Pab) + 0.5f * (Ap * hb + ApR * hbR + Bp * ha + BpR * haR);
-            } else {
-                mixed = true;
             }
+            PabP = Pab;
+            Ap = A; ApR = AR; Bp = B; BpR = BR;
+            mP = m;
         }
-        const unsigned mc = __ballot_sync(FULL, mixed);
-        if (mixed) sh.qc[qc + __popc(mc & lt)] = (unsigned short)((slot << 5) | lane);
-        qc += __popc(mc);
-        Ap = A; ApR = AR; Bp = B; BpR = BR;
-        PaaP = Paa; PabP = Pab; PbbP = Pbb;
-        slowP = slow; slowPR = slowR;
+        sh.mom[7][lane] = qab;
+    } else {
+        float qdd = 0.f;
         if (withQ) {
-            const float dRx = __shfl_down_sync(FULL, dm.x, 1), dRy = __shfl_down_sync(FULL, dm.y, 1);
-            const float qx = dRx - dm.x, qy = dRy - dm.y;
-            const float rx = dm.x - dPx, ry = dm.y - dPy;
-            const float sx = __shfl_down_sync(FULL, rx, 1), sy = __shfl_down_sync(FULL, ry, 1);
-            if (g.cellCol && r > g.r0) qdd += pform(pdx, qx) + pform(rx, sx) + pform(pdy, qy) + pform(ry, sy);
-            pdx = qx; pdy = qy; dPx = dm.x; dPy = dm.y;
+#pragma unroll 8
+            for (int i = 1; i < nr; i++)
+                if (g.cellCol) qdd += sh.qt[i][lane];
         }
-        nrow++;
-        if (nrow == TW || qn > TQ - 32 || qc > TC - 32 || r == g.rEnd) {
-            if (qn > q0 || qc > 0) trial_flush<BF16, JM>(T, g, V, tau, J, sh, lane, r, nrow, q0, qn, qc);
-            else {
-                // nothing new queued (so the last row has no exact nodes): only
-                // its A, B move to slot 0
-                const float a = sh.A[nrow][lane], b = sh.B[nrow][lane];
-                __syncwarp();
-                sh.A[0][lane] = a;
-                sh.B[0][lane] = b;
-                sh.qi[0][lane] = 0;
-                q0 = qn = 0;
-                __syncwarp();
+        const float tot = warp_sum(qdd / 3.f);
+        if (lane == 0) {
+            b.partT[(int64_t)part * PT_STRIDE + 3 * REG_MAX_TRIALS + 2] = tot;
+            if (rq.tn) atomicAdd(&b.work[KW_TEXACT], (unsigned long long)rq.tn);
+        }
+    }
+    __syncthreads();
+    // two step sizes per warp: the exact nodes and cells, window by window, then the
+    // sums
+    for (int j = 2 * wid; j < J; j += 2 * TRIAL_WARPS) {
+        const float2 t = f2(s.tau[j], j + 1 < J ? s.tau[j + 1] : 0.f);
+        float2 sn0 = f2(0.f, 0.f), sn1 = sn0, sn2 = sn0, sq = sn0;
+        // a node's two changes: at word 2 (j / 2 mod 2) of its entry in plane j / 4, or
+        // from A and B in the first words of its entry
+        const float2 *plane = reinterpret_cast<const float2 *>(&sh.node[0][0][0]);
+        const int dofs = (j >> 2) * (TWR + 1) * 64 + ((j >> 1) & 1);
+        if (rq.tn > 0) {
+            int a = 0, carry = 0, pna = 0, pca = 0;
+            for (;;) {
+                const bool trig = lane >= a && lane < nr &&
+                                  (lane - a == TW - 1 || carry + rq.pn - pna > TQ - 32 || rq.pc - pca > TC - 32 ||
+                                   lane == nr - 1);
+                const unsigned bt = __ballot_sync(FULL, trig);
+                const int e = bt ? __ffs(bt) - 1 : 32;  // the window's last row
+                const int pne = e < 32 ? __shfl_sync(FULL, rq.pn, e) : rq.tn;
+                const int pce = e < 32 ? __shfl_sync(FULL, rq.pc, e) : rq.tc;
+                for (int k = pna + lane; k < pne; k += 32) {
+                    const int en = sh.qn[k], i = en >> 5, ln = en & 31;
+                    const int r = w0 + i, c = g.c - lane + ln;
+                    if ((ln < REG_CW || c == n - 1) && (r < g.r0 + g.h || r == n - 1)) {
+                        const float2 zw = reinterpret_cast<const float2 *>(V + 2 * (r * pitch + c) + 1)[1];
+                        const float w = ((c == 0 || c == n - 1) ? 0.5f : 1.f) * ((r == 0 || r == n - 1) ? 0.5f : 1.f);
+                        const float2 d = plane[2 * en + dofs];
+                        sn0 = __ffma2_rn(f2(w, w), d, sn0);
+                        sn1 = __ffma2_rn(f2(zw.x, zw.x), d, sn1);
+                        sn2 = __ffma2_rn(f2(zw.y, zw.y), d, sn2);
+                    }
+                }
+                for (int k = pca + lane; k < pce; k += 32) {
+                    const int en = sh.qc[k], i = en >> 5, ln = en & 31;
+                    const unsigned mt = sh.slow[i - 1] >> ln, mb = sh.slow[i] >> ln;
+                    auto corner = [&](unsigned slow, int node) {
+                        const float2 q = plane[2 * node + ((slow & 1) ? dofs : 0)];
+                        const float2 pl = __fmul2_rn(t, __ffma2_rn(t, f2(q.y, q.y), f2(q.x, q.x)));
+                        return (slow & 1) ? q : pl;
+                    };
+                    const float2 tl = corner(mt, en - 32), tr = corner(mt >> 1, en - 31);
+                    const float2 bl = corner(mb, en), br = corner(mb >> 1, en + 1);
+                    sq = __fadd2_rn(sq, cell2(pform2(tl, tr), pform2(bl, br), tl, tr, bl, br));
+                }
+                if (e >= nr - 1) break;
+                carry = __popc(__shfl_sync(FULL, rq.s, e));
+                a = e + 1;
+                pna = pne;
+                pca = pce;
             }
-            nrow = 0;
         }
+        const float mWA = sh.mom[0][lane], mWB = sh.mom[1][lane], mTA = sh.mom[2][lane], mTB = sh.mom[3][lane];
+        const float mRA = sh.mom[4][lane], mRB = sh.mom[5][lane];
+        const float qaa = sh.mom[6][lane], qab = sh.mom[7][lane], qbb = sh.mom[8][lane];
+        auto sums = [&](int jj, float t, float sn0, float sn1, float sn2, float sq) {
+            const float v0 = t * (mWA + t * mWB) + sn0;
+            const float v1 = (t * (mTA + t * mTB) + t * t * (qaa + t * (2.f * qab + t * qbb)) + sn1 +
+                              sq) / 18.f;
+            const float v2 = t * (mRA + t * mRB) + sn2;
+            const float t0 = warp_sum(v0), t1 = warp_sum(v1), t2 = warp_sum(v2);
+            if (lane < 3) b.partT[(int64_t)part * PT_STRIDE + 3 * jj + lane] = lane == 0 ? t0 : (lane == 1 ? t1 : t2);
+        };
+        sums(j, t.x, sn0.x, sn1.x, sn2.x, sq.x);
+        if (j + 1 < J) sums(j + 1, t.y, sn0.y, sn1.y, sn2.y, sq.y);
     }
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < JM; j++) {
-        const float t = tau[j];
-        v[3 * j] = t * (mWA + t * mWB) + sh.sn[0][j][lane];
-        v[3 * j + 1] = (t * (mTA + t * mTB) + t * t * (qaa + t * (2.f * qab + t * qbb)) + sh.sn[1][j][lane] +
-                        sh.sq[j][lane]) / 18.f;
-        v[3 * j + 2] = t * (mRA + t * mRB) + sh.sn[2][j][lane];
-    }
-    v[3 * REG_MAX_TRIALS + 2] = qdd / 3.f;
-}
-
-// Warp sums of a tile's partial record; lane k stores entry k.
-template <int JM>
-__device__ __forceinline__ void write_partials(const BatchDev &b, int item, const float *v, int nused, int lane)
-{
-    const unsigned FULL = 0xffffffffu;
-    if constexpr (JM <= 4) {
-        // The (at most) 15 sums by one transpose-reduction: at each butterfly
-        // step (lane offsets 16, 8, 4, 2) a lane keeps half of its values and
-        // adds the partner's copy of them, so that after the last step (offset
-        // 1) lanes 2 k and 2 k + 1 hold sum k.  Every sum pairs the same lanes
-        // in the same order as warp_sum, so the totals are the same floats.
-        float x[16];
-#pragma unroll
-        for (int k = 0; k < 12; k++) x[k] = (k < 3 * JM && k < nused) ? v[k] : 0.f;
-#pragma unroll
-        for (int k = 0; k < 3; k++) x[12 + k] = v[3 * REG_MAX_TRIALS + k];
-        x[15] = 0.f;
-#pragma unroll
-        for (int o = 16, h = 8; h >= 1; o >>= 1, h >>= 1) {
-            const bool up = (lane & o) != 0;
-#pragma unroll
-            for (int i = 0; i < h; i++) {
-                const float send = up ? x[i] : x[h + i], keep = up ? x[h + i] : x[i];
-                x[i] = keep + __shfl_xor_sync(FULL, send, o);
-            }
-        }
-        x[0] += __shfl_xor_sync(FULL, x[0], 1);
-        // entry e of the record: sums 0..11 from lanes 0, 2, .., 22; entries
-        // 3 MAXT .. 3 MAXT + 2 from lanes 24, 26, 28; the rest zero
-        const int src = lane < 12 ? 2 * lane : (lane >= 3 * REG_MAX_TRIALS ? 2 * (12 + lane - 3 * REG_MAX_TRIALS) : 0);
-        const float tot = __shfl_sync(FULL, x[0], src & 31);
-        const bool has = lane < 12 || (lane >= 3 * REG_MAX_TRIALS && lane < PT_STRIDE);
-        if (lane < PT_STRIDE) b.partT[(int64_t)item * PT_STRIDE + lane] = has ? (double)tot : 0.0;
-        return;
-    }
-    double mine = 0.0;
-#pragma unroll
-    for (int k = 0; k < PT_STRIDE; k++) {
-        if ((k < 3 * JM && k < nused) || k >= 3 * REG_MAX_TRIALS) {
-            const float tot = warp_sum(v[k]);
-            if (lane == k) mine = tot;
-        }
-    }
-    if (lane < PT_STRIDE) b.partT[(int64_t)item * PT_STRIDE + lane] = mine;
 }
 
 }  // namespace
 
 template <bool BF16, int JM>
-__global__ void __launch_bounds__(REG_STRIP_THREADS, 4) k_trial(BatchDev b)
+__global__ void __launch_bounds__(REG_STRIP_THREADS, TRIAL_BLOCKS) k_trial(BatchDev b)
 {
-    __shared__ TrialScratch<JM> scratch[REG_STRIP_THREADS / 32];
-    const int lane = threadIdx.x & 31;
-    const int nwarps = gridDim.x * (REG_STRIP_THREADS / 32);
-    const WorkPlan wp = work_plan<false>(b, lane);
-    for (int item = blockIdx.x * (REG_STRIP_THREADS / 32) + (threadIdx.x >> 5); item < wp.items; item += nwarps) {
+    __shared__ TrialTile<JM> sh;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int item = blockIdx.x;; item += gridDim.x) {
+        const WorkPlan wp = work_plan<false>(b, lane);
+        if (item >= wp.items) break;
         int tile;
         const StepDesc &s = b.st[find_item<false>(b, wp, item, tile)].step;
         const StripGeom g = strip_geom(s, tile, lane);
         const int part = s.part0 + tile;
-        const bool start = (s.phase == PH_START || s.phase == PH_PROLONG);
-        if (start) {
+        if (s.phase == PH_START || s.phase == PH_PROLONG) {
             // sums in double, reduced in double: [0..2] and the Dirichlet form of u
             double v[4];
-            start_tile<BF16>(s, g, v);
-            double mine = 0.0;
+            const int rows = g.rEnd - g.r0 + 1, per = (rows + TRIAL_WARPS - 1) / TRIAL_WARPS;
+            const int ra = g.r0 + min(wid * per, rows);
+            start_rows<BF16>(s, g, ra, min(ra + per, g.rEnd + 1), v);
 #pragma unroll
             for (int k = 0; k < 4; k++) {
                 const double tot = warp_sum_d(v[k]);
-                if (lane == (k < 3 ? k : 3 * REG_MAX_TRIALS)) mine = tot;
+                if (lane == 0) sh.start[wid][k] = tot;
             }
-            if (lane < PT_STRIDE) b.partT[(int64_t)part * PT_STRIDE + lane] = mine;
-        } else {
-            float v[PT_STRIDE];
+            __syncthreads();
+            if (threadIdx.x < 4) {
+                double t = 0.0;
 #pragma unroll
-            for (int k = 0; k < PT_STRIDE; k++) v[k] = 0.f;
-            unsigned nexact = 0;
-            steps_tile<BF16, JM>(s, g, v, scratch[threadIdx.x >> 5], lane, nexact);
-            write_partials<JM>(b, part, v, 3 * min(s.ntr, JM), lane);
-            if (lane == 0 && nexact) atomicAdd(&b.work[KW_TEXACT], (unsigned long long)nexact);
+                for (int w = 0; w < TRIAL_WARPS; w++) t += sh.start[w][threadIdx.x];
+                b.partT[(int64_t)part * PT_STRIDE + (threadIdx.x < 3 ? threadIdx.x : 3 * REG_MAX_TRIALS)] = t;
+            }
+        } else {
+            trial_tile<BF16, JM>(b, s, g, sh, part, wid, lane);
         }
+        __syncthreads();
     }
 }
 

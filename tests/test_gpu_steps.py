@@ -79,3 +79,28 @@ def test_smoothed_direction_is_the_tensor_product_solve(reg, syn, side):
         f = w[:, None] * w[None, :] * d_l2[c].astype(np.float64)
         want = solve_banded((1, 1), ab, solve_banded((1, 1), ab, f).T).T
         assert np.abs(got[c] - want).max() <= 1e-5 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("side,rows", [(32, 4), (32, 8), (64, 16), (64, 32), (64, 64), (128, 32)])
+@pytest.mark.parametrize("amp", [1e-3, 0.4, 1.6])
+def test_trial_sums_against_fp64_energies(reg, orc, syn, side, rows, amp):
+    """The trial pass's energy changes against the oracle's FP64 energies at tile
+    heights from four rows to more than a tile holds, with moves from far below
+    a cell (no node on the exact path) to beyond one (every node on it, full
+    queues): 1e-4 relative, the bound of the trial parity test."""
+    rng = np.random.default_rng(side + rows)
+    fr = syn.series(9, 2, side, peak=20.0, spacing=9.0, sigma=1.8)
+    L, n = int(np.log2(side)), side + 1
+    u = (0.3 * rng.standard_normal((2, n, n))).astype(np.float32)
+    with reg.Series(fr, reg.default_params(n_levels=1, lam=10.0)) as s:
+        s.set_tile_rows(L, rows, rows)
+        d, _ = s.eval_direction(0, 1, L, u)
+        t0 = amp / np.abs(d).max()
+        taus = [t0, 0.5 * t0, 0.25 * t0, 0.1 * t0]
+        d, dE = s.eval_trials(0, 1, L, u, taus)
+    g = [orc.embed(f) for f in fr]
+    E = lambda v: orc.energy(g[0], g[1], v / side, 10.0)[0]
+    e0 = E(u.astype(np.float64))
+    for t, got in zip(taus, dE):
+        want = E(u.astype(np.float64) + t * d.astype(np.float64)) - e0
+        assert abs(got - want) <= 1e-4 * abs(want) + 1e-9 * abs(e0), (t, got, want)
