@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <array>
 #include <chrono>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -29,7 +30,7 @@ __global__ void k_zero_u(BatchDev);
 __global__ void k_init_state(BatchDev, int);
 __global__ void k_plan(BatchDev);
 __global__ void k_final(BatchDev);
-void launch_grad(int bf16, int grid, cudaStream_t st, const BatchDev &b);
+void launch_grad(int bf16, bool few, int grid, cudaStream_t st, const BatchDev &b);
 void launch_trial(int bf16, int J, int grid, cudaStream_t st, const BatchDev &b);
 void launch_smooth(int nsm, int ops, int n, cudaStream_t st, const BatchDev &b);
 int smooth_row_chunks(int n);
@@ -148,7 +149,7 @@ struct reg_series {
     reg_params p{};
     int bf16 = 0;
     int nsm = 0;
-    int grid_G = 0, grid_T = 0;  // resident-block grids of the step kernels
+    int grid_G = 0, grid_F = 0, grid_T = 0;  // resident-block grids of the step kernels (F: gradient, few tiles)
     // strip rows of the gradient and trial tiles per level l (2^l + 1 nodes)
     int tile_hg[REG_TILE_LEVELS] = {0}, tile_ht[REG_TILE_LEVELS] = {0};
     std::vector<SeriesInfo> S;
@@ -171,8 +172,8 @@ struct reg_series {
     OpState *h_st = nullptr;
     int h_st_cap = 0;
     // graph of GRAPH_STEPS steps
-    cudaGraphExec_t gexec = nullptr;
-    int graph_gen = -1, buf_gen = 0;
+    cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // wide batches, narrow ones
+    int graph_gen[2] = {-1, -1}, buf_gen = 0;
     // profiling
     cudaEvent_t ev[GRAPH_STEPS][NFAM];
     cudaEvent_t ev_end[GRAPH_STEPS];
@@ -310,10 +311,12 @@ BatchDev make_batch(reg_series *s)
 
 // Work items per operator at a level of n nodes per side: the larger of the
 // gradient and trial strip tiles.
+int grad_tiles(const reg_series *s, int n) { return cdiv(n, REG_GW) * cdiv(n, s->tile_hg[level_of(n)]); }
+
 int max_tiles(const reg_series *s, int n)
 {
     const int l = level_of(n);
-    int g = cdiv(n, REG_GW) * cdiv(n, s->tile_hg[l]);
+    int g = grad_tiles(s, n);
     int t = cdiv(n - 1, REG_CW) * cdiv(n - 1, std::min(s->tile_ht[l], REG_TRIAL_ROWS));
     return std::max(g, t);
 }
@@ -384,13 +387,25 @@ reg_status ensure_capacity(reg_series *s, int n_ops, size_t ws_total, int64_t it
     return REG_OK;
 }
 
-// Capture GRAPH_STEPS steps [G T C] into one executable graph.
-reg_status build_graph(reg_series *s)
+// A batch is narrow if none of its steps has more than GRAD_FEW_WAVES gradient tiles
+// per resident block of the few-tiles form of the gradient pass: up to there that form
+// is the faster one (a 21 x 512^2 scan's passes, 3060 to 6120 tiles: 14.7 us with one
+// tile per block as the limit, 13.8 with two, 13.1 with four).
+constexpr int GRAD_FEW_WAVES = 4;
+
+void launch_gradient(reg_series *s, bool narrow, cudaStream_t st, const BatchDev &b)
 {
-    if (s->gexec && s->graph_gen == s->buf_gen) return REG_OK;
-    if (s->gexec) {
-        cudaGraphExecDestroy(s->gexec);
-        s->gexec = nullptr;
+    launch_grad(s->bf16, narrow, narrow ? s->grid_F : s->grid_G, st, b);
+}
+
+// Capture GRAPH_STEPS steps [G T C] into an executable graph.
+reg_status build_graph(reg_series *s, bool narrow)
+{
+    cudaGraphExec_t &gexec = s->gexec[narrow];
+    if (gexec && s->graph_gen[narrow] == s->buf_gen) return REG_OK;
+    if (gexec) {
+        cudaGraphExecDestroy(gexec);
+        gexec = nullptr;
     }
     BatchDev b = make_batch(s);
     cudaGraph_t g;
@@ -400,17 +415,17 @@ reg_status build_graph(reg_series *s)
     cudaStream_t cs = s->cap_stream;
     CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < GRAPH_STEPS; k++) {
-        launch_grad(s->bf16, s->grid_G, cs, b);
+        launch_gradient(s, narrow, cs, b);
         if (b.smooth) launch_smooth(s->nsm, s->cap_ops, s->sm_n, cs, b);
         launch_trial(s->bf16, s->p.trials_per_pass, s->grid_T, cs, b);
         k_control<<<std::min(s->cap_ops, 2048), REG_CTL_THREADS, 0, cs>>>(b);
     }
     cudaError_t e = cudaStreamEndCapture(cs, &g);
     if (e != cudaSuccess) return fail(REG_ECUDA, "graph capture: %s", cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&s->gexec, g, 0);
+    e = cudaGraphInstantiate(&gexec, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return fail(REG_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
-    s->graph_gen = s->buf_gen;
+    s->graph_gen[narrow] = s->buf_gen;
     return REG_OK;
 }
 
@@ -457,7 +472,7 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
     std::vector<size_t> ws_off(n);
     std::vector<int> part0(n);  // first tile record of each op
     size_t ws = 0;
-    int64_t items = 0;
+    int64_t items = 0, gtiles = 0;
     int nl = 0, nLmax = 0;
     for (int i = 0; i < n; i++) {
         const OpReq &o = ops[i];
@@ -466,11 +481,14 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
         ws += (si.ws_bytes + 255) / 256 * 256;
         part0[i] = (int)items;
         items += max_tiles_series(s, si, o.skip);
+        gtiles += grad_tiles(s, si.n[si.nl - 1]);
         nl = std::max(nl, si.nl);
         nLmax = std::max(nLmax, si.n[si.nl - 1]);
     }
     if (items > INT32_MAX) return fail(REG_EINVAL, "batch of %d ops has too many tiles", n);
     RET(ensure_capacity(s, n, ws, items));
+    // no step has more gradient tiles than one with every op on its finest level
+    const bool narrow = gtiles <= (int64_t)GRAD_FEW_WAVES * s->grid_F;
     for (int i = 0; i < n; i++) {
         const OpReq &o = ops[i];
         const SeriesInfo &si = s->S[o.series];
@@ -550,7 +568,7 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
     s->fam[F_SETUP].launches += 3 + nl;
     s->fam[F_PLAN].launches++;
     const bool prof = (s->p.flags & REG_FLAG_PROFILE) && s->ev_ok;
-    if (!prof) RET(build_graph(s));  // profiling launches the same kernels directly
+    if (!prof) RET(build_graph(s, narrow));  // profiling launches the same kernels directly
     int max_steps = s->p.max_steps > 0 ? s->p.max_steps
                                        : nl * (s->p.iter_max * (2 + 48 / std::max(1, s->p.trials_per_pass)) + 4) + 64;
     int steps = 0;
@@ -559,7 +577,7 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
             // profiling: the same step kernels launched one by one between events
             for (int k = 0; k < GRAPH_STEPS; k++) {
                 cudaEventRecord(s->ev[k][F_G], s->stream);
-                launch_grad(s->bf16, s->grid_G, s->stream, b);
+                launch_gradient(s, narrow, s->stream, b);
                 if (b.smooth) launch_smooth(s->nsm, s->cap_ops, s->sm_n, s->stream, b);  // timed with the gradient family
                 cudaEventRecord(s->ev[k][F_T], s->stream);
                 launch_trial(s->bf16, s->p.trials_per_pass, s->grid_T, s->stream, b);
@@ -569,7 +587,7 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
             }
             CK(cudaGetLastError());
         } else {
-            CK(cudaGraphLaunch(s->gexec, s->stream));
+            CK(cudaGraphLaunch(s->gexec[narrow], s->stream));
         }
         CK(cudaMemcpyAsync(s->h_ctr, s->d_ctr, sizeof(int) * 16, cudaMemcpyDeviceToHost, s->stream));
         CK(cudaStreamSynchronize(s->stream));
@@ -939,6 +957,7 @@ void set_grids(reg_series *s)
         return s->nsm * std::max(1, std::min(occ, 32));
     };
     s->grid_G = grid_of(1);
+    s->grid_F = grid_of(0);
     s->grid_T = grid_of(2);
 }
 
@@ -1232,7 +1251,8 @@ reg_status reg_create_series(const float *frames, int32_t n_series, const int32_
 reg_status reg_destroy_series(reg_series_t s)
 {
     if (!s) return REG_OK;
-    if (s->gexec) cudaGraphExecDestroy(s->gexec);
+    for (cudaGraphExec_t g : s->gexec)
+        if (g) cudaGraphExecDestroy(g);
     if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
     if (s->copy_stream) cudaStreamDestroy(s->copy_stream);
     for (int i = 0; i < 2; i++) {
@@ -1773,7 +1793,7 @@ reg_status reg_eval_direction(reg_series_t s, int32_t series, int32_t frame_i, i
     RET(diag_setup(s, series, frame_i, frame_k, level, u_grid, k));
     BatchDev b = make_batch(s);
     // state is now PH_GRAD with src = 0, cur = 1 (no pending step)
-    launch_grad(s->bf16, s->grid_G, s->stream, b);
+    launch_gradient(s, true, s->stream, b);
     CK(cudaGetLastError());
     OpState st;
     CK(cudaMemcpyAsync(&st, s->d_st, sizeof(OpState), cudaMemcpyDeviceToHost, s->stream));
@@ -1812,7 +1832,7 @@ reg_status reg_eval_trials(reg_series_t s, int32_t series, int32_t frame_i, int3
     BatchDev b = make_batch(s);
     // gradient pass at u (state PH_GRAD, no pending step), then one trial pass
     // over the given step sizes (still PH_GRAD, so that it also forms d^T K d)
-    launch_grad(s->bf16, s->grid_G, s->stream, b);
+    launch_gradient(s, true, s->stream, b);
     CK(cudaGetLastError());
     OpState st;
     CK(cudaMemcpyAsync(&st, s->d_st, sizeof(OpState), cudaMemcpyDeviceToHost, s->stream));

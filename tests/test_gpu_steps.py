@@ -104,3 +104,26 @@ def test_trial_sums_against_fp64_energies(reg, orc, syn, side, rows, amp):
     for t, got in zip(taus, dE):
         want = E(u.astype(np.float64) + t * d.astype(np.float64)) - e0
         assert abs(got - want) <= 1e-4 * abs(want) + 1e-9 * abs(e0), (t, got, want)
+
+
+@pytest.mark.parametrize("side,rows", [(32, 4), (64, 8), (128, 32), (128, 64), (256, 16)])
+def test_narrow_and_wide_batches_take_the_same_steps(reg, syn, side, rows):
+    """The gradient pass's two forms (a tile per warp in wide batches, a tile per
+    block in narrow ones) add their sums in the same order: an operator run alone
+    and in a batch wide enough for the other form ends on the same bits."""
+    L, n = int(np.log2(side)), side + 1
+    tiles = -(-n // 30) * -(-n // rows)
+    width = 4 * 6 * 160 // tiles + 2  # more tiles than any grid of the narrow form takes
+    fr = syn.series(13, 3, side, peak=20.0, spacing=9.0, sigma=1.8)
+    p = reg.default_params(n_levels=2, iter_max=6, lam=10.0)
+    m = -(-width // 2)
+    ops = [(k // 2, -1, -1, k % 2, k % 2, k % 2 + 1) for k in range(2 * m)]
+    with reg.Series([fr] * m, p) as s:
+        s.set_tile_rows(L, rows, min(rows, 32))
+        s.apply_operator_batch(ops)
+        wide = [s.get_slot(e, series=m - 1)[0] for e in range(2)]
+    with reg.Series(fr, p) as s:
+        s.set_tile_rows(L, rows, min(rows, 32))
+        s.apply_operator_batch([(0, -1, -1, e, e, e + 1) for e in range(2)])
+        for e in range(2):
+            assert np.array_equal(s.get_slot(e)[0], wide[e])
