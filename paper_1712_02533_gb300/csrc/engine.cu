@@ -163,7 +163,8 @@ struct reg_series {
     int *d_lists = nullptr;  // listG, listT, prefG, prefT
     int2 *d_plan = nullptr;  // per op: its work of the next step
     int *d_ctr = nullptr;
-    double *d_partG = nullptr, *d_partT = nullptr;
+    float *d_partG = nullptr, *d_partT = nullptr;
+    double *d_partU = nullptr;
     unsigned long long *d_work = nullptr;
     char *d_ws = nullptr;
     double *d_scratch = nullptr;
@@ -191,7 +192,7 @@ struct reg_series {
     size_t d_lock_cap = 0;
     // H1-type smoother: Thomas pivots per level l (2^l + 1 nodes), partial sums
     float2 *d_smtab[REG_TILE_LEVELS] = {nullptr};
-    double *d_partS = nullptr;
+    float *d_partS = nullptr;
     int sm_rch = 0, sm_cch = 0, sm_n = 0;  // row and column chunks per op, largest level
     // rigid variant buffers
     RigidLevel *d_rlv = nullptr, *h_rlv = nullptr;
@@ -284,6 +285,7 @@ BatchDev make_batch(reg_series *s)
     b.ctr = s->d_ctr;
     b.partG = s->d_partG;
     b.partT = s->d_partT;
+    b.partU = s->d_partU;
     b.work = s->d_work;
     b.trace = s->d_trace;
     b.trace_len = s->d_trace_len;
@@ -361,7 +363,7 @@ reg_status ensure_capacity(reg_series *s, int n_ops, size_t ws_total, int64_t it
         RET(track(s, (void **)&s->d_plan, sizeof(int2) * std::max(c, 32)));
         if (s->p.smooth > 0.0) {
             untrack(s, s->d_partS);
-            RET(track(s, (void **)&s->d_partS, sizeof(double) * 2 * (size_t)s->sm_cch * c));
+            RET(track(s, (void **)&s->d_partS, sizeof(float) * 2 * (size_t)s->sm_cch * c));
         }
         CK(cudaMallocHost((void **)&s->h_ops, sizeof(OpDesc) * c));
         s->cap_ops = c;
@@ -372,8 +374,10 @@ reg_status ensure_capacity(reg_series *s, int n_ops, size_t ws_total, int64_t it
         int64_t c = std::max(items, (int64_t)(1.25 * s->cap_items));
         untrack(s, s->d_partG);
         untrack(s, s->d_partT);
-        RET(track(s, (void **)&s->d_partG, sizeof(double) * PG_STRIDE * c));
-        RET(track(s, (void **)&s->d_partT, sizeof(double) * PT_STRIDE * c));
+        untrack(s, s->d_partU);
+        RET(track(s, (void **)&s->d_partG, sizeof(float) * PG_STRIDE * c));
+        RET(track(s, (void **)&s->d_partT, sizeof(float) * PT_STRIDE * c));
+        RET(track(s, (void **)&s->d_partU, sizeof(double) * 4 * c));
         s->cap_items = c;
         changed = true;
     }
@@ -1769,15 +1773,15 @@ reg_status reg_eval_energy(reg_series_t s, int32_t series, int32_t frame_i, int3
     CK(cudaMemcpy(&st, s->d_st, sizeof(OpState), cudaMemcpyDeviceToHost));
     if (parts) {
         parts[0] = st.E;
-        parts[1] = st.ncc;
-        parts[2] = st.E + st.ncc;
-        parts[3] = st.Tbar;
-        parts[4] = st.sigT;
+        parts[1] = st.cur_ev.ncc;
+        parts[2] = st.E + st.cur_ev.ncc;
+        parts[3] = st.cur_ev.S1;
+        parts[4] = st.cur_ev.sig;
     }
     return REG_OK;
 }
 
-__global__ void k_sum_range(const double *v, int stride, int b, int e, double *out)
+__global__ void k_sum_range(const float *v, int stride, int b, int e, double *out)
 {
     double s = 0.0;
     for (int i = b + threadIdx.x; i < e; i += 32) s += v[(int64_t)i * stride];
@@ -1846,10 +1850,10 @@ reg_status reg_eval_trials(reg_series_t s, int32_t series, int32_t frame_i, int3
     CK(cudaMemcpyAsync(s->d_st, &st, sizeof(OpState), cudaMemcpyHostToDevice, s->stream));
     launch_trial(s->bf16, s->p.trials_per_pass, s->grid_T, s->stream, b);
     CK(cudaGetLastError());
-    std::vector<double> pt((size_t)st.tT * PT_STRIDE), pg((size_t)st.tG * PG_STRIDE);
-    CK(cudaMemcpyAsync(pt.data(), s->d_partT, pt.size() * sizeof(double),
+    std::vector<float> pt((size_t)st.tT * PT_STRIDE), pg((size_t)st.tG * PG_STRIDE);
+    CK(cudaMemcpyAsync(pt.data(), s->d_partT, pt.size() * sizeof(float),
                        cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(pg.data(), s->d_partG, pg.size() * sizeof(double),
+    CK(cudaMemcpyAsync(pg.data(), s->d_partG, pg.size() * sizeof(float),
                        cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
     double S[PT_STRIDE] = {0.0}, qud = 0.0;
@@ -1859,10 +1863,10 @@ reg_status reg_eval_trials(reg_series_t s, int32_t series, int32_t frame_i, int3
     const SeriesInfo &si = s->S[series];
     const double hh = 1.0 / (si.n[k] - 1), h2 = hh * hh, qdd = S[3 * REG_MAX_TRIALS + 2];
     for (int j = 0; j < n_tau; j++) {
-        double S1 = st.S1 + h2 * S[3 * j], S2 = st.S2 + h2 * S[3 * j + 1], S3 = st.S3 + h2 * S[3 * j + 2];
+        double S1 = st.cur_ev.S1 + h2 * S[3 * j], S2 = st.cur_ev.S2 + h2 * S[3 * j + 1], S3 = st.cur_ev.S3 + h2 * S[3 * j + 2];
         double var = S2 - S1 * S1;
         double nc = S3 / (var > 0.0 ? std::sqrt(var) : 0.0);
-        dE_out[j] = -(nc - st.ncc) + 0.5 * s->p.lambda * h2 * (2.0 * taus[j] * qud + taus[j] * taus[j] * qdd);
+        dE_out[j] = -(nc - st.cur_ev.ncc) + 0.5 * s->p.lambda * h2 * (2.0 * taus[j] * qud + taus[j] * taus[j] * qdd);
     }
     if (d_out) {
         int n = si.n[k];

@@ -524,6 +524,9 @@ __device__ __forceinline__ void set_step(OpState &s, const OpDesc &op)
     d.ntr = s.ntr;
     d.part0 = op.part0;
     d.ih2 = 1.f / L.h2;
+    d.isig = s.cur_ev.isig;
+    d.c36 = s.cur_ev.c36;
+    d.cT = s.cur_ev.cT;
 }
 
 // A warp's view of the step's work items (tiles of one family).  Batches of up to
@@ -1929,7 +1932,7 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, TRIAL_BLOCKS) k_trial(Batch
                 double t = 0.0;
 #pragma unroll
                 for (int w = 0; w < TRIAL_WARPS; w++) t += sh.start[w][threadIdx.x];
-                b.partT[(int64_t)part * PT_STRIDE + (threadIdx.x < 3 ? threadIdx.x : 3 * REG_MAX_TRIALS)] = t;
+                b.partU[4 * (int64_t)part + threadIdx.x] = t;
             }
         } else {
             trial_tile<BF16, JM>(b, s, g, sh, part, wid, lane);
@@ -1939,272 +1942,305 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, TRIAL_BLOCKS) k_trial(Batch
 }
 
 // ---------------------------------------------------------------------------
-// C: per-operator FP64 reduction, the Armijo state machine, and the plan of the
-// next step
+// C: per-operator sums, the Armijo state machine, and the plan of the next step
 // ---------------------------------------------------------------------------
 namespace {
 
-// An evaluated energy: the FE sums S1 = int That, S2 = int That^2, S3 = int That
-// R~ (R~ normalised: mean 0, FE sigma 1), sigma = sqrt(S2 - S1^2), NCC = S3 /
-// sigma, the gradient pass's coefficients there, and of a trial the energy
-// change, the Armijo test and the stopping test.
-struct EvalAt {
-    double S1, S2, S3, ncc, sig, dE;
-    float isig, c36, cT;
-    int acc, conv;
-};
+// 1 / sqrt(v), v within float's range: the single-precision value (2^-22) and one
+// third-order step (Halley's iteration for v^-1/2), to 1-2 ulp.  The double-precision
+// instructions behind sqrt and the division take 600 cycles each here, these four
+// dependent multiply-adds 250.
+__device__ __forceinline__ double rsqrt_step(double v)
+{
+    const double r = (double)rsqrtf((float)v);
+    const double t = v * r, e = fma(-t, r, 1.0);
+    return fma(r * e, fma(e, 0.375, 0.5), r);
+}
 
-// One reciprocal square root serves sigma, NCC and the coefficients: a double
-// division or square root takes 600-670 cycles on this chip (a multiplication
-// 62), and a chain of five of them was a third of the control kernel.
+// sigma, NCC and the gradient pass's coefficients from the FE sums.
 __device__ __forceinline__ void eval_at(EvalAt &v, double S1, double S2, double S3)
 {
     const double var = S2 - S1 * S1;
     v.S1 = S1;
     v.S2 = S2;
     v.S3 = S3;
-    if (var > 0.0 && var < 1e300) {
-        const double r = rsqrt(var);
+    if (var > 1e-30 && var < 1e30) {
+        const double r = rsqrt_step(var);
         v.sig = var * r;
         v.ncc = S3 * r;
         v.isig = (float)r;
         const double q = v.ncc * (r * r);
         v.c36 = (float)(q * (1.0 / 36.0));
         v.cT = (float)(q * S1);
-    } else {  // no variance, or not finite: no energy
+    } else {  // (almost) no variance, or not finite
         v.sig = var > 0.0 ? sqrt(var) : 0.0;
         v.ncc = S3 / v.sig;
-        v.isig = v.c36 = v.cT = 0.f;
+        v.isig = (float)(1.0 / v.sig);
+        v.c36 = (float)(v.ncc / (v.sig * v.sig) / 36.0);
+        v.cT = (float)(v.ncc / (v.sig * v.sig) * S1);
     }
 }
 
 // Positive doubles compare like their bits, and doubling one adds to its
 // exponent field: the step sizes of the search stay off the slow FP64 pipe.
 // (Numbers near the ends of the exponent range take the multiplication.)
-__device__ __forceinline__ double pow2_scale(double x, int e, double f)
+__device__ __forceinline__ double pow2_scale(double x, int e)
 {
     const long long w = __double_as_longlong(x);
     const int ex = (int)(w >> 52);
-    return ex >= 2 && ex <= 0x7fc ? __longlong_as_double(w + ((long long)e << 52)) : x * f;
+    return ex > 8 && ex < 0x7f0 ? __longlong_as_double(w + ((long long)e << 52)) : scalbn(x, e);
 }
-__device__ __forceinline__ double twice(double x) { return pow2_scale(x, 1, 2.0); }
-__device__ __forceinline__ double half_of(double x) { return pow2_scale(x, -1, 0.5); }
+__device__ __forceinline__ double twice(double x) { return pow2_scale(x, 1); }
+__device__ __forceinline__ double half_of(double x) { return pow2_scale(x, -1); }
 __device__ __forceinline__ bool pos_le(double a, double b) { return __double_as_longlong(a) <= __double_as_longlong(b); }
 __device__ __forceinline__ bool pos_eq(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
 
-__device__ __forceinline__ void level_end(OpState &s, const OpDesc &op, int status, double pending)
-{
-    if (status == OPST_NONFINITE) s.nonfinite_seen = 1;
-    s.status = status;
-    s.tau_acc = pending;
-    s.step.tau_acc = (float)pending;
-    s.src = s.cur;
-    if (s.lvl < op.nl - 1) {
-        s.phase = PH_PROLONG;
-        s.lvl += 1;
-        s.cur = 0;
-    } else {
-        s.phase = PH_DONE;
-    }
-}
-
-// Lockstep replay: the step size the given search of iteration s.iter takes.
-__device__ __forceinline__ double lock_step(const OpState &s, const OpDesc &op)
-{
-    return op.lock_tau[op.lock_off[s.lvl] + s.iter];
-}
-
-__device__ __forceinline__ int lock_count(const OpState &s, const OpDesc &op)
-{
-    return op.lock_off[s.lvl + 1] - op.lock_off[s.lvl];
-}
-
-__device__ __forceinline__ void set_trial(OpState &s, int k, double t)
-{
-    s.trial_tau[k] = t;
-    s.step.tau[k] = (float)t;
-}
-
-__device__ __forceinline__ void schedule_grad(OpState &s, const BatchDev &b, const OpDesc &op, double pending)
-{
-    s.phase = PH_GRAD;
-    s.tau_acc = pending;
-    s.step.tau_acc = (float)pending;
-    s.src = s.cur;
-    s.cur = 1 - s.cur;
-    s.search = SEARCH_INIT;
-    if (op.lock_tau) {
-        // replay: the one step size the reference sequence accepted here
-        set_trial(s, 0, lock_step(s, op));
-        s.ntr = 1;
-        return;
-    }
-    // sequential Armijo order: tau, then 2 tau (if accepted), else tau/2; the
-    // pass covers the most likely continuations of both branches.
-    const int J = b.J;
-    int k = 0;
-    double up = s.tau, dn = s.tau;
-    set_trial(s, k++, up);
-    while (k < J) {
-        const double u2 = twice(up), d2 = half_of(dn);
-        const bool canUp = pos_le(u2, b.tau_max), canDn = pos_le(b.tau_min, d2);
-        if (!canUp && !canDn) break;
-        if (canUp) { up = u2; set_trial(s, k++, up); }
-        if (k < J && canDn) { dn = d2; set_trial(s, k++, dn); }
-    }
-    s.ntr = k;
-}
-
-__device__ __forceinline__ void trace_trial(const BatchDev &b, const OpState &s, int o, int n, double want,
+__device__ __forceinline__ void trace_trial(const BatchDev &b, int o, int n, int iter, double want, double slope,
                                             const EvalAt &v)
 {
-    if (!b.trace) return;
     unsigned long long k = atomicAdd(b.trace_len, 1ull);
     if ((long long)k < b.trace_cap) {
         double *rec = b.trace + 7 * k;
-        rec[0] = o; rec[1] = n; rec[2] = s.iter - 1; rec[3] = want;
-        rec[4] = v.dE; rec[5] = b.sigma * want * s.slope; rec[6] = v.acc;
+        rec[0] = o; rec[1] = n; rec[2] = iter - 1; rec[3] = want;
+        rec[4] = v.dE; rec[5] = b.sigma * want * slope; rec[6] = v.acc;
     }
 }
 
-// The Armijo state machine of one operator after a step (one thread; s and op in
-// shared memory).  ev: the evaluated trials, or ev[0] the level's start (dE: its
-// energy).  sgn: 1 the slope of a new search is negative, 0 it is zero, -1 else.
-__device__ __forceinline__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int o, int n,
-                                           const EvalAt *ev, double slope, int sgn)
+// The Armijo state machine of one operator after a step, by one warp (s and op in
+// shared memory, s written by this warp only).  Lane j holds trial j (lane 0 a
+// level's start, its energy in dE); the decisions are uniform, taken from ballots
+// over the lanes.
+__device__ __forceinline__ void control_op(const BatchDev &b, OpState &s, const OpDesc &op, int o, int n, int lane,
+                                           const EvalAt &ev, double mytau, double slope)
 {
-    const int ph = s.phase;
-    auto take = [&](const EvalAt &v) {
-        s.S1 = v.S1; s.S2 = v.S2; s.S3 = v.S3;
-        s.Tbar = v.S1;
-        s.sigT = v.sig;
-        s.ncc = v.ncc;
-        s.step.isig = v.isig; s.step.c36 = v.c36; s.step.cT = v.cT;
-    };
+    const unsigned FULL = 0xffffffffu;
+    const int ph = s.phase, ntr = s.ntr;
+    int iter = s.iter, status = -1;  // status >= 0: the level ends
+    bool go = false;                 // next: a gradient pass at the level
+    double pending = 0.0, tau = s.tau;
+    const unsigned long long nn = (unsigned long long)n * n;
+    int evals = ph == PH_START || ph == PH_PROLONG ? 1 : ntr, seq = 0;
     if (ph == PH_START || ph == PH_PROLONG) {
-        take(ev[0]);
-        s.E = ev[0].dE;
-        s.iter = 0;
-        s.tau = b.tau_init;
-        s.evals += 1;
-        if (!isfinite(s.E)) level_end(s, op, OPST_NONFINITE, 0.0);
-        else if (op.lock_tau && lock_count(s, op) == 0) level_end(s, op, OPST_MAXITER, 0.0);
-        else schedule_grad(s, b, op, 0.0);
-        return;
-    }
-    if (ph == PH_GRAD) {
-        s.iter += 1;
-        s.iters_total += 1;
-        s.slope = slope;
-        if (sgn != 1) {
-            level_end(s, op, sgn == 0 ? OPST_ZERO_GRAD : OPST_NONFINITE, 0.0);
-            return;
+        if (lane == 0) {
+            s.cur_ev = ev;
+            s.E = ev.dE;
+        }
+        iter = 0;
+        tau = b.tau_init;
+        const bool fin = __shfl_sync(FULL, (int)isfinite(ev.dE), 0);
+        if (!fin) status = OPST_NONFINITE;
+        else if (op.lock_tau && op.lock_off[s.lvl + 1] == op.lock_off[s.lvl]) status = OPST_MAXITER;
+        else go = true;
+    } else {
+        bool search_on = true;
+        if (ph == PH_GRAD) {
+            iter++;
+            if (!(slope < 0.0)) {
+                status = slope == 0.0 ? OPST_ZERO_GRAD : OPST_NONFINITE;
+                search_on = false;
+                evals = 0;
+            }
+        }
+        const unsigned accs = __ballot_sync(FULL, lane < ntr && ev.acc);
+        if (search_on && op.lock_tau) {
+            // lockstep replay: take the given step whatever the test says (the
+            // trace records the test), end the level after the last given step
+            seq = 1;
+            if (lane == 0) {
+                if (b.trace) trace_trial(b, o, n, iter, mytau, slope, ev);
+                s.E += ev.dE;
+                s.cur_ev = ev;
+            }
+            tau = pending = s.trial_tau[0];
+            if (iter >= op.lock_off[s.lvl + 1] - op.lock_off[s.lvl]) status = OPST_MAXITER;
+            else go = true;
+        } else if (search_on) {
+            // walk the sequential Armijo search over the step sizes evaluated this pass
+            int search = s.search, best = -1;  // best: the last trial accepted in this pass
+            double btau = s.btau, sh_tau = s.sh_tau;
+            bool finish = false, more = false;
+            int guard = 0;
+            for (; guard < 4 * REG_MAX_TRIALS + 8 && !finish && status < 0; guard++) {
+                const double want =
+                    search == SEARCH_INIT ? tau : (search == SEARCH_WIDEN ? twice(btau) : half_of(sh_tau));
+                if (search == SEARCH_WIDEN && !pos_le(want, b.tau_max)) { finish = true; break; }
+                if (search == SEARCH_SHRINK && !pos_le(b.tau_min, want)) { status = OPST_STALLED; break; }
+                const unsigned at = __ballot_sync(FULL, lane < ntr && pos_eq(mytau, want));
+                if (!at) {
+                    // continue the search in another pass
+                    int k = 0;
+                    double t = want;
+                    while (k < b.J && (search == SEARCH_WIDEN ? pos_le(t, b.tau_max) : pos_le(b.tau_min, t))) {
+                        if (lane == k) {
+                            s.trial_tau[k] = t;
+                            s.step.tau[k] = (float)t;
+                        }
+                        t = search == SEARCH_WIDEN ? twice(t) : half_of(t);
+                        k++;
+                    }
+                    if (lane == 0) {
+                        s.ntr = k;
+                        s.phase = PH_TRIAL;
+                    }
+                    more = true;
+                    break;
+                }
+                const int j = __ffs(at) - 1;
+                seq++;
+                if (b.trace && lane == j) trace_trial(b, o, n, iter, want, slope, ev);
+                const bool acc = accs >> j & 1;
+                if (acc) best = j;
+                if (search == SEARCH_SHRINK) {
+                    if (acc) { btau = want; finish = true; }
+                    else sh_tau = want;
+                } else if (acc) {
+                    search = SEARCH_WIDEN;
+                    btau = want;
+                } else if (search == SEARCH_INIT) {
+                    search = SEARCH_SHRINK;
+                    sh_tau = want;
+                } else {
+                    finish = true;
+                }
+            }
+            if (finish) {
+                const bool conv = best >= 0 ? __shfl_sync(FULL, ev.conv, best) != 0 : s.best_ev.conv != 0;
+                __syncwarp();
+                if (best >= 0) {
+                    if (lane == best) {
+                        s.cur_ev = ev;
+                        s.E += ev.dE;
+                    }
+                } else if (lane == 0) {
+                    s.cur_ev = s.best_ev;
+                    s.E += s.best_ev.dE;
+                }
+                tau = pending = btau;
+                if (conv) status = OPST_CONVERGED;
+                else if (iter >= b.iter_max) status = OPST_MAXITER;
+                else go = true;
+            } else if (more) {
+                if (lane == max(best, 0) && best >= 0) s.best_ev = ev;
+                if (lane == 0) {
+                    s.search = search;
+                    s.btau = btau;
+                    s.sh_tau = sh_tau;
+                }
+            } else if (status < 0) {  // the search did not terminate: internal error
+                if (lane == 0) {
+                    atomicExch(&b.ctr[8], 1);
+                    s.phase = PH_DONE;
+                }
+            }
         }
     }
-    s.evals += s.ntr;
-    const unsigned long long nn = (unsigned long long)n * n;
-    if (op.lock_tau) {
-        // lockstep replay: take the given step whatever the test says (the
-        // trace records the test), end the level after the last given step
-        const double want = s.trial_tau[0];
-        s.trials_seq += 1;
-        atomicAdd(&b.work[KW_TSEQ], nn);
-        trace_trial(b, s, o, n, want, ev[0]);
-        s.E += ev[0].dE;
-        take(ev[0]);
-        s.tau = want;
-        if (s.iter >= lock_count(s, op)) level_end(s, op, OPST_MAXITER, want);
-        else schedule_grad(s, b, op, want);
-        return;
-    }
-    // Walk the sequential Armijo search over the step sizes evaluated this pass.
-    const int ntr = s.ntr;
-    int search = s.search, seq = 0, best = -1;  // best: the last trial accepted in this pass
-    double btau = s.btau, sh_tau = s.sh_tau;
-    bool finish = false, stall = false;
-    int guard = 0;
-    for (; guard < 4 * REG_MAX_TRIALS + 8 && !finish && !stall; guard++) {
-        const double want = search == SEARCH_INIT ? s.tau : (search == SEARCH_WIDEN ? twice(btau) : half_of(sh_tau));
-        if (search == SEARCH_WIDEN && !pos_le(want, b.tau_max)) { finish = true; break; }
-        if (search == SEARCH_SHRINK && !pos_le(b.tau_min, want)) { stall = true; break; }
-        int j = -1;
-        for (int k = 0; k < ntr; k++)
-            if (pos_eq(s.trial_tau[k], want)) { j = k; break; }
-        if (j < 0) {
-            // continue the search in another pass
-            int k = 0;
-            double t = want;
-            if (search == SEARCH_WIDEN) {
-                while (k < b.J && pos_le(t, b.tau_max)) { set_trial(s, k++, t); t = twice(t); }
+    __syncwarp();
+    if (status >= 0) {
+        const int lvl = s.lvl, cur = s.cur, last = op.nl - 1;
+        __syncwarp();
+        if (lane == 0) {
+            if (status == OPST_NONFINITE) s.nonfinite_seen = 1;
+            s.status = status;
+            s.tau_acc = pending;
+            s.step.tau_acc = (float)pending;
+            s.src = cur;
+            if (lvl < last) {
+                s.phase = PH_PROLONG;
+                s.lvl = lvl + 1;
+                s.cur = 0;
             } else {
-                while (k < b.J && pos_le(b.tau_min, t)) { set_trial(s, k++, t); t = half_of(t); }
+                s.phase = PH_DONE;
+            }
+        }
+    } else if (go) {
+        if (lane == 0) {
+            s.phase = PH_GRAD;
+            s.tau_acc = pending;
+            s.step.tau_acc = (float)pending;
+            s.src = s.cur;
+            s.cur = 1 - s.cur;
+            s.search = SEARCH_INIT;
+        }
+        // step sizes in the sequential Armijo order: tau, then 2 tau (if accepted), else
+        // tau / 2; the pass covers the most likely continuations of both branches
+        const int J = b.J;
+        if (op.lock_tau) {
+            // replay: the one step size the reference sequence accepted here
+            if (lane == 0) {
+                const double t = op.lock_tau[op.lock_off[s.lvl] + iter];
+                s.trial_tau[0] = t;
+                s.step.tau[0] = (float)t;
+                s.ntr = 1;
+            }
+        } else if (pos_le(pow2_scale(tau, J / 2), b.tau_max) && pos_le(b.tau_min, pow2_scale(tau, -((J - 1) / 2)))) {
+            if (lane < J) {
+                const double t = pow2_scale(tau, (lane & 1) ? (lane + 1) / 2 : -(lane / 2));
+                s.trial_tau[lane] = t;
+                s.step.tau[lane] = (float)t;
+            }
+            if (lane == 0) s.ntr = J;
+        } else if (lane == 0) {  // at the ends of the admitted range
+            int k = 0;
+            double up = tau, dn = tau;
+            auto put = [&](double t) {
+                s.trial_tau[k] = t;
+                s.step.tau[k++] = (float)t;
+            };
+            put(up);
+            while (k < J) {
+                const double u2 = twice(up), d2 = half_of(dn);
+                const bool canUp = pos_le(u2, b.tau_max), canDn = pos_le(b.tau_min, d2);
+                if (!canUp && !canDn) break;
+                if (canUp) { up = u2; put(up); }
+                if (k < J && canDn) { dn = d2; put(dn); }
             }
             s.ntr = k;
-            s.phase = PH_TRIAL;
-            break;
-        }
-        seq++;
-        trace_trial(b, s, o, n, want, ev[j]);
-        const bool acc = ev[j].acc != 0;
-        if (acc) best = j;
-        if (search == SEARCH_SHRINK) {
-            if (acc) { btau = want; finish = true; }
-            else sh_tau = want;
-        } else if (acc) {
-            search = SEARCH_WIDEN;
-            btau = want;
-        } else if (search == SEARCH_INIT) {
-            search = SEARCH_SHRINK;
-            sh_tau = want;
-        } else {
-            finish = true;
         }
     }
-    s.trials_seq += seq;
-    if (seq) atomicAdd(&b.work[KW_TSEQ], nn * seq);
-    if (best >= 0) {
-        const EvalAt &v = ev[best];
-        s.bS1 = v.S1; s.bS2 = v.S2; s.bS3 = v.S3; s.bncc = v.ncc; s.bdE = v.dE;
-        s.bsig = v.sig;
-        s.b_isig = v.isig; s.b_c36 = v.c36; s.b_cT = v.cT;
-        s.b_conv = v.conv;
+    if (lane == 0) {
+        s.tau = tau;
+        s.iter = iter;
+        if (ph == PH_GRAD) {
+            s.iters_total += 1;
+            s.slope = slope;
+        }
+        s.evals += evals;
+        s.trials_seq += seq;
+        if (seq) atomicAdd(&b.work[KW_TSEQ], nn * seq);
     }
-    s.search = search;
-    s.btau = btau;
-    s.sh_tau = sh_tau;
-    if (stall) {
-        level_end(s, op, OPST_STALLED, 0.0);
-    } else if (finish) {
-        s.E += s.bdE;
-        s.S1 = s.bS1; s.S2 = s.bS2; s.S3 = s.bS3;
-        s.Tbar = s.bS1;
-        s.sigT = s.bsig;
-        s.ncc = s.bncc;
-        s.step.isig = s.b_isig; s.step.c36 = s.b_c36; s.step.cT = s.b_cT;
-        s.tau = btau;
-        if (s.b_conv) level_end(s, op, OPST_CONVERGED, btau);
-        else if (s.iter >= b.iter_max) level_end(s, op, OPST_MAXITER, btau);
-        else schedule_grad(s, b, op, btau);
-    } else if (s.phase != PH_TRIAL || guard >= 4 * REG_MAX_TRIALS + 8) {
-        atomicExch(&b.ctr[8], 1);  // the search did not terminate: internal error
-        s.phase = PH_DONE;
+    __syncwarp();
+}
+
+// Adds over the 32 lanes (the sum in every lane, not split alike).
+__device__ __forceinline__ void warp_sum3(Sum3 &v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float a = __shfl_xor_sync(0xffffffffu, v.a, o), c = __shfl_xor_sync(0xffffffffu, v.b, o),
+                    d = __shfl_xor_sync(0xffffffffu, v.c, o);
+        v.add(a);
+        v.add(c);
+        v.add(d);
     }
 }
 
 }  // namespace
 
 // One block per operator (grid stride): the block sums the operator's tile
-// partials in FP64, the lanes of a warp evaluate all trials side by side, and
-// thread 0 runs the state machine on copies of the state and the descriptor in
-// shared memory.  Batches of more than PLAN_WARP operators: the last block to
-// finish makes the lists of the next step (narrower ones need none).  Latency
-// bound at every size; what was spent was chains of FP64 operations (62 cycles
-// each, 600 and more for a square root or a division) and of dependent loads.
+// partials, the lanes of a warp evaluate all trials side by side and run the state
+// machine on copies of the state and the descriptor in shared memory.  Batches of
+// more than PLAN_WARP operators: the last block to finish makes the lists of the next
+// step (narrower ones need none).  Latency bound at every size.
 //
-// The sums: thread (g, kk) adds entry kk of every ng-th record (kk fastest, so a
-// warp reads neighbouring doubles), only the entries that the pass wrote: 3 per
-// step size and one Dirichlet form, at most 16 for up to four step sizes (32
-// groups), 32 otherwise (16 groups); then one warp per entry adds the groups.
+// The FP64 pipe takes 16 cycles for a warp's operation and 62 until its result: sums
+// and reductions of the tiles' floats in FP64 were 6000 of 15000 cycles at 65^2 nodes
+// and 18000 of 28000 at 1025^2, a chain of square roots and divisions 2900, the state
+// machine as one thread's loads and stores 3000 to 4700.  The sums run in float
+// triples now (exact to 2^-72, more than FP64 keeps): thread (g, kk) adds entry kk of
+// every ng-th record (kk fastest, so a warp reads neighbouring floats), only the
+// entries that the pass wrote, 3 per step size and one Dirichlet form (at most 13
+// for up to four step sizes: 32 groups; else 16 groups), and the gradient pass's two
+// sums as two more entries; then one warp per entry adds the groups.
 __global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
 {
     constexpr int NW = REG_CTL_THREADS / 32;
@@ -2212,24 +2248,26 @@ __global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
     static_assert(sizeof(OpState) % 8 == 0 && sizeof(OpDesc) % 8 == 0 && NS + ND <= REG_CTL_THREADS,
                   "state and descriptor copied in one pass");
     __shared__ __align__(16) double sbuf[NS], dbuf[ND];
-    __shared__ double red[REG_CTL_THREADS + 32];
-    __shared__ double redG[NW][2];
-    __shared__ double S[32];
-    __shared__ double SG[2];
-    __shared__ EvalAt ev[REG_MAX_TRIALS];
+    __shared__ float red[3][REG_CTL_THREADS + 32];
+    __shared__ float sums[3][32];
+    __shared__ double startS[4];
     __shared__ int last;
     OpState &s = *reinterpret_cast<OpState *>(sbuf);
     const OpDesc &op = *reinterpret_cast<const OpDesc *>(dbuf);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int n_ops = b.ctr[0];
-    if ((int)blockIdx.x >= n_ops) return;
-    for (int o = blockIdx.x; o < n_ops; o += gridDim.x) {
+    const int lg = b.J <= 4 ? 4 : 5, ng = REG_CTL_THREADS >> lg;
+    int n_ops = 0;
+    // (the first operator's state is read beside the operator count: a grid never has
+    // more blocks than there is room for operators)
+    for (int o = blockIdx.x; o == (int)blockIdx.x || o < n_ops; o += gridDim.x) {
         if (tid < NS) sbuf[tid] = reinterpret_cast<const double *>(b.st + o)[tid];
         else if (tid < NS + ND) dbuf[tid - NS] = reinterpret_cast<const double *>(b.ops + o)[tid - NS];
+        n_ops = b.ctr[0];
+        if (o >= n_ops) return;
         __syncthreads();
         const int ph = s.phase;
         if (ph != PH_DONE) {
-            const int n = s.step.n, ntr = s.ntr;
+            const int n = s.step.n, ntr = s.ntr, nt = s.tT;
             const double h2 = op.lv[s.lvl].h2d;
             const bool start = ph == PH_START || ph == PH_PROLONG;
             if (tid == REG_CTL_THREADS - 1) {
@@ -2243,89 +2281,108 @@ __global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
                     atomicAdd(&b.work[KW_TSAMPLES], nn * (unsigned long long)ntr);
                 }
             }
-            const int lg = b.J <= 4 ? 4 : 5, ng = REG_CTL_THREADS >> lg;
-            const int kk = tid & ((1 << lg) - 1), g = tid >> lg;
-            // entries 0 .. ne-2 of a record, then the Dirichlet form: of u
-            // (level start) or of d (first pass of a search)
-            const int ne = (start ? 3 : 3 * ntr) + 1;
-            if (kk < ne) {
-                const double *rec = b.partT + (int64_t)op.part0 * PT_STRIDE +
-                                    (kk < ne - 1 ? kk : 3 * REG_MAX_TRIALS + (start ? 0 : 2));
-                const int nt = s.tT;
-                double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0, acc3 = 0.0;
+            // entries 0 .. 3 ntr - 1 and the Dirichlet form of d; the last two of a group
+            // are the gradient pass's (or the smoother's)
+            const int ne = 3 * ntr + 1, e0 = (1 << lg) - 2;
+            if (start) {
+                // doubles: three sums and the Dirichlet form of u
+                if (wid < 4) {
+                    double v = 0.0;
+                    for (int it = lane; it < nt; it += 32) v += b.partU[4 * ((int64_t)op.part0 + it) + wid];
+                    v = warp_sum_d(v);
+                    if (lane == 0) startS[wid] = v;
+                }
+                __syncthreads();
+            } else {
+                const int kk = tid & ((1 << lg) - 1), g = tid >> lg;
+                const float *rec = nullptr;
+                int stride = PT_STRIDE, cnt = 0;
+                if (kk < ne) {
+                    rec = b.partT + (int64_t)op.part0 * PT_STRIDE + (kk < ne - 1 ? kk : 3 * REG_MAX_TRIALS + 2);
+                    cnt = nt;
+                } else if (kk >= e0 && ph == PH_GRAD) {
+                    // gradient tiles, or the smoother's column chunks
+                    rec = (b.smooth ? b.partS + (int64_t)o * b.cch * 2 : b.partG + (int64_t)op.part0 * PG_STRIDE) + (kk - e0);
+                    stride = PG_STRIDE;
+                    cnt = b.smooth ? (n + REG_GW - 1) / REG_GW : s.tG;
+                }
+                Sum3 v;
                 int it = g;
-#pragma unroll 2
-                for (; it + 3 * ng < nt; it += 4 * ng) {
-                    acc0 += rec[(int64_t)it * PT_STRIDE];
-                    acc1 += rec[(int64_t)(it + ng) * PT_STRIDE];
-                    acc2 += rec[(int64_t)(it + 2 * ng) * PT_STRIDE];
-                    acc3 += rec[(int64_t)(it + 3 * ng) * PT_STRIDE];
+                for (; it + 3 * ng < cnt; it += 4 * ng) {
+                    const float x0 = rec[(int64_t)it * stride], x1 = rec[(int64_t)(it + ng) * stride],
+                                x2 = rec[(int64_t)(it + 2 * ng) * stride], x3 = rec[(int64_t)(it + 3 * ng) * stride];
+                    v.add(x0);
+                    v.add(x1);
+                    v.add(x2);
+                    v.add(x3);
                 }
-                if (it < nt) acc0 += rec[(int64_t)it * PT_STRIDE];
-                if (it + ng < nt) acc1 += rec[(int64_t)(it + ng) * PT_STRIDE];
-                if (it + 2 * ng < nt) acc2 += rec[(int64_t)(it + 2 * ng) * PT_STRIDE];
-                red[kk * (ng + 1) + g] = (acc0 + acc1) + (acc2 + acc3);
-            }
-            if (ph == PH_GRAD) {
-                double slope = 0.0, qud = 0.0;
-                // the gradient pass's tiles, or the smoother's column chunks
-                const double2 *p = b.smooth ? reinterpret_cast<const double2 *>(b.partS) + (int64_t)o * b.cch
-                                            : reinterpret_cast<const double2 *>(b.partG) + op.part0;
-                const int np = b.smooth ? (n + REG_GW - 1) / REG_GW : s.tG;
-#pragma unroll 4
-                for (int it = tid; it < np; it += REG_CTL_THREADS) {
-                    const double2 v = p[it];
-                    slope += v.x;
-                    qud += v.y;
-                }
-                slope = warp_sum_d(slope);
-                qud = warp_sum_d(qud);
-                if (lane == 0) {
-                    redG[wid][0] = slope;
-                    redG[wid][1] = qud;
-                }
-            }
-            __syncthreads();
-            for (int k = wid; k < ne; k += NW) {
-                const double v = warp_sum_d(lane < ng ? red[k * (ng + 1) + lane] : 0.0);
-                if (lane == 0) S[k] = v;
-            }
-            if (ph == PH_GRAD && wid >= NW - 2) {
-                // (the two last warps have no entry of a pass with four step sizes)
-                const int w = wid - (NW - 2);
-                const double v = warp_sum_d(lane < NW ? redG[lane][w] : 0.0);
-                if (lane == 0) SG[w] = w == 0 && b.smooth ? -h2 * h2 * v : v;
-            }
-            __syncthreads();
-            if (wid == 0) {
-                // the Dirichlet forms of the search: u^T K d from the gradient pass
-                // (or the smoother), d^T K d from its first trial pass
-                const double Qud = ph == PH_GRAD ? SG[1] : s.Qud, Qdd = ph == PH_GRAD ? S[ne - 1] : s.Qdd;
-                const double slope = ph == PH_GRAD ? SG[0] : s.slope;
-                if (start) {
-                    if (lane == 0) {
-                        eval_at(ev[0], h2 * S[0], h2 * S[1], h2 * S[2]);
-                        ev[0].dE = -ev[0].ncc + 0.5 * b.lambda * h2 * S[3];
+                for (; it < cnt; it += ng) v.add(rec[(int64_t)it * stride]);
+                const int at = kk * (ng + 1) + g;
+                red[0][at] = v.a;
+                red[1][at] = v.b;
+                red[2][at] = v.c;
+                __syncthreads();
+                for (int k = wid; k < (1 << lg); k += NW) {
+                    if (k >= ne && k < e0) continue;
+                    Sum3 w;
+                    if (lane < ng) {
+                        const int i = k * (ng + 1) + lane;
+                        w.a = red[0][i];
+                        w.b = red[1][i];
+                        w.c = red[2][i];
                     }
-                } else if (lane < ntr) {
-                    EvalAt v;
-                    const double want = s.trial_tau[lane], E = s.E;
-                    const double reg = 0.5 * b.lambda * h2 * (2.0 * want * Qud + want * want * Qdd);
-                    const double bound = b.sigma * want * slope, stop = b.eps * (fabs(E) > 1.0 ? fabs(E) : 1.0);
-                    eval_at(v, s.S1 + h2 * S[3 * lane], s.S2 + h2 * S[3 * lane + 1], s.S3 + h2 * S[3 * lane + 2]);
+                    warp_sum3(w);
+                    if (lane == 0) {  // (one lane's triple: the lanes split the sum differently)
+                        sums[0][k] = w.a;
+                        sums[1][k] = w.b;
+                        sums[2][k] = w.c;
+                    }
+                }
+                __syncthreads();
+            }
+            if (wid == 0) {
+                const unsigned FULL = 0xffffffffu;
+                EvalAt v;
+                v.dE = 0.0;
+                v.acc = v.conv = 0;
+                double slope = s.slope, mytau = 0.0;
+                if (start) {
+                    eval_at(v, h2 * startS[0], h2 * startS[1], h2 * startS[2]);
+                    v.dE = -v.ncc + 0.5 * b.lambda * h2 * startS[3];
+                } else {
+                    // lane k: entry k's sum
+                    const double e = (double)sums[0][lane] + ((double)sums[1][lane] + (double)sums[2][lane]);
+                    double Qud = s.Qud, Qdd = s.Qdd;
+                    const double eq = __shfl_sync(FULL, e, ne - 1), es = __shfl_sync(FULL, e, e0),
+                                 eu = __shfl_sync(FULL, e, e0 + 1);
+                    if (ph == PH_GRAD) {
+                        // the Dirichlet forms of the search: u^T K d from the gradient pass
+                        // (or the smoother), d^T K d from its first trial pass
+                        slope = b.smooth ? -h2 * h2 * es : es;
+                        Qud = eu;
+                        Qdd = eq;
+                    }
+                    const int j3 = 3 * min(lane, ntr - 1);
+                    const double d1 = __shfl_sync(FULL, e, j3), d2 = __shfl_sync(FULL, e, j3 + 1),
+                                 d3 = __shfl_sync(FULL, e, j3 + 2);
+                    mytau = s.trial_tau[min(lane, REG_MAX_TRIALS - 1)];
+                    const double E = s.E, hl = 0.5 * b.lambda * h2;
+                    const double reg = hl * (mytau * fma(mytau, Qdd, 2.0 * Qud));
+                    const double bound = b.sigma * mytau * slope, stop = b.eps * (fabs(E) > 1.0 ? fabs(E) : 1.0);
+                    eval_at(v, s.cur_ev.S1 + h2 * d1, s.cur_ev.S2 + h2 * d2, s.cur_ev.S3 + h2 * d3);
                     // energy change E(u + tau d) - E(u) from the accumulated sums at u
-                    v.dE = -(v.ncc - s.ncc) + reg;
+                    v.dE = -(v.ncc - s.cur_ev.ncc) + reg;
                     v.acc = v.dE <= bound;
                     v.conv = -v.dE < stop;
-                    ev[lane] = v;
-                }
-                __syncwarp();
-                if (lane == 0) {
-                    if (ph == PH_GRAD) {
+                    __syncwarp();
+                    if (lane == 0 && ph == PH_GRAD) {
                         s.Qud = Qud;
                         s.Qdd = Qdd;
                     }
-                    control_op(b, s, op, o, n, ev, slope, slope < 0.0 ? 1 : (slope == 0.0 ? 0 : -1));
+                }
+                __syncwarp();
+                control_op(b, s, op, o, n, lane, v, mytau, slope);
+                if (lane == 0) {
                     set_step(s, op);
                     b.plan[o] = make_int2(s.tG, s.tT);
                     if (s.phase == PH_DONE) atomicAdd(&b.ctr[7], -1);

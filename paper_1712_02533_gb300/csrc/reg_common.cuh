@@ -22,8 +22,8 @@
 // pick others per level): short strips where a tile's row walk is latency
 // bound, long ones where there are enough tiles.
 __host__ __device__ __forceinline__ int strip_rows(int n) { return n <= 65 ? 8 : (n <= 257 ? 16 : 32); }
-#define PT_STRIDE (3 * REG_MAX_TRIALS + 3)  // doubles per trial-tile partial record
-#define PG_STRIDE 2                         // doubles per gradient-tile partial record
+#define PT_STRIDE (3 * REG_MAX_TRIALS + 3)  // floats per trial-tile partial record
+#define PG_STRIDE 2                         // floats per gradient-tile partial record
 
 // Phases of the per-operator state machine.
 enum {
@@ -109,6 +109,16 @@ struct __align__(16) StepDesc {
     float tau[REG_MAX_TRIALS];  // step sizes of the trial pass
 };
 
+// An evaluated energy: the FE sums S1 = int That, S2 = int That^2, S3 = int That
+// R~ (R~ normalised: mean 0, FE sigma 1; S1 is That's mean), sigma = sqrt(S2 - S1^2),
+// NCC = S3 / sigma, the gradient pass's coefficients there, and of a trial the energy
+// change, the Armijo test and the stopping test.
+struct EvalAt {
+    double S1, S2, S3, ncc, sig, dE;
+    float isig, c36, cT;
+    int acc, conv, pad;
+};
+
 struct OpState {
     StepDesc step;
     int phase, lvl, cur, src;
@@ -116,19 +126,15 @@ struct OpState {
     int status, nonfinite_seen, search, ntr;
     int tG, tT;       // gradient and trial tiles of this step
     double tau;       // base step of the current search
-    double tau_acc;   // step to apply at the start of the next G/P pass
+    double tau_acc;   // step to apply at the start of the next gradient pass, prolongation or result
     double sh_tau;    // shrinking: last rejected step
-    double E, Tbar, sigT, ncc;      // at the current u
-    double S1, S2, S3;              // FE sums int That, int That^2, int That R~ at the current u
-    double bS1, bS2, bS3, bncc, bsig, bdE;  // last accepted trial of the search
-    double btau;
+    double btau;      // last accepted step of the search
+    double E;         // at the current u
     double slope;
     double Qud, Qdd;  // Dirichlet forms u^T K d and d^T K d of the current search
+    EvalAt cur_ev;    // at the current u
+    EvalAt best_ev;   // last accepted trial of a search that goes on in another pass
     double trial_tau[REG_MAX_TRIALS];
-    // of the last accepted trial of the search: the gradient pass's coefficients
-    // there, and whether its energy decrease meets the stopping rule
-    float b_isig, b_c36, b_cT;
-    int b_conv;
     double corr;  // judged ops: sum over finest nodes of |u_final - u_start| (x + y, px)
 };
 
@@ -143,8 +149,9 @@ struct BatchDev {
     int *prefG, *prefT;          // and exclusive prefix of tile counts (n+1 entries)
     int *ctr;                    // [0] n_ops [2] nG [3] nT [5] itemsG [6] itemsT [7] n_active
                                  // [8] error flag [9] blocks of the control kernel that are done
-    double *partG;               // per gradient tile: slope and u^T K d partials (PG_STRIDE)
-    double *partT;               // per trial tile: 3 sums per step size, then 3 Dirichlet forms (PT_STRIDE)
+    float *partG;                // per gradient tile: slope and u^T K d partials (PG_STRIDE)
+    float *partT;                // per trial tile: 3 sums per step size, .., the Dirichlet form of d (PT_STRIDE)
+    double *partU;               // per tile of a level-start pass: 3 sums and the Dirichlet form of u
     unsigned long long *work;    // per kernel family: nodes processed
     double *trace;               // optional Armijo trial records (7 doubles each)
     unsigned long long *trace_len;
@@ -154,7 +161,7 @@ struct BatchDev {
     int iter_max, J, bf16;
     // H1-type smoother (smooth != 0): per op and column chunk of
     // REG_GW columns, the partial sums {sum omega d_L2 . d, sum d . 6 K u}
-    double *partS;
+    float *partS;
     int smooth, rch, cch;  // row chunks and column chunks of REG_GW per op (maxima)
     float sm_a;            // off-diagonal of the dimensionless 1D system (1/6 - s^2/2)
 };
