@@ -1957,6 +1957,17 @@ __device__ __forceinline__ double rsqrt_step(double v)
     return fma(r * e, fma(e, 0.375, 0.5), r);
 }
 
+// (The rare paths are calls: the code of a step's common path runs once per launch, and
+// its length in instruction fetches counts.)
+__device__ __noinline__ void eval_rare(EvalAt &v, double var)
+{
+    v.sig = var > 0.0 ? sqrt(var) : 0.0;
+    v.ncc = v.S3 / v.sig;
+    v.isig = (float)(1.0 / v.sig);
+    v.c36 = (float)(v.ncc / (v.sig * v.sig) / 36.0);
+    v.cT = (float)(v.ncc / (v.sig * v.sig) * v.S1);
+}
+
 // sigma, NCC and the gradient pass's coefficients from the FE sums.
 __device__ __forceinline__ void eval_at(EvalAt &v, double S1, double S2, double S3)
 {
@@ -1973,22 +1984,21 @@ __device__ __forceinline__ void eval_at(EvalAt &v, double S1, double S2, double 
         v.c36 = (float)(q * (1.0 / 36.0));
         v.cT = (float)(q * S1);
     } else {  // (almost) no variance, or not finite
-        v.sig = var > 0.0 ? sqrt(var) : 0.0;
-        v.ncc = S3 / v.sig;
-        v.isig = (float)(1.0 / v.sig);
-        v.c36 = (float)(v.ncc / (v.sig * v.sig) / 36.0);
-        v.cT = (float)(v.ncc / (v.sig * v.sig) * S1);
+        EvalAt w = v;
+        eval_rare(w, var);
+        v = w;
     }
 }
 
 // Positive doubles compare like their bits, and doubling one adds to its
 // exponent field: the step sizes of the search stay off the slow FP64 pipe.
 // (Numbers near the ends of the exponent range take the multiplication.)
+__device__ __noinline__ double pow2_rare(double x, int e) { return scalbn(x, e); }
 __device__ __forceinline__ double pow2_scale(double x, int e)
 {
     const long long w = __double_as_longlong(x);
     const int ex = (int)(w >> 52);
-    return ex > 8 && ex < 0x7f0 ? __longlong_as_double(w + ((long long)e << 52)) : scalbn(x, e);
+    return ex > 8 && ex < 0x7f0 ? __longlong_as_double(w + ((long long)e << 52)) : pow2_rare(x, e);
 }
 __device__ __forceinline__ double twice(double x) { return pow2_scale(x, 1); }
 __device__ __forceinline__ double half_of(double x) { return pow2_scale(x, -1); }
@@ -2060,6 +2070,7 @@ __device__ __forceinline__ void control_op(const BatchDev &b, OpState &s, const 
             double btau = s.btau, sh_tau = s.sh_tau;
             bool finish = false, more = false;
             int guard = 0;
+#pragma unroll 1
             for (; guard < 4 * REG_MAX_TRIALS + 8 && !finish && status < 0; guard++) {
                 const double want =
                     search == SEARCH_INIT ? tau : (search == SEARCH_WIDEN ? twice(btau) : half_of(sh_tau));
@@ -2308,15 +2319,15 @@ __global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
                 }
                 Sum3 v;
                 int it = g;
-                for (; it + 3 * ng < cnt; it += 4 * ng) {
-                    const float x0 = rec[(int64_t)it * stride], x1 = rec[(int64_t)(it + ng) * stride],
-                                x2 = rec[(int64_t)(it + 2 * ng) * stride], x3 = rec[(int64_t)(it + 3 * ng) * stride];
-                    v.add(x0);
-                    v.add(x1);
-                    v.add(x2);
-                    v.add(x3);
+                // eight loads in flight
+                for (; it < cnt; it += 8 * ng) {
+                    float x[8];
+#pragma unroll
+                    for (int q = 0; q < 8; q++) x[q] = it + q * ng < cnt ? rec[(it + q * ng) * stride] : 0.f;
+#pragma unroll
+                    for (int q = 0; q < 8; q++)
+                        if (it + q * ng < cnt) v.add(x[q]);
                 }
-                for (; it < cnt; it += ng) v.add(rec[(int64_t)it * stride]);
                 const int at = kk * (ng + 1) + g;
                 red[0][at] = v.a;
                 red[1][at] = v.b;
