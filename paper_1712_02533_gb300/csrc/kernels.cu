@@ -2427,11 +2427,14 @@ __global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
 // stored finest level with its normalisation undone (F = F~ sigma_k + mean_k),
 // sampled bilinearly and clamped to the grid; u_k from fields[k] (float2 grid
 // units of the finest level; null = the identity), as sums in double give it.
-// Three FP64 operations per sample (16 cycles of an SM each for a warp) took 345 of
-// the 415 us for 64 frames of 1025^2 (255 us now, bound by issue and the latency of
-// field -> texel chains), so the products and their sum run in float
-// pairs (to 2^-44 of the terms' sum, the means' sum is one FP64 constant); a node
-// whose rounding that does not settle, about one in 10^5, is summed again in FP64.
+// Three FP64 operations per sample and the division (16 cycles of an SM each for a
+// warp) took 345 of the 415 us for 64 frames of 1025^2, so the products, their sum
+// and its product with 1/m run in float pairs (to 2^-43 of the terms' sum; the
+// means' sum and 1/m are two constants of the block); a node whose rounding that
+// does not settle, about one in 10^5, is summed again in FP64.  A call for 64 frames
+// takes 276 us (443 with FP64 sums, 308 with the end of a node in FP64: two
+// divisions), for 3 frames in BF16 47 us (67, 93); bound by issue and the latency of
+// field -> texel chains.
 constexpr int AVG_FRAMES = 128;  // frames staged in shared memory at a time
 constexpr int AVG_BATCH = 2;     // frames whose fields, then texels, a thread has in flight
 template <bool BF16>
@@ -2443,7 +2446,7 @@ __global__ void __launch_bounds__(256) k_average(const void *__restrict__ pyr, i
     __shared__ const float2 *fld[AVG_FRAMES];
     __shared__ const void *img[AVG_FRAMES];
     __shared__ float2 sig[AVG_FRAMES];  // sigma_k as two floats
-    __shared__ double mean_sum;
+    __shared__ float2 mean_sum, inv_m;  // as two floats
     const int c = blockIdx.x * 32 + threadIdx.x, r = blockIdx.y * 8 + threadIdx.y;
     const int tid = threadIdx.y * 32 + threadIdx.x;
     const bool in = r < n && c < n;
@@ -2456,7 +2459,10 @@ __global__ void __launch_bounds__(256) k_average(const void *__restrict__ pyr, i
         double s = 0.0;
         for (int k = tid; k < m; k += 32) s += fstats[2 * k];
         s = warp_sum_d(s);
-        if (tid == 0) mean_sum = s;
+        if (tid == 0) mean_sum = make_float2((float)s, (float)(s - (double)(float)s));
+    } else if (tid == 32) {
+        const double s = 1.0 / m;
+        inv_m = make_float2((float)s, (float)(s - (double)(float)s));
     }
     float hi = 0.f, lo = 0.f, mag = 0.f;
     for (int k0 = 0; k0 < m; k0 += AVG_FRAMES) {
@@ -2507,11 +2513,14 @@ __global__ void __launch_bounds__(256) k_average(const void *__restrict__ pyr, i
         }
     }
     if (!in) return;
-    const double t = ((double)hi + (double)lo) + mean_sum;
-    const double tol = ((double)mag + fabs(mean_sum)) * 5.6843418860808015e-14;  // 2^-44
-    const float a = (float)((t - tol) / m), b = (float)((t + tol) / m);
+    float t, te;
+    two_sum(hi, mean_sum.x, t, te);
+    te += lo + mean_sum.y;
+    const float p = __fmul_rn(t, inv_m.x), pl = fmaf(t, inv_m.y, fmaf(te, inv_m.x, fmaf(t, inv_m.x, -p)));
+    const float size = (mag + fabsf(mean_sum.x)) * inv_m.x, tol = size * 1.1368683772161603e-13f;  // 2^-43
+    const float a = p + (pl - tol), b = p + (pl + tol);
     float res = a;
-    if (!(a == b)) {
+    if (!(a == b) || !(size > 1e-25f)) {  // (the low parts of tiny values underflow)
         double acc = 0.0;
         for (int k = 0; k < m; k++) {
             const float2 *f = fields[k];

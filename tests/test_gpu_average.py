@@ -56,6 +56,22 @@ def test_average_of_given_deformations_matches_oracle(reg, orc, syn, side, stora
     assert err <= tol * rng_, (err, rng_)
 
 
+@pytest.mark.parametrize("nf", [2, 3, 131])
+def test_average_of_few_and_many_frames_matches_oracle(reg, orc, syn, nf):
+    """As above in FP32 storage at the frame counts where the sums begin and end: a
+    last pair of frames that is half empty (3), more frames than are staged at a time
+    (131).  Same tolerance: the stored frames' rounding, 1e-5 of the range."""
+    side = 32
+    fr = syn.series(43, nf, side, peak=20.0, spacing=10.0, sigma=2.0) + np.float32(50.0)
+    fields = _fields(nf, side + 1, 5)
+    with reg.Series(fr, reg.default_params(n_levels=2, lam=10.0)) as s:
+        for k in range(1, nf):
+            s.set_slot(k - 1, fields[k - 1], 0, k)
+        got = s.average(iterations=0)
+    want = orc.average([orc.embed(f) for f in fr], [None] + [f.astype(np.float64) / side for f in fields])[:side, :side]
+    assert np.abs(got - want).max() <= 1e-5 * float(want.max() - want.min())
+
+
 def test_averaging_procedure_matches_oracle_on_a_stable_series(reg, orc, syn):
     """The whole procedure on the config-1 series without shot noise (the
     oracle's result is stable there): registration, average, one iteration of
