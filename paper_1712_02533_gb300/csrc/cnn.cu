@@ -702,6 +702,22 @@ int wgrad_small_grid(int n_tiles)
     return std::max(1, std::min(n_tiles, 2 * nsm));
 }
 
+// Floats of a layer's partial records (the tensor-core kernel writes one record per
+// SM, the others up to two), and of all layers: the records stay until one launch
+// adds them all.
+size_t wpart_floats(int k)
+{
+    const size_t rec = k == 0 ? WF_REC : k == NL - 1 ? WL_REC : WG32_REC, n = wgrad_small_grid(1 << 30) * rec;
+    return k == 0 || k == NL - 1 ? n : std::max(n, (size_t)cnn_wgrad32_umma_part_floats());
+}
+
+size_t wpart_offset(int k)
+{
+    size_t n = 0;
+    for (int j = 0; j < k; j++) n += wpart_floats(j);
+    return n;
+}
+
 // Mean squared error: per-block partial sums (double), then one block adds them
 // in order; gy = 2 (y - t) / N.
 __global__ void k_mse(const float *__restrict__ y, const float *__restrict__ t, int64_t n, float *__restrict__ gy,
@@ -774,23 +790,23 @@ void fwd(int k, const float *in, int H, const float *theta, float *out, int B, c
     else k_conv_fwd32<32, 1><<<grid, 128, 0, st>>>(in, H, theta, out, Ho, nyg, total);
 }
 
-// FP32 weight gradient of layer k into grad and, for k > 0, its data gradient with
+// FP32 weight gradient of layer k (records to part, entered in sums for grad) and, for k > 0, its data gradient with
 // the ReLU mask of the layer below into gx.
 void bwd(int k, const float *in, int H, const float *gz, const float *theta, float *gx, float *grad, int B,
-         cudaStream_t st, float *part)
+         cudaStream_t st, float *part, CnnSumList &sums)
 {
     const int Ho = (H + 2 - 3) / LAYERS[k].S + 1;
     auto tiles = [&](int tr, int tc) { return B * ((Ho + tr - 1) / tr) * ((Ho + tc - 1) / tc); };
     if (k == 0) {
         const int grid = wgrad_small_grid(tiles(WF_TR, WF_TW));
         k_wgrad_first<<<grid, 256, 0, st>>>(in, H, gz, Ho, B, part);
-        cnn_sum_records(part, grid, WF_REC, grad, st);
+        sums.add(part, grid, WF_REC, grad, false);
         return;
     }
     if (k == NL - 1) {
         const int grid = wgrad_small_grid(tiles(WL_TR, WL_TW)), total = B * H * H;
         k_wgrad_last<false><<<grid, 256, 0, st>>>(in, H, gz, B, part);
-        cnn_sum_records(part, grid, WL_REC, grad, st);
+        sums.add(part, grid, WL_REC, grad, false);
         k_conv_bwd_data<32, 2, 1><<<(total + 127) / 128, 128, 0, st>>>(gz, Ho, theta, in, gx, H, total);
         return;
     }
@@ -799,12 +815,12 @@ void bwd(int k, const float *in, int H, const float *gz, const float *theta, flo
     if (S == 2) {
         const int wg = wgrad_small_grid(tiles(Wg32<2>::TR, Wg32<2>::TC));
         k_wgrad32<2><<<wg, 256, 0, st>>>(in, H, gz, Ho, B, part);
-        cnn_sum_records(part, wg, WG32_REC, grad, st);
+        sums.add(part, wg, WG32_REC, grad, false);
         k_conv_bwd_data32<2><<<grid, 128, 0, st>>>(gz, Ho, theta, in, gx, H, nyg, total);
     } else {
         const int wg = wgrad_small_grid(tiles(Wg32<1>::TR, Wg32<1>::TC));
         k_wgrad32<1><<<wg, 256, 0, st>>>(in, H, gz, Ho, B, part);
-        cnn_sum_records(part, wg, WG32_REC, grad, st);
+        sums.add(part, wg, WG32_REC, grad, false);
         k_conv_bwd_data32<1><<<grid, 128, 0, st>>>(gz, Ho, theta, in, gx, H, nyg, total);
     }
 }
@@ -824,12 +840,12 @@ struct reg_cnn {
     uint32_t *wpack_u = nullptr;  // the 32 -> 32 layers' weights in the tcgen05 operand layout
     uint32_t *wpack_d = nullptr;  // the same, flipped and transposed for the data gradients
     uint32_t *wpack_first = nullptr, *wpack_last = nullptr;  // the first and last layers, tcgen05 layouts
-    // parameter version (set_params, adam_step) and the version each packed
-    // copy was made from (forward: layers 0..5): the packing runs only after a change
-    int64_t version = 0, packed_fwd[6] = {-1, -1, -1, -1, -1, -1}, packed_dgrad[4] = {-1, -1, -1, -1};
+    // parameter version (set_params, adam_step) and the version the packed
+    // copies were made from: the packing runs only after a change
+    int64_t version = 0, packed = -1;
     int *uerr = nullptr;          // error word of the tcgen05 kernels (a wait ran out): device view
     int *uerr_host = nullptr;     // the same word, pinned host memory mapped into the device
-    float *wpart = nullptr;     // per-block partial weight gradients of the tensor-core training
+    float *wpart = nullptr;     // per-block partial weight gradients, a region per layer
     int64_t step = 0;
 };
 
@@ -878,6 +894,13 @@ reg_status cnn_forward(reg_cnn *h, const float *x, int B, float *y, cudaStream_t
 {
     const int S = h->side;
     const float *a = x;
+    if (tc && h->packed != h->version) {
+        const float *th[NL];
+        for (int k = 0; k < NL; k++) th[k] = h->theta + param_offset(k);
+        const reg_status rs = cnn_pack_umma(th, h->wpack_first, h->wpack_u, h->wpack_last, h->wpack_d, st);
+        if (rs != REG_OK) return rs;
+        h->packed = h->version;
+    }
     for (int k = 0; k < NL; k++) {
         const int H = in_side(k, S);
         const float *th = h->theta + param_offset(k);
@@ -886,17 +909,15 @@ reg_status cnn_forward(reg_cnn *h, const float *x, int B, float *y, cudaStream_t
             // tensor-core path, all six layers on tcgen05: layer 0 from the FP32
             // input, the others from the BF16 planar activations, which layers
             // 0..4 write; layer 5 writes the FP32 output
-            const bool pack = h->packed_fwd[k] != h->version;
             reg_status rs;
             if (k == 0)
-                rs = cnn_first_umma(a, H, th, h->actb[0], B, st, h->wpack_first, pack, h->uerr);
+                rs = cnn_first_umma(a, H, th, h->actb[0], B, st, h->wpack_first, h->uerr);
             else if (k == NL - 1)
-                rs = cnn_last_umma(h->actb[k - 1], H, th, out, B, st, h->wpack_last, pack, h->uerr);
+                rs = cnn_last_umma(h->actb[k - 1], H, th, out, B, st, h->wpack_last, h->uerr);
             else
                 rs = cnn_conv32_umma(h->actb[k - 1], H, th, h->actb[k], false, B, LAYERS[k].S, st,
-                                     h->wpack_u + (k - 1) * cnn_conv32_umma_words(), pack, h->uerr);
+                                     h->wpack_u + (k - 1) * cnn_conv32_umma_words(), h->uerr);
             if (rs != REG_OK) return rs;
-            h->packed_fwd[k] = h->version;
         } else {
             fwd(k, a, H, th, out, B, st);
         }
@@ -942,7 +963,7 @@ reg_status reg_cnn_create(int32_t side, int32_t max_batch, void *cuda_stream, re
          alloc((void **)&h->wpack_last, sizeof(uint32_t) * cnn_last_umma_words()) &&
          cudaHostAlloc((void **)&h->uerr_host, sizeof(int), cudaHostAllocMapped) == cudaSuccess &&
          cudaHostGetDevicePointer((void **)&h->uerr, h->uerr_host, 0) == cudaSuccess &&
-         alloc((void **)&h->wpart, sizeof(float) * (size_t)std::max(cnn_wgrad32_umma_part_floats(), wgrad_small_grid(1 << 30) * WG32_REC));
+         alloc((void **)&h->wpart, sizeof(float) * wpart_offset(NL));
     if (!ok) {
         reg_cnn_destroy(h);
         return cnn_fail(REG_ENOMEM, "device allocation failed");
@@ -1024,23 +1045,23 @@ static reg_status loss_grad(reg_cnn_t h, const float *x, const float *target, in
     k_sum_partials<<<1, 256, 0, st>>>(h->partial, nb, 1.0 / (double)ny, h->loss);
     const float *gz = h->gy;
     float *bufs[2] = {h->g0, h->g1};
+    CnnSumList sums;
     for (int k = NL - 1; k >= 0; k--) {
         const int H = in_side(k, S);
         const float *in = k == 0 ? x : h->act[k - 1];
         const float *th = h->theta + param_offset(k);
         float *gr = h->grad + param_offset(k);
         float *gx = k == 0 ? nullptr : bufs[k & 1];
+        float *part = h->wpart + wpart_offset(k);
         if (tc && k >= 1 && k <= 4) {
             // the layer's input and the mask below: BF16 planar
             const uint16_t *inb = h->actb[k - 1];
-            rs = cnn_wgrad32_umma(inb, H, gz, B, LAYERS[k].S, gr, h->wpart, st, h->uerr);
+            rs = cnn_wgrad32_umma(inb, H, gz, B, LAYERS[k].S, gr, part, sums, st, h->uerr);
             if (rs != REG_OK) return rs;
-            const bool pack = h->packed_dgrad[k - 1] != h->version;
-            uint32_t *wp = h->wpack_d + (k - 1) * cnn_conv32_umma_words();
-            if (LAYERS[k].S == 1) rs = cnn_dgrad32_umma(gz, H, th, inb, gx, B, st, wp, pack, h->uerr);
-            else rs = cnn_dgrad32s2_umma(gz, H / 2, th, inb, gx, B, st, wp, pack, h->uerr);
+            const uint32_t *wp = h->wpack_d + (k - 1) * cnn_conv32_umma_words();
+            if (LAYERS[k].S == 1) rs = cnn_dgrad32_umma(gz, H, th, inb, gx, B, st, wp, h->uerr);
+            else rs = cnn_dgrad32s2_umma(gz, H / 2, th, inb, gx, B, st, wp, h->uerr);
             if (rs != REG_OK) return rs;
-            h->packed_dgrad[k - 1] = h->version;
             gz = gx;
             continue;
         }
@@ -1048,8 +1069,8 @@ static reg_status loss_grad(reg_cnn_t h, const float *x, const float *target, in
             // the last layer's input (and the mask below) is the planar BF16
             // output of layer 4
             const int nt = B * ((H + WL_TW - 1) / WL_TW) * ((H + WL_TR - 1) / WL_TR), grid = wgrad_small_grid(nt);
-            k_wgrad_last<true><<<grid, 256, 0, st>>>(h->actb[k - 1], H, gz, B, h->wpart);
-            cnn_sum_records(h->wpart, grid, WL_REC, gr, st);
+            k_wgrad_last<true><<<grid, 256, 0, st>>>(h->actb[k - 1], H, gz, B, part);
+            sums.add(part, grid, WL_REC, gr, false);
             const int total = B * H * H;
             k_conv_bwd_data<32, 2, 1, true><<<(total + 127) / 128, 128, 0, st>>>(gz, H, th, h->actb[k - 1], gx, H, total);
             gz = gx;
@@ -1058,13 +1079,14 @@ static reg_status loss_grad(reg_cnn_t h, const float *x, const float *target, in
         if (tc && k == 0) {
             const int Ho = H / 2, nt = B * ((Ho + WF_TW - 1) / WF_TW) * ((Ho + WF_TR - 1) / WF_TR);
             const int grid = wgrad_small_grid(nt);
-            k_wgrad_first<<<grid, 256, 0, st>>>(x, H, gz, Ho, B, h->wpart);
-            cnn_sum_records(h->wpart, grid, WF_REC, gr, st);
+            k_wgrad_first<<<grid, 256, 0, st>>>(x, H, gz, Ho, B, part);
+            sums.add(part, grid, WF_REC, gr, false);
             continue;
         }
-        bwd(k, in, H, gz, th, gx, gr, B, st, h->wpart);
+        bwd(k, in, H, gz, th, gx, gr, B, st, part, sums);
         gz = gx;
     }
+    cnn_sum_records(sums, st);
     CKC(cudaGetLastError());
     if (loss) CKC(cudaMemcpyAsync(loss, h->loss, sizeof(double), cudaMemcpyDeviceToHost, st));
     if (grad_out) CKC(cudaMemcpyAsync(grad_out, h->grad, sizeof(float) * h->n, cudaMemcpyDeviceToHost, st));

@@ -22,7 +22,7 @@
 // matrices" of 8 rows x 16 bytes (8 BF16 values along k), each stored as 128
 // contiguous bytes, rows 16 bytes apart.  A descriptor gives the start address
 // and two strides: between core matrices adjacent along M (or N) and along K.
-//   - Weights, packed by k_pack_umma when the parameters change: [tap][cg][o][8
+//   - Weights, packed by k_pack when the parameters change: [tap][cg][o][8
 //     channels] BF16.  For a k-step (tap, half h) the operand starts at
 //     ((4 tap + 2 h) N) 16 bytes; N-stride 128 B, K-stride 16 N bytes.  They
 //     reach shared memory by a bulk asynchronous copy (cp.async.bulk).
@@ -272,10 +272,9 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi)
 // stride-1 32 -> 32 layer as a forward convolution of the output gradient
 // with K'[c][o][tap] = W[o][c][8 - tap] (output channel c, reduction channel o).
 template <bool DGRAD, int N, int O>
-__global__ void k_pack_umma(const float *__restrict__ theta, uint32_t *__restrict__ wpack)
+__device__ __forceinline__ void pack_umma(const float *__restrict__ theta, uint32_t *__restrict__ wpack, int i)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;  // one pair of reduction channels
-    if (i >= Wts<N>::bytes / 4) return;
+    if (i >= Wts<N>::bytes / 4) return;  // i: one pair of reduction channels
     const int jp = i & 3, n = (i >> 2) % N, r = (i >> 2) / N, cg = r & 3, tap = r >> 2;
     const int k0 = 8 * cg + 2 * jp;  // reduction channel of the low half
     float lo = 0.f, hi = 0.f;
@@ -300,9 +299,8 @@ __host__ __device__ constexpr int l0_tap(int j, int h)
 
 // W[o][c][dy][dx] of the first layer (32 x 2 x 3 x 3) -> [step][half][o][8
 // channels] (BF16), channels 2..7 and the missing tap zero.
-__global__ void k_pack_l0(const float *__restrict__ theta, uint32_t *__restrict__ wpack)
+__device__ __forceinline__ void pack_l0(const float *__restrict__ theta, uint32_t *__restrict__ wpack, int i)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= L0_WBYTES / 4) return;
     const int jp = i & 3, o = (i >> 2) & 31, h = (i >> 7) & 1, j = i >> 8;
     const int tap = l0_tap(j, h);
@@ -312,6 +310,24 @@ __global__ void k_pack_l0(const float *__restrict__ theta, uint32_t *__restrict_
         hi = theta[(o * 2 + 1) * 9 + tap];
     }
     wpack[i] = pack2(lo, hi);
+}
+
+// All layers' packed weights in one launch when the parameters have changed (block
+// row y: 0 the first layer, 1..4 the 32 -> 32 layers, 5 the last, 6..9 the 32 -> 32
+// layers flipped and transposed for the data gradients).  A launch per layer and
+// direction took ten times 2.8 us of a training pass.
+struct PackLayers {
+    const float *theta[6];
+    uint32_t *first, *fwd, *last, *dgrad;
+};
+__global__ void __launch_bounds__(256) k_pack(const __grid_constant__ PackLayers p)
+{
+    const int i = blockIdx.x * 256 + threadIdx.x, y = blockIdx.y;
+    constexpr int words = Wts<UC>::bytes / 4;
+    if (y == 0) pack_l0(p.theta[0], p.first, i);
+    else if (y < 5) pack_umma<false, UC, UC>(p.theta[y], p.fwd + (y - 1) * words, i);
+    else if (y == 5) pack_umma<false, 16, 2>(p.theta[5], p.last, i);
+    else pack_umma<true, UC, UC>(p.theta[y - 5], p.dgrad + (y - 6) * words, i);
 }
 
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
@@ -813,8 +829,8 @@ __global__ void __launch_bounds__(128) k_conv_umma_staged(const float *__restric
 // its tiles (tile = block + k grid) with two staging buffers, so that the MMAs
 // of one tile run while the next is staged; the bias sums (of the unrounded
 // FP32 gradient) are formed from the staging registers.  Each CTA writes one
-// record in the parameter layout ((o 32 + c) 9 + tap, then the 32 biases);
-// cnn_sum_records adds the records.
+// record (entry (tap 32 + c) 32 + o, then the 32 biases); cnn_sum_records adds the
+// records into the parameter layout.
 constexpr int WG_TH = 8, WG_TW = 16, WG_N = 96, WG_COLS = 512;
 constexpr int WG_REC = UC * UC * 9 + UC;
 
@@ -960,18 +976,22 @@ __global__ void __launch_bounds__(256, 1) k_wgrad32_umma(const uint4 *__restrict
         bad = __syncthreads_or(!ok);
     }
     float *rec = part + (int64_t)blockIdx.x * WG_REC;
-    if (warp == 0) {
-        // lane o of the accumulators: column 32 (3 dy + dx) + c = tap (dy, dx), channel c
+    if ((warp & 3) == 0) {
+        // lane o of the accumulators (warps 0 and 4 read the lanes 0..31): column
+        // 32 (3 dy + dx) + c = tap (dy, dx), channel c.  A store instruction writes
+        // the 32 output channels of one entry: one line, where the parameter
+        // layout's (o 32 + c) 9 + tap took 32 sectors of 32 lines and the other
+        // warps waited for it: 31 -> 22.4 us per launch (32 x 64^2 output pixels).
         tc_fence_after();
 #pragma unroll 1
-        for (int tap = 0; tap < 9; tap++) {
+        for (int tap = warp >> 2; tap < 9; tap += 2) {
             float v[UC];
             if (!bad && it > 0) tmem_ld<UC>(tmem + 32 * tap, v);
             else
 #pragma unroll
                 for (int c = 0; c < UC; c++) v[c] = 0.f;
 #pragma unroll
-            for (int c = 0; c < UC; c++) rec[(lane * UC + c) * 9 + tap] = v[c];
+            for (int c = 0; c < UC; c++) rec[(tap * UC + c) * UC + lane] = v[c];
         }
     }
     // bias: the four lanes of a pixel-pair group, then the eight warps
@@ -992,27 +1012,43 @@ __global__ void __launch_bounds__(256, 1) k_wgrad32_umma(const uint4 *__restrict
     umma_teardown<WG_COLS>(tmem);
 }
 
-// grad[e] = sum of the records' entries e < rec: a warp's lanes on adjacent
-// entries, 32 groups of records side by side (a chain of a few loads each), the
-// groups in order.  9.3 -> 3.5 us for the 152 records of a 32 -> 32 layer against
-// one thread per entry walking all records.
-__global__ void __launch_bounds__(1024) k_sum_records(const float *__restrict__ part, int nrec, int rec,
-                                                      float *__restrict__ grad)
+// The layers' weight and bias gradients from their records, one launch for all
+// layers: block b works in the last layer of the list with block0 <= b, on 32
+// adjacent pairs of entries (a warp's lanes; records are of even length), 16 groups
+// of records side by side, the groups added in order: one wave of blocks.  One launch per layer took 5.8 us
+// for each 32 -> 32 layer and 4.7 for the others (32 us a pass of 32 x 256^2), a
+// launch's own length more than its 5.6 MB.
+__global__ void __launch_bounds__(512) k_sum_records(const __grid_constant__ CnnSumList list)
 {
-    __shared__ float red[32][32];
-    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
-    float s = 0.f;
-    if (e < rec) {
+    __shared__ float2 red[16][32];
+    int q = 0;
+    while (q + 1 < list.n && (int)blockIdx.x >= list.s[q + 1].block0) q++;
+    const CnnSumSeg sg = list.s[q];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, e = ((int)blockIdx.x - sg.block0) * 64 + 2 * lane;
+    float2 s = make_float2(0.f, 0.f);
+    if (e < sg.rec) {
 #pragma unroll 8
-        for (int k = g; k < nrec; k += 32) s += part[(int64_t)k * rec + e];
+        for (int k = g; k < sg.nrec; k += 16) {
+            const float2 v = *reinterpret_cast<const float2 *>(sg.part + (int64_t)k * sg.rec + e);
+            s.x += v.x;
+            s.y += v.y;
+        }
     }
     red[g][lane] = s;
     __syncthreads();
-    if (g == 0 && e < rec) {
-        float tot = 0.f;
+    if (g == 0 && e < sg.rec) {
+        float tot[2] = {0.f, 0.f};
 #pragma unroll
-        for (int w = 0; w < 32; w++) tot += red[w][lane];
-        grad[e] = tot;
+        for (int w = 0; w < 16; w++) {
+            tot[0] += red[w][lane].x;
+            tot[1] += red[w][lane].y;
+        }
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+            const int i = e + j;
+            const bool perm = sg.tap_major && i < UC * UC * 9;
+            sg.grad[perm ? ((i & 31) * UC + ((i >> 5) & 31)) * 9 + (i >> 10) : i] = tot[j];
+        }
     }
 }
 
@@ -1084,12 +1120,11 @@ bool grid_for(K kern, int bytes, int cols, int n_tiles, int &grid)
 
 template <int S, int N, int NR, bool RELU, bool OUT_F32>
 reg_status launch_fwd(const uint16_t *in, int H, const float *theta, void *out, int B, cudaStream_t st,
-                      uint32_t *wpack, bool pack, int *err)
+                      const uint32_t *wpack, int *err)
 {
     CUtensorMap map;
     if (!encode_input_map(&map, in, H, B, S))
         return reg_internal_fail(REG_ECUDA, "tcgen05 convolution: tensor map of the input");
-    if (pack) k_pack_umma<false, N, NR><<<(Wts<N>::bytes / 4 + 255) / 256, 256, 0, st>>>(theta, wpack);
     const int Ho = (H + 2 - 3) / S + 1;
     const int tx = (Ho + UTW - 1) / UTW, ty = (Ho + UTH - 1) / UTH, nt = B * tx * ty;
     auto kern = k_conv_umma_ws<S, N, NR, RELU, OUT_F32>;
@@ -1104,31 +1139,40 @@ reg_status launch_fwd(const uint16_t *in, int H, const float *theta, void *out, 
 
 }  // namespace
 
+reg_status cnn_pack_umma(const float *const theta[6], uint32_t *first, uint32_t *fwd, uint32_t *last, uint32_t *dgrad,
+                         cudaStream_t st)
+{
+    PackLayers p{{}, first, fwd, last, dgrad};
+    for (int k = 0; k < 6; k++) p.theta[k] = theta[k];
+    static_assert(Wts<UC>::bytes >= Wts<16>::bytes && Wts<UC>::bytes >= L0_WBYTES, "the largest layer sets the grid");
+    k_pack<<<dim3((Wts<UC>::bytes / 4 + 255) / 256, 10), 256, 0, st>>>(p);
+    return cudaGetLastError() == cudaSuccess ? REG_OK : reg_internal_fail(REG_ECUDA, "tcgen05 weight packing launch");
+}
+
 int cnn_conv32_umma_words() { return Wts<UC>::bytes / 4; }
 
 reg_status cnn_conv32_umma(const uint16_t *in, int H, const float *theta, void *out, bool out_f32, int B, int S,
-                           cudaStream_t st, uint32_t *wpack, bool pack, int *err)
+                           cudaStream_t st, const uint32_t *wpack, int *err)
 {
     if (S == 1)
-        return out_f32 ? launch_fwd<1, UC, UC, true, true>(in, H, theta, out, B, st, wpack, pack, err)
-                       : launch_fwd<1, UC, UC, true, false>(in, H, theta, out, B, st, wpack, pack, err);
+        return out_f32 ? launch_fwd<1, UC, UC, true, true>(in, H, theta, out, B, st, wpack, err)
+                       : launch_fwd<1, UC, UC, true, false>(in, H, theta, out, B, st, wpack, err);
     if (S == 2)
-        return out_f32 ? launch_fwd<2, UC, UC, true, true>(in, H, theta, out, B, st, wpack, pack, err)
-                       : launch_fwd<2, UC, UC, true, false>(in, H, theta, out, B, st, wpack, pack, err);
+        return out_f32 ? launch_fwd<2, UC, UC, true, true>(in, H, theta, out, B, st, wpack, err)
+                       : launch_fwd<2, UC, UC, true, false>(in, H, theta, out, B, st, wpack, err);
     return reg_internal_fail(REG_EINVAL, "tcgen05 convolution: stride must be 1 or 2");
 }
 
 reg_status cnn_last_umma(const uint16_t *in, int H, const float *theta, float *out, int B, cudaStream_t st,
-                         uint32_t *wpack, bool pack, int *err)
+                         const uint32_t *wpack, int *err)
 {
-    return launch_fwd<1, 16, 2, false, true>(in, H, theta, out, B, st, wpack, pack, err);
+    return launch_fwd<1, 16, 2, false, true>(in, H, theta, out, B, st, wpack, err);
 }
 
 reg_status cnn_first_umma(const float *x, int H, const float *theta, uint16_t *out, int B, cudaStream_t st,
-                          uint32_t *wpack, bool pack, int *err)
+                          const uint32_t *wpack, int *err)
 {
     if (H % 2) return reg_internal_fail(REG_EINVAL, "tcgen05 first layer: odd input side");
-    if (pack) k_pack_l0<<<(L0_WBYTES / 4 + 255) / 256, 256, 0, st>>>(theta, wpack);
     const int Ho = (H + 2 - 3) / 2 + 1;
     const int tx = (Ho + UTW - 1) / UTW, ty = (Ho + UTH - 1) / UTH, nt = B * tx * ty;
     int grid = 0;
@@ -1141,9 +1185,8 @@ reg_status cnn_first_umma(const float *x, int H, const float *theta, uint16_t *o
 }
 
 reg_status cnn_dgrad32_umma(const float *gz, int H, const float *theta, const uint16_t *mask, float *gx, int B,
-                            cudaStream_t st, uint32_t *wpack, bool pack, int *err)
+                            cudaStream_t st, const uint32_t *wpack, int *err)
 {
-    if (pack) k_pack_umma<true, UC, UC><<<(Wts<UC>::bytes / 4 + 255) / 256, 256, 0, st>>>(theta, wpack);
     const int tx = (H + UTW - 1) / UTW, ty = (H + UTH - 1) / UTH, nt = B * tx * ty;
     int grid = 0;
     if (!grid_for(k_conv_umma_staged<ST_DGRAD1>, DgradSmem::bytes, staged_cols<ST_DGRAD1>(), nt, grid))
@@ -1156,9 +1199,8 @@ reg_status cnn_dgrad32_umma(const float *gz, int H, const float *theta, const ui
 }
 
 reg_status cnn_dgrad32s2_umma(const float *gz, int Hg, const float *theta, const uint16_t *mask, float *gx, int B,
-                              cudaStream_t st, uint32_t *wpack, bool pack, int *err)
+                              cudaStream_t st, const uint32_t *wpack, int *err)
 {
-    if (pack) k_pack_umma<true, UC, UC><<<(Wts<UC>::bytes / 4 + 255) / 256, 256, 0, st>>>(theta, wpack);
     const int tx = (Hg + UTW - 1) / UTW, ty = (Hg + UTH - 1) / UTH, nt = B * tx * ty;
     int grid = 0;
     if (!grid_for(k_conv_umma_staged<ST_DGRAD2>, DgradSmem::bytes, staged_cols<ST_DGRAD2>(), nt, grid))
@@ -1174,7 +1216,7 @@ namespace {
 
 template <int S>
 reg_status launch_wgrad_umma(const uint16_t *in, int H, const float *gz, int B, float *grad, float *part,
-                             cudaStream_t st, int *err)
+                             CnnSumList &sums, cudaStream_t st, int *err)
 {
     const int Ho = (H + 2 - 3) / S + 1;
     const int tx = (Ho + WG_TW - 1) / WG_TW, ty = (Ho + WG_TH - 1) / WG_TH, nt = B * tx * ty;
@@ -1183,7 +1225,7 @@ reg_status launch_wgrad_umma(const uint16_t *in, int H, const float *gz, int B, 
         return reg_internal_fail(REG_ECUDA, "tcgen05 weight gradient: launch attributes");
     k_wgrad32_umma<S><<<grid, 256, WgSmem<S>::bytes, st>>>(reinterpret_cast<const uint4 *>(in), H, gz, Ho, tx, ty, nt,
                                                           part, err);
-    cnn_sum_records(part, grid, WG_REC, grad, st);
+    sums.add(part, grid, WG_REC, grad, true);
     if (cudaGetLastError() != cudaSuccess) return reg_internal_fail(REG_ECUDA, "tcgen05 weight gradient launch");
     return REG_OK;
 }
@@ -1191,16 +1233,16 @@ reg_status launch_wgrad_umma(const uint16_t *in, int H, const float *gz, int B, 
 }  // namespace
 
 reg_status cnn_wgrad32_umma(const uint16_t *in, int H, const float *gz, int B, int S, float *grad, float *part,
-                            cudaStream_t st, int *err)
+                            CnnSumList &sums, cudaStream_t st, int *err)
 {
-    if (S == 1) return launch_wgrad_umma<1>(in, H, gz, B, grad, part, st, err);
-    if (S == 2) return launch_wgrad_umma<2>(in, H, gz, B, grad, part, st, err);
+    if (S == 1) return launch_wgrad_umma<1>(in, H, gz, B, grad, part, sums, st, err);
+    if (S == 2) return launch_wgrad_umma<2>(in, H, gz, B, grad, part, sums, st, err);
     return reg_internal_fail(REG_EINVAL, "tcgen05 weight gradient: stride must be 1 or 2");
 }
 
-void cnn_sum_records(const float *part, int nrec, int rec, float *grad, cudaStream_t st)
+void cnn_sum_records(const CnnSumList &list, cudaStream_t st)
 {
-    k_sum_records<<<(rec + 31) / 32, 1024, 0, st>>>(part, nrec, rec, grad);
+    if (list.n > 0) k_sum_records<<<list.blocks, 512, 0, st>>>(list);
 }
 
 int cnn_wgrad32_umma_part_floats()
