@@ -682,7 +682,7 @@ __host__ __device__ constexpr int staged_cols()
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(128) k_conv_umma_staged(const float *__restrict__ in, int H,
+__global__ void __launch_bounds__(128, MODE == ST_DGRAD1 ? 5 : MODE == ST_DGRAD2 ? 2 : 8) k_conv_umma_staged(const float *__restrict__ in, int H,
                                                           const uint32_t *__restrict__ wpack,
                                                           const float *__restrict__ bias_g,
                                                           const uint4 *__restrict__ mask, void *__restrict__ out,
@@ -713,29 +713,50 @@ __global__ void __launch_bounds__(128) k_conv_umma_staged(const float *__restric
             constexpr int C = L0 ? 2 : UC;
             const float *img = in + (int64_t)b * C * H * H;
             const int64_t plane = (int64_t)H * H;
+            // A thread's loads of the tile are all issued before its first store.
             if (L0) {
                 // halo columns ix0 + 2 j (copy 0) and ix0 + 1 + 2 j (copy 1), j < 9
-                for (int i = tid; i < 2 * HL::rows * HL::cols; i += 128) {
-                    const int j = i % HL::cols, r3 = i / HL::cols, iy = r3 % HL::rows, par = r3 / HL::rows;
+                constexpr int ITEMS = 2 * HL::rows * HL::cols, NI = (ITEMS + 127) / 128;
+                float v[NI][2];
+#pragma unroll
+                for (int k = 0; k < NI; k++) {
+                    const int i = tid + 128 * k, j = i % HL::cols, r3 = i / HL::cols, iy = r3 % HL::rows,
+                              par = r3 / HL::rows;
                     const int gy = iy0 + iy, gxx = ix0 + par + 2 * j;
-                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                    if (gy >= 0 && gy < H && gxx >= 0 && gxx < H) {
-                        const float *p = img + (int64_t)gy * H + gxx;
-                        v.x = pack2(p[0], p[plane]);
-                    }
-                    *reinterpret_cast<uint4 *>(hbuf + par * HL::copy_stride + (iy * HL::cols + j) * 16) = v;
+                    const bool in_img = i < ITEMS && gy >= 0 && gy < H && gxx >= 0 && gxx < H;
+                    const float *p = img + (int64_t)gy * H + gxx;
+#pragma unroll
+                    for (int c = 0; c < 2; c++) v[k][c] = in_img ? p[c * plane] : 0.f;
+                }
+#pragma unroll
+                for (int k = 0; k < NI; k++) {
+                    const int i = tid + 128 * k, j = i % HL::cols, r3 = i / HL::cols, iy = r3 % HL::rows,
+                              par = r3 / HL::rows;
+                    if (i < ITEMS)
+                        *reinterpret_cast<uint4 *>(hbuf + par * HL::copy_stride + (iy * HL::cols + j) * 16) =
+                            make_uint4(pack2(v[k][0], v[k][1]), 0u, 0u, 0u);
                 }
             } else {
-                for (int i = tid; i < 4 * HL::rows * HL::cols; i += 128) {
-                    const int ix = i % HL::cols, r3 = i / HL::cols, iy = r3 % HL::rows, cg = r3 / HL::rows;
+                constexpr int ITEMS = 4 * HL::rows * HL::cols, NI = (ITEMS + 127) / 128;
+                float v[NI][8];
+#pragma unroll
+                for (int k = 0; k < NI; k++) {
+                    const int i = tid + 128 * k, ix = i % HL::cols, r3 = i / HL::cols, iy = r3 % HL::rows,
+                              cg = r3 / HL::rows;
                     const int gy = iy0 + iy, gxx = ix0 + ix;
-                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                    if (gy >= 0 && gy < H && gxx >= 0 && gxx < H) {
-                        const float *p = img + (int64_t)(8 * cg) * plane + (int64_t)gy * H + gxx;
-                        v = make_uint4(pack2(p[0], p[plane]), pack2(p[2 * plane], p[3 * plane]),
-                                       pack2(p[4 * plane], p[5 * plane]), pack2(p[6 * plane], p[7 * plane]));
-                    }
-                    *reinterpret_cast<uint4 *>(hbuf + cg * HL::cg_bytes + (iy * HL::cols + ix) * 16) = v;
+                    const bool in_img = i < ITEMS && gy >= 0 && gy < H && gxx >= 0 && gxx < H;
+                    const float *p = img + (int64_t)(8 * cg) * plane + (int64_t)gy * H + gxx;
+#pragma unroll
+                    for (int c = 0; c < 8; c++) v[k][c] = in_img ? p[c * plane] : 0.f;
+                }
+#pragma unroll
+                for (int k = 0; k < NI; k++) {
+                    const int i = tid + 128 * k, ix = i % HL::cols, r3 = i / HL::cols, iy = r3 % HL::rows,
+                              cg = r3 / HL::rows;
+                    if (i < ITEMS)
+                        *reinterpret_cast<uint4 *>(hbuf + cg * HL::cg_bytes + (iy * HL::cols + ix) * 16) =
+                            make_uint4(pack2(v[k][0], v[k][1]), pack2(v[k][2], v[k][3]), pack2(v[k][4], v[k][5]),
+                                       pack2(v[k][6], v[k][7]));
                 }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
