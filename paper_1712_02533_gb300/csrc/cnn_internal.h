@@ -19,7 +19,7 @@ int cnn_max_batch(const reg_cnn *h);
 //
 // The partial records of the layers' weight and bias gradients, added by one
 // launch at the end of a backward pass: grad[e] = the sum of entry e < rec of nrec
-// records part[record][rec] (rec even; fixed order); tap_major: entry (tap 32 + c) 32 + o of
+// records part[record][rec] (rec even; fixed order); tap_major: entry (tap 32 + o) 32 + c of
 // a 32 -> 32 layer goes to (o 32 + c) 9 + tap.
 struct CnnSumSeg {
     const float *part;

@@ -836,40 +836,49 @@ __global__ void __launch_bounds__(128, MODE == ST_DGRAD1 ? 5 : MODE == ST_DGRAD2
 // the sum over all output pixels p = (y, x) of the batch, as GEMMs with the
 // pixels as the reduction: for every output row y of a tile of WG_TH x WG_TW
 // pixels and every dy, one MMA with K = the row's 16 pixels,
-//   D_dy[o][(dx, c)] += A[o][k] B_dy[(dx, c)][k],   M = 128, N = 96,
-// A = the output gradient (BF16; rows 32..127 read padding, so lanes 32..127
-// of D are unused), B_dy = the input row S y + dy at the columns S x + dx - 1.
+//   D_dy[(dx, c)][o] += B_dy[(dx, c)][k] A[o][k],   M = 128, N = 32,
+// A = the output gradient (BF16), B_dy = the input row S y + dy at the columns
+// S x + dx - 1, (dx, c) along M (rows 96..127 read whatever follows in shared
+// memory; lanes 96..127 of D are unused), so that three quarters of the M lanes
+// work and an MMA has 32 columns: with the gradient along M (a quarter of the
+// lanes, 96 columns) a tile's 24 MMAs bounded the kernel, and its accumulators took
+// all TMEM columns: one CTA per SM, 22.2 us per launch (32 x 64^2 output pixels),
+// against 17.9.
 // Both operands are K-major core matrices staged by the CTA's threads:
-//   A: [tile row][k half][8-channel group of o][8 o x 8 pixels], 1536 B of
-//      padding after it for the unused rows;
+//   A: [tile row][k half][8-channel group of o][8 o x 8 pixels];
 //   B: [dx, 8-channel group of c][input row of the tile][k half][8 c x 8
 //      pixels], one copy per dx (so that every MMA reads 16-byte aligned core
 //      matrices), from the planar BF16 input.
-// The three accumulators D_0, D_1, D_2 take TMEM columns 0, 96 and 192, so
-// column 32 (3 dy + dx) + c holds tap (dy, dx) of channel c.  The CTA walks
+// The three accumulators D_0, D_1, D_2 take TMEM columns 0, 32 and 64, so
+// column 32 dy + o of lane 32 dx + c holds tap (dy, dx).  The CTA walks
 // its tiles (tile = block + k grid) with two staging buffers, so that the MMAs
-// of one tile run while the next is staged; the bias sums (of the unrounded
-// FP32 gradient) are formed from the staging registers.  Each CTA writes one
-// record (entry (tap 32 + c) 32 + o, then the 32 biases); cnn_sum_records adds the
-// records into the parameter layout.
-constexpr int WG_TH = 8, WG_TW = 16, WG_N = 96, WG_COLS = 512;
+// of one tile run while the next is staged: 8 staging warps load, round and
+// store, a ninth issues.  The bias sums (of the unrounded FP32 gradient) are
+// formed from the staging registers.  Each CTA writes one record (entry
+// (tap 32 + o) 32 + c, then the 32 biases); cnn_sum_records adds the records into
+// the parameter layout.
+constexpr int WG_TH = 8, WG_TW = 16, WG_N = 32, WG_COLS = 128;
 constexpr int WG_REC = UC * UC * 9 + UC;
+constexpr int WG_THREADS = 288;  // 8 staging warps and the issuing one
+constexpr int WG_CTAS = 2;       // per SM, at most (stride 2: one, by shared memory)
 
 template <int S>
 struct WgSmem {
     static constexpr int ir = S * (WG_TH - 1) + 3;      // input rows of a tile
-    static constexpr int a_bytes = WG_TH * 1024 + 1536;  // 8 rows x 2 halves x 4 groups x 128 B + padding
+    static constexpr int a_bytes = WG_TH * 1024;         // 8 rows x 2 halves x 4 groups x 128 B
     static constexpr int b_bytes = 12 * ir * 256;        // 12 groups x rows x 2 halves x 128 B
-    static constexpr int a0 = 0, b0 = 2 * a_bytes;
-    static constexpr int bars = b0 + 2 * b_bytes;        // MMA done, per buffer
+    static constexpr int b0 = 0, a0 = 2 * b_bytes;
+    static constexpr int bars = a0 + 2 * a_bytes;        // MMA done, per buffer
     static constexpr int taddr = bars + 16;
     static constexpr int red = taddr + 16;               // bias sums: [warp][8 o][4 groups]
-    static constexpr int bytes = red + 8 * 8 * 4 * 4;
+    static constexpr int end = red + 8 * 8 * 4 * 4;
+    static constexpr int m_end = b_bytes + 16 * ir * 256;  // what the 128 rows of the second buffer's MMAs read
+    static constexpr int bytes = end > m_end ? end : m_end;
     static_assert(a_bytes % 128 == 0 && b_bytes % 128 == 0, "core matrices 16-byte aligned");
 };
 
 template <int S>
-__global__ void __launch_bounds__(256, 1) k_wgrad32_umma(const uint4 *__restrict__ in, int H,
+__global__ void __launch_bounds__(WG_THREADS, S == 1 ? WG_CTAS : 1) k_wgrad32_umma(const uint4 *__restrict__ in, int H,
                                                          const float *__restrict__ gz, int Ho, int tiles_x,
                                                          int tiles_y, int n_tiles, float *__restrict__ part,
                                                          int *__restrict__ err)
@@ -898,94 +907,101 @@ __global__ void __launch_bounds__(256, 1) k_wgrad32_umma(const uint4 *__restrict
     // stores), then k half, tile row and group og = o / 8 (= slot k / 2)
     const int a_jp = tid & 3, a_r = (tid >> 2) & 7;
     float bsum[4] = {0.f, 0.f, 0.f, 0.f};
+    const bool pairs = Ho % 2 == 0;  // the gradient's pixel pairs 8-byte aligned
     int bad = 0, it = 0;
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
         const int buf = it & 1;
-        int b, ty, tx;
-        tile_coords(tile, tiles_x, tiles_y, b, ty, tx);
-        const int oy0 = ty * WG_TH, ox0 = tx * WG_TW;
-        // the gradient's and the input's values of this tile, loaded before
-        // the buffer is free
-        float2 av[8];
+        bool ok = true;
+        if (warp < 8) {
+            int b, ty, tx;
+            tile_coords(tile, tiles_x, tiles_y, b, ty, tx);
+            const int oy0 = ty * WG_TH, ox0 = tx * WG_TW;
+            // the gradient's and the input's values of this tile, loaded before
+            // the buffer is free
+            float2 av[8];
 #pragma unroll
-        for (int k = 0; k < 8; k++) {
-            const int item = tid + 256 * k, kap = (item >> 5) & 1, y = (item >> 6) & 7, o = 8 * (item >> 9) + a_r;
-            const int oy = oy0 + y, ox = ox0 + 8 * kap + 2 * a_jp;
-            float2 v = make_float2(0.f, 0.f);
-            if (oy < Ho) {
-                const float *row = gz + (((int64_t)b * UC + o) * Ho + oy) * Ho;
-                if (ox < Ho) v.x = row[ox];
-                if (ox + 1 < Ho) v.y = row[ox + 1];
+            for (int k = 0; k < 8; k++) {
+                const int item = tid + 256 * k, kap = (item >> 5) & 1, y = (item >> 6) & 7, o = 8 * (item >> 9) + a_r;
+                const int oy = oy0 + y, ox = ox0 + 8 * kap + 2 * a_jp;
+                float2 v = make_float2(0.f, 0.f);
+                if (oy < Ho) {
+                    const float *row = gz + (((int64_t)b * UC + o) * Ho + oy) * Ho;
+                    if (pairs) {
+                        if (ox < Ho) v = *reinterpret_cast<const float2 *>(row + ox);
+                    } else {
+                        if (ox < Ho) v.x = row[ox];
+                        if (ox + 1 < Ho) v.y = row[ox + 1];
+                    }
+                }
+                av[k] = v;
             }
-            av[k] = v;
-        }
-        uint4 q0[NB], q1[NB];
+            uint4 q0[NB], q1[NB];
 #pragma unroll
-        for (int k = 0; k < NB; k++) {
-            const int item = tid + 256 * k, jp = item & 3, kap = (item >> 2) & 1, r2 = item >> 3;
-            const int ir = r2 % IR, g = r2 / IR, dx = g >> 2, cg = g & 3;
-            const int iy = S * oy0 - 1 + ir, x = ox0 + 8 * kap + 2 * jp;
-            const int ix0 = S * x + dx - 1, ix1 = S * (x + 1) + dx - 1;
-            q0[k] = q1[k] = make_uint4(0u, 0u, 0u, 0u);
-            if (item < 96 * IR && iy >= 0 && iy < H) {
-                const uint4 *row = in + ((int64_t)(4 * b + cg) * H + iy) * H;
-                if (ix0 >= 0 && ix0 < H) q0[k] = row[ix0];
-                if (ix1 >= 0 && ix1 < H) q1[k] = row[ix1];
+            for (int k = 0; k < NB; k++) {
+                const int item = tid + 256 * k, jp = item & 3, kap = (item >> 2) & 1, r2 = item >> 3;
+                const int ir = r2 % IR, g = r2 / IR, dx = g >> 2, cg = g & 3;
+                const int iy = S * oy0 - 1 + ir, x = ox0 + 8 * kap + 2 * jp;
+                const int ix0 = S * x + dx - 1, ix1 = S * (x + 1) + dx - 1;
+                q0[k] = q1[k] = make_uint4(0u, 0u, 0u, 0u);
+                if (item < 96 * IR && iy >= 0 && iy < H) {
+                    const uint4 *row = in + ((int64_t)(4 * b + cg) * H + iy) * H;
+                    if (ix0 >= 0 && ix0 < H) q0[k] = row[ix0];
+                    if (ix1 >= 0 && ix1 < H) q1[k] = row[ix1];
+                }
             }
-        }
-        if (it >= 2) {
-            // the MMAs of tile it - 2 have read this buffer
-            const bool ok = bad ? true : mbar_wait(bar_mma + 8 * buf, ((it - 2) >> 1) & 1);
-            if (!ok) *reinterpret_cast<volatile int *>(err) = 3;
-            bad = __syncthreads_or(!ok || bad);
-            if (bad) break;
-        }
-        uint8_t *abuf = smem + SM::a0 + buf * SM::a_bytes;
-#pragma unroll
-        for (int k = 0; k < 8; k++) {
-            const int item = tid + 256 * k, kap = (item >> 5) & 1, y = (item >> 6) & 7, og = item >> 9;
-            bsum[k >> 1] += av[k].x + av[k].y;
-            *reinterpret_cast<uint32_t *>(abuf + ((y * 2 + kap) * 4 + og) * 128 + a_r * 16 + a_jp * 4) =
-                pack2(av[k].x, av[k].y);
-        }
-        uint8_t *bbuf = smem + SM::b0 + buf * SM::b_bytes;
-#pragma unroll
-        for (int k = 0; k < NB; k++) {
-            const int item = tid + 256 * k, jp = item & 3, kap = (item >> 2) & 1, r2 = item >> 3;
-            if (item >= 96 * IR) continue;
-            const int ir = r2 % IR, g = r2 / IR;
-            uint8_t *cm = bbuf + ((g * IR + ir) * 2 + kap) * 128 + jp * 4;
-            const uint32_t w0[4] = {q0[k].x, q0[k].y, q0[k].z, q0[k].w}, w1[4] = {q1[k].x, q1[k].y, q1[k].z, q1[k].w};
-            // wd[c]: channel c of the two pixels (row c of the core matrix)
-            uint32_t wd[8];
-#pragma unroll
-            for (int c = 0; c < 8; c++) wd[c] = __byte_perm(w0[c >> 1], w1[c >> 1], (c & 1) ? 0x7632 : 0x5410);
-            // rotated by the lane group (rot = lane / 4), so that the 8 lane
-            // groups of a store instruction write 8 different rows: 32 banks
-            const int rot = lane >> 2;
-#pragma unroll
-            for (int sh = 1; sh < 8; sh <<= 1) {
-                uint32_t t[8];
-#pragma unroll
-                for (int i = 0; i < 8; i++) t[i] = (rot & sh) ? wd[(i + sh) & 7] : wd[i];
-#pragma unroll
-                for (int i = 0; i < 8; i++) wd[i] = t[i];
+            if (it >= 2) {
+                // the MMAs of tile it - 2 have read this buffer
+                ok = mbar_wait(bar_mma + 8 * buf, ((it - 2) >> 1) & 1);
+                if (!ok) *reinterpret_cast<volatile int *>(err) = 3;
             }
+            uint8_t *abuf = smem + SM::a0 + buf * SM::a_bytes;
 #pragma unroll
-            for (int i = 0; i < 8; i++) *reinterpret_cast<uint32_t *>(cm + ((i + rot) & 7) * 16) = wd[i];
+            for (int k = 0; k < 8; k++) {
+                const int item = tid + 256 * k, kap = (item >> 5) & 1, y = (item >> 6) & 7, og = item >> 9;
+                bsum[k >> 1] += av[k].x + av[k].y;
+                *reinterpret_cast<uint32_t *>(abuf + ((y * 2 + kap) * 4 + og) * 128 + a_r * 16 + a_jp * 4) =
+                    pack2(av[k].x, av[k].y);
+            }
+            uint8_t *bbuf = smem + SM::b0 + buf * SM::b_bytes;
+#pragma unroll
+            for (int k = 0; k < NB; k++) {
+                const int item = tid + 256 * k, jp = item & 3, kap = (item >> 2) & 1, r2 = item >> 3;
+                if (item >= 96 * IR) continue;
+                const int ir = r2 % IR, g = r2 / IR;
+                uint8_t *cm = bbuf + ((g * IR + ir) * 2 + kap) * 128 + jp * 4;
+                const uint32_t w0[4] = {q0[k].x, q0[k].y, q0[k].z, q0[k].w}, w1[4] = {q1[k].x, q1[k].y, q1[k].z, q1[k].w};
+                // wd[c]: channel c of the two pixels (row c of the core matrix)
+                uint32_t wd[8];
+#pragma unroll
+                for (int c = 0; c < 8; c++) wd[c] = __byte_perm(w0[c >> 1], w1[c >> 1], (c & 1) ? 0x7632 : 0x5410);
+                // rotated by the lane group (rot = lane / 4), so that the 8 lane
+                // groups of a store instruction write 8 different rows: 32 banks
+                const int rot = lane >> 2;
+#pragma unroll
+                for (int sh = 1; sh < 8; sh <<= 1) {
+                    uint32_t t[8];
+#pragma unroll
+                    for (int i = 0; i < 8; i++) t[i] = (rot & sh) ? wd[(i + sh) & 7] : wd[i];
+#pragma unroll
+                    for (int i = 0; i < 8; i++) wd[i] = t[i];
+                }
+#pragma unroll
+                for (int i = 0; i < 8; i++) *reinterpret_cast<uint32_t *>(cm + ((i + rot) & 7) * 16) = wd[i];
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
-        __syncthreads();
-        if (tid == 0) {
+        bad = __syncthreads_or(!ok);
+        if (bad) break;
+        if (tid == 256) {
             tc_fence_after();
             const uint32_t abase = s_base + SM::a0 + buf * SM::a_bytes, bbase = s_base + SM::b0 + buf * SM::b_bytes;
 #pragma unroll 1
             for (int y = 0; y < WG_TH; y++)
 #pragma unroll
                 for (int dy = 0; dy < 3; dy++)
-                    umma_bf16<WG_N>(tmem + WG_N * dy, sdesc(abase + y * 1024, 512, 128),
-                                    sdesc(bbase + (S * y + dy) * 256, 128, IR * 256), (it > 0 || y > 0) ? 1u : 0u);
+                    umma_bf16<WG_N>(tmem + WG_N * dy, sdesc(bbase + (S * y + dy) * 256, 128, IR * 256),
+                                    sdesc(abase + y * 1024, 512, 128), (it > 0 || y > 0) ? 1u : 0u);
             umma_commit(bar_mma + 8 * buf);
         }
     }
@@ -997,22 +1013,19 @@ __global__ void __launch_bounds__(256, 1) k_wgrad32_umma(const uint4 *__restrict
         bad = __syncthreads_or(!ok);
     }
     float *rec = part + (int64_t)blockIdx.x * WG_REC;
-    if ((warp & 3) == 0) {
-        // lane o of the accumulators (warps 0 and 4 read the lanes 0..31): column
-        // 32 (3 dy + dx) + c = tap (dy, dx), channel c.  A store instruction writes
-        // the 32 output channels of one entry: one line, where the parameter
-        // layout's (o 32 + c) 9 + tap took 32 sectors of 32 lines and the other
-        // warps waited for it: 31 -> 22.4 us per launch (32 x 64^2 output pixels).
+    if (warp < 3) {
+        // lane c of warp dx's accumulator lanes: column 32 dy + o = tap (dy, dx).  A
+        // store instruction writes the 32 input channels of one entry: one line.
         tc_fence_after();
 #pragma unroll 1
-        for (int tap = warp >> 2; tap < 9; tap += 2) {
+        for (int dy = 0; dy < 3; dy++) {
             float v[UC];
-            if (!bad && it > 0) tmem_ld<UC>(tmem + 32 * tap, v);
+            if (!bad && it > 0) tmem_ld<UC>(tmem + ((uint32_t)(32 * warp) << 16) + WG_N * dy, v);
             else
 #pragma unroll
-                for (int c = 0; c < UC; c++) v[c] = 0.f;
+                for (int o = 0; o < UC; o++) v[o] = 0.f;
 #pragma unroll
-            for (int c = 0; c < UC; c++) rec[(tap * UC + c) * UC + lane] = v[c];
+            for (int o = 0; o < UC; o++) rec[((3 * dy + warp) * UC + o) * UC + lane] = v[o];
         }
     }
     // bias: the four lanes of a pixel-pair group, then the eight warps
@@ -1022,7 +1035,7 @@ __global__ void __launch_bounds__(256, 1) k_wgrad32_umma(const uint4 *__restrict
         float v = bsum[g];
         v += __shfl_xor_sync(0xffffffffu, v, 1);
         v += __shfl_xor_sync(0xffffffffu, v, 2);
-        if (a_jp == 0) red[(warp * 8 + a_r) * 4 + g] = v;
+        if (warp < 8 && a_jp == 0) red[(warp * 8 + a_r) * 4 + g] = v;
     }
     __syncthreads();
     if (tid < UC) {
@@ -1068,7 +1081,7 @@ __global__ void __launch_bounds__(512) k_sum_records(const __grid_constant__ Cnn
         for (int j = 0; j < 2; j++) {
             const int i = e + j;
             const bool perm = sg.tap_major && i < UC * UC * 9;
-            sg.grad[perm ? ((i & 31) * UC + ((i >> 5) & 31)) * 9 + (i >> 10) : i] = tot[j];
+            sg.grad[perm ? (((i >> 5) & 31) * UC + (i & 31)) * 9 + (i >> 10) : i] = tot[j];
         }
     }
 }
@@ -1244,7 +1257,8 @@ reg_status launch_wgrad_umma(const uint16_t *in, int H, const float *gz, int B, 
     int grid = 0;
     if (!grid_for(k_wgrad32_umma<S>, WgSmem<S>::bytes, WG_COLS, nt, grid))
         return reg_internal_fail(REG_ECUDA, "tcgen05 weight gradient: launch attributes");
-    k_wgrad32_umma<S><<<grid, 256, WgSmem<S>::bytes, st>>>(reinterpret_cast<const uint4 *>(in), H, gz, Ho, tx, ty, nt,
+    static_assert(3 * WgSmem<1>::bytes > 228 * 1024, "two CTAs per SM: WG_CTAS records of each SM in part");
+    k_wgrad32_umma<S><<<grid, WG_THREADS, WgSmem<S>::bytes, st>>>(reinterpret_cast<const uint4 *>(in), H, gz, Ho, tx, ty, nt,
                                                           part, err);
     sums.add(part, grid, WG_REC, grad, true);
     if (cudaGetLastError() != cudaSuccess) return reg_internal_fail(REG_ECUDA, "tcgen05 weight gradient launch");
@@ -1271,7 +1285,7 @@ int cnn_wgrad32_umma_part_floats()
     int dev = 0, nsm = 152;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         nsm = 152;
-    return nsm * WG_REC;
+    return WG_CTAS * nsm * WG_REC;
 }
 
 int cnn_last_umma_words() { return Wts<16>::bytes / 4; }

@@ -313,3 +313,32 @@ def test_fp32_gradient_at_ragged_sides(reg, syn, side, batch):
     grad = torch.autograd.grad(want, th)[0].numpy()
     assert abs(loss - float(want.detach())) <= 1e-5 * float(want.detach())
     assert np.abs(got - grad).max() <= 1e-5 * np.abs(grad).max()
+
+
+@pytest.mark.parametrize("tensor_cores", [False, True])
+@pytest.mark.parametrize("side,batch", [(256, 32), (100, 128)])
+def test_batch_gradient_is_the_mean_of_its_pairs(reg, syn, side, batch, tensor_cores):
+    """The loss is a mean over the batch, so its gradient is the mean of the
+    pairs' own.  A pair alone gives every block at most a tile or two; the batch
+    makes each walk several (three and more of the tensor-core weight gradient's,
+    whose staging buffers are then reused), with the gradient's rows 16-byte
+    aligned (side 256) and not (side 100: 50 and 25 columns).  The batch sizes
+    are powers of two, so the pairs' output gradients differ from the batch's by
+    an exact factor, BF16 operands round alike, and only the order of the FP32
+    sums differs: chains of at most some 300 terms, 300 * 2^-24 = 2e-5 of the
+    sums' size at worst, under 1e-4 of the layer's largest gradient."""
+    import torch
+    from oracle import cnn as ocnn
+    theta = syn.cnn_params(11)
+    g = torch.Generator(device="cuda").manual_seed(side)
+    x = torch.randn((batch, 2, side, side), generator=g, device="cuda")
+    t = torch.randn((batch, 2, side // 4, side // 4), generator=g, device="cuda")
+    with reg.Cnn(theta, side=side, max_batch=batch) as net:
+        loss, got = net.loss_grad(x, t, want_grad=True, tensor_cores=tensor_cores)
+        one = [net.loss_grad(x[i:i + 1].contiguous(), t[i:i + 1].contiguous(), want_grad=True,
+                             tensor_cores=tensor_cores) for i in range(batch)]
+    ref = np.mean([o[1].astype(np.float64) for o in one], axis=0)
+    assert abs(loss - np.mean([o[0] for o in one])) <= 1e-6 * loss
+    for k, ((gw, gb), (rw, rb)) in enumerate(zip(ocnn.unpack(got.astype(np.float64)), ocnn.unpack(ref))):
+        assert np.abs(gw - rw).max() <= 1e-4 * np.abs(rw).max(), k
+        assert np.abs(gb - rb).max() <= 1e-4 * np.abs(rb).max(), k
