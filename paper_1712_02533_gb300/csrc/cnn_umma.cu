@@ -1046,37 +1046,52 @@ __global__ void __launch_bounds__(WG_THREADS, S == 1 ? WG_CTAS : 1) k_wgrad32_um
     umma_teardown<WG_COLS>(tmem);
 }
 
+// s + lo += v, the addition's rounding error kept in lo.
+__device__ __forceinline__ void comp_add(float &s, float &lo, float v)
+{
+    const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+    lo += __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z));
+    s = t;
+}
+
 // The layers' weight and bias gradients from their records, one launch for all
 // layers: block b works in the last layer of the list with block0 <= b, on 32
 // adjacent pairs of entries (a warp's lanes; records are of even length), 16 groups
-// of records side by side, the groups added in order: one wave of blocks.  One launch per layer took 5.8 us
-// for each 32 -> 32 layer and 4.7 for the others (32 us a pass of 32 x 256^2), a
-// launch's own length more than its 5.6 MB.
+// of records side by side, the groups added in order: one wave of blocks.  The
+// records are read at the memory's rate, so the sums carry their rounding errors
+// along.  One launch per layer took 5.8 us for each 32 -> 32 layer and 4.7 for the
+// others (32 us a pass of 32 x 256^2), a launch's own length more than its 5.6 MB;
+// now 9 us.
 __global__ void __launch_bounds__(512) k_sum_records(const __grid_constant__ CnnSumList list)
 {
-    __shared__ float2 red[16][32];
+    __shared__ float2 red[16][32], rlo[16][32];
     int q = 0;
     while (q + 1 < list.n && (int)blockIdx.x >= list.s[q + 1].block0) q++;
     const CnnSumSeg sg = list.s[q];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, e = ((int)blockIdx.x - sg.block0) * 64 + 2 * lane;
-    float2 s = make_float2(0.f, 0.f);
+    float2 s = make_float2(0.f, 0.f), lo = s;
     if (e < sg.rec) {
 #pragma unroll 8
         for (int k = g; k < sg.nrec; k += 16) {
             const float2 v = *reinterpret_cast<const float2 *>(sg.part + (int64_t)k * sg.rec + e);
-            s.x += v.x;
-            s.y += v.y;
+            comp_add(s.x, lo.x, v.x);
+            comp_add(s.y, lo.y, v.y);
         }
     }
     red[g][lane] = s;
+    rlo[g][lane] = lo;
     __syncthreads();
     if (g == 0 && e < sg.rec) {
-        float tot[2] = {0.f, 0.f};
+        float tot[2] = {0.f, 0.f}, tl[2] = {0.f, 0.f};
 #pragma unroll
         for (int w = 0; w < 16; w++) {
-            tot[0] += red[w][lane].x;
-            tot[1] += red[w][lane].y;
+            comp_add(tot[0], tl[0], red[w][lane].x);
+            comp_add(tot[1], tl[1], red[w][lane].y);
+            tl[0] += rlo[w][lane].x;
+            tl[1] += rlo[w][lane].y;
         }
+#pragma unroll
+        for (int j = 0; j < 2; j++) tot[j] += tl[j] == tl[j] ? tl[j] : 0.f;  // (NaN: the sum is infinite or NaN itself)
 #pragma unroll
         for (int j = 0; j < 2; j++) {
             const int i = e + j;

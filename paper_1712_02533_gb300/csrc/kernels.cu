@@ -2656,7 +2656,7 @@ __global__ void __launch_bounds__(256) k_rigid_eval(const RigidLevel *__restrict
 // Per operator: the tiles' partial sums in a fixed order (one block per op): warp by
 // warp of 32 tiles, then the warps' sums in order, up to 256 tiles; beyond, a lane
 // first adds every 256th.  Each warp takes (sum, group of 32 tiles) pairs of the sums
-// this round asked for; one sum after the other through the whole block took 21 us.
+// the request asks for; one sum after the other through the whole block took 21 us.
 __global__ void __launch_bounds__(1024) k_rigid_reduce(const double *__restrict__ part, int tiles_stride,
                                                        const RigidLevel *__restrict__ lv,
                                                        const RigidReq *__restrict__ req, double *__restrict__ sums)
