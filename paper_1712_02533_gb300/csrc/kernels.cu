@@ -739,7 +739,7 @@ __global__ void __launch_bounds__(256) k_final(BatchDev b)
 // length; the rows' terms of the two sums go through shared memory and are added
 // in row order, so that both forms give the same sums.  Per launch of a single 1024^2
 // operator 14.5 -> 8 us, of 7 operators of 64^2 8.2 -> 4.9, of a 21 x 512^2 scan 20 ->
-// 14; of a 33 x 1024^2 scan 67 us as it is, 83 us with tiles shared.
+// 14; of a 33 x 1024^2 scan 67 us as it was (57 now), 83 us with tiles shared.
 constexpr int GRAD_WARPS = REG_STRIP_THREADS / 32;
 template <bool BF16, bool FEW>
 __global__ void __launch_bounds__(REG_STRIP_THREADS, FEW ? 6 : 8) k_grad(BatchDev b)
