@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "reg_common.cuh"
+#include "tile_rows.h"
 
 namespace {
 
@@ -757,8 +758,9 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, FEW ? 6 : 8) k_grad(BatchDe
         const int n = s.n, pitch = s.pitch, ntx = (n + REG_GW - 1) / REG_GW, h = s.hg;
         const int part = s.part0 + t;
         const int tile0 = (t / ntx) * h, c = (t % ntx) * REG_GW - 1 + lane;
-        const int r0 = FEW ? tile0 + (threadIdx.x >> 5) * (h / GRAD_WARPS) : tile0;  // (h is 4, 8, .. 64)
-        const int rLast = min(r0 + (FEW ? h / GRAD_WARPS : h) - 1, n - 1);
+        // (h is 4, 8, .. 64; in the last row of tiles of the FEW form warps 1 .. 3 have no rows)
+        const GradRows g = grad_rows(tile0, h, n, FEW ? (int)(threadIdx.x >> 5) : 0, FEW ? GRAD_WARPS : 1);
+        const int r0 = g.r0;
         const bool colIn = c >= 0 && c < n;
         const bool own = colIn && lane >= 1 && lane <= REG_GW;
         const bool cEdge = (c == 0 || c == n - 1);
@@ -781,19 +783,19 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, FEW ? 6 : 8) k_grad(BatchDe
         float4 nu = make_float4(0.f, 0.f, 0.f, 0.f);
         float2 nd = make_float2(0.f, 0.f);
         float nmr = 0.f;
-        if (colIn && r0 - 1 >= 0) {
-            const int idx = (r0 - 1) * pitch + c;
+        if (colIn && grad_loads(g, g.first, n)) {
+            const int idx = g.first * pitch + c;
             const float4 *rec = reinterpret_cast<const float4 *>(s.Vs + idx);
             nu = rec[0];
             nd = *reinterpret_cast<const float2 *>(rec + 1);
             nmr = s.MR[idx];
         }
-        for (int r = r0 - 1; r <= rLast + 1; r++) {
+        for (int r = g.first; r <= g.last; r++) {
             const bool in = colIn && r >= 0 && r < n;
             float4 u = nu;
             const float2 dp = make_float2(nd.x, nd.y);
             const float mr = nmr;
-            if (colIn && r + 1 < n && r + 1 <= rLast + 1) {
+            if (colIn && grad_loads(g, r + 1, n)) {
                 const int idx = (r + 1) * pitch + c;
                 const float4 *rec = reinterpret_cast<const float4 *>(s.Vs + idx);
                 nu = rec[0];
