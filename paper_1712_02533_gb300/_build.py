@@ -14,7 +14,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libreg.so")
 
 SOURCES = ["kernels.cu", "engine.cu", "schedule.cpp", "noalloc.cu", "cnn.cu", "cnn_umma.cu"]
-HEADERS = ["reg_common.cuh", "schedule.h", "cnn_internal.h", "tile_rows.h"]
+HEADERS = ["reg_common.cuh", "schedule.h", "cnn_internal.h", "tile_rows.h", "arith.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

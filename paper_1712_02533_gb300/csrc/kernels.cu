@@ -2431,12 +2431,12 @@ __global__ void __launch_bounds__(REG_CTL_THREADS) k_control(BatchDev b)
 // units of the finest level; null = the identity), as sums in double give it.
 // Three FP64 operations per sample and the division (16 cycles of an SM each for a
 // warp) took 345 of the 415 us for 64 frames of 1025^2, so the products, their sum
-// and its product with 1/m run in float pairs (to 2^-43 of the terms' sum; the
-// means' sum and 1/m are two constants of the block); a node whose rounding that
-// does not settle, about one in 10^5, is summed again in FP64.  A call for 64 frames
-// takes 276 us (443 with FP64 sums, 308 with the end of a node in FP64: two
-// divisions), for 3 frames in BF16 47 us (67, 93); bound by issue and the latency of
-// field -> texel chains.
+// and its product with 1/m run in float pairs (PairSum, whose bound grows with the
+// number of frames; the means' sum and 1/m are two constants of the block); a node
+// whose rounding that does not settle, one in 10^4 at 64 frames, is summed again in
+// FP64 by its warp.  A call for 64 frames takes 258 us (443 with FP64 sums, 308 with the
+// end of a node in FP64: two divisions); bound by issue and the latency of field ->
+// texel chains.
 constexpr int AVG_FRAMES = 128;  // frames staged in shared memory at a time
 constexpr int AVG_BATCH = 2;     // frames whose fields, then texels, a thread has in flight
 template <bool BF16>
@@ -2466,7 +2466,7 @@ __global__ void __launch_bounds__(256) k_average(const void *__restrict__ pyr, i
         const double s = 1.0 / m;
         inv_m = make_float2((float)s, (float)(s - (double)(float)s));
     }
-    float hi = 0.f, lo = 0.f, mag = 0.f;
+    PairSum sum;
     for (int k0 = 0; k0 < m; k0 += AVG_FRAMES) {
         const int mk = min(AVG_FRAMES, m - k0);
         __syncthreads();
@@ -2479,14 +2479,8 @@ __global__ void __launch_bounds__(256) k_average(const void *__restrict__ pyr, i
         }
         __syncthreads();
         if (in) {
-            auto add = [&](int k, float v) {
-                const float2 s = sig[k];
-                const float p = v * s.x, pl = fmaf(v, s.y, fmaf(v, s.x, -p));
-                float e;
-                two_sum(hi, p, hi, e);
-                lo += e + pl;
-                mag += fabsf(p);
-            };
+            static_assert(AVG_BATCH <= 2, "folded after at most two products");
+            auto add = [&](int k, float v) { sum.add(v, sig[k].x, sig[k].y); };
             for (int k = 0; k < mk; k += AVG_BATCH) {
                 float2 u[AVG_BATCH];
                 float far = 0.f;
@@ -2511,28 +2505,33 @@ __global__ void __launch_bounds__(256) k_average(const void *__restrict__ pyr, i
                     for (int q = 0; q < AVG_BATCH && k + q < mk; q++)
                         add(k + q, sample<BF16, false>(img[k + q], n, pitch, c, r, u[q].x, u[q].y, nullptr, nullptr));
                 }
+                sum.fold();
             }
         }
     }
-    if (!in) return;
-    float t, te;
-    two_sum(hi, mean_sum.x, t, te);
-    te += lo + mean_sum.y;
-    const float p = __fmul_rn(t, inv_m.x), pl = fmaf(t, inv_m.y, fmaf(te, inv_m.x, fmaf(t, inv_m.x, -p)));
-    const float size = (mag + fabsf(mean_sum.x)) * inv_m.x, tol = size * 1.1368683772161603e-13f;  // 2^-43
+    float p, pl;
+    sum.scaled(mean_sum.x, mean_sum.y, inv_m.x, inv_m.y, p, pl);
+    const float size = (sum.mag + fabsf(mean_sum.x)) * inv_m.x, tol = sum.tolerance(m, mean_sum.x, inv_m.x);
     const float a = p + (pl - tol), b = p + (pl + tol);
     float res = a;
-    if (!(a == b) || !(size > 1e-25f)) {  // (the low parts of tiny values underflow)
+    // Open nodes (the low parts of tiny values underflow: open too) in FP64, the frames
+    // over the lanes of the node's warp: one thread's chain of m gathers was 20 us for
+    // 64 frames, as long as it takes at the end of the launch.
+    unsigned open = __ballot_sync(0xffffffffu, in && (!(a == b) || !(size > 1e-25f)));
+    while (open) {
+        const int src = __ffs(open) - 1, cs = blockIdx.x * 32 + src;
+        open &= open - 1;
         double acc = 0.0;
-        for (int k = 0; k < m; k++) {
+        for (int k = threadIdx.x; k < m; k += 32) {
             const float2 *f = fields[k];
-            const float2 u = f ? f[(int64_t)r * slot_pitch + c] : make_float2(0.f, 0.f);
-            const float v = sample<BF16, false>(image(k), n, pitch, c, r, u.x, u.y, nullptr, nullptr);
+            const float2 u = f ? f[(int64_t)r * slot_pitch + cs] : make_float2(0.f, 0.f);
+            const float v = sample<BF16, false>(image(k), n, pitch, cs, r, u.x, u.y, nullptr, nullptr);
             acc += (double)v * fstats[2 * k + 1] + fstats[2 * k];
         }
-        res = (float)(acc / m);
+        acc = warp_sum_d(acc);
+        if ((int)threadIdx.x == src) res = (float)(acc / m);
     }
-    out[(int64_t)r * opitch + c] = res;
+    if (in) out[(int64_t)r * opitch + c] = res;
 }
 
 void launch_average(int bf16, cudaStream_t st, const void *pyr, int64_t frame_block, int64_t img_off, int n,

@@ -4,6 +4,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "arith.h"
+
 #define REG_MAX_LEVELS 8
 #define REG_MAX_TRIALS 8
 #define REG_CTL_THREADS 512  // threads per block of the control kernel
@@ -203,14 +205,6 @@ static inline int cdiv(int a, int b) { return (a + b - 1) / b; }
 // a level shrink to ~1e-6 grid units while |u| is several units: one float
 // cannot take such a step without rounding it by percents, so u is kept as an
 // unevaluated sum hi + lo of two floats and updated with an exact two-sum.
-// (explicitly rounded adds: the compiler must not contract them into FMAs)
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
-{
-    s = __fadd_rn(a, b);
-    float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
 // (hi + lo) + v, renormalised so that |lo| <= ulp(hi) / 2
 __device__ __forceinline__ void df_add(float &hi, float &lo, float v)
 {

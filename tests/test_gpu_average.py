@@ -72,6 +72,22 @@ def test_average_of_few_and_many_frames_matches_oracle(reg, orc, syn, nf):
     assert np.abs(got - want).max() <= 1e-5 * float(want.max() - want.min())
 
 
+def test_average_of_many_equal_frames_is_the_frame(reg, syn):
+    """The same frame 2000 times: every node's sum is 2000 equal terms of one sign, so
+    the average in double is the term itself to 1e-13 and its float the one that two
+    frames give, bit for bit."""
+    f = syn.series(45, 1, 128, peak=20.0, spacing=10.0, sigma=2.0)[0] + np.float32(50.0)
+    p = reg.default_params(n_levels=2, lam=10.0)
+
+    def average(n):
+        with reg.Series(np.repeat(f[None], n, axis=0), p) as s:
+            for k in range(1, n):
+                s.set_slot(k - 1, np.zeros((2, 129, 129), np.float32), 0, k)
+            return s.average(iterations=0)
+
+    assert np.array_equal(average(2000), average(2))
+
+
 def test_averaging_procedure_matches_oracle_on_a_stable_series(reg, orc, syn):
     """The whole procedure on the config-1 series without shot noise (the
     oracle's result is stable there): registration, average, one iteration of

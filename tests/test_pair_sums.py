@@ -1,0 +1,71 @@
+"""Float-pair arithmetic of the kernels (csrc/arith.h), compiled for the host:
+errors against the same sums in extended precision."""
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1712_02533_gb300", "csrc")
+
+AVERAGE = r"""
+#include <cmath>
+#include <cstdio>
+#include <random>
+#include "arith.h"
+// 3000 nodes averaged over m frames as the averaging kernel does it: the largest error
+// over the stated tolerance, and the nodes whose rounding stays open (those are summed
+// again in double).
+int main()
+{
+    const int m = M, mode = MODE, nodes = 3000;
+    std::mt19937 g(7);
+    std::normal_distribution<double> z(0, 1);
+    std::uniform_real_distribution<double> u(0.5, 4);
+    double worst = 0;
+    int open = 0;
+    for (int t = 0; t < nodes; t++) {
+        const double base = u(g), s0 = 5 + 3 * u(g), mean = 10 * u(g);
+        PairSum s;
+        long double exact = 0;
+        double means = 0;
+        for (int k = 0; k < m; k++) {
+            // one sign and frames that differ; the same value in every frame; both signs
+            const float v = (float)(mode == 0 ? base + 0.1 * z(g) : mode == 1 ? base : (k & 1 ? base : -base) + 1e-3 * z(g));
+            const double sigma = mode == 1 ? s0 : s0 + 0.05 * z(g);
+            const float sh = (float)sigma;
+            s.add(v, sh, (float)(sigma - (double)sh));
+            if ((k & 1) || k == m - 1) s.fold();
+            exact += (long double)v * sigma;
+            means += mean;
+        }
+        const double inv = 1.0 / m;
+        const float ch = (float)means, cl = (float)(means - (double)ch), fh = (float)inv, fl = (float)(inv - (double)fh);
+        float p, pl;
+        s.scaled(ch, cl, fh, fl, p, pl);
+        const float tol = s.tolerance(m, ch, fh);
+        worst = std::fmax(worst, (double)std::fabs((long double)p + pl - (exact + means) / m) / tol);
+        open += !(p + (pl - tol) == p + (pl + tol));
+    }
+    printf("%.9f %d\n", worst, open);
+}
+"""
+
+
+def _run(tmp_path, src):
+    (tmp_path / "t.cpp").write_text(src)
+    subprocess.run(["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-I", CSRC, str(tmp_path / "t.cpp"), "-o",
+                    str(tmp_path / "t")], check=True)
+    return subprocess.run([str(tmp_path / "t")], check=True, capture_output=True, text=True).stdout.split()
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2])
+@pytest.mark.parametrize("m", [1, 2, 3, 64, 400, 4000])
+def test_average_of_any_number_of_frames_keeps_its_tolerance(tmp_path, m, mode):
+    """The error of the pair sum is at most the tolerance that decides whether a node's
+    rounding is settled (derived beside the code; it grows with the number of frames m),
+    and the open nodes stay few: a node is open with probability 2 (m + 4) 2^-45 / 2^-24
+    times at most 4 (the result may be that much smaller than the terms' sum), 2% at
+    4000 frames."""
+    worst, n_open = _run(tmp_path, AVERAGE.replace("M,", f"{m},").replace("MODE,", f"{mode},"))
+    assert float(worst) <= 1.0
+    assert int(n_open) <= 0.05 * 3000
