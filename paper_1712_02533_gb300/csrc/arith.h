@@ -30,6 +30,22 @@ REG_HD float mul_rn(float a, float b)
     return a * b;
 #endif
 }
+REG_HD double add_rn(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    return __dadd_rn(a, b);
+#else
+    return a + b;
+#endif
+}
+REG_HD double mul_rn(double a, double b)
+{
+#ifdef __CUDA_ARCH__
+    return __dmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
 
 // a + b = s + e exactly.
 REG_HD void two_sum(float a, float b, float &s, float &e)
@@ -77,3 +93,28 @@ struct PairSum {
         pl = fmaf(t, fl, fmaf(te, fh, fmaf(t, fh, -ph)));
     }
 };
+
+// 1 / sqrt(v) as an unevaluated pair r + lo from a float value r0 of it (rsqrtf: within
+// 2 ulp), v within float's range: one third-order step (Halley's iteration for v^-1/2),
+// whose residual 1 - v r0^2 carries the rounding of v r0.  r is the pair rounded; what
+// the step leaves is below 2^-63.
+struct RootInv {
+    double r, lo;
+};
+REG_HD RootInv rsqrt_step(double v, float r0)
+{
+    const double r = (double)r0, t = mul_rn(v, r), tl = fma(v, r, -t);
+    const double e = fma(-tl, r, fma(-t, r, 1.0)), re = r * e, c = fma(e, 0.375, 0.5);
+    RootInv q;
+    q.r = fma(re, c, r);
+    q.lo = fma(re, c, r - q.r);
+    return q;
+}
+
+// s / sqrt(v), and sqrt(v) for s = v, rounded once (a square root and a division round
+// twice: up to 2 2^-53 off).
+REG_HD double times(double s, const RootInv &q)
+{
+    const double p = mul_rn(s, q.r);
+    return add_rn(p, fma(s, q.lo, fma(s, q.r, -p)));
+}

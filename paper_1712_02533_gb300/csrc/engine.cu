@@ -1776,7 +1776,8 @@ reg_status reg_eval_energy(reg_series_t s, int32_t series, int32_t frame_i, int3
         parts[1] = st.cur_ev.ncc;
         parts[2] = st.E + st.cur_ev.ncc;
         parts[3] = st.cur_ev.S1;
-        parts[4] = st.cur_ev.sig;
+        const double var = st.cur_ev.S2 - st.cur_ev.S1 * st.cur_ev.S1;
+        parts[4] = var > 0.0 ? std::sqrt(var) : 0.0;
     }
     return REG_OK;
 }

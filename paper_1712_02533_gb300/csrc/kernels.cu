@@ -1948,29 +1948,20 @@ __global__ void __launch_bounds__(REG_STRIP_THREADS, TRIAL_BLOCKS) k_trial(Batch
 // ---------------------------------------------------------------------------
 namespace {
 
-// 1 / sqrt(v), v within float's range: the single-precision value (2^-22) and one
-// third-order step (Halley's iteration for v^-1/2), to 1-2 ulp.  The double-precision
-// instructions behind sqrt and the division take 600 cycles each here, these four
-// dependent multiply-adds 250.
-__device__ __forceinline__ double rsqrt_step(double v)
-{
-    const double r = (double)rsqrtf((float)v);
-    const double t = v * r, e = fma(-t, r, 1.0);
-    return fma(r * e, fma(e, 0.375, 0.5), r);
-}
-
 // (The rare paths are calls: the code of a step's common path runs once per launch, and
 // its length in instruction fetches counts.)
 __device__ __noinline__ void eval_rare(EvalAt &v, double var)
 {
-    v.sig = var > 0.0 ? sqrt(var) : 0.0;
-    v.ncc = v.S3 / v.sig;
-    v.isig = (float)(1.0 / v.sig);
-    v.c36 = (float)(v.ncc / (v.sig * v.sig) / 36.0);
-    v.cT = (float)(v.ncc / (v.sig * v.sig) * v.S1);
+    const double sig = var > 0.0 ? sqrt(var) : 0.0;
+    v.ncc = v.S3 / sig;
+    v.isig = (float)(1.0 / sig);
+    v.c36 = (float)(v.ncc / (sig * sig) / 36.0);
+    v.cT = (float)(v.ncc / (sig * sig) * v.S1);
 }
 
-// sigma, NCC and the gradient pass's coefficients from the FE sums.
+// NCC and the gradient pass's coefficients from the FE sums.  The square root and
+// division of double precision take 600 cycles each here, the chain of rsqrt_step and
+// times nine dependent operations of 62.
 __device__ __forceinline__ void eval_at(EvalAt &v, double S1, double S2, double S3)
 {
     const double var = S2 - S1 * S1;
@@ -1978,11 +1969,10 @@ __device__ __forceinline__ void eval_at(EvalAt &v, double S1, double S2, double 
     v.S2 = S2;
     v.S3 = S3;
     if (var > 1e-30 && var < 1e30) {
-        const double r = rsqrt_step(var);
-        v.sig = var * r;
-        v.ncc = S3 * r;
-        v.isig = (float)r;
-        const double q = v.ncc * (r * r);
+        const RootInv r = rsqrt_step(var, rsqrtf((float)var));
+        v.ncc = times(S3, r);
+        v.isig = (float)r.r;
+        const double q = v.ncc * (r.r * r.r);
         v.c36 = (float)(q * (1.0 / 36.0));
         v.cT = (float)(q * S1);
     } else {  // (almost) no variance, or not finite

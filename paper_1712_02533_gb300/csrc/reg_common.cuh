@@ -112,11 +112,11 @@ struct __align__(16) StepDesc {
 };
 
 // An evaluated energy: the FE sums S1 = int That, S2 = int That^2, S3 = int That
-// R~ (R~ normalised: mean 0, FE sigma 1; S1 is That's mean), sigma = sqrt(S2 - S1^2),
-// NCC = S3 / sigma, the gradient pass's coefficients there, and of a trial the energy
+// R~ (R~ normalised: mean 0, FE sigma 1; S1 is That's mean), NCC = S3 / sigma with
+// sigma = sqrt(S2 - S1^2), the gradient pass's coefficients there, and of a trial the energy
 // change, the Armijo test and the stopping test.
 struct EvalAt {
-    double S1, S2, S3, ncc, sig, dE;
+    double S1, S2, S3, ncc, dE;
     float isig, c36, cT;
     int acc, conv, pad;
 };
