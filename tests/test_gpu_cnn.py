@@ -25,6 +25,80 @@ def reg():
     return r
 
 
+def _single_taps(rng):
+    """Parameters whose first and last layers have one weight per 32-channel index (a
+    random value at a random tap) and whose 32 -> 32 layers are the identity: every
+    activation and every gradient down to the second layer is then one FP32 product."""
+    w0, w5 = np.zeros((32, 2, 3, 3), np.float32), np.zeros((2, 32, 3, 3), np.float32)
+    tap0, tap5 = rng.integers(0, 3, (32, 2)), rng.integers(0, 3, (32, 2))
+    v0, v5 = (rng.uniform(0.5, 1.5, 32).astype(np.float32) for _ in range(2))
+    eye = np.zeros((32, 32, 3, 3), np.float32)
+    for c in range(32):
+        w0[c, c % 2, tap0[c, 0], tap0[c, 1]] = v0[c]
+        w5[c % 2, c, tap5[c, 0], tap5[c, 1]] = v5[c]
+        eye[c, c, 1, 1] = 1
+    mid = np.concatenate([eye.ravel(), np.zeros(32, np.float32)])
+    theta = np.concatenate([w0.ravel(), np.zeros(32, np.float32)] + [mid] * 4 + [w5.ravel(), np.zeros(2, np.float32)])
+    return theta, (v0, tap0), (v5, tap5)
+
+
+def _strided_sums(g, v):
+    """sum_p g[p, o] v[p, c] in FP32 as 256 strided chains and a tree over them."""
+    n = -(-g.shape[0] // 256) * 256
+    g, v = (np.pad(a, ((0, n - a.shape[0]), (0, 0))).reshape(-1, 256, a.shape[1]).astype(np.float64) for a in (g, v))
+    acc = np.zeros((256, g.shape[2], v.shape[2]), np.float32)
+    for k in range(g.shape[0]):
+        acc = (g[k][:, :, None] * v[k][:, None, :] + acc).astype(np.float32)
+    acc = acc.reshape(8, 32, *acc.shape[1:])
+    while acc.shape[1] > 1:
+        h = acc.shape[1] // 2
+        acc = acc[:, :h] + acc[:, h:]
+    tot = np.zeros(acc.shape[2:], np.float32)
+    for w in range(8):
+        tot = tot + acc[w, 0]
+    return tot
+
+
+@pytest.mark.parametrize("batch", [1, 2])
+def test_weight_sums_are_as_accurate_as_strided_sums_and_a_tree(reg, batch):
+    """The FP32 weight gradients of the 32 -> 32 layers (strides 1 and 2) from exactly
+    known operands: their root-mean-square error against FP64 is no larger than that of
+    256 strided FP32 sums added by a tree over the same products."""
+    import torch
+    from oracle import cnn as ocnn
+    rng = np.random.default_rng(batch)
+    theta, (v0, tap0), (v5, tap5) = _single_taps(rng)
+    x = rng.uniform(0.5, 2.0, (batch, 2, 256, 256)).astype(np.float32)
+    t = (2e4 * rng.standard_normal((batch, 2, 64, 64))).astype(np.float32)
+    with reg.Cnn(theta, side=256, max_batch=batch) as net:
+        xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+        y = net.forward(xd).cpu().numpy()
+        _, grad = net.loss_grad(xd, td, want_grad=True)
+    xp = np.pad(x, ((0, 0), (0, 0), (1, 1), (1, 1)))
+    a0 = np.stack([v0[c] * xp[:, c % 2, tap0[c, 0]:tap0[c, 0] + 255:2, tap0[c, 1]:tap0[c, 1] + 255:2] for c in range(32)], 1)
+    a1 = a0[:, :, ::2, ::2]
+    gy = np.float32(2) / np.float32(y.size) * (y - t)
+    gp = np.pad(gy, ((0, 0), (0, 0), (1, 1), (1, 1)))
+    gz = np.stack([v5[c] * gp[:, c % 2, 2 - tap5[c, 0]:66 - tap5[c, 0], 2 - tap5[c, 1]:66 - tap5[c, 1]] for c in range(32)], 1)
+    gz = np.where(a1 > 0, gz, np.float32(0))
+    assert a0.dtype == gz.dtype == np.float32
+    got = ocnn.unpack(grad)
+    g = gz.transpose(0, 2, 3, 1).reshape(-1, 32)
+    for layer, a, st in ((1, a0, 2), (2, a1, 1), (4, a1, 1)):
+        ap = np.pad(a, ((0, 0), (0, 0), (1, 1), (1, 1)))
+        err, ref = [], []
+        for dy in range(3):
+            for dx in range(3):
+                v = ap[:, :, dy:dy + st * 63 + 1:st, dx:dx + st * 63 + 1:st].transpose(0, 2, 3, 1).reshape(-1, 32)
+                want = g.astype(np.float64).T @ v.astype(np.float64)
+                scale = np.sqrt((g.astype(np.float64) ** 2).T @ (v.astype(np.float64) ** 2))
+                err.append((got[layer][0][:, :, dy, dx] - want) / scale)
+                ref.append((_strided_sums(g, v) - want) / scale)
+        e, r = (float(np.sqrt(np.mean(np.square(q)))) for q in (err, ref))
+        print(f"layer {layer}: {e:.3e} of {r:.3e}")
+        assert e <= r, (layer, e, r)
+
+
 def test_forward_loss_and_gradients_match_the_oracle(reg):
     import torch
     import synth
