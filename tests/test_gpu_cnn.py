@@ -99,6 +99,87 @@ def test_weight_sums_are_as_accurate_as_strided_sums_and_a_tree(reg, batch):
         assert e <= r, (layer, e, r)
 
 
+def _spread_second_layer(theta):
+    """Ones at four taps of the second layer's diagonal instead of one: its data gradient
+    is then still one product, at every pixel of the first layer's output."""
+    from oracle import cnn as ocnn
+    layers = ocnn.unpack(theta)
+    for c in range(32):
+        layers[1][0][c, c, 1:, 1:] = 1
+    return np.concatenate([np.concatenate([w.ravel(), b]) for w, b in layers]).astype(np.float32)
+
+
+def _known_gradient(y, t, v5, tap5, mask, bf16=False):
+    """The gradient with respect to the last layer's input, masked by its sign."""
+    import torch
+    q = y.shape[2]
+    gy = np.float32(2) / np.float32(y.size) * (y - t)
+    gp = np.pad(gy, ((0, 0), (0, 0), (1, 1), (1, 1)))
+    gz = np.stack([v5[c] * gp[:, c % 2, 2 - tap5[c, 0]:q + 2 - tap5[c, 0], 2 - tap5[c, 1]:q + 2 - tap5[c, 1]]
+                   for c in range(32)], 1)
+    if bf16:
+        gz = torch.from_numpy(gz).bfloat16().float().numpy()
+    return gy, np.where(mask > 0, gz, np.float32(0))
+
+
+def _rms(sums, g, v):
+    want = g.astype(np.float64).T @ v.astype(np.float64)
+    scale = np.sqrt((g.astype(np.float64) ** 2).T @ (v.astype(np.float64) ** 2))
+    return np.mean(np.square((sums - want) / scale))
+
+
+def test_first_layer_weight_sums_of_many_pairs(reg):
+    """The first layer's weight gradient of 32 pairs in the tensor-core pass (its operands
+    are FP32 and exactly known here): no larger a root-mean-square error against FP64 than
+    32 chains per block over a quarter of a warp's pixels each, four pixels of a 2 x 64
+    tile at a time."""
+    import torch
+    from oracle import cnn as ocnn
+    B = 32
+    rng = np.random.default_rng(5)
+    theta, _, (v5, tap5) = _single_taps(rng)
+    theta = _spread_second_layer(theta)
+    theta[32 * 18:32 * 19] = 20  # biases: the first layer's output is positive everywhere
+    x = rng.standard_normal((B, 2, 256, 256)).astype(np.float32)
+    t = (2e4 * rng.standard_normal((B, 2, 64, 64))).astype(np.float32)
+    with reg.Cnn(theta, side=256, max_batch=B) as net:
+        xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+        y = net.forward(xd, tensor_cores=True).cpu().numpy()
+        _, grad = net.loss_grad(xd, td, want_grad=True, tensor_cores=True)
+    got = ocnn.unpack(grad)[0][0]
+    xp = np.pad(x, ((0, 0), (0, 0), (1, 1), (1, 1)))
+    _, gz = _known_gradient(y, t, v5, tap5, np.ones((B, 32, 64, 64)), bf16=True)
+    gz = gz.repeat(2, axis=2).repeat(2, axis=3)
+    blocks = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+
+    def tiles(a):  # (B, C, 128, 128) -> (rounds, blocks, 4, 32, C), pixel 32 k + chain of a tile
+        a = a.transpose(0, 2, 3, 1).reshape(B, 64, 2, 2, 64, -1).transpose(0, 1, 3, 2, 4, 5).reshape(-1, 4, 32, a.shape[1])
+        n = -(-a.shape[0] // blocks) * blocks
+        return np.pad(a, ((0, n - a.shape[0]),) + ((0, 0),) * 3).reshape(-1, blocks, 4, 32, a.shape[3])
+
+    err, ref = [], []
+    gt, g = tiles(gz), gz.transpose(0, 2, 3, 1).reshape(-1, 32)
+    for dy in range(3):
+        for dx in range(3):
+            vv = xp[:, :, dy:dy + 255:2, dx:dx + 255:2]
+            v, vt = vv.transpose(0, 2, 3, 1).reshape(-1, 2), tiles(vv)
+            acc = np.zeros((blocks, 32, 32, 2), np.float32)
+            for r in range(gt.shape[0]):
+                for k in range(4):
+                    acc = (gt[r, :, k][..., None].astype(np.float64) * vt[r, :, k][:, :, None] + acc).astype(np.float32)
+            acc = acc.reshape(blocks, 8, 4, 32, 2)
+            acc = (acc[:, :, 0] + acc[:, :, 1]) + (acc[:, :, 2] + acc[:, :, 3])
+            tot = np.zeros((blocks, 32, 2), np.float32)
+            for w in range(8):
+                tot = tot + acc[:, w]
+            tot = tot.astype(np.float64).sum(0).astype(np.float32)  # the blocks' sums exactly added
+            err.append(_rms(got[:, :, dy, dx], g, v))
+            ref.append(_rms(tot, g, v))
+    e, r = np.sqrt(np.mean(err)), np.sqrt(np.mean(ref))
+    print(f"first layer: {e:.3e} of {r:.3e}")
+    assert e <= r
+
+
 def test_forward_loss_and_gradients_match_the_oracle(reg):
     import torch
     import synth
