@@ -180,6 +180,41 @@ def test_first_layer_weight_sums_of_many_pairs(reg):
     assert e <= r
 
 
+def test_last_layer_weight_sums_of_many_pairs(reg):
+    """The last layer's FP32 weight gradient of 128 pairs: no larger a root-mean-square
+    error than 16 parts of the pixels in turn, each as 256 strided sums and a tree."""
+    import torch
+    from oracle import cnn as ocnn
+    B = 128
+    rng = np.random.default_rng(6)
+    theta, (v0, tap0), (v5, tap5) = _single_taps(rng)
+    x = rng.uniform(0.5, 2.0, (B, 2, 256, 256)).astype(np.float32)
+    t = (2e4 * rng.standard_normal((B, 2, 64, 64))).astype(np.float32)
+    with reg.Cnn(theta, side=256, max_batch=B) as net:
+        xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+        y = net.forward(xd).cpu().numpy()
+        _, grad = net.loss_grad(xd, td, want_grad=True)
+    got = ocnn.unpack(grad)[5][0]
+    xp = np.pad(x, ((0, 0), (0, 0), (1, 1), (1, 1)))
+    a1 = np.stack([v0[c] * xp[:, c % 2, tap0[c, 0]:tap0[c, 0] + 253:4, tap0[c, 1]:tap0[c, 1] + 253:4] for c in range(32)], 1)
+    gy, _ = _known_gradient(y, t, v5, tap5, a1)
+    g = gy.transpose(0, 2, 3, 1).reshape(-1, 2)
+    ap = np.pad(a1, ((0, 0), (0, 0), (1, 1), (1, 1)))
+    part = g.shape[0] // 16
+    err, ref = [], []
+    for dy in range(3):
+        for dx in range(3):
+            v = ap[:, :, dy:dy + 64, dx:dx + 64].transpose(0, 2, 3, 1).reshape(-1, 32)
+            tot = np.zeros((2, 32), np.float32)
+            for k in range(16):
+                tot = tot + _strided_sums(g[k * part:(k + 1) * part], v[k * part:(k + 1) * part])
+            err.append(_rms(got[:, :, dy, dx], g, v))
+            ref.append(_rms(tot, g, v))
+    e, r = np.sqrt(np.mean(err)), np.sqrt(np.mean(ref))
+    print(f"last layer: {e:.3e} of {r:.3e}")
+    assert e <= r
+
+
 def test_forward_loss_and_gradients_match_the_oracle(reg):
     import torch
     import synth
