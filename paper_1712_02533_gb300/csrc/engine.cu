@@ -311,6 +311,9 @@ BatchDev make_batch(reg_series *s)
     return b;
 }
 
+// Rows of a trial tile where `rows` are asked for: its nodes lie in shared memory.
+int trial_rows_used(int rows) { return std::min(rows, REG_TRIAL_ROWS); }
+
 // Work items per operator at a level of n nodes per side: the larger of the
 // gradient and trial strip tiles.
 int grad_tiles(const reg_series *s, int n) { return cdiv(n, REG_GW) * cdiv(n, s->tile_hg[level_of(n)]); }
@@ -319,7 +322,7 @@ int max_tiles(const reg_series *s, int n)
 {
     const int l = level_of(n);
     int g = grad_tiles(s, n);
-    int t = cdiv(n - 1, REG_CW) * cdiv(n - 1, std::min(s->tile_ht[l], REG_TRIAL_ROWS));
+    int t = cdiv(n - 1, REG_CW) * cdiv(n - 1, trial_rows_used(s->tile_ht[l]));
     return std::max(g, t);
 }
 
@@ -336,7 +339,7 @@ void fill_level(const reg_series *s, LevelDesc &L, int n, int pitch)
     L.n = n;
     L.pitch = pitch;
     L.hg = s->tile_hg[level_of(n)];
-    L.ht = std::min(s->tile_ht[level_of(n)], REG_TRIAL_ROWS);
+    L.ht = trial_rows_used(s->tile_ht[level_of(n)]);
     L.tg = cdiv(n, REG_GW) * cdiv(n, L.hg);
     L.tt = cdiv(n - 1, REG_CW) * cdiv(n - 1, L.ht);
     const double h = 1.0 / (n - 1);
@@ -2097,7 +2100,9 @@ reg_status reg_autotune(reg_series_t s, int32_t series, int32_t n_pairs, int32_t
             double best = ps;
             int keep = keep0;
             for (int c : cand) {
+                // (trial rows that come to the same tiles as those in place are not timed)
                 if (c == keep0 || c > si.n[k]) continue;
+                if (which && (c > REG_TRIAL_ROWS || c == trial_rows_used(keep0))) continue;
                 tab[l] = c;
                 RET(measure(ps, tot));
                 if (ps < 0.98 * best) { best = ps; keep = c; }

@@ -102,3 +102,19 @@ def test_autotune_picks_valid_tiles_and_keeps_results(reg, syn):
         s.prefix_scan(reg.SKLANSKY)
         got = s.get_deformations()
     assert np.abs(got - base).max() <= 0.05
+
+
+@pytest.mark.parametrize("trial_rows", [16, 32, 64])
+def test_autotune_times_only_tiles_that_differ(reg, syn, trial_rows):
+    """A trial tile has at most 32 rows, so 64 is no candidate beside 32, and 32 none
+    where 64 was asked for: the runs are one for the times before and after, per level
+    of at least 129 nodes the tiles in place and the other rows (three for the gradient
+    pass; for the trial pass two of 8, 16, 32), and the step sizes."""
+    fr = syn.series(12, 3, 256, spacing=12.0, sigma=2.0, peak=10.0, noise=False)
+    with reg.Series(fr, reg.default_params(n_levels=3, iter_max=4, lam=10.0)) as s:
+        for lvl in (7, 8):
+            s.set_tile_rows(lvl, 16, trial_rows)
+        rep = s.autotune(n_pairs=2, repeats=1)
+        for lv in rep["levels"][1:]:
+            assert lv["trial_rows"] in (8, 16, 32) + (() if trial_rows < 64 else (64,))
+    assert rep["runs"] == 1 + 2 * ((1 + 3) + (1 + 2)) + (1 + 3) + 1
