@@ -18,6 +18,7 @@
 #include "reg_common.cuh"
 #include "schedule.h"
 #include "cnn_internal.h"
+#include "tile_rows.h"
 
 // kernels (kernels.cu)
 __global__ void k_restrict_img(const float *, int64_t, int64_t, int, int, float *, int64_t, int);
@@ -316,12 +317,10 @@ int trial_rows_used(int rows) { return std::min(rows, REG_TRIAL_ROWS); }
 
 // Work items per operator at a level of n nodes per side: the larger of the
 // gradient and trial strip tiles.
-int grad_tiles(const reg_series *s, int n) { return cdiv(n, REG_GW) * cdiv(n, s->tile_hg[level_of(n)]); }
-
 int max_tiles(const reg_series *s, int n)
 {
     const int l = level_of(n);
-    int g = grad_tiles(s, n);
+    int g = grad_tiles(n, s->tile_hg[l], REG_GW);
     int t = cdiv(n - 1, REG_CW) * cdiv(n - 1, trial_rows_used(s->tile_ht[l]));
     return std::max(g, t);
 }
@@ -334,13 +333,24 @@ int max_tiles_series(const reg_series *s, const SeriesInfo &si, int k0 = 0)
     return m;
 }
 
+// The most gradient tiles that a step has for an operator of a series (from level index k0).
+int grad_tiles_series(const reg_series *s, const SeriesInfo &si, int k0 = 0)
+{
+    int n[REG_MAX_LEVELS], rows[REG_MAX_LEVELS], nl = 0;
+    for (int k = k0; k < si.nl; k++, nl++) {
+        n[nl] = si.n[k];
+        rows[nl] = s->tile_hg[level_of(si.n[k])];
+    }
+    return most_grad_tiles(n, rows, nl, REG_GW);
+}
+
 void fill_level(const reg_series *s, LevelDesc &L, int n, int pitch)
 {
     L.n = n;
     L.pitch = pitch;
     L.hg = s->tile_hg[level_of(n)];
     L.ht = trial_rows_used(s->tile_ht[level_of(n)]);
-    L.tg = cdiv(n, REG_GW) * cdiv(n, L.hg);
+    L.tg = grad_tiles(n, L.hg, REG_GW);
     L.tt = cdiv(n - 1, REG_CW) * cdiv(n - 1, L.ht);
     const double h = 1.0 / (n - 1);
     L.h2d = h * h;
@@ -488,13 +498,13 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
         ws += (si.ws_bytes + 255) / 256 * 256;
         part0[i] = (int)items;
         items += max_tiles_series(s, si, o.skip);
-        gtiles += grad_tiles(s, si.n[si.nl - 1]);
+        gtiles += grad_tiles_series(s, si, o.skip);
         nl = std::max(nl, si.nl);
         nLmax = std::max(nLmax, si.n[si.nl - 1]);
     }
     if (items > INT32_MAX) return fail(REG_EINVAL, "batch of %d ops has too many tiles", n);
     RET(ensure_capacity(s, n, ws, items));
-    // no step has more gradient tiles than one with every op on its finest level
+    // no step has more gradient tiles than one with every op on the level where it has most
     const bool narrow = gtiles <= (int64_t)GRAD_FEW_WAVES * s->grid_F;
     for (int i = 0; i < n; i++) {
         const OpReq &o = ops[i];

@@ -30,3 +30,18 @@ REG_HD GradRows grad_rows(int tile0, int h, int n, int part, int parts)
 
 // Whether the walk loads row r.
 REG_HD bool grad_loads(const GradRows &g, int r, int n) { return r >= g.first && r <= g.last && r >= 0 && r < n; }
+
+// Gradient tiles of an operator at a level of n rows and columns, and the most that any
+// of its nl levels has, tiles of `width` owned columns by rows[k] rows: with rows set
+// per level a coarser level can have more tiles than the finest.
+REG_HD int grad_tiles(int n, int rows, int width) { return ((n + width - 1) / width) * ((n + rows - 1) / rows); }
+
+REG_HD int most_grad_tiles(const int *n, const int *rows, int nl, int width)
+{
+    int m = 0;
+    for (int k = 0; k < nl; k++) {
+        const int t = grad_tiles(n[k], rows[k], width);
+        m = t > m ? t : m;
+    }
+    return m;
+}

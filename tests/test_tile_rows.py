@@ -64,3 +64,19 @@ def test_gradient_walks_stay_on_their_level(compile_host):
     a tile shared by four: no load off the level, every completed row with its
     neighbours at hand, every row completed by exactly one warp."""
     assert compile_host(WALK) == ["0", "0", "0"]
+
+
+def test_a_batch_is_judged_by_its_widest_level(compile_host):
+    """The most gradient tiles of an operator: on the finest level under the default
+    rows (33 and 65 rows of 8, 129 and 257 of 16, 513 of 32), on the next one where the
+    finest has 64 rows and that one 4."""
+    src = """
+#include <cstdio>
+#include "tile_rows.h"
+int main()
+{
+    const int n[5] = {33, 65, 129, 257, 513}, rows[5] = {8, 8, 16, 16, 32}, other[5] = {8, 8, 16, 4, 64};
+    printf("%d %d %d\\n", most_grad_tiles(n, rows, 5, 30), most_grad_tiles(n, other, 5, 30), most_grad_tiles(n + 4, other + 4, 1, 30));
+}
+"""
+    assert compile_host(src) == [str(18 * 17), str(9 * 65), str(18 * 9)]
