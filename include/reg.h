@@ -348,7 +348,8 @@ reg_status reg_cnn_init_series(reg_series_t s, int32_t series, reg_cnn_t h, int3
 reg_status reg_set_tile_rows(reg_series_t s, int32_t level, int32_t grad_rows, int32_t trial_rows);
 reg_status reg_get_tile_rows(reg_series_t s, int32_t level, int32_t *grad_rows, int32_t *trial_rows);
 /* Tile autotuner: times a sample batch of function A on the neighbour pairs
- * 0..n_pairs-1 of `series` (best of `repeats` runs) and picks, level by level
+ * 0..n_pairs-1 of `series` (best of `repeats` runs; the gradient pass in the form
+ * that a batch of all the series' pairs takes) and picks, level by level
  * from the finest (levels of at least 129 nodes), the gradient and trial tile
  * rows with the shortest time per device step, then the step sizes per trial
  * pass (2, 3, 4 or 8) with the shortest batch time; a change must gain 2%.  The
@@ -356,7 +357,8 @@ reg_status reg_get_tile_rows(reg_series_t s, int32_t level, int32_t *grad_rows, 
  * trials_per_pass as the handle uses it).  It overwrites the data slots
  * 0..n_pairs-1 (and drops a pending learned start): call it before
  * reg_prefix_scan, reg_set_slot or reg_cnn_init_series.  report (may be NULL):
- * a JSON object with the chosen table and the sample's time before and after. */
+ * a JSON object with the chosen table, whether that form is the one of narrow
+ * batches, and the sample's time before and after. */
 reg_status reg_autotune(reg_series_t s, int32_t series, int32_t n_pairs, int32_t repeats, char *report,
                         size_t buf_len);
 

@@ -175,6 +175,7 @@ struct reg_series {
     int h_st_cap = 0;
     // graph of GRAPH_STEPS steps
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // wide batches, narrow ones
+    int grad_form = -1;  // while tiles are tuned: 0 wide, 1 narrow, whatever the batch; else -1
     int graph_gen[2] = {-1, -1}, buf_gen = 0;
     // profiling
     cudaEvent_t ev[GRAPH_STEPS][NFAM];
@@ -410,6 +411,8 @@ reg_status ensure_capacity(reg_series *s, int n_ops, size_t ws_total, int64_t it
 // tile per block as the limit, 13.8 with two, 13.1 with four).
 constexpr int GRAD_FEW_WAVES = 4;
 
+bool is_narrow(const reg_series *s, int64_t grad_tiles) { return grad_tiles <= (int64_t)GRAD_FEW_WAVES * s->grid_F; }
+
 void launch_gradient(reg_series *s, bool narrow, cudaStream_t st, const BatchDev &b)
 {
     launch_grad(s->bf16, narrow, narrow ? s->grid_F : s->grid_G, st, b);
@@ -505,7 +508,7 @@ reg_status run_batch(reg_series *s, const std::vector<OpReq> &ops, F pre_iter, i
     if (items > INT32_MAX) return fail(REG_EINVAL, "batch of %d ops has too many tiles", n);
     RET(ensure_capacity(s, n, ws, items));
     // no step has more gradient tiles than one with every op on the level where it has most
-    const bool narrow = gtiles <= (int64_t)GRAD_FEW_WAVES * s->grid_F;
+    const bool narrow = s->grad_form >= 0 ? s->grad_form : is_narrow(s, gtiles);
     for (int i = 0; i < n; i++) {
         const OpReq &o = ops[i];
         const SeriesInfo &si = s->S[o.series];
@@ -2095,6 +2098,15 @@ reg_status reg_autotune(reg_series_t s, int32_t series, int32_t n_pairs, int32_t
         }
         return REG_OK;
     };
+    // The sample runs the form of the gradient pass that a batch of all the series' pairs
+    // runs, for every candidate: the two forms prefer different rows, and rows that take
+    // a small sample from one form to the other would be timed by that.
+    struct Form {
+        reg_series *s;
+        ~Form() { s->grad_form = -1; }
+    } form{s};
+    s->grad_form = is_narrow(s, (int64_t)si.n_data * grad_tiles_series(s, si));
+    const int narrow = s->grad_form;
     double ps, tot, ps0, tot0;
     RET(run_batch(s, ops, [] { return REG_OK; }, nullptr, nullptr));  // warm-up: buffers, graph
     RET(measure(ps0, tot0));
@@ -2154,9 +2166,9 @@ reg_status reg_autotune(reg_series_t s, int32_t series, int32_t n_pairs, int32_t
         }
         char b[256];
         snprintf(b, sizeof b,
-                 "], \"trials_per_pass\": %d, \"sample_ops\": %d, \"runs\": %d, \"ms_before\": %.3f, "
+                 "], \"trials_per_pass\": %d, \"sample_ops\": %d, \"narrow\": %s, \"runs\": %d, \"ms_before\": %.3f, "
                  "\"ms_after\": %.3f}",
-                 s->p.trials_per_pass, n_pairs, runs, tot0, tot1);
+                 s->p.trials_per_pass, n_pairs, narrow ? "true" : "false", runs, tot0, tot1);
         js += b;
         snprintf(report, buf_len, "%s", js.c_str());
     }

@@ -118,3 +118,17 @@ def test_autotune_times_only_tiles_that_differ(reg, syn, trial_rows):
         for lv in rep["levels"][1:]:
             assert lv["trial_rows"] in (8, 16, 32) + (() if trial_rows < 64 else (64,))
     assert rep["runs"] == 1 + 2 * ((1 + 3) + (1 + 2)) + (1 + 3) + 1
+
+
+@pytest.mark.parametrize("frames,narrow", [(3, True), (80, False)])
+def test_autotune_samples_the_form_of_the_whole_series(reg, syn, frames, narrow):
+    """A sample of two pairs is timed with the form of the gradient pass that a batch of
+    all the series' pairs takes: 79 pairs of 5 x 33 tiles are wide (more than four tiles
+    for each of 152 x 21 blocks), two narrow.  Batches after it run as ever."""
+    fr = np.tile(syn.series(12, 3, 128, spacing=12.0, sigma=2.0, peak=10.0), (frames // 3 + 1, 1, 1))[:frames]
+    with reg.Series(fr, reg.default_params(n_levels=2, iter_max=3, lam=10.0)) as s:
+        s.set_tile_rows(7, 4, 16)  # 5 x 33 tiles per pair
+        rep = s.autotune(n_pairs=2, repeats=1)
+        assert rep["narrow"] is narrow
+        st, it = s.apply_operator_batch([(0, -1, -1, 0, 0, 1)])
+        assert it[0] > 0
