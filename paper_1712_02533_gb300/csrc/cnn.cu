@@ -48,127 +48,93 @@ int64_t total_params() { return param_offset(NL); }
 
 
 // ---------------------------------------------------------------------------
-// Forward: one thread per output pixel (b, y, x) computes all O channels.
+// Last layer (32 -> 2, stride 1, no ReLU), forward: one thread per output pixel
+// (b, y, x) computes both channels.
 // ---------------------------------------------------------------------------
-template <int C, int O, int S, bool RELU>
-__global__ void __launch_bounds__(128) k_conv_fwd(const float *__restrict__ in, int H, const float *__restrict__ theta,
-                                                  float *__restrict__ out, int Ho, int total)
+__global__ void __launch_bounds__(128) k_conv_last(const float *__restrict__ in, int H, const float *__restrict__ theta,
+                                                   float *__restrict__ out, int total)
 {
-    // weights as [c][tap][o], so that one vector load brings the weights of
-    // several output channels for an input value
-    __shared__ __align__(16) float w[O * C * 9];
-    __shared__ float bias[O];
-    for (int i = threadIdx.x; i < O * C * 9; i += blockDim.x) {
-        const int o = i / (C * 9), ck = i - o * (C * 9);
-        w[ck * O + o] = theta[i];
-    }
-    for (int i = threadIdx.x; i < O; i += blockDim.x) bias[i] = theta[O * C * 9 + i];
+    __shared__ float2 w[32 * 9];  // [c][tap], both output channels
+    for (int i = threadIdx.x; i < 32 * 9; i += blockDim.x) w[i] = make_float2(theta[i], theta[32 * 9 + i]);
+    const float b0 = theta[2 * 32 * 9], b1 = theta[2 * 32 * 9 + 1];
     __syncthreads();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= total) return;
-    const int x = p % Ho, y = (p / Ho) % Ho, b = p / (Ho * Ho);
-    float acc[O];
-#pragma unroll
-    for (int o = 0; o < O; o++) acc[o] = bias[o];
-    for (int c = 0; c < C; c++) {
-        const float *src = in + ((int64_t)b * C + c) * H * H;
+    const int x = p % H, y = (p / H) % H, b = p / (H * H);
+    float acc0 = b0, acc1 = b1;
+    for (int c = 0; c < 32; c++) {
+        const float *src = in + ((int64_t)b * 32 + c) * H * H;
         float v[9];
 #pragma unroll
         for (int dy = 0; dy < 3; dy++)
 #pragma unroll
             for (int dx = 0; dx < 3; dx++) {
-                const int iy = S * y + dy - 1, ix = S * x + dx - 1;
+                const int iy = y + dy - 1, ix = x + dx - 1;
                 v[dy * 3 + dx] = (iy >= 0 && iy < H && ix >= 0 && ix < H) ? src[iy * H + ix] : 0.f;
             }
         // per output channel the products are added in the order (c, tap)
 #pragma unroll
         for (int k = 0; k < 9; k++) {
-            const float *wk = w + (c * 9 + k) * O;
-            if constexpr (O % 4 == 0) {
-#pragma unroll
-                for (int q = 0; q < O / 4; q++) {
-                    const float4 wv = reinterpret_cast<const float4 *>(wk)[q];
-                    acc[4 * q] = fmaf(wv.x, v[k], acc[4 * q]);
-                    acc[4 * q + 1] = fmaf(wv.y, v[k], acc[4 * q + 1]);
-                    acc[4 * q + 2] = fmaf(wv.z, v[k], acc[4 * q + 2]);
-                    acc[4 * q + 3] = fmaf(wv.w, v[k], acc[4 * q + 3]);
-                }
-            } else if constexpr (O == 2) {
-                const float2 wv = *reinterpret_cast<const float2 *>(wk);
-                acc[0] = fmaf(wv.x, v[k], acc[0]);
-                acc[1] = fmaf(wv.y, v[k], acc[1]);
-            } else {
-#pragma unroll
-                for (int o = 0; o < O; o++) acc[o] = fmaf(wk[o], v[k], acc[o]);
-            }
+            const float2 wv = w[c * 9 + k];
+            acc0 = fmaf(wv.x, v[k], acc0);
+            acc1 = fmaf(wv.y, v[k], acc1);
         }
     }
-#pragma unroll
-    for (int o = 0; o < O; o++)
-        if (RELU) acc[o] = fmaxf(acc[o], 0.f);
-#pragma unroll
-    for (int o = 0; o < O; o++) out[(((int64_t)b * O + o) * Ho + y) * Ho + x] = acc[o];
+    out[(((int64_t)b * 2) * H + y) * H + x] = acc0;
+    out[(((int64_t)b * 2 + 1) * H + y) * H + x] = acc1;
 }
 
 // ---------------------------------------------------------------------------
-// Backward, data: gx[b, c, iy, ix] = sum over (o, dy, dx) with S oy + dy - 1 = iy
-// and S ox + dx - 1 = ix of W[o, c, dy, dx] gz[b, o, oy, ox], times the ReLU
-// mask of the layer below (its output a > 0).  One thread per input pixel.
+// Last layer, data gradient: gx[b, c, iy, ix] = sum over (o, dy, dx) of W[o, c, dy, dx]
+// gz[b, o, iy + 1 - dy, ix + 1 - dx], times the ReLU mask of the layer below (its
+// output a > 0).  One thread per pixel, all 32 channels.
+// MASK_PLANAR: a_below is BF16 in the planar layout of the tensor-core layers instead of
+// FP32 NCHW.
 // ---------------------------------------------------------------------------
-// MASK_PLANAR: a_below is BF16 in the planar layout of the tensor-core layers
-// (C = 32) instead of FP32 NCHW.
-template <int C, int O, int S, bool MASK_PLANAR = false>
-__global__ void __launch_bounds__(128) k_conv_bwd_data(const float *__restrict__ gz, int Ho,
-                                                       const float *__restrict__ theta,
+template <bool MASK_PLANAR>
+__global__ void __launch_bounds__(128) k_bwd_data_last(const float *__restrict__ gz, const float *__restrict__ theta,
                                                        const void *__restrict__ a_below, float *__restrict__ gx,
                                                        int H, int total)
 {
     // weights as [o][tap][c], so that one vector load brings the weights of
     // several input channels for an output gradient value
-    __shared__ __align__(16) float w[O * C * 9];
-    for (int i = threadIdx.x; i < O * C * 9; i += blockDim.x) {
-        const int o = i / (C * 9), r = i - o * (C * 9), c = r / 9, k = r - c * 9;
-        w[(o * 9 + k) * C + c] = theta[i];
+    __shared__ __align__(16) float w[2 * 9 * 32];
+    for (int i = threadIdx.x; i < 2 * 9 * 32; i += blockDim.x) {
+        const int o = i / (32 * 9), r = i - o * (32 * 9), c = r / 9, k = r - c * 9;
+        w[(o * 9 + k) * 32 + c] = theta[i];
     }
     __syncthreads();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= total) return;
     const int ix = p % H, iy = (p / H) % H, b = p / (H * H);
-    float acc[C];
+    float acc[32];
 #pragma unroll
-    for (int c = 0; c < C; c++) acc[c] = 0.f;
+    for (int c = 0; c < 32; c++) acc[c] = 0.f;
 #pragma unroll
     for (int dy = 0; dy < 3; dy++) {
-        const int ty = iy + 1 - dy;
-        if (ty < 0 || ty % S != 0 || ty / S >= Ho) continue;
-        const int oy = ty / S;
+        const int oy = iy + 1 - dy;
+        if (oy < 0 || oy >= H) continue;
 #pragma unroll
         for (int dx = 0; dx < 3; dx++) {
-            const int tx = ix + 1 - dx;
-            if (tx < 0 || tx % S != 0 || tx / S >= Ho) continue;
-            const int ox = tx / S;
-            for (int o = 0; o < O; o++) {
-                const float g = gz[(((int64_t)b * O + o) * Ho + oy) * Ho + ox];
-                const float *wk = w + (o * 9 + dy * 3 + dx) * C;
-                if constexpr (C % 4 == 0) {
+            const int ox = ix + 1 - dx;
+            if (ox < 0 || ox >= H) continue;
+            for (int o = 0; o < 2; o++) {
+                const float g = gz[(((int64_t)b * 2 + o) * H + oy) * H + ox];
+                const float4 *wk = reinterpret_cast<const float4 *>(w + (o * 9 + dy * 3 + dx) * 32);
 #pragma unroll
-                    for (int q = 0; q < C / 4; q++) {
-                        const float4 wv = reinterpret_cast<const float4 *>(wk)[q];
-                        acc[4 * q] = fmaf(wv.x, g, acc[4 * q]);
-                        acc[4 * q + 1] = fmaf(wv.y, g, acc[4 * q + 1]);
-                        acc[4 * q + 2] = fmaf(wv.z, g, acc[4 * q + 2]);
-                        acc[4 * q + 3] = fmaf(wv.w, g, acc[4 * q + 3]);
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < C; c++) acc[c] = fmaf(wk[c], g, acc[c]);
+                for (int q = 0; q < 8; q++) {
+                    const float4 wv = wk[q];
+                    acc[4 * q] = fmaf(wv.x, g, acc[4 * q]);
+                    acc[4 * q + 1] = fmaf(wv.y, g, acc[4 * q + 1]);
+                    acc[4 * q + 2] = fmaf(wv.z, g, acc[4 * q + 2]);
+                    acc[4 * q + 3] = fmaf(wv.w, g, acc[4 * q + 3]);
                 }
             }
         }
     }
 #pragma unroll
-    for (int c = 0; c < C; c++) {
-        const int64_t i = (((int64_t)b * C + c) * H + iy) * H + ix;
+    for (int c = 0; c < 32; c++) {
+        const int64_t i = (((int64_t)b * 32 + c) * H + iy) * H + ix;
         bool pos;
         if (MASK_PLANAR) {
             const uint16_t v = reinterpret_cast<const uint16_t *>(
@@ -211,7 +177,7 @@ __device__ __forceinline__ void fma_group(float2 (&acc)[PX][OC / 2], const float
 }
 
 // Forward, 32 outputs with ReLU: out[b][o][y][x], rows y = 4 yg .. 4 yg + 3.  grid
-// (column-and-row-group blocks, channel halves).  Sum order (c, tap), as k_conv_fwd.
+// (column-and-row-group blocks, channel halves).  Sum order (c, tap), as k_conv_last.
 template <int C, int S>
 __global__ void __launch_bounds__(128, 4) k_conv_fwd32(const float *__restrict__ in, int H,
                                                        const float *__restrict__ theta, float *__restrict__ out,
@@ -270,7 +236,7 @@ __global__ void __launch_bounds__(128, 4) k_conv_fwd32(const float *__restrict__
 // FP32 output > 0).  Stride 2: an input pixel takes the taps dy with iy + 1 - dy
 // even, likewise along x, so the pixels of one parity class (blockIdx.z = 2 py +
 // px) share their taps; a thread's rows and the lanes' columns are two apart.  Sum
-// order (dy, dx, o), as k_conv_bwd_data.
+// order (dy, dx, o), as k_bwd_data_last.
 template <int S>
 __global__ void __launch_bounds__(128, 4) k_conv_bwd_data32(const float *__restrict__ gz, int Ho,
                                                             const float *__restrict__ theta,
@@ -849,7 +815,7 @@ void fwd(int k, const float *in, int H, const float *theta, float *out, int B, c
     const int Ho = (H + 2 - 3) / LAYERS[k].S + 1;
     if (k == NL - 1) {
         const int total = B * Ho * Ho;
-        k_conv_fwd<32, 2, 1, false><<<(total + 127) / 128, 128, 0, st>>>(in, H, theta, out, Ho, total);
+        k_conv_last<<<(total + 127) / 128, 128, 0, st>>>(in, H, theta, out, total);
         return;
     }
     const int nyg = (Ho + PX - 1) / PX, total = B * nyg * Ho;
@@ -876,7 +842,7 @@ void bwd(int k, const float *in, int H, const float *gz, const float *theta, flo
         const int grid = wgrad_small_grid(tiles(WL_TR, WL_TW)), total = B * H * H;
         k_wgrad_last<false><<<grid, 256, 0, st>>>(in, H, gz, B, part);
         sums.add(part, grid, WL_REC, grad, false);
-        k_conv_bwd_data<32, 2, 1><<<(total + 127) / 128, 128, 0, st>>>(gz, Ho, theta, in, gx, H, total);
+        k_bwd_data_last<false><<<(total + 127) / 128, 128, 0, st>>>(gz, theta, in, gx, H, total);
         return;
     }
     const int S = LAYERS[k].S, nx = H / S, nyg = (nx + PX - 1) / PX, total = B * nyg * nx;
@@ -984,7 +950,7 @@ reg_status cnn_forward(reg_cnn *h, const float *x, int B, float *y, cudaStream_t
             else if (k == NL - 1)
                 rs = cnn_last_umma(h->actb[k - 1], H, th, out, B, st, h->wpack_last, h->uerr);
             else
-                rs = cnn_conv32_umma(h->actb[k - 1], H, th, h->actb[k], false, B, LAYERS[k].S, st,
+                rs = cnn_conv32_umma(h->actb[k - 1], H, th, h->actb[k], B, LAYERS[k].S, st,
                                      h->wpack_u + (k - 1) * cnn_conv32_umma_words(), h->uerr);
             if (rs != REG_OK) return rs;
         } else {
@@ -1128,8 +1094,8 @@ static reg_status loss_grad(reg_cnn_t h, const float *x, const float *target, in
             rs = cnn_wgrad32_umma(inb, H, gz, B, LAYERS[k].S, gr, part, sums, st, h->uerr);
             if (rs != REG_OK) return rs;
             const uint32_t *wp = h->wpack_d + (k - 1) * cnn_conv32_umma_words();
-            if (LAYERS[k].S == 1) rs = cnn_dgrad32_umma(gz, H, th, inb, gx, B, st, wp, h->uerr);
-            else rs = cnn_dgrad32s2_umma(gz, H / 2, th, inb, gx, B, st, wp, h->uerr);
+            if (LAYERS[k].S == 1) rs = cnn_dgrad32_umma(gz, H, inb, gx, B, st, wp, h->uerr);
+            else rs = cnn_dgrad32s2_umma(gz, H / 2, inb, gx, B, st, wp, h->uerr);
             if (rs != REG_OK) return rs;
             gz = gx;
             continue;
@@ -1141,7 +1107,7 @@ static reg_status loss_grad(reg_cnn_t h, const float *x, const float *target, in
             k_wgrad_last<true><<<grid, 256, 0, st>>>(h->actb[k - 1], H, gz, B, part);
             sums.add(part, grid, WL_REC, gr, false);
             const int total = B * H * H;
-            k_conv_bwd_data<32, 2, 1, true><<<(total + 127) / 128, 128, 0, st>>>(gz, H, th, h->actb[k - 1], gx, H, total);
+            k_bwd_data_last<true><<<(total + 127) / 128, 128, 0, st>>>(gz, th, h->actb[k - 1], gx, H, total);
             gz = gx;
             continue;
         }

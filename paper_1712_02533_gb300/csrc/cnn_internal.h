@@ -47,25 +47,25 @@ int cnn_wgrad32_umma_part_floats();
 // 32 -> 32 channel 3x3 convolution (zero padding 1, stride S = 1 or 2) with
 // bias and ReLU on the fifth-generation tensor cores (tcgen05.mma, accumulator
 // in TMEM, BF16 operands, FP32 accumulation): in (planar, B x 32 x H x H, read
-// by TMA; H even for S = 2), out (B x 32 x Ho x Ho) planar, or FP32 NCHW with
-// out_f32; theta: the layer's W then b; wpack: its packed weights
-// (cnn_pack_umma; cnn_conv32_umma_words() words, 16-byte aligned);
+// by TMA; H even for S = 2), out (B x 32 x Ho x Ho) planar; theta: the layer's W
+// then b; wpack: its packed weights (cnn_pack_umma; cnn_conv32_umma_words() words,
+// 16-byte aligned);
 // err: a device word set to nonzero when a wait of the kernel ran out (the
 // result is then invalid).
-reg_status cnn_conv32_umma(const uint16_t *in, int H, const float *theta, void *out, bool out_f32, int B, int S,
-                           cudaStream_t st, const uint32_t *wpack, int *err);
+reg_status cnn_conv32_umma(const uint16_t *in, int H, const float *theta, uint16_t *out, int B, int S, cudaStream_t st,
+                           const uint32_t *wpack, int *err);
 // Data gradient of a stride-1 32 -> 32 layer on the tensor cores: gx (FP32
 // NCHW, B x 32 x H x H) = (mask > 0) * conv(gz, W flipped and transposed), gz
 // (FP32 NCHW) the gradient with respect to the layer's pre-activation output,
 // mask the activation below (planar).
-reg_status cnn_dgrad32_umma(const float *gz, int H, const float *theta, const uint16_t *mask, float *gx, int B,
+reg_status cnn_dgrad32_umma(const float *gz, int H, const uint16_t *mask, float *gx, int B,
                             cudaStream_t st, const uint32_t *wpack, int *err);
 // Data gradient of a stride-2 32 -> 32 layer on the tensor cores: gz (FP32
 // NCHW, B x 32 x Hg x Hg) the gradient with respect to the layer's
 // pre-activation output, gx (FP32 NCHW, B x 32 x 2Hg x 2Hg) = (mask > 0) *
 // the transposed convolution, mask the activation below (planar, side 2 Hg);
 // wpack as cnn_dgrad32_umma's (the same packing).
-reg_status cnn_dgrad32s2_umma(const float *gz, int Hg, const float *theta, const uint16_t *mask, float *gx, int B,
+reg_status cnn_dgrad32s2_umma(const float *gz, int Hg, const uint16_t *mask, float *gx, int B,
                               cudaStream_t st, const uint32_t *wpack, int *err);
 int cnn_conv32_umma_words();
 // The last layer (32 -> 2, stride 1, no ReLU) on the same kernel with N = 16

@@ -1200,15 +1200,11 @@ reg_status cnn_pack_umma(const float *const theta[6], uint32_t *first, uint32_t 
 
 int cnn_conv32_umma_words() { return Wts<UC>::bytes / 4; }
 
-reg_status cnn_conv32_umma(const uint16_t *in, int H, const float *theta, void *out, bool out_f32, int B, int S,
-                           cudaStream_t st, const uint32_t *wpack, int *err)
+reg_status cnn_conv32_umma(const uint16_t *in, int H, const float *theta, uint16_t *out, int B, int S, cudaStream_t st,
+                           const uint32_t *wpack, int *err)
 {
-    if (S == 1)
-        return out_f32 ? launch_fwd<1, UC, UC, true, true>(in, H, theta, out, B, st, wpack, err)
-                       : launch_fwd<1, UC, UC, true, false>(in, H, theta, out, B, st, wpack, err);
-    if (S == 2)
-        return out_f32 ? launch_fwd<2, UC, UC, true, true>(in, H, theta, out, B, st, wpack, err)
-                       : launch_fwd<2, UC, UC, true, false>(in, H, theta, out, B, st, wpack, err);
+    if (S == 1) return launch_fwd<1, UC, UC, true, false>(in, H, theta, out, B, st, wpack, err);
+    if (S == 2) return launch_fwd<2, UC, UC, true, false>(in, H, theta, out, B, st, wpack, err);
     return reg_internal_fail(REG_EINVAL, "tcgen05 convolution: stride must be 1 or 2");
 }
 
@@ -1233,7 +1229,7 @@ reg_status cnn_first_umma(const float *x, int H, const float *theta, uint16_t *o
     return REG_OK;
 }
 
-reg_status cnn_dgrad32_umma(const float *gz, int H, const float *theta, const uint16_t *mask, float *gx, int B,
+reg_status cnn_dgrad32_umma(const float *gz, int H, const uint16_t *mask, float *gx, int B,
                             cudaStream_t st, const uint32_t *wpack, int *err)
 {
     const int tx = (H + UTW - 1) / UTW, ty = (H + UTH - 1) / UTH, nt = B * tx * ty;
@@ -1247,7 +1243,7 @@ reg_status cnn_dgrad32_umma(const float *gz, int H, const float *theta, const ui
     return REG_OK;
 }
 
-reg_status cnn_dgrad32s2_umma(const float *gz, int Hg, const float *theta, const uint16_t *mask, float *gx, int B,
+reg_status cnn_dgrad32s2_umma(const float *gz, int Hg, const uint16_t *mask, float *gx, int B,
                               cudaStream_t st, const uint32_t *wpack, int *err)
 {
     const int tx = (Hg + UTW - 1) / UTW, ty = (Hg + UTH - 1) / UTH, nt = B * tx * ty;

@@ -1435,7 +1435,6 @@ __device__ __forceinline__ bool patch_delta(const Patch &P, int n, float ex, flo
 // Shared memory of one block of the trial pass (one tile).
 constexpr int TRIAL_WARPS = REG_STRIP_THREADS / 32;
 constexpr int TRIAL_BLOCKS = 7;   // resident blocks per SM
-constexpr int TRIAL_RB = 1;       // node rows a warp has in flight
 constexpr int TWR = REG_TRIAL_ROWS;  // most cell rows of a tile
 template <int JM>
 struct TrialTile {
@@ -1632,9 +1631,8 @@ __device__ __forceinline__ RowQueues row_queues(const TrialTile<JM> &sh, int nr,
 // gathered once for all step sizes.  A node whose largest move leaves the cell, and
 // every cell touching one, is summed exactly for each step size.  Phases, the tile's
 // nodes in shared memory between them:
-//   1. every warp walks some rows, TRIAL_RB at a time without a branch, their texel
-//      loads and the next rows' records in flight together: A, B, and which
-//      nodes take the exact path;
+//   1. every warp walks some rows without a branch, a row's texel loads and the next
+//      row's records in flight together: A, B, and which nodes take the exact path;
 //   2. lists of those nodes and of the cells that touch one;
 //   3. exact changes, one node per thread; beside them the moments, one kind per
 //      warp, each down the rows;
@@ -1673,63 +1671,42 @@ __device__ __forceinline__ void trial_tile(const BatchDev &b, const StepDesc &s,
             pdx = __shfl_down_sync(FULL, dPx, 1) - dPx;
             pdy = __shfl_down_sync(FULL, dPy, 1) - dPy;
         }
-        constexpr int RB = TRIAL_RB;
-        float4 nu[RB], nd[RB];
-#pragma unroll
-        for (int k = 0; k < RB; k++) {
-            const int o = 2 * (w0 + min(i0 + k, cells)) * pitch;
-            nu[k] = Vcol[o];
-            nd[k] = Vcol[o + 1];
-        }
-        for (int i = i0; i < i1; i += RB) {
-            float4 dmr[RB];  // d, 36 M~That, M~R~
-            Texel4 t[RB];
-            bool slw[RB];
-#pragma unroll
-            for (int k = 0; k < RB; k++) {
-                const int r = w0 + min(i + k, cells);
-                dmr[k] = nd[k];
-                int ix, iy;
-                df_split(nu[k].x, nu[k].z, ix, t[k].ax);
-                df_split(nu[k].y, nu[k].w, iy, t[k].ay);
-                const int jx = cc + ix, jy = r + iy;
-                // a base point outside the grid, or a largest move that leaves the
-                // cell (then every smaller one along the ray stays inside)
-                const float ax1 = t[k].ax + tmax * dmr[k].x, ay1 = t[k].ay + tmax * dmr[k].y;
-                slw[k] = (unsigned)jx > (unsigned)(n - 2) || (unsigned)jy > (unsigned)(n - 2) ||
-                         !(ax1 >= 0.f && ax1 < 1.f) || !(ay1 >= 0.f && ay1 < 1.f);
-                t[k].jx = min(max(jx, 0), n - 2);
-                t[k].jy = min(max(jy, 0), n - 2);
-                fetch<BF16>(t[k], T, pitch);
-            }
-#pragma unroll
-            for (int k = 0; k < RB; k++) {
-                const int o = 2 * (w0 + min(i + RB + k, cells)) * pitch;
-                nu[k] = Vcol[o];
-                nd[k] = Vcol[o + 1];
-            }
-#pragma unroll
-            for (int k = 0; k < RB; k++) {
-                if (k > 0 && i + k >= i1) break;  // warp-uniform
-                const Texel4 &q = t[k];
-                const float4 dm = dmr[k];
-                const float dtx = q.t01 - q.t00, dtx1 = q.t11 - q.t10;
-                const float sx = dtx + q.ay * (dtx1 - dtx);                            // dThat/dx
-                const float sy = (q.t10 - q.t00) + q.ax * ((q.t11 - q.t01) - (q.t10 - q.t00));  // dThat/dy
-                const float A = dm.x * sx + dm.y * sy;
-                const float B = dm.x * dm.y * (dtx1 - dtx);
-                const unsigned ms = __ballot_sync(FULL, slw[k] && g.colIn);
-                if (lane == 0) sh.slow[i + k] = ms;
-                sh.node[0][i + k][lane] = make_float4(A, B, dm.z, dm.w);
-                if (withQ) {
-                    // Dirichlet form of d over the cells between rows r-1 and r
-                    const float dRx = __shfl_down_sync(FULL, dm.x, 1), dRy = __shfl_down_sync(FULL, dm.y, 1);
-                    const float qx = dRx - dm.x, qy = dRy - dm.y;
-                    const float rx = dm.x - dPx, ry = dm.y - dPy;
-                    const float sx = __shfl_down_sync(FULL, rx, 1), sy = __shfl_down_sync(FULL, ry, 1);
-                    sh.qt[i + k][lane] = pform(pdx, qx) + pform(rx, sx) + pform(pdy, qy) + pform(ry, sy);
-                    pdx = qx; pdy = qy; dPx = dm.x; dPy = dm.y;
-                }
+        float4 nu = Vcol[2 * (w0 + min(i0, cells)) * pitch], nd = Vcol[2 * (w0 + min(i0, cells)) * pitch + 1];
+        for (int i = i0; i < i1; i++) {
+            const int r = w0 + i;
+            const float4 dm = nd;  // d, 36 M~That, M~R~
+            Texel4 q;
+            int ix, iy;
+            df_split(nu.x, nu.z, ix, q.ax);
+            df_split(nu.y, nu.w, iy, q.ay);
+            const int jx = cc + ix, jy = r + iy;
+            // a base point outside the grid, or a largest move that leaves the
+            // cell (then every smaller one along the ray stays inside)
+            const float ax1 = q.ax + tmax * dm.x, ay1 = q.ay + tmax * dm.y;
+            const bool slw = (unsigned)jx > (unsigned)(n - 2) || (unsigned)jy > (unsigned)(n - 2) ||
+                             !(ax1 >= 0.f && ax1 < 1.f) || !(ay1 >= 0.f && ay1 < 1.f);
+            q.jx = min(max(jx, 0), n - 2);
+            q.jy = min(max(jy, 0), n - 2);
+            fetch<BF16>(q, T, pitch);
+            const int o = 2 * (w0 + min(i + 1, cells)) * pitch;
+            nu = Vcol[o];
+            nd = Vcol[o + 1];
+            const float dtx = q.t01 - q.t00, dtx1 = q.t11 - q.t10;
+            const float sx = dtx + q.ay * (dtx1 - dtx);                            // dThat/dx
+            const float sy = (q.t10 - q.t00) + q.ax * ((q.t11 - q.t01) - (q.t10 - q.t00));  // dThat/dy
+            const float A = dm.x * sx + dm.y * sy;
+            const float B = dm.x * dm.y * (dtx1 - dtx);
+            const unsigned ms = __ballot_sync(FULL, slw && g.colIn);
+            if (lane == 0) sh.slow[i] = ms;
+            sh.node[0][i][lane] = make_float4(A, B, dm.z, dm.w);
+            if (withQ) {
+                // Dirichlet form of d over the cells between rows r-1 and r
+                const float dRx = __shfl_down_sync(FULL, dm.x, 1), dRy = __shfl_down_sync(FULL, dm.y, 1);
+                const float qx = dRx - dm.x, qy = dRy - dm.y;
+                const float rx = dm.x - dPx, ry = dm.y - dPy;
+                const float sx = __shfl_down_sync(FULL, rx, 1), sy = __shfl_down_sync(FULL, ry, 1);
+                sh.qt[i][lane] = pform(pdx, qx) + pform(rx, sx) + pform(pdy, qy) + pform(ry, sy);
+                pdx = qx; pdy = qy; dPx = dm.x; dPy = dm.y;
             }
         }
     }
