@@ -8,28 +8,26 @@
 #endif
 
 // Node rows of one warp in a gradient tile of h rows from row tile0 of a level of n
-// rows, the tile cut into `parts` runs of rows (1: one warp walks all of it).  The warp
-// owns [r0, rEnd); its walk visits first .. last, one halo row on either side of them,
-// and a visited row is loaded if it lies on the level.  Since n = 2^l + 1 and h divides
-// 2^l, the last row of tiles owns the single row n - 1: every other warp of such a tile
-// starts past the level, owns nothing and visits nothing (last < first).
+// rows, the tile cut into `parts` runs of rows.  The warp owns r0 .. rLast; its walk
+// visits r0 - 1 .. rLast + 1, one halo row on either side, and loads those of them that
+// lie on the level: the first one before the walk (grad_loads_first), row r + 1 while it
+// works on row r (r + 1 < n && r + 1 <= rLast + 1).  Since n = 2^l + 1 and h divides 2^l,
+// the last row of tiles owns the single row n - 1: every other warp of a tile there starts
+// past the level, owns nothing and visits nothing (r0 - 1 > rLast + 1).
 struct GradRows {
-    int r0, rEnd, first, last;
+    int r0, rLast;
 };
 
 REG_HD GradRows grad_rows(int tile0, int h, int n, int part, int parts)
 {
-    const int len = h / parts;
     GradRows g;
-    g.r0 = tile0 + part * len;
-    g.rEnd = g.r0 + len < n ? g.r0 + len : n;
-    g.first = g.r0 - 1;
-    g.last = g.r0 < n ? g.rEnd : g.first - 1;
+    g.r0 = tile0 + part * (h / parts);
+    g.rLast = g.r0 + h / parts - 1 < n - 1 ? g.r0 + h / parts - 1 : n - 1;
+    if (g.r0 >= n) g.r0 = n + 2;
     return g;
 }
 
-// Whether the walk loads row r.
-REG_HD bool grad_loads(const GradRows &g, int r, int n) { return r >= g.first && r <= g.last && r >= 0 && r < n; }
+REG_HD bool grad_loads_first(int r0, int n) { return r0 - 1 >= 0 && r0 - 1 < n; }
 
 // Gradient tiles of an operator at a level of n rows and columns, and the most that any
 // of its nl levels has, tiles of `width` owned columns by rows[k] rows: with rows set

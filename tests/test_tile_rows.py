@@ -29,9 +29,9 @@ int main()
                             if (r < 0 || r >= n) off++;
                             else got[r] = 1;
                         };
-                        if (grad_loads(g, g.first, n)) load(g.first);
-                        for (int r = g.first; r <= g.last; r++) {
-                            if (grad_loads(g, r + 1, n)) load(r + 1);
+                        if (grad_loads_first(g.r0, n)) load(g.r0 - 1);
+                        for (int r = g.r0 - 1; r <= g.rLast + 1; r++) {
+                            if (r + 1 < n && r + 1 <= g.rLast + 1) load(r + 1);
                             const int m = r - 1;  // completed by row r
                             if (m < g.r0) continue;
                             if (m >= n) { owners++; continue; }
