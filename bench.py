@@ -146,7 +146,7 @@ def roofline_of(stats, cfg, bf16=False):
 def cnn_roofline(reg, s, torch, batch=64, reps=20):
     """Tensor-core roofline of the learned initialiser's forward pass: the 64
     network inputs of the series' first neighbour pairs through the 6-layer
-    CNN (the four 32->32 layers on the BF16 tensor cores), timed with CUDA
+    CNN (all layers on the BF16 tensor cores), timed with CUDA
     events; FLOPs = 2 x multiply-adds of all six layers (0.326 GFLOP per pair)."""
     import synth
     peak = None
@@ -175,8 +175,8 @@ def cnn_roofline(reg, s, torch, batch=64, reps=20):
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1) / reps
     tflops = flop_pair * batch / (ms * 1e-3) / 1e12
-    return {"bound": "tensor", "kernel": "CNN forward (k_conv32_umma_fwd, tcgen05 + TMA, on the four 32->32 layers, BF16 operands, FP32 "
-                                        "accumulation; the 2->32 and 32->2 layers on the CUDA cores)",
+    return {"bound": "tensor", "kernel": "CNN forward (k_conv_umma_ws, tcgen05 + TMA, layers 2 to 6; k_conv_umma_staged, tcgen05, the "
+                                        "first layer; BF16 operands, FP32 accumulation)",
             "achieved": round(tflops, 2), "peak": peak, "unit": "TFLOP/s", "frac": round(tflops / peak, 5),
             "peak_source": src, "batch": batch, "ms_per_forward": round(ms, 4),
             "gflop_per_pair": round(flop_pair / 1e9, 4), "traffic": None}

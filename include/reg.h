@@ -343,8 +343,8 @@ reg_status reg_cnn_init_series(reg_series_t s, int32_t series, reg_cnn_t h, int3
  * chosen per pyramid level l (2^l + 1 nodes per side); defaults 8 (l <= 6),
  * 16 (l <= 8), 32.  Rows must be 4, 8, 16, 32 or 64 (REG_EINVAL otherwise); the
  * trial pass uses at most 32 of them.
- * The rows change which FP32 partial sums are formed before the FP64 sum over
- * tiles, so results can differ at the rounding level. */
+ * The rows change which FP32 partial sums are formed before the sum over tiles
+ * (float triples, rounded to FP64), so results can differ at the rounding level. */
 reg_status reg_set_tile_rows(reg_series_t s, int32_t level, int32_t grad_rows, int32_t trial_rows);
 reg_status reg_get_tile_rows(reg_series_t s, int32_t level, int32_t *grad_rows, int32_t *trial_rows);
 /* Tile autotuner: times a sample batch of function A on the neighbour pairs

@@ -737,9 +737,8 @@ int wgrad_small_grid(int n_tiles)
     return std::max(1, std::min(n_tiles, 2 * nsm));
 }
 
-// Floats of a layer's partial records (the tensor-core kernel writes one record per
-// SM, the others up to two), and of all layers: the records stay until one launch
-// adds them all.
+// Floats of a layer's partial records (one per block, at most two blocks per SM), and
+// of all layers: the records stay until one launch adds them all.
 size_t wpart_floats(int k)
 {
     const size_t rec = k == 0 ? WF_REC : k == NL - 1 ? WL_REC : WG32_REC, n = wgrad_small_grid(1 << 30) * rec;

@@ -11,8 +11,9 @@
 //
 // Energies are sums over cells of the Q1 element integrals (exact FE mass and
 // stiffness forms); per-cell values are float, per-warp and per-tile sums
-// float, and the per-operator sum over tiles is double (the global energy and
-// normalisation reductions that the Armijo test compares).
+// float (level-start sums: float triples), and the per-operator sum over tiles
+// runs in float triples, exact to 2^-72, and goes on in double (the energies that
+// the Armijo test compares).
 #include <algorithm>
 
 #include "reg_common.cuh"
@@ -919,8 +920,9 @@ constexpr int SM_BATCH = 8;     // elements of a sweep held in registers at a ti
 constexpr int SM_RING = 32;     // rows of the column sweeps' ring, filled SM_GROUP at a time
 constexpr int SM_GROUP = 8;
 
-// Rows per block of the row pass: what fits 131 KB of shared memory at a side of
-// n nodes, at most 16 (one warp sweeps 16 rows x 2 components).
+// Rows per block of the row pass: 16 (one warp sweeps 16 rows x 2 components) up to
+// 1025 nodes per side, where they and the pivots take 139 KB of shared memory; fewer
+// beyond, 164 KB at 4097.
 __host__ __device__ __forceinline__ int smooth_row_chunk(int n) { return n <= 1025 ? 16 : (n <= 2049 ? 8 : 4); }
 
 __device__ __forceinline__ void copy_async8(void *dst, const void *src)
@@ -1645,7 +1647,9 @@ __device__ __forceinline__ RowQueues row_queues(const TrialTile<JM> &sh, int nr,
 // One warp per tile doing all of this row by row held 128 registers (16 warps on an
 // SM) and waited for the record -> template gather of every row: per launch of a 33 x
 // 1024^2 scan 122 -> 104 us, of a 21 x 512^2 one 37 -> 23, of a single 1024^2 operator
-// 24 -> 15, of 7 operators of 64^2 12.6 -> 8.  Seven blocks per SM at one row in flight
+// 24 -> 15, of 7 operators of 64^2 12.6 -> 8.  It pays where tiles are few: with the 200
+// operators of a 400 x 1024^2 scan's batches a launch is bound by its instructions and
+// takes what it took (0.96 ms, 0.95 before, the prolongation now among it).  Seven blocks per SM at one row in flight
 // (72 registers) beat six (80) at one or two rows, 104 against 112 and 109 us.
 template <bool BF16, int JM>
 __device__ __forceinline__ void trial_tile(const BatchDev &b, const StepDesc &s, const StripGeom &g, TrialTile<JM> &sh,

@@ -15,7 +15,8 @@
 #define REG_GW 30  // gradient tile: owned node columns (lanes 1..30; lanes 0, 31 are halo)
 #define REG_CW 31  // trial tile: owned cell columns (lanes 0..30; lane 31 is the right corner)
 #define REG_TRIAL_ROWS 32  // most cell rows of a trial tile (its nodes lie in shared memory)
-#define REG_STRIP_THREADS 128  // threads per block of the strip kernels (warps work independently)
+#define REG_STRIP_THREADS 128  // threads per block of the strip kernels (a tile per block, or per warp in the
+                               // gradient pass of many tiles)
 // Rows per strip tile at a level of n nodes per side (owned node rows of a
 // gradient tile, owned cell rows of a trial tile): short strips on the coarse
 // levels, where a tile's row walk is latency bound, long ones on the fine
