@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(128, 4) k_conv_bwd_data32(const float *__restr
 // weight of one pair of 256^2 was 1.6 times that of 256 strided sums and a tree, in
 // runs it is 0.83 times that.  With a block per (o, c) pair, which
 // read input and gradient 32 times over from L2, a layer took 1155 us (32 pairs);
-// now 66 us and 4 us for the records' sum.
+// now 69 us (66 in one chain) and 4 us for the records' sum.
 // Blocks take tiles block, block + grid, ..; each writes one record.
 constexpr int WG32_RUN = 16;
 template <int S>
@@ -481,7 +481,8 @@ constexpr int WF_REC = 32 * 2 * 9 + 32;                       // weights (o, c, 
 // registers, the window) run under this tile's sums.
 // It reads each byte once (84 MB at 32 x 256^2, 12.4 us at the copy rate).  With
 // threads over (4 output channels, pixel), the channels' 19 scalar reads a pixel
-// and the copies waited for before each tile's sums it took 51.3 us; now 27.5 us.
+// and the copies waited for before each tile's sums it took 51.3 us; now 28.9 us (27.6
+// without the totals).
 __global__ void __launch_bounds__(256, 2) k_wgrad_first(const float *__restrict__ x, int H,
                                                      const float *__restrict__ gz, int Ho, int B,
                                                      float *__restrict__ part)
